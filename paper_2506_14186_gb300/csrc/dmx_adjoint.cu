@@ -256,7 +256,7 @@ __global__ void k_body_invweight_tangent(const DevModel* mp, const double* qpos0
   crba(g, m, w);
   Dual* H = w.at(sL.H); const Dual* M = w.at(sL.M);
   for (int i = 0; i < m.nv * m.nv; ++i) H[i] = M[i];
-  cholesky(g, H, w.at(sL.tmp2), m.nv);
+  cholesky(g, H, w.at(sL.tmp2), m.nv, m.nv);
   const Dual* S = w.at(sL.sd); const Dual* C = w.at(sL.com);
   for (int b = 0; b < m.nbody; ++b) {
     Dual tr = 0.0;

@@ -19,10 +19,16 @@
 //                           quaternions integrated exactly
 //   Fig. 12                 Tsitouras 5(4) and fixed-step semi-implicit Euler
 //
-// GB300 notes: FP64 runs at 1/62 of the FP32 rate and a warp instruction costs
-// the same whatever its active lanes, so work is split across the group where
-// it parallelises and divisions are avoided (reciprocals, division-free
-// breakpoint comparisons).  The Newton search starts from the active set of
+// GB300 notes: an FP64 warp instruction takes 64 cycles of its SM
+// sub-partition whatever its active lanes (a division 565, a reciprocal square
+// root 350, a shared-memory read about 30, a model read through the L1 about
+// 40), so the cost of a phase is the number of FP64 instructions on its
+// longest path plus its dependent reads.  Work is therefore split into equal
+// tasks of one matrix or vector component (branches inside a task cost the sum
+// of their sides), tree recursions run along chains without meeting the other
+// lanes, and indices come packed or from tables.  Every split keeps the
+// operations of each result and their order, so that results do not depend on
+// the lane count.  The Newton search starts from the active set of
 // the previous right-hand side of the same environment (the minimiser is
 // unique, so the start only changes the number of iterations).
 #pragma once
@@ -76,19 +82,28 @@ struct Grp {
 };
 
 // (row, column) of the t-th entry of a lower triangle enumerated row by row
-// ((0,0), (1,0), (1,1), (2,0), ...): the same for every matrix size.
+// ((0,0), (1,0), (1,1), (2,0), ...): the same for every matrix size.  In
+// global memory (read through the L1): the lanes of a group read different
+// entries, which the constant cache would serve one after the other.
+constexpr int NTRI = (MAXV + 1) * (MAXV + 2) / 2;
 struct TriTab {
-  unsigned char e[MAXV * (MAXV + 1) / 2][2];
+  unsigned short e[NTRI];            // row << 8 | column
 };
-__host__ __device__ constexpr TriTab make_tri() {
+constexpr TriTab make_tri() {
   TriTab t{};
   int k = 0;
-  for (int i = 0; i < MAXV; ++i)
-    for (int j = 0; j <= i; ++j) { t.e[k][0] = (unsigned char)i; t.e[k][1] = (unsigned char)j; ++k; }
+  for (int i = 0; i <= MAXV; ++i)
+    for (int j = 0; j <= i; ++j) t.e[k++] = (unsigned short)(i << 8 | j);
   return t;
 }
-static __constant__ TriTab c_tri_tab = make_tri();
-#define c_tri c_tri_tab.e
+static __device__ const TriTab d_tri = make_tri();
+struct Tri {
+  int i, j;
+};
+__device__ __forceinline__ Tri tri(int t) {
+  const int p = __ldg(&d_tri.e[t]);
+  return {p >> 8, p & 255};
+}
 
 // ------------------------------------------------------------------ small helpers
 // Templated on the scalar types so that the same code runs on doubles (the
@@ -273,21 +288,21 @@ struct Par<Dual> {
 using Ws = WsT<double>;
 
 // Entry e (row-major) of the rotation of the quaternion x (w, x, y, z) with
-// s = 2 / |x|^2 (the normalisation folded into the products).
+// s = 2 / |x|^2 (the normalisation folded into the products).  Every entry is
+// s u1 u3 +- s u2 u4 (one minus it on the diagonal) with components picked by
+// e, so that the nine lanes of a body run one instruction sequence: a switch
+// over e costs the sum of its nine sides.
+__device__ __forceinline__ double mul_add(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ Dual mul_add(const Dual& a, const Dual& b, const Dual& c) { return a * b + c; }
 template <class T>
 __device__ __forceinline__ T quat_entry(const T* x, const T& s, int e) {
-  const T w = x[0], a = x[1], b = x[2], c = x[3];
-  switch (e) {
-    case 0: return 1.0 - (s * b * b + s * c * c);
-    case 1: return s * a * b - s * w * c;
-    case 2: return s * a * c + s * w * b;
-    case 3: return s * a * b + s * w * c;
-    case 4: return 1.0 - (s * a * a + s * c * c);
-    case 5: return s * b * c - s * w * a;
-    case 6: return s * a * c - s * w * b;
-    case 7: return s * b * c + s * w * a;
-    default: return 1.0 - (s * a * a + s * b * b);
-  }
+  // per entry 8 bits: u1, u3, u2, u4 (2 bits each, lowest first; 0 = w)
+  const unsigned k = e < 8 ? (unsigned)(0x4E8D4EF5C98DC9FAull >> (8 * e)) & 255u : 0xA5u;
+  const T t1 = s * x[k & 3], t2 = s * x[(k >> 4) & 3];
+  T p = t2 * x[(k >> 6) & 3];
+  if ((0x062u >> e) & 1u) p = -p;                      // entries 1, 5, 6
+  const T v = mul_add(t1, x[(k >> 2) & 3], p);
+  return ((0x111u >> e) & 1u) ? 1.0 - v : v;           // entries 0, 4, 8
 }
 // Entry (i, j) of the hinge rotation about the unit axis a by the angle with
 // sine sn and cosine cs (Rodrigues: I + sin K + (1 - cos) K^2, K = [a]x).
@@ -301,6 +316,55 @@ __device__ __forceinline__ T hinge_entry(const double* a, const T& sn, const T& 
   return pos ? v - sn * a[k] : v + sn * a[k];
 }
 
+// Sums along the body tree of one NC-component vector per body, in place, one
+// lane per (chain, component): tree_down adds each body's parent into it
+// (parents first), tree_up each body's children into it (children first, in
+// order).  A chain is one loop of dependent additions in a register; the
+// lanes meet once per chain level instead of once per body level.
+template <int NC, int G, class T>
+__device__ __forceinline__ void tree_down(const Grp<G>& g, const DevModel& m, T* X) {
+  if (m.nlevel == 1) return;
+  for (int cl = 0; cl < m.nchlev; ++cl) {
+    const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
+    for (int t = g.lane; t < n; t += G) {
+      const int c = c0 + t / NC, e = t % NC;
+      const int k0 = m.ch_start[c], k1 = m.ch_start[c + 1], par = m.ch_par[c];
+      const int b0 = m.ch_list[k0];
+      T x = X[NC * b0 + e];
+      if (par >= 0) { x += X[NC * par + e]; X[NC * b0 + e] = x; }
+      for (int k = k0 + 1; k < k1; ++k) {
+        T* p = X + NC * m.ch_list[k] + e;
+        x = *p + x;
+        *p = x;
+      }
+    }
+    g.sync();
+  }
+}
+template <int NC, int G, class T>
+__device__ __forceinline__ void tree_up(const Grp<G>& g, const DevModel& m, T* X) {
+  if (m.nlevel == 1) return;
+  for (int cl = m.nchlev - 1; cl >= 0; --cl) {
+    const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
+    for (int t = g.lane; t < n; t += G) {
+      const int c = c0 + t / NC, e = t % NC;
+      const int k0 = m.ch_start[c], k1 = m.ch_start[c + 1] - 1;
+      const int tail = m.ch_list[k1], nc = m.child_count[tail], cs = m.child_start[tail];
+      T x = X[NC * tail + e];
+      if (nc > 0) {
+        for (int j = 0; j < nc; ++j) x += X[NC * m.child_list[cs + j] + e];
+        X[NC * tail + e] = x;
+      }
+      for (int k = k1 - 1; k >= k0; --k) {
+        T* p = X + NC * m.ch_list[k] + e;
+        x = *p + x;
+        *p = x;
+      }
+    }
+    g.sync();
+  }
+}
+
 // Kinematics: body poses, COMs, dof motion vectors, body spatial inertias, geom poses.
 // Work is split into small tasks so that a group's lanes stay busy even for a
 // single body: per-body scalars (hinge sine and cosine, the free joint's
@@ -311,7 +375,7 @@ template <int G, class T>
 __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* q) {
   const Layout& L = *w.L;
   T* R = w.at(L.R); T* P = w.at(L.p); T* C = w.at(L.com);
-  T* S = w.at(L.sd); T* Ib = w.at(L.Ib);
+  T* S = w.at(L.sd); T* Ib = w.at(L.Ib); T* Ic = w.at(L.Ic);
   T* X = w.at(L.xl); T* SC = w.at(L.sc);
   const int nb = m.nbody;
   for (int b = g.lane; b < nb; b += G) {
@@ -351,120 +415,133 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
     else X[12 * b + e] = v;
   }
   g.sync();
-  // world poses: R = R_parent R_local, p = p_parent + R_parent p_local
+  // world poses: R = R_parent R_local, p = p_parent + R_parent p_local: entries
+  // 0..8 of R and 9..11 of p are the same product of a row of R_parent with a
+  // column of the local transform
   for (int lev = 1; lev < m.nlevel; ++lev) {
-    for (int t = 12 * m.level_start[lev] + g.lane; t < 12 * m.level_start[lev + 1]; t += G) {
+    const int k0 = m.level_start[lev], n = 12 * (m.level_start[lev + 1] - k0);
+    for (int t = g.lane; t < n; t += G) {
       const int k = t / 12, e = t - 12 * k;
-      const int b = m.level_list[k], par = m.b_parent[b];
-      const T* Rp = R + 9 * par; const T* xl = X + 12 * b;
-      if (e < 9) {
-        const int i = e / 3, j = e - 3 * (e / 3);
-        R[9 * b + e] = Rp[3 * i] * xl[j] + Rp[3 * i + 1] * xl[3 + j] + Rp[3 * i + 2] * xl[6 + j];
-      } else {
-        const int i = e - 9;
-        P[3 * b + i] = P[3 * par + i] + (Rp[3 * i] * xl[9] + Rp[3 * i + 1] * xl[10] + Rp[3 * i + 2] * xl[11]);
-      }
+      const int pk = m.lv_pack[k0 + k], b = pk & 255, par = pk >> 8;
+      const bool pos = e >= 9;
+      const int i = pos ? e - 9 : e / 3, j = pos ? 9 : e - 3 * (e / 3), st = pos ? 1 : 3;
+      const T* Rp = R + 9 * par + 3 * i; const T* xl = X + 12 * b + j;
+      T v = Rp[0] * xl[0] + Rp[1] * xl[st] + Rp[2] * xl[2 * st];
+      if (pos) v = P[3 * par + i] + v;
+      *(pos ? P + 3 * b + i : R + 9 * b + e) = v;
     }
     g.sync();
   }
-  // COMs (one component per task), geom poses (one entry per task), dof
-  // motion vectors (w; v at the world origin, one dof per task)
+  // COMs and geom poses, one component per task, all of them a row of R times
+  // a model vector (plus p): com, gpos, the columns of Roff
   T* gR = w.at(L.gR); T* gp = w.at(L.gp);
-  const int n1 = 3 * nb, n2 = n1 + 12 * m.ngeom, n3 = n2 + m.nv;
-  for (int t = g.lane; t < n3; t += G) {
+  const int n1 = 3 * nb, n2 = n1 + 12 * m.ngeom;
+  for (int t = g.lane; t < n2; t += G) {
+    int b, i, st = 1;
+    const double* c;
+    T* out;
+    bool rot = false, same = false;
     if (t < n1) {
-      const int b = t / 3, i = t - 3 * b;
-      const T* Rb = R + 9 * b; const double* c = m.b_com[b];
-      C[t] = (Rb[3 * i] * c[0] + Rb[3 * i + 1] * c[1] + Rb[3 * i + 2] * c[2]) + P[t];
-    } else if (t < n2) {
-      const int gi = (t - n1) / 12, e = t - n1 - 12 * gi;
-      const int b = m.g_body[gi];
-      const T* Rb = R + 9 * b;
-      if (e < 9) {
-        const int i = e / 3, j = e - 3 * (e / 3);
-        const double* Ro = m.g_Roff[gi];
-        gR[9 * gi + e] = m.g_ident[gi] ? Rb[e] : Rb[3 * i] * Ro[j] + Rb[3 * i + 1] * Ro[3 + j] + Rb[3 * i + 2] * Ro[6 + j];
-      } else {
-        const int i = e - 9;
-        const double* gpos = m.g_pos[gi];
-        gp[3 * gi + i] = m.g_zpos[gi] ? P[3 * b + i]
-                                      : P[3 * b + i] + (Rb[3 * i] * gpos[0] + Rb[3 * i + 1] * gpos[1] + Rb[3 * i + 2] * gpos[2]);
-      }
+      b = t / 3; i = t - 3 * b;
+      c = m.b_com[b]; out = C + t;
     } else {
-      const int i = t - n2;
-      const int b = m.dof_body[i];
-      const T* Rb = R + 9 * b; const T* pb = P + 3 * b;
-      T* st = S + 6 * i;
-      if (m.b_jtype[b] == JNT_FREE) {
-        const int d = i - m.b_vadr[b];
-        if (d < 3) {
-          st[0] = 0.0; st[1] = 0.0; st[2] = 0.0; st[3] = d == 0 ? 1.0 : 0.0; st[4] = d == 1 ? 1.0 : 0.0;
-          st[5] = d == 2 ? 1.0 : 0.0;
-        } else {
-          st[0] = Rb[d - 3]; st[1] = Rb[d]; st[2] = Rb[d + 3];
-          cross3(pb, st, st + 3);
-        }
+      const int gi = (t - n1) / 12, e = t - n1 - 12 * gi;
+      b = m.g_body[gi];
+      rot = e < 9;
+      i = rot ? e / 3 : e - 9;
+      const int j = e - 3 * i;
+      c = rot ? m.g_Roff[gi] + j : m.g_pos[gi];
+      if (rot) st = 3;
+      same = rot ? m.g_ident[gi] : m.g_zpos[gi];
+      out = rot ? gR + 9 * gi + e : gp + 3 * gi + i;
+      if (same) { *out = rot ? R[9 * b + e] : P[3 * b + i]; continue; }
+    }
+    const T* Rb = R + 9 * b + 3 * i;
+    T v = Rb[0] * c[0] + Rb[1] * c[st] + Rb[2] * c[2 * st];
+    if (!rot) v = v + P[3 * b + i];
+    *out = v;
+  }
+  // dof motion vectors (w; v at the world origin), one dof per task
+  for (int i = g.lane; i < m.nv; i += G) {
+    const int b = m.dof_body[i];
+    const T* Rb = R + 9 * b; const T* pb = P + 3 * b;
+    T* st = S + 6 * i;
+    if (m.b_jtype[b] == JNT_FREE) {
+      const int d = i - m.b_vadr[b];
+      if (d < 3) {
+        st[0] = 0.0; st[1] = 0.0; st[2] = 0.0; st[3] = d == 0 ? 1.0 : 0.0; st[4] = d == 1 ? 1.0 : 0.0;
+        st[5] = d == 2 ? 1.0 : 0.0;
       } else {
-        matvec3(Rb, m.b_axis[b], st);
+        st[0] = Rb[d - 3]; st[1] = Rb[d]; st[2] = Rb[d + 3];
         cross3(pb, st, st + 3);
       }
+    } else {
+      matvec3(Rb, m.b_axis[b], st);
+      cross3(pb, st, st + 3);
     }
   }
   g.sync();
   // spatial inertias about the world origin (m, m c, R diag(I) R^T + m (|c|^2 1 - c c^T)),
-  // one entry per task
-  for (int k = g.lane; k < 10 * nb; k += G) {
-    const int b = k / 10, e = k - 10 * b;
+  // one entry per task: the six moments of every body first (12 operations
+  // each), then mass and first moments, so that a pass of the lanes mostly
+  // meets one kind.  Ic starts as a copy (composite inertias, crba).
+  for (int k = g.lane; k < 6 * nb; k += G) {
+    const int b = k / 6, e = k - 6 * b;
     const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
     const T* c = C + 3 * b;
-    T v;
-    if (e == 0) v = ms;
-    else if (e < 4) v = ms * c[e - 1];
-    else {
-      const int ii[6] = {0, 1, 2, 0, 0, 1}, jj[6] = {0, 1, 2, 1, 2, 2};
-      const int i = ii[e - 4], j = jj[e - 4];
-      const T* Rb = R + 9 * b;
-      const double* In = m.b_inertia[b];
-      v = Rb[3 * i] * Rb[3 * j] * In[0] + Rb[3 * i + 1] * Rb[3 * j + 1] * In[1] + Rb[3 * i + 2] * Rb[3 * j + 2] * In[2];
-      if (Par<T>::mass_dir(m, w.pdir, b)) v = v * (ms / m.b_mass[b]);   // inertia proportional to the mass
-      if (Par<T>::side_dir(m, w.pdir, b)) {                             // ... and to the side squared
-        const int gs = m.b_solebox[b];
-        const double l0 = 2.0 * m.g_size[gs][0];
-        const auto lam = Par<T>::get(w.pdir, par_side(m, m.g_box[gs]), l0) / l0;
-        v = v * (lam * lam);
-      }
-      const T cc = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
-      v += ms * ((i == j ? cc : T(0.0)) - c[i] * c[j]);
+    const int i = e < 3 ? e : (e == 5 ? 1 : 0), j = e < 3 ? e : (e == 3 ? 1 : 2);   // xx yy zz xy xz yz
+    const T* Rb = R + 9 * b;
+    const double* In = m.b_inertia[b];
+    T v = Rb[3 * i] * Rb[3 * j] * In[0] + Rb[3 * i + 1] * Rb[3 * j + 1] * In[1] + Rb[3 * i + 2] * Rb[3 * j + 2] * In[2];
+    if (Par<T>::mass_dir(m, w.pdir, b)) v = v * (ms / m.b_mass[b]);   // inertia proportional to the mass
+    if (Par<T>::side_dir(m, w.pdir, b)) {                             // ... and to the side squared
+      const int gs = m.b_solebox[b];
+      const double l0 = 2.0 * m.g_size[gs][0];
+      const auto lam = Par<T>::get(w.pdir, par_side(m, m.g_box[gs]), l0) / l0;
+      v = v * (lam * lam);
     }
+    const T cc = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
+    v += ms * ((i == j ? cc : T(0.0)) - c[i] * c[j]);
+    Ib[10 * b + 4 + e] = v;
+    Ic[10 * b + 4 + e] = v;
+  }
+  for (int k = g.lane; k < 4 * nb; k += G) {
+    const int b = k / 4, e = k - 4 * b;
+    const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
+    T v;
+    if (e == 0) v = ms; else v = ms * C[3 * b + e - 1];
     Ib[10 * b + e] = v;
+    Ic[10 * b + e] = v;
   }
   g.sync();
+}
+
+// Task t of 6 n tasks (n vectors of 6 components), angular components of
+// every vector first: the two kinds of component have different formulas.
+struct Comp6 {
+  int i, e;
+};
+__device__ __forceinline__ Comp6 comp6(int t, int n) {
+  const int h = t < 3 * n ? t : t - 3 * n, i = h / 3;
+  return {i, h - 3 * i + (t < 3 * n ? 0 : 3)};
 }
 
 // Composite-rigid-body algorithm: M (dense, both triangles).
 template <int G, class T>
 __device__ void crba(const Grp<G>& g, const DevModel& m, const WsT<T>& w) {
   const Layout& L = *w.L;
-  const T* Ib = w.at(L.Ib); T* Ic = w.at(L.Ic);
+  T* Ic = w.at(L.Ic);
   const T* S = w.at(L.sd); T* F = w.at(L.F); T* M = w.at(L.M);
   const int nv = m.nv;
-  for (int lev = m.nlevel - 1; lev >= 0; --lev) {
-    for (int k = m.level_start[lev] + g.lane; k < m.level_start[lev + 1]; k += G) {
-      const int b = m.level_list[k];
-      T acc[10];
-      for (int e = 0; e < 10; ++e) acc[e] = Ib[10 * b + e];
-      for (int c = 0; c < m.child_count[b]; ++c) {
-        const int ch = m.child_list[m.child_start[b] + c];
-        for (int e = 0; e < 10; ++e) acc[e] += Ic[10 * ch + e];
-      }
-      for (int e = 0; e < 10; ++e) Ic[10 * b + e] = acc[e];
-    }
-    g.sync();
+  tree_up<10>(g, m, Ic);             // Ic starts as Ib (kinematics)
+  for (int t = g.lane; t < 6 * nv; t += G) {
+    const Comp6 c = comp6(t, nv);
+    F[6 * c.i + c.e] = inertia_comp(Ic + 10 * m.dof_body[c.i], S + 6 * c.i, c.e);
   }
-  for (int i = g.lane; i < nv; i += G) inertia_apply(Ic + 10 * m.dof_body[i], S + 6 * i, F + 6 * i);
   g.sync();
   for (int t = g.lane; t < nv * (nv + 1) / 2; t += G) {   // lower triangle
-    const int i = c_tri[t][0], j = c_tri[t][1];
+    const Tri ij = tri(t);
+    const int i = ij.i, j = ij.j;
     T v = 0.0;
     if ((m.b_anc[m.dof_body[i]] >> m.dof_body[j]) & 1u) {
       const T* s = S + 6 * j; const T* f = F + 6 * i;
@@ -479,15 +556,15 @@ __device__ void crba(const Grp<G>& g, const DevModel& m, const WsT<T>& w) {
 // Recursive Newton-Euler with zero joint acceleration: rhs0 = tau - c.
 // Body velocities and velocity-product accelerations are sums along the path
 // from the root: each body's own joint term is computed for all bodies at
-// once, then added down the tree level by level (6 additions per body).  The
-// per-body work is split by component (one body component per task).
+// once, then added down the tree.  The per-body work is split by component
+// (one body component per task).
 template <int G, class T>
 __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* q, const T* v,
                                const T* u) {
   const Layout& L = *w.L;
   const T* Ib = w.at(L.Ib); const T* S = w.at(L.sd);
   T* V = w.at(L.Vb); T* A = w.at(L.Ab); T* Fb = w.at(L.Fb); T* IV = w.at(L.iv);
-  const int nt = 6 * m.nbody;
+  const int nb = m.nbody, nt = 6 * nb;
   // own joint velocity S v
   for (int t = g.lane; t < nt; t += G) {
     const int b = t / 6, e = t - 6 * b;
@@ -497,68 +574,46 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
     V[t] = x;
   }
   g.sync();
-  for (int lev = 1; lev < m.nlevel; ++lev) {
-    for (int t = 6 * m.level_start[lev] + g.lane; t < 6 * m.level_start[lev + 1]; t += G) {
-      const int k = t / 6, e = t - 6 * k;
-      const int b = m.level_list[k], par = m.b_parent[b];
-      if (par >= 0) V[6 * b + e] += V[6 * par + e];
-    }
-    g.sync();
-  }
+  tree_down<6>(g, m, V);
   // own velocity-product acceleration (vb x S_d) v_d (gravity at the roots)
   for (int t = g.lane; t < nt; t += G) {
-    const int b = t / 6, e = t - 6 * b;
+    const Comp6 c = comp6(t, nb);
+    const int b = c.i, e = c.e;
     const int va = m.b_vadr[b], nd = m.b_nv[b];
     T x = (m.b_parent[b] < 0 && e >= 3) ? T(-m.grav[e - 3]) : T(0.0);
     const int d0 = (m.b_jtype[b] == JNT_FREE) ? 3 : 0;   // world-fixed translation axes
     for (int d = d0; d < nd; ++d) x += crm_comp(V + 6 * b, S + 6 * (va + d), e) * v[va + d];
-    A[t] = x;
+    A[6 * b + e] = x;
   }
   g.sync();
-  for (int lev = 1; lev < m.nlevel; ++lev) {
-    for (int t = 6 * m.level_start[lev] + g.lane; t < 6 * m.level_start[lev + 1]; t += G) {
-      const int k = t / 6, e = t - 6 * k;
-      const int b = m.level_list[k], par = m.b_parent[b];
-      if (par >= 0) A[6 * b + e] += A[6 * par + e];
-    }
-    g.sync();
-  }
+  tree_down<6>(g, m, A);
   // body forces I a + v x* (I v)
   for (int t = g.lane; t < nt; t += G) {
-    const int b = t / 6, e = t - 6 * b;
-    Fb[t] = inertia_comp(Ib + 10 * b, A + 6 * b, e);
-    IV[t] = inertia_comp(Ib + 10 * b, V + 6 * b, e);
+    const Comp6 c = comp6(t, nb);
+    const int b = c.i, e = c.e;
+    Fb[6 * b + e] = inertia_comp(Ib + 10 * b, A + 6 * b, e);
+    IV[6 * b + e] = inertia_comp(Ib + 10 * b, V + 6 * b, e);
   }
   g.sync();
   for (int t = g.lane; t < nt; t += G) {
-    const int b = t / 6, e = t - 6 * b;
-    Fb[t] += crf_comp(V + 6 * b, IV + 6 * b, e);
+    const Comp6 c = comp6(t, nb);
+    const int b = c.i, e = c.e;
+    Fb[6 * b + e] += crf_comp(V + 6 * b, IV + 6 * b, e);
   }
   g.sync();
-  for (int lev = m.nlevel - 1; lev >= 1; --lev) {
-    // children add into their parents; parents of one level are distinct bodies
-    // of the level above, so sweep the level above and gather its children
-    for (int t = 6 * m.level_start[lev - 1] + g.lane; t < 6 * m.level_start[lev]; t += G) {
-      const int k = t / 6, e = t - 6 * k;
-      const int b = m.level_list[k];
-      for (int c = 0; c < m.child_count[b]; ++c) Fb[6 * b + e] += Fb[6 * m.child_list[m.child_start[b] + c] + e];
-    }
-    g.sync();
-  }
+  tree_up<6>(g, m, Fb);
   T* rhs0 = w.at(L.rhs0);
   for (int i = g.lane; i < m.nv; i += G) {
-    const T* s = S + 6 * i; const T* f = Fb + 6 * m.dof_body[i];
+    const int b = m.dof_body[i];
+    const T* s = S + 6 * i; const T* f = Fb + 6 * b;
     const T c = s[0] * f[0] + s[1] * f[1] + s[2] * f[2] + s[3] * f[3] + s[4] * f[4] + s[5] * f[5];
-    const T tau = -m.b_damping[m.dof_body[i]] * v[i];
-    rhs0[i] = tau - c;
-  }
-  g.sync();
-  if (g.lane == 0) {
-    for (int a = 0; a < m.nact; ++a) {
-      const int vi = m.a_vadr[a];
-      if (m.a_type[a] == ACT_MOTOR) rhs0[vi] += m.a_gear[a] * u[a];
-      else rhs0[vi] += m.a_kp[a] * (u[a] - q[m.a_qadr[a]]) - m.a_kd[a] * v[vi];
+    const T tau = -m.b_damping[b] * v[i];
+    T x = tau - c;
+    for (int a = m.dof_act[i]; a >= 0; a = m.act_next[a]) {
+      if (m.a_type[a] == ACT_MOTOR) x += m.a_gear[a] * u[a];
+      else x += m.a_kp[a] * (u[a] - q[m.a_qadr[a]]) - m.a_kd[a] * v[i];
     }
+    rhs0[i] = x;
   }
   g.sync();
 }
@@ -792,6 +847,29 @@ __device__ __forceinline__ T spline_shape(const T& x, double mid, double pw) {
   const T num = (pw == 2.0) ? y * y : (pw == 4.0 ? (y * y) * (y * y) : pow(y, pw));
   return 1.0 - num / ((pw == 2.0) ? (1.0 - mid) : ::pow(1.0 - mid, pw - 1.0));
 }
+// a / b for a model constant b > 0 whose reciprocal rb was rounded on the host
+// and 0 <= a <= 2 b: the quotient estimate a rb corrected by its exact
+// remainder, three FP64 instructions instead of nine.
+__device__ __forceinline__ double div_const(double a, double b, double rb) {
+  const double q = a * rb;
+  return __fma_rn(__fma_rn(-b, q, a), rb, q);
+}
+// impedance(r) of the forward right-hand side, r < 0, in doubles, for the
+// quadratic spline (power 2, every shipped setting): the same value, with the
+// divisions by the width and the midpoint done by div_const.
+__device__ __forceinline__ double impedance_quadratic(const DevModel& m, double r) {
+  const double width = m.solimp[2], mid = m.solimp[3], a = fabs(r);
+  const double x = a < width ? div_const(a, width, m.imp_rwidth) : 1.0;
+  const bool low = x <= mid && mid > 0;
+  const double y = low ? x : 1.0 - x, den = low ? mid : 1.0 - mid;
+  const double num = y * y;
+  double sh = den > 0 ? div_const(num, den, low ? m.imp_rmid : m.imp_rmid1) : num / den;
+  if (!low) sh = 1.0 - sh;
+  const double d = m.solimp[0] + (m.solimp[1] - m.solimp[0]) * sh;
+  if (d < 0.0) return 0.0;
+  if (d > 0.9999) return 0.9999;
+  return d;
+}
 // The same shape with a derivative-scalar midpoint (parameter tangents).
 __device__ __forceinline__ Dual spline_shape(const Dual& x, const Dual& mid, double pw) {
   if (value(x) <= value(mid) && value(mid) > 0) {
@@ -873,7 +951,9 @@ __device__ void collide(const Grp<G>& g, const DevModel& m, const WsT<T>& w, boo
     w.i[L.sinc + s] = inc ? 1 : 0;
     if (inc) {
       const T r = ct[0];
-      const T d = impedance(m, r, cfd, w.pdir);
+      T d;
+      if constexpr (std::is_same<T, double>::value) d = (!cfd && m.solimp[4] == 2.0) ? impedance_quadratic(m, r) : impedance(m, r, cfd);
+      else d = impedance(m, r, cfd, w.pdir);
       const int pr = m.s_pair[s];
       const auto ahat = m.p_condim[pr] == 1 ? Par<T>::ahat(m, w.pdir, pr) : Par<T>::ahat_edge(m, w.pdir, pr);
       const auto kc = Par<T>::kcoef(m, w.pdir);
@@ -895,28 +975,30 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
   const int nv = m.nv;
   int* rowslot = w.i + L.rowslot;
   const int* sinc = w.i + L.sinc;
-  if (g.lane == 0) {
-    int n = 0, ns = 0;
-    for (int s = 0; s < m.nslot; ++s) {
-      const bool inc = sinc[s] != 0;
-      slotrow[s] = inc ? n : -1;
-      if (inc) {
-        const int nrow = (m.p_condim[m.s_pair[s]] == 1) ? 1 : 4;
-        for (int e = 0; e < nrow && n + e < L.rcap; ++e) rowslot[n + e] = s;
-        n += nrow;
-        slist[ns++] = s;
-      }
+  // row and slot prefixes by group ballots (every slot has 1 or 4 rows)
+  int n = 0, ns = 0;
+  for (int s0 = 0; s0 < m.nslot; s0 += G) {
+    const int s = s0 + g.lane;
+    const bool inc = s < m.nslot && sinc[s] != 0;
+    const int nrow = s < m.nslot ? m.s_rows[s] : 0;
+    const unsigned b1 = g.ballot(inc && nrow == 1), b4 = g.ballot(inc && nrow != 1);
+    const unsigned below = (1u << g.lane) - 1u;
+    const int r0 = n + __popc(b1 & below) + 4 * __popc(b4 & below);
+    if (s < m.nslot) slotrow[s] = inc ? r0 : -1;
+    if (inc) {
+      for (int e = 0; e < nrow && r0 + e < L.rcap; ++e) rowslot[r0 + e] = s;
+      slist[ns + __popc((b1 | b4) & below)] = s;
     }
-    slotrow[m.nslot] = n;
-    w.i[L.misc] = ns;
+    n += __popc(b1) + 4 * __popc(b4);
+    ns += __popc(b1 | b4);
   }
+  if (g.lane == 0) slotrow[m.nslot] = n;
   g.sync();
-  const int nr = slotrow[m.nslot];
-  const int nincl = w.i[L.misc];
+  const int nr = n, nincl = ns;
   if (nr > L.rcap) return -1;
   T* J = w.at(L.J);
-  for (int idx = g.lane; idx < nincl * nv; idx += G) {   // included slots only
-    const int si = idx / nv, i = idx - si * nv;
+  for (int idx = g.lane, si = g.lane / nv, i = g.lane - si * nv; idx < nincl * nv;   // included slots only
+       idx += G, i += G % nv, si += G / nv + (i >= nv), i -= (i >= nv) ? nv : 0) {
     const int s = slist[si];
     const int r0 = slotrow[s];
     const T* ct = CT + 16 * s;
@@ -964,41 +1046,57 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
     rowid[r] = m.p_row0[p] + m.s_idx[s] * nrow + e;
   }
   g.sync();
-  (void)nincl;
   return nr;
 }
 
 // ------------------------------------------------------------------ dense kernels
 // H <- its Cholesky factor below the diagonal, invd <- 1 / diagonal of the
-// factor.  Returns false if not SPD.
+// factor.  With rows = n + 1 the row after H's last (a right side) takes part
+// as another row of the factor: it leaves as L^-1 of the right side, the
+// forward half of the solve, without steps of its own.  Returns false if not SPD.
 template <int G, class T>
-__device__ bool cholesky(const Grp<G>& g, T* H, T* invd, int n) {
+__device__ bool cholesky(const Grp<G>& g, T* H, T* invd, int n, int rows) {
   bool ok = true;
   for (int k = 0; k < n; ++k) {
     const T hkk = H[k * n + k];
     ok = ok && (value(hkk) > 0);
     const T il = rsqrt_t(hkk);   // the diagonal of the factor is kept as its reciprocal
-    for (int i = k + 1 + g.lane; i < n; i += G) H[i * n + k] *= il;
+    for (int i = k + 1 + g.lane; i < rows; i += G) H[i * n + k] *= il;
     if (g.lane == 0) invd[k] = il;
     g.sync();
-    const int nt = n - k - 1;
-    for (int t = g.lane; t < nt * (nt + 1) / 2; t += G) {   // lower triangle of the trailing block
-      const int i = k + 1 + c_tri[t][0], j = k + 1 + c_tri[t][1];
-      H[i * n + j] -= H[i * n + k] * H[j * n + k];
+    const int nt = rows - k - 1, cnt = nt * (nt + 1) / 2 - (rows - n);
+    T* Hk = H + (k + 1) * n + k;   // column k below the diagonal
+    for (int t = g.lane; t < cnt; t += G) {   // lower triangle of the trailing block
+      const Tri ij = tri(t);
+      Hk[ij.i * n + 1 + ij.j] -= Hk[ij.i * n] * Hk[ij.j * n];
     }
     g.sync();
   }
   return ok;
 }
-// x <- H^-1 x with the factor from cholesky().
+// x <- L^-T x (the backward half of the solve).  With a lane per component
+// the vector stays in registers and each step broadcasts one of them (two
+// shuffles instead of two group meetings and a trip through shared memory:
+// 155 against 270 cycles a step).
+template <int G>
+__device__ __forceinline__ double chol_back_lanes(const Grp<G>& g, const double* H, const double* invd, double xi,
+                                                  int n) {
+  for (int k = n - 1; k >= 0; --k) {
+    const double xk = g.bcast(xi, k) * invd[k];
+    if (g.lane == k) xi = xk;
+    else if (g.lane < k) xi -= H[k * n + g.lane] * xk;
+  }
+  return xi;
+}
 template <int G, class T>
-__device__ void chol_solve(const Grp<G>& g, const T* H, const T* invd, T* x, int n) {
-  for (int k = 0; k < n; ++k) {
-    const T xk = x[k] * invd[k];
-    g.sync();
-    if (g.lane == 0) x[k] = xk;
-    for (int i = k + 1 + g.lane; i < n; i += G) x[i] -= H[i * n + k] * xk;
-    g.sync();
+__device__ void chol_back(const Grp<G>& g, const T* H, const T* invd, T* x, int n) {
+  if constexpr (G > 1 && std::is_same<T, double>::value) {
+    if (n <= G) {
+      const double xi = chol_back_lanes(g, H, invd, g.lane < n ? x[g.lane] : 0.0, n);
+      if (g.lane < n) x[g.lane] = xi;
+      g.sync();
+      return;
+    }
   }
   for (int k = n - 1; k >= 0; --k) {
     const T xk = x[k] * invd[k];
@@ -1007,6 +1105,32 @@ __device__ void chol_solve(const Grp<G>& g, const T* H, const T* invd, T* x, int
     for (int i = g.lane; i < k; i += G) x[i] -= H[k * n + i] * xk;
     g.sync();
   }
+}
+// x <- H^-1 x with the factor from cholesky().
+template <int G, class T>
+__device__ void chol_solve(const Grp<G>& g, const T* H, const T* invd, T* x, int n) {
+  if constexpr (G > 1 && std::is_same<T, double>::value) {
+    if (n <= G) {
+      double xi = g.lane < n ? x[g.lane] : 0.0;
+      for (int k = 0; k < n; ++k) {
+        const double xk = g.bcast(xi, k) * invd[k];
+        if (g.lane == k) xi = xk;
+        else if (g.lane > k && g.lane < n) xi -= H[g.lane * n + k] * xk;
+      }
+      xi = chol_back_lanes(g, H, invd, xi, n);
+      if (g.lane < n) x[g.lane] = xi;
+      g.sync();
+      return;
+    }
+  }
+  for (int k = 0; k < n; ++k) {
+    const T xk = x[k] * invd[k];
+    g.sync();
+    if (g.lane == 0) x[k] = xk;
+    for (int i = k + 1 + g.lane; i < n; i += G) x[i] -= H[i * n + k] * xk;
+    g.sync();
+  }
+  chol_back(g, H, invd, x, n);
 }
 
 __device__ __forceinline__ bool mask_has(const int* mk, int id) { return (mk[id >> 5] >> (id & 31)) & 1; }
@@ -1031,30 +1155,37 @@ __device__ bool solve_active(const Grp<G>& g, const DevModel& m, const WsT<T>& w
     na += __popc(bits);
   }
   g.sync();
-  // lower triangle of H, then b: one entry per task
-  const int ntri = nv * (nv + 1) / 2;
-  for (int t = g.lane; t < ntri + nv; t += G) {
-    if (t < ntri) {
-      const int i = c_tri[t][0], j = c_tri[t][1];
-      T h = M[i * nv + j];
-      for (int k = 0; k < na; ++k) {
-        const int r = alist[k];
-        h += Dr[r] * J[r * nv + i] * J[r * nv + j];
+  // Lower triangle of H, then b as its extra row: one entry per task, entry
+  // (i, j) = M_ij + sum_r X_ri J_rj with the D-scaled rows X = (D J, D a_ref)
+  // of hb active rows at a time, so that a row costs an entry one
+  // multiply-add (scaling inside costs two and a second pass for b).
+  T* X = w.at(L.xd);
+  const int nx1 = nv + 1, nent = nv * (nv + 1) / 2 + nv;
+  const int hb = L.hb;
+  for (int k0 = 0; k0 == 0 || k0 < na; k0 += hb) {
+    const int nk = min(hb, na - k0);
+    for (int t = g.lane; t < nk * nx1; t += G) {
+      const int k = t / nx1, i = t - k * nx1;
+      const int r = alist[k0 + k];
+      X[t] = Dr[r] * (i < nv ? J[r * nv + i] : aref[r]);
+    }
+    g.sync();
+    for (int t = g.lane; t < nent; t += G) {
+      const Tri ij = tri(t);
+      const int i = ij.i, j = ij.j;
+      T h = k0 ? H[i * nv + j] : (i < nv ? M[i * nv + j] : rhs0[j]);
+      if (nk == HBLK) {
+#pragma unroll
+        for (int k = 0; k < HBLK; ++k) h += X[k * nx1 + i] * J[alist[k0 + k] * nv + j];
+      } else {
+        for (int k = 0; k < nk; ++k) h += X[k * nx1 + i] * J[alist[k0 + k] * nv + j];
       }
       H[i * nv + j] = h;
-    } else {
-      const int i = t - ntri;
-      T b = rhs0[i];
-      for (int k = 0; k < na; ++k) {
-        const int r = alist[k];
-        b += Dr[r] * aref[r] * J[r * nv + i];
-      }
-      an[i] = b;
     }
+    g.sync();
   }
-  g.sync();
-  const bool ok = cholesky(g, H, w.at(L.tmp2), nv);
-  chol_solve(g, H, w.at(L.tmp2), an, nv);
+  const bool ok = cholesky(g, H, w.at(L.tmp2), nv, nv + 1);
+  chol_back(g, (const T*)H, (const T*)w.at(L.tmp2), an, nv);
   return ok;
 }
 
@@ -1311,6 +1442,21 @@ static __constant__ TabSet c_tabs = make_tabs();
 #define TAB(mt) (c_tabs.t[(mt)])
 
 // q (+) dq for every joint (free: translation + body-frame rotation exponential).
+template <class T>
+__device__ __forceinline__ void rot_exp(const T& th2, T& cw, T& sk) {   // cos(th / 2), sin(th / 2) / th
+  if (value(th2) < 1e-2) {
+    // |dq| < 0.1 rad: Taylor series of cos(th/2) and sin(th/2)/th in th^2
+    // (the next terms are below 3e-20): no square root, sine or division
+    cw = 1.0 + th2 * (-1.0 / 8.0 + th2 * (1.0 / 384.0 + th2 * (-1.0 / 46080.0 + th2 * (1.0 / 10321920.0))));
+    sk = 0.5 + th2 * (-1.0 / 48.0 + th2 * (1.0 / 3840.0 + th2 * (-1.0 / 645120.0 + th2 * (1.0 / 185794560.0))));
+  } else {
+    const T th = sqrt(th2);
+    T sn, cs;
+    sincos(0.5 * th, &sn, &cs);
+    cw = cs;
+    sk = sn / th;
+  }
+}
 template <int G, class T>
 __device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, const T* dq, T* out) {
   for (int b = g.lane; b < m.nbody; b += G) {
@@ -1320,18 +1466,7 @@ __device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, co
     const T* d = dq + va + 3;
     const T th2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
     T cw, sk;
-    if (value(th2) < 1e-2) {
-      // |dq| < 0.1 rad: Taylor series of cos(th/2) and sin(th/2)/th in th^2
-      // (the next terms are below 3e-20): no square root, sine or division
-      cw = 1.0 + th2 * (-1.0 / 8.0 + th2 * (1.0 / 384.0 + th2 * (-1.0 / 46080.0 + th2 * (1.0 / 10321920.0))));
-      sk = 0.5 + th2 * (-1.0 / 48.0 + th2 * (1.0 / 3840.0 + th2 * (-1.0 / 645120.0 + th2 * (1.0 / 185794560.0))));
-    } else {
-      const T th = sqrt(th2);
-      T sn, cs;
-      sincos(0.5 * th, &sn, &cs);
-      cw = cs;
-      sk = sn / th;
-    }
+    rot_exp(th2, cw, sk);
     const T ex = sk * d[0], ey = sk * d[1], ez = sk * d[2];
     const T w0 = q[qa + 3], a0 = q[qa + 4], b0 = q[qa + 5], c0 = q[qa + 6];
     const T rw = w0 * cw - a0 * ex - b0 * ey - c0 * ez;

@@ -35,7 +35,7 @@ __global__ void k_body_invweight(const DevModel* mp, const double* qpos0, double
   crba(g, m, w);
   double* H = w.at(sL.H); const double* M = w.at(sL.M);
   for (int i = 0; i < m.nv * m.nv; ++i) H[i] = M[i];
-  cholesky(g, H, w.at(sL.tmp2), m.nv);
+  cholesky(g, H, w.at(sL.tmp2), m.nv, m.nv);
   const double* S = w.at(sL.sd); const double* C = w.at(sL.com);
   double* col = scratch;
   double* x = scratch + m.nv;

@@ -29,6 +29,7 @@ constexpr int MAXROWID = 128; // constraint rows over all slots (stable row ids)
 constexpr int ROWCAP = 64;
 constexpr int MAXLEV = 12;    // depth of the body tree
 constexpr int MASKW = MAXROWID / 32;
+constexpr int HBLK = 8;       // active rows per block of the Newton matrix assembly, at most
 
 enum { JNT_FREE = 0, JNT_HINGE = 1 };
 enum { GEOM_SPHERE = 0, GEOM_CAPSULE = 1, GEOM_BOX = 2 };
@@ -48,6 +49,7 @@ struct DevModel {
   double solimp[5];                  // d_o, d_w, width, midpoint, power
   double cfd[5];                     // d_c, d_0, w_c, m_c, p_c
   double softplus;
+  double imp_rwidth, imp_rmid, imp_rmid1;   // reciprocals of the spline's width, midpoint and 1 - midpoint
   // bodies (topological order)
   int b_parent[MAXB], b_jtype[MAXB], b_qadr[MAXB], b_vadr[MAXB], b_nv[MAXB];
   unsigned b_anc[MAXB];              // bit j: body j is this body or an ancestor
@@ -57,6 +59,14 @@ struct DevModel {
   int child_start[MAXB], child_count[MAXB], child_list[MAXB];
   int level_start[MAXLEV + 1], level_list[MAXB];
   int dof_body[MAXV];
+  // Chains of the body tree: maximal runs in which every body but the last has
+  // exactly one child, ordered by levels (a chain's head hangs on a chain of an
+  // earlier level, or on the world), so that one lane can carry a component
+  // down or up a whole run without meeting the others.
+  int nchlev, chlev_start[MAXLEV + 1];                 // chain levels: ranges of chains
+  int ch_start[MAXB + 1], ch_list[MAXB], ch_par[MAXB]; // bodies of each chain (head first), parent of its head (-1 = world)
+  int lv_pack[MAXB];                 // k-th body in level order: body | parent << 8 (parent 255 = world)
+  int dof_act[MAXV], act_next[MAXU]; // first actuator on a dof (-1 = none), next one on the same dof
   // geoms
   int g_type[MAXG], g_body[MAXG];
   double g_pos[MAXG][3], g_Roff[MAXG][9], g_size[MAXG][3];
@@ -70,6 +80,7 @@ struct DevModel {
   double p_mu[MAXP], p_ahat[MAXP], p_ahat_edge[MAXP];
   double p_dahat[MAXP][MAXB + MAXBOX];   // d A_hat / d (mass of each body, then side of each box)
   int s_pair[MAXS], s_idx[MAXS];
+  int s_rows[MAXS];                  // constraint rows of the slot (1 or 4)
   int s_barofs[MAXS], nslotbar;      // adjoint: offset / total of the per-slot pose cotangents
                                      // (12 doubles for a plane slot, 24 for a geom pair)
   // actuators
@@ -83,6 +94,7 @@ struct Layout {
   int R, p, com, sd, Ib, Ic, F, Vb, Ab, Fb, iv, gR, gp;
   int M, H, rhs0, a, an, tmp, tmp2;
   int ct, csv, J, aref, Dr, z, s, u;   // csv: closest-point parameters of each geom-pair slot (2 per slot)
+  int xd, hb;                        // D-scaled rows (J, a_ref) of hb active rows (Newton matrix assembly)
   int nd;                            // doubles per environment (padded to even)
   int xl, sc;                        // kinematics scratch, aliases of Ab..Fb (12 per body) and iv (2 per body)
   int rowid, slotrow, slist, amask, pmask, misc;
@@ -92,6 +104,13 @@ struct Layout {
   int xbar;                          // adjoint layout: state cotangent (nq + nv), else -1
   int ovl;                           // adjoint layout: start of the arrays the VJP never reads, else nd
 };
+
+// Active rows per block of the Newton matrix assembly: as many D-scaled rows
+// of nv + 1 as two row arrays hold.
+DMX_HD inline int newton_block(int nv, int rcap) {
+  const int h = 2 * rcap / (nv + 1);
+  return h < 1 ? 1 : (h > HBLK ? HBLK : h);
+}
 
 DMX_HD inline Layout make_layout(const DevModel& m, int rcap) {
   Layout L{};
@@ -108,9 +127,13 @@ DMX_HD inline Layout make_layout(const DevModel& m, int rcap) {
   L.xl = L.Ab; L.sc = L.iv;
   L.gR = take(9 * ng); L.gp = take(3 * ng);
   L.M = take(nv * nv); L.H = take(nv * nv);
-  L.rhs0 = take(nv); L.a = take(nv); L.an = take(nv); L.tmp = take(nv); L.tmp2 = take(nv);
+  L.an = take(nv);                   // directly after H: its extra row (cholesky)
+  L.rhs0 = take(nv); L.a = take(nv); L.tmp = take(nv); L.tmp2 = take(nv);
   L.ct = take(16 * ns); L.csv = take(2 * ns);
   L.J = take(rcap * nv); L.aref = take(rcap); L.Dr = take(rcap); L.z = take(rcap); L.s = take(rcap);
+  // the residuals and line-search slopes are free while H is assembled
+  L.hb = newton_block(nv, rcap); L.xd = L.z;
+  if (L.hb * (nv + 1) > 2 * rcap) take(L.hb * (nv + 1) - 2 * rcap);
   L.u = take(m.nu > 0 ? m.nu : 1);
   L.nd = (o + 1) & ~1;
   int i = 0;
@@ -146,7 +169,8 @@ DMX_HD inline Layout make_layout_adj(const DevModel& m, int rcap) {
   L.xl = L.Ab; L.sc = L.iv;
   L.gR = take(9 * ng); L.gp = take(3 * ng);
   L.H = take(nv * nv);
-  L.rhs0 = take(nv); L.a = take(nv); L.an = take(nv); L.tmp = take(nv); L.tmp2 = take(nv);
+  L.an = take(nv);                   // directly after H, as above
+  L.rhs0 = take(nv); L.a = take(nv); L.tmp = take(nv); L.tmp2 = take(nv);
   L.csv = take(2 * ns); L.Dr = take(rcap); L.z = take(rcap);
   L.u = take(m.nu > 0 ? m.nu : 1);
   L.xbar = take(nq + nv);
@@ -156,6 +180,7 @@ DMX_HD inline Layout make_layout_adj(const DevModel& m, int rcap) {
   L.M = take(nv * nv);
   L.ct = take(16 * ns);
   L.J = take(rcap * nv); L.aref = take(rcap); L.s = take(rcap);
+  L.xd = take(L.hb * (nv + 1));
   L.nd = (o + 1) & ~1;
   return L;
 }

@@ -118,6 +118,32 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
       if (depth[b] == l) m.level_list[pos++] = b;
   }
   m.level_start[m.nlevel] = pos;
+  for (int k = 0; k < m.nbody; ++k) {
+    const int b = m.level_list[k];
+    m.lv_pack[k] = b | ((m.b_parent[b] < 0 ? 255 : m.b_parent[b]) << 8);
+  }
+  // chains: a body heads one unless it is its parent's only child
+  int nch = 0, chpos = 0, chlev_of[MAXB];
+  for (int b = 0; b < m.nbody; ++b) chlev_of[b] = MAXB;   // not placed yet
+  for (int lev = 0, done = 0; done < m.nbody; ++lev) {
+    m.chlev_start[lev] = nch;
+    for (int b = 0; b < m.nbody; ++b) {
+      const int par = m.b_parent[b];
+      if (par >= 0 && m.child_count[par] == 1) continue;            // inside its parent's chain
+      if ((par < 0 ? 0 : chlev_of[par] + 1) != lev) continue;
+      m.ch_par[nch] = par;
+      m.ch_start[nch++] = chpos;
+      for (int x = b;; x = m.child_list[m.child_start[x]]) {
+        m.ch_list[chpos++] = x;
+        chlev_of[x] = lev;
+        ++done;
+        if (m.child_count[x] != 1) break;
+      }
+    }
+    m.nchlev = lev + 1;
+    m.chlev_start[lev + 1] = nch;
+  }
+  m.ch_start[nch] = chpos;
   for (int b = 0; b < m.nbody; ++b)
     for (int k = 0; k < m.b_nv[b]; ++k) m.dof_body[m.b_vadr[b] + k] = b;
   for (int g = 0; g < m.ngeom; ++g) {
@@ -162,6 +188,7 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
     if (m.nslot + ns > MAXS) return "too many contact slots";
     for (int j = 0; j < ns; ++j) {
       m.s_pair[m.nslot + j] = p; m.s_idx[m.nslot + j] = j;
+      m.s_rows[m.nslot + j] = P.condim == 1 ? 1 : 4;
       m.s_barofs[m.nslot + j] = m.nslotbar;
       m.nslotbar += P.geom2 >= 0 ? 24 : 12;     // a plane slot moves one geom
     }
@@ -177,6 +204,11 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
     m.a_type[a] = A.type; m.a_qadr[a] = m.b_qadr[A.body]; m.a_vadr[a] = m.b_vadr[A.body];
     m.a_gear[a] = A.gear; m.a_kp[a] = A.kp; m.a_kd[a] = A.kd;
   }
+  for (int i = 0; i < m.nv; ++i) m.dof_act[i] = -1;
+  for (int a = m.nact - 1; a >= 0; --a) {   // in actuator order along each dof's list
+    m.act_next[a] = m.dof_act[m.a_vadr[a]];
+    m.dof_act[m.a_vadr[a]] = a;
+  }
   m.nu = m.nact;
   for (int i = 0; i < 3; ++i) m.grav[i] = d->gravity[i];
   const double tc = d->solref[0], damp = d->solref[1], dw = d->solimp[1];
@@ -187,6 +219,7 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
   m.solref[0] = tc; m.solref[1] = damp;
   for (int i = 0; i < 5; ++i) { m.solimp[i] = d->solimp[i]; m.cfd[i] = d->solimp_cfd[i]; }
   m.softplus = d->softplus;
+  m.imp_rwidth = 1.0 / m.solimp[2]; m.imp_rmid = 1.0 / m.solimp[3]; m.imp_rmid1 = 1.0 / (1.0 - m.solimp[3]);
   return "";
 }
 
