@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS) k_adjoint(AdjParams P) {
         if (n == n1 - 1) break;
         const double h = P.hlog[(size_t)n * P.B + env];
         int st;
-        rk_attempt(g, m, wp, (const double*)u, h, P.method, 1.0, 1.0, &st);
+        rk_attempt(g, m, wp, (const double*)u, h, P.method, 1.0, 1.0, 1, &st);
         const double tn = adj_boundary(T, P.NI, k + 1);
         const bool reached = (h == tn - t) || (t + h >= tn);
         t = reached ? tn : t + h;

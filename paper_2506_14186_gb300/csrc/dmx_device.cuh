@@ -1526,13 +1526,36 @@ __device__ int rk_stages(const Grp<G>& g, const DevModel& m, const Ws& w, const 
   return st;
 }
 
+// Sum of x[0..n) (shared memory, consumed) in the order of a shuffle
+// reduction over C lanes: component i first joins lane i mod C's partial sum,
+// then the partial sums meet in a binary tree.  The order is C's whatever the
+// group's own lane count, so that the lane count can follow the hardware
+// without touching a single step decision.
+template <int G>
+__device__ double sum_as_lanes(const Grp<G>& g, double* x, int n, int C) {
+  for (int c = g.lane; c < C && c + C < n; c += G) {
+    double acc = x[c];
+    for (int i = c + C; i < n; i += C) acc += x[i];
+    x[c] = acc;
+  }
+  g.sync();
+  const int np = min(n, C);          // partial sums that exist
+  for (int o = C >> 1; o > 0; o >>= 1) {
+    if (o >= np) continue;
+    for (int c = g.lane; c < o && c + o < np; c += G) x[c] += x[c + o];
+    g.sync();
+  }
+  return x[0];
+}
+
 // One attempt of scheme mt of size h from (qn, vn) with ka[0] = F(qn, vn).
 // Leaves the result in (qs, vs) and its derivative in ka[(S-1) nv]; returns
 // the RMS error norm of the embedded estimate (NaN-safe: non-finite -> +inf;
-// 0 for a fixed-step scheme) and the worst stage status.
+// 0 for a fixed-step scheme; summed in the order of `red` lanes) and the
+// worst stage status.
 template <int G>
 __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
-                             double rtol, double atol, int* st_out) {
+                             double rtol, double atol, int red, int* st_out) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   const double* qn = w.at(L.qn); const double* vn = w.at(L.vn);
@@ -1542,7 +1565,7 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
   *st_out = st;
   if (!TAB(mt).adaptive) return 0.0;
   const unsigned enz = TAB(mt).enz;
-  double acc = 0;
+  double* terms = w.at(L.dq);        // free after the last stage
   for (int i = g.lane; i < nv; i += G) {
     double ep = 0, ev = 0;
     for (int j = 0; j < 7; ++j) {
@@ -1555,9 +1578,11 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
     const double sp = atol + rtol * fmax(pos_mag(m, qn, i), pos_mag(m, qs, i));
     const double sv = atol + rtol * fmax(fabs(vn[i]), fabs(vs[i]));
     const double r1 = ep / sp, r2 = ev / sv;
-    acc += r1 * r1 + r2 * r2;
+    terms[i] = r1 * r1 + r2 * r2;
   }
-  acc = g.sum(acc);
+  g.sync();
+  const double acc = sum_as_lanes(g, terms, nv, red);
+  g.sync();
   const double err = sqrt(acc / (2.0 * nv));
   return isfinite(err) ? err : INFINITY;
 }

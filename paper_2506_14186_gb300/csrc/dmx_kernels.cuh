@@ -86,7 +86,7 @@ __device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, con
   if (ht < 1e-12) { s.st = ENV_H_UNDERFLOW; s.done = 1; return; }
   int stage_st = 0;
   const int mt = P.method;
-  const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, &stage_st);
+  const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, P.red, &stage_st);
   ++s.att;
   if (err <= 1.0) {
     if (stage_st != ENV_OK) { s.st = stage_st; s.done = 1; return; }

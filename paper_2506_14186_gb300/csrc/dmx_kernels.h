@@ -11,6 +11,7 @@ struct RolloutParams {
   Layout L;
   int B, NI, max_steps, K;
   int method;           // METHOD_* integration scheme (dmx_device.cuh)
+  int red;              // lanes whose summation order the error norm follows (sum_as_lanes)
   double rtol, atol, h0;
   const double* x0;     // [nx][B]
   const double* ctrl;   // [NI][nu][B]

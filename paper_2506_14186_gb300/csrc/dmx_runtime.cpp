@@ -343,13 +343,40 @@ bool launch_config_layout(const dmx_model* m, const dmx::Layout& L, int G, int* 
   return true;
 }
 
-int default_lanes(const dmx_model* m, int B) {
-  // enough lanes to give every SM sub-partition one warp of FP64 work
+int reduction_lanes(const dmx_model* m, int B) {
   const int want = 4 * 32 * m->nsm;
   int G = 1;
   while (G < 32 && (long long)B * G < want) G <<= 1;
   int t; size_t s;
   while (G < 32 && !launch_config(m, G, &t, &s)) G <<= 1;
+  return G;
+}
+
+// Lanes for `per` bytes of workspace per environment: the most lanes (gmin at
+// least) that leave an SM at most `warps` warps of the environments it holds
+// (its share of the batch, or what its shared memory takes).  Fewer lanes leave
+// an SM's few environments on too few warps to cover their dependent reads
+// (quadruped rollouts, 3000 for 0.1 s: 172 ms with 32 lanes, 197 with 16, 358
+// with 8); more lanes spread the same FP64 instructions thinner once the FP64
+// unit is busy (box pushes, 4096 for 0.05 s: 55 ms with 8 lanes, 63 with 16,
+// 94 with 32; tosses, 20001 for 0.2 s: 250, 287, 385).
+int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
+  const long long share = ((long long)B + m->nsm - 1) / m->nsm;
+  const long long fit = (long long)((size_t)(m->smem_max + 1024) / (per + 256));
+  const long long e = std::max(1LL, std::min(share, fit));
+  int G = 32;
+  while (G > gmin && e * G > warps * 32) G >>= 1;
+  return G;
+}
+// Rollouts: two warps per sub-partition fill the FP64 unit with a single
+// body's short phases (8 to 36 tasks); the phases of larger models (100 tasks)
+// use 32 lanes, and four warps still gain (arms, 4000 for 0.1 s: 74 ms with 32
+// lanes, 83 with 16).  Below 4 lanes nothing was faster.
+int default_lanes(const dmx_model* m, int B) { return layout_lanes(m, m->L, B, m->host.nv > 8 ? 16 : 8); }
+int layout_lanes(const dmx_model* m, const dmx::Layout& L, int B, int warps) {
+  int G = fill_lanes(m, B, (size_t)L.nd * 8 + (size_t)L.ni * 4, warps, 4);
+  int t; size_t s;
+  while (G < 32 && !launch_config_layout(m, L, G, &t, &s)) G <<= 1;
   return G;
 }
 
@@ -490,11 +517,12 @@ extern "C" dmx_status dmx_rollout(dmx_model* m, const dmx_rollout_args* a, void*
   int cur = 0;
   CK(cudaGetDevice(&cur));
   if (cur != m->device) return dmx_fail(DMX_ERR_INVALID, "model belongs to another device");
-  const int G = a->lanes ? a->lanes : tuned_lanes(m, a->B, 0);
+  int red = 0;
+  const int G = a->lanes ? a->lanes : tuned_lanes(m, a->B, 0, &red);
   const size_t B = a->B;
   RolloutParams P{};
   P.model = m->dev; P.L = m->L; P.B = a->B; P.NI = a->NI; P.max_steps = a->max_steps; P.K = a->K > 0 ? a->K : 1;
-  P.rtol = a->rtol; P.atol = a->atol; P.h0 = a->h0; P.method = a->method;
+  P.rtol = a->rtol; P.atol = a->atol; P.h0 = a->h0; P.method = a->method; P.red = a->lanes ? G : red;
   P.x0 = a->x0; P.ctrl = a->ctrl; P.T = a->T; P.xT = a->xT; P.xb = a->xb;
   P.nsteps = a->nsteps; P.nrej = a->nrej; P.status = a->status;
   if (a->host && B > 0) {
@@ -542,17 +570,21 @@ extern "C" dmx_status dmx_rollout(dmx_model* m, const dmx_rollout_args* a, void*
 }
 
 // ------------------------------------------------------------------ autotuner
-int tuned_lanes(dmx_model* m, int B, int grad) {
+int tuned_lanes(dmx_model* m, int B, int grad, int* red) {
   std::lock_guard<std::mutex> lk(m->mu);
   auto it = m->tuned.find({B, grad});
-  if (it != m->tuned.end()) return it->second;
+  if (it != m->tuned.end()) {
+    if (red) *red = it->second;
+    return it->second;
+  }
+  if (red) *red = reduction_lanes(m, B);
   return default_lanes(m, B);
 }
 
 extern "C" dmx_status dmx_autotune(dmx_model* m, int32_t B, int32_t grad, int32_t* lanes, void* stream) {
   (void)stream;
   if (!m || B < 0) return dmx_fail(DMX_ERR_INVALID, "bad argument");
-  if (lanes) *lanes = tuned_lanes(m, B, grad);
+  if (lanes) *lanes = tuned_lanes(m, B, grad, nullptr);
   return DMX_OK;
 }
 
@@ -582,9 +614,14 @@ static bool adj_launch_config(const dmx_model* m, const dmx::Layout& L, const dm
   return true;
 }
 
-// Lanes of the reverse-mode adjoint: the recorded choice, else enough lanes
-// to give every SM sub-partition a warp (at least 2), within shared memory.
-static int adjoint_lanes(dmx_model* m, int B, const dmx::Layout& L) {
+// Lanes of the reverse-mode kernels: the recorded choice, else by fill_lanes.
+// `sweep`: the adjoint of a tape, whose groups stay resident (0: one VJP per
+// environment).  Larger models run their sweep on 32 lanes; a single body's
+// has 8 tasks in its longest phase (the vertices), so one warp per
+// sub-partition of 8-lane groups is the better use (tosses, 2048 for 0.25 s,
+// forward and adjoint: 270 ms with 16 lanes, 192 with 8).  Single VJPs keep
+// one warp per sub-partition, too (arms, 16384: 17.0 -> 10.8 ms).
+static int adjoint_lanes(dmx_model* m, int B, const dmx::Layout& L, bool sweep) {
   const dmx::LayoutBar LB = dmx::make_bar_layout(m->host, L.rcap);
   int t; size_t s;
   {
@@ -593,9 +630,8 @@ static int adjoint_lanes(dmx_model* m, int B, const dmx::Layout& L) {
     if (it != m->tuned.end() && valid_adj_lanes(it->second) && adj_launch_config(m, L, LB, it->second, &t, &s))
       return it->second;
   }
-  const int want = 4 * 32 * m->nsm;
-  int G = 2;
-  while (G < 32 && (long long)B * G < want) G <<= 1;
+  const size_t per = (size_t)(L.nd + LB.nd) * 8 + (size_t)L.ni * 4;
+  int G = fill_lanes(m, B, per, sweep ? (m->host.nv > 8 ? 16 : 4) : 5, 8);
   while (G < 32 && !adj_launch_config(m, L, LB, G, &t, &s)) G <<= 1;
   return G;
 }
@@ -710,7 +746,7 @@ extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, c
   P.ckpt = t->ckpt; P.hlog = t->hlog; P.tape_n = t->n; P.ctrl = t->ctrl; P.T = t->T;
   P.xT_bar = xT_bar; P.xb_bar = xb_bar; P.x0_bar = x0_bar; P.ctrl_bar = m->host.nu ? ctrl_bar : nullptr;
   if (mode == DMX_ADJ_TANGENT) return run_tangent_adjoint(m, t, P, st);
-  const int G = adjoint_lanes(m, t->B, L);
+  const int G = adjoint_lanes(m, t->B, L, true);
   P.LB = dmx::make_bar_layout(m->host, L.rcap);
   const int gpb = 32 / G, threads = 32;
   const int RW = dmx::rev_row_doubles(m->host);
@@ -774,7 +810,7 @@ extern "C" dmx_status dmx_eval_rhs_vjp(dmx_model* m, int32_t B, const double* q,
   const bool act = m->host.nu > 0;
   if (!q || !v || !abar || !qbar || !vbar || !status || (act && (!u || !ubar))) return dmx_fail(DMX_ERR_INVALID, "null array");
   const dmx::Layout& L = layout_for(m, cfd);
-  const int G = lanes ? lanes : adjoint_lanes(m, B, L);
+  const int G = lanes ? lanes : adjoint_lanes(m, B, L, false);
   if (!valid_adj_lanes(G)) return dmx_fail(DMX_ERR_INVALID, "lanes must be 0, 2, 4, 8, 16 or 32");
   dmx::AdjParams P{};
   P.model = m->dev; P.L = L; P.LB = dmx::make_bar_layout(m->host, L.rcap); P.B = B; P.cfd = cfd;
@@ -790,7 +826,7 @@ extern "C" dmx_status dmx_eval_rhs(dmx_model* m, int32_t B, const double* q, con
   if (!m || B < 0) return dmx_fail(DMX_ERR_INVALID, "bad argument");
   if (B == 0) return DMX_OK;
   if (!q || !v || !a || !info || (m->host.nu && !u)) return dmx_fail(DMX_ERR_INVALID, "null array");
-  const int G = lanes ? lanes : default_lanes(m, B);
+  const int G = lanes ? lanes : layout_lanes(m, layout_for(m, cfd), B, 8);
   if (!valid_lanes(G)) return dmx_fail(DMX_ERR_INVALID, "lanes must be 0, 1, 2, 4, 8, 16 or 32");
   int threads; size_t smem;
   const dmx::Layout& L = layout_for(m, cfd);

@@ -51,8 +51,19 @@ bool launch_config_layout(const dmx_model* m, const dmx::Layout& L, int G, int* 
 // Workspace layout of a right-hand side with (cfd = 1) or without the CFD
 // contacts: F~ includes every slot within w_c, so it may need more rows.
 inline const dmx::Layout& layout_for(const dmx_model* m, int cfd) { return cfd ? m->Lc : m->L; }
+// Lanes per environment: fill_lanes for `per` bytes each, layout_lanes for a
+// right-hand-side layout, default_lanes for a rollout.
+int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin);
+int layout_lanes(const dmx_model* m, const dmx::Layout& L, int B, int warps);
 int default_lanes(const dmx_model* m, int B);
-int tuned_lanes(dmx_model* m, int B, int grad);
+// Lanes whose summation order the error norm follows when the caller names no
+// lane count: the fewest that give every SM sub-partition a warp.  Kept apart
+// from the lanes a call runs on, so that these can follow the hardware while
+// step decisions, hence trajectories, stay the same bit for bit.
+int reduction_lanes(const dmx_model* m, int B);
+// The recorded lane count of (model, B, grad), else default_lanes; *red (if
+// not null) receives the matching summation order.
+int tuned_lanes(dmx_model* m, int B, int grad, int* red);
 dmx_status run_rollout(dmx_model* m, const dmx::RolloutParams& P, int form, int G, cudaStream_t st);
 int model_smem_bytes(const dmx_model* m, int groups);
 // Upper bound of the device scratch that dmx_rollout_grad allocates for B

@@ -88,6 +88,7 @@ extern "C" dmx_status dmx_rollout_static(dmx_model* m, const dmx_rollout_args* a
   RolloutParams P{};
   P.model = m->dev; P.L = m->L; P.B = a->B; P.NI = a->NI; P.max_steps = a->max_steps; P.K = 1;
   P.rtol = a->rtol; P.atol = a->atol; P.h0 = a->h0; P.method = a->method;
+  P.red = a->lanes ? G : reduction_lanes(m, a->B);
   P.x0 = a->x0; P.ctrl = a->ctrl; P.T = a->T; P.xT = a->xT; P.xb = a->xb;
   P.nsteps = a->nsteps; P.nrej = a->nrej; P.status = a->status;
   // the unfinished-environment counter must start at B; every other field is
