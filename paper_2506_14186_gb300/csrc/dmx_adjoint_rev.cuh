@@ -41,6 +41,21 @@ __device__ __forceinline__ int rev_interval(double T, int NI, double t) {
   return k;
 }
 
+// dst[i] = src[i], i < n, eight loads in flight per lane (the snapshots live in
+// device memory: one round trip per eight passes instead of one per pass).
+template <int G>
+__device__ __forceinline__ void copy_run(const Grp<G>& g, const double* __restrict__ src, double* __restrict__ dst,
+                                         int n) {
+  for (int i0 = g.lane; i0 < n; i0 += 8 * G) {
+    double x[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i0 + k * G < n) x[k] = src[i0 + k * G];
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (i0 + k * G < n) dst[i0 + k * G] = x[k];
+  }
+}
 // Workspace of the right-hand side just evaluated (status st) -> snapshot dst.
 template <int G>
 __device__ void snap_save(const Grp<G>& g, const DevModel& m, const Ws& w, double* dst, int st) {
@@ -70,8 +85,8 @@ __device__ int snap_restore(const Grp<G>& g, const DevModel& m, const Ws& w, con
   const int* si = reinterpret_cast<const int*>(src + o.oi);
   const int st = si[0], nr = si[1];
   double* d = w.d;
-  for (int i = g.lane; i < o.n1; i += G) d[L.R + i] = src[i];
-  for (int i = g.lane; i < o.n2; i += G) d[L.H + i] = src[o.o2 + i];
+  copy_run(g, src, d + L.R, o.n1);
+  copy_run(g, src + o.o2, d + L.H, o.n2);
   for (int i = g.lane; i < 2 * m.nslot; i += G) d[L.csv + i] = src[o.o3 + 16 * m.nslot + i];
   for (int i = g.lane; i < nr; i += G) { d[L.Dr + i] = src[o.o5 + i]; d[L.z + i] = src[o.o6 + i]; }
   for (int i = g.lane; i <= m.nslot; i += G) w.i[L.slotrow + i] = si[2 + i];

@@ -81,6 +81,10 @@ struct DevModel {
   double p_dahat[MAXP][MAXB + MAXBOX];   // d A_hat / d (mass of each body, then side of each box)
   int s_pair[MAXS], s_idx[MAXS];
   int s_rows[MAXS];                  // constraint rows of the slot (1 or 4)
+  unsigned s_move[MAXS];             // bodies that move geom 1 of the slot (bit mask: its body and its ancestors)
+  unsigned g_slots1[MAXG], g_slots2[MAXG];   // bit s: the geom is geom 1 / geom 2 of slot s
+  unsigned b_geoms[MAXB];            // bit g: geom g is fixed to the body
+  unsigned dof_anc[MAXV], dof_desc[MAXV];    // dofs j <= i of the dof's ancestor bodies, k >= i of its descendants (with its own)
   int s_barofs[MAXS], nslotbar;      // adjoint: offset / total of the per-slot pose cotangents
                                      // (12 doubles for a plane slot, 24 for a geom pair)
   // actuators
@@ -106,9 +110,10 @@ struct Layout {
 };
 
 // Active rows per block of the Newton matrix assembly: as many D-scaled rows
-// of nv + 1 as two row arrays hold.
-DMX_HD inline int newton_block(int nv, int rcap) {
-  const int h = 2 * rcap / (nv + 1);
+// of nv + 1 as fit the larger of the arrays that are free meanwhile (residuals
+// and line-search slopes, 2 per row; I V of the bias force, 6 per body).
+DMX_HD inline int newton_block(int nv, int nb, int rcap) {
+  const int h = (6 * nb > 2 * rcap ? 6 * nb : 2 * rcap) / (nv + 1);
   return h < 1 ? 1 : (h > HBLK ? HBLK : h);
 }
 
@@ -131,9 +136,9 @@ DMX_HD inline Layout make_layout(const DevModel& m, int rcap) {
   L.rhs0 = take(nv); L.a = take(nv); L.tmp = take(nv); L.tmp2 = take(nv);
   L.ct = take(16 * ns); L.csv = take(2 * ns);
   L.J = take(rcap * nv); L.aref = take(rcap); L.Dr = take(rcap); L.z = take(rcap); L.s = take(rcap);
-  // the residuals and line-search slopes are free while H is assembled
-  L.hb = newton_block(nv, rcap); L.xd = L.z;
-  if (L.hb * (nv + 1) > 2 * rcap) take(L.hb * (nv + 1) - 2 * rcap);
+  L.hb = newton_block(nv, nb, rcap);
+  L.xd = 6 * nb > 2 * rcap ? L.iv : L.z;
+  if (nv + 1 > 6 * nb && nv + 1 > 2 * rcap) L.xd = take(nv + 1);   // a free body with a row or two
   L.u = take(m.nu > 0 ? m.nu : 1);
   L.nd = (o + 1) & ~1;
   int i = 0;
@@ -189,7 +194,7 @@ DMX_HD inline Layout make_layout_adj(const DevModel& m, int rcap) {
 // adjoint kernel): cotangents of the right-hand side's intermediates, then
 // the stage data and cotangents of one Dormand-Prince step.
 struct LayoutBar {
-  int R, p, cR, cp, S, F, Ib, Ic, V, A, Fb, slot, y, jy, cz, cj, q, v, u;   // right-hand side
+  int R, p, cR, cp, S, F, Ic, V, A, Fb, slot, y, jy, cz, cj, q, v, u;   // right-hand side
   int gb, iv, ivb;                   // geom pose cotangents, I V and its cotangent per body
   int sc, tk;                        // hinge sine and cosine, theta-cotangent terms per body
   int qn, vst, dq, dqb, Qs, kab, kvb, Qb, Vb, qnb, vnb, ub, xb;            // one step
@@ -203,7 +208,7 @@ DMX_HD inline LayoutBar make_bar_layout(const DevModel& m, int rcap) {
   const int nq = m.nq, nv = m.nv, nb = m.nbody, ns = m.nslot > 0 ? m.nslot : 1, nu = m.nu > 0 ? m.nu : 1;
   auto take = [&](int n) { int r = o; o += n; return r; };
   B.R = take(9 * nb); B.p = take(3 * nb); B.cR = take(9 * nb); B.cp = take(3 * nb);
-  B.S = take(6 * nv); B.F = take(6 * nv); B.Ib = take(10 * nb); B.Ic = take(10 * nb);
+  B.S = take(6 * nv); B.F = take(6 * nv); B.Ic = take(10 * nb);
   B.V = take(6 * nb); B.A = take(6 * nb); B.Fb = take(6 * nb);
   B.slot = take(m.nslotbar > 0 ? m.nslotbar : SLOTBAR * ns);
   B.y = take(nv); B.jy = take(rcap); B.cz = take(rcap); B.cj = take(rcap);

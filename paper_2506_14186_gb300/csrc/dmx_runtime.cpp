@@ -189,6 +189,9 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
     for (int j = 0; j < ns; ++j) {
       m.s_pair[m.nslot + j] = p; m.s_idx[m.nslot + j] = j;
       m.s_rows[m.nslot + j] = P.condim == 1 ? 1 : 4;
+      m.s_move[m.nslot + j] = m.b_anc[m.g_body[P.geom1]];
+      m.g_slots1[P.geom1] |= 1u << (m.nslot + j);
+      if (P.geom2 >= 0) m.g_slots2[P.geom2] |= 1u << (m.nslot + j);
       m.s_barofs[m.nslot + j] = m.nslotbar;
       m.nslotbar += P.geom2 >= 0 ? 24 : 12;     // a plane slot moves one geom
     }
@@ -204,6 +207,10 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
     m.a_type[a] = A.type; m.a_qadr[a] = m.b_qadr[A.body]; m.a_vadr[a] = m.b_vadr[A.body];
     m.a_gear[a] = A.gear; m.a_kp[a] = A.kp; m.a_kd[a] = A.kd;
   }
+  for (int g = 0; g < m.ngeom; ++g) m.b_geoms[m.g_body[g]] |= 1u << g;
+  for (int i = 0; i < m.nv; ++i)
+    for (int j = 0; j <= i; ++j)
+      if ((m.b_anc[m.dof_body[i]] >> m.dof_body[j]) & 1u) { m.dof_anc[i] |= 1u << j; m.dof_desc[j] |= 1u << i; }
   for (int i = 0; i < m.nv; ++i) m.dof_act[i] = -1;
   for (int a = m.nact - 1; a >= 0; --a) {   // in actuator order along each dof's list
     m.act_next[a] = m.dof_act[m.a_vadr[a]];

@@ -24,7 +24,13 @@
 //   Jbar_r = -D_r (z_r y + (J_r y) an)   (+ the a_ref term -bcoef a_refbar_r v).
 // Every intermediate's cotangent is written by one lane of the group
 // (reductions over children, dofs or slots are gathers by the owner), so the
-// result does not depend on scheduling.
+// result does not depend on scheduling.  As in the forward code a group is
+// bound by its chain of FP64 instructions and dependent reads, so the phases
+// are loops over equal one-component tasks, ordered so that a pass of the
+// lanes meets one formula; sums over slots follow bit masks of the included
+// ones; sums along the tree run in chains (tree_down, tree_up).  On stiff
+// pushing contacts the gradient amplifies a rounding difference to 1e-8 of
+// its norm, so every split keeps each result's operations and their order.
 #pragma once
 #include "dmx_device.cuh"
 
@@ -42,50 +48,31 @@ __device__ __forceinline__ void acc_cross(const double* a, const double* b, doub
   out[1] += a[2] * b[0] - a[0] * b[2];
   out[2] += a[0] * b[1] - a[1] * b[0];
 }
-// Ibar += d/dI (ybar . inertia_apply(I, x)) for the 10-number spatial inertia.
-__device__ __forceinline__ void inertia_grad(const double* yb, const double* x, double* Ibar) {
-  const double w0 = x[0], w1 = x[1], w2 = x[2], v0 = x[3], v1 = x[4], v2 = x[5];
-  Ibar[0] += yb[3] * v0 + yb[4] * v1 + yb[5] * v2;
-  // h enters as h x v (angular part) and -(h x w) (linear part)
-  Ibar[1] += (v1 * yb[2] - v2 * yb[1]) - (w1 * yb[5] - w2 * yb[4]);
-  Ibar[2] += (v2 * yb[0] - v0 * yb[2]) - (w2 * yb[3] - w0 * yb[5]);
-  Ibar[3] += (v0 * yb[1] - v1 * yb[0]) - (w0 * yb[4] - w1 * yb[3]);
-  Ibar[4] += yb[0] * w0; Ibar[5] += yb[1] * w1; Ibar[6] += yb[2] * w2;
-  Ibar[7] += yb[0] * w1 + yb[1] * w0; Ibar[8] += yb[0] * w2 + yb[2] * w0; Ibar[9] += yb[1] * w2 + yb[2] * w1;
-}
-// Component e of d/dI (ybar . inertia_apply(I, x)) (the terms inertia_grad adds).
+// Component e of d/dI (ybar . inertia_apply(I, x)) for the 10-number spatial
+// inertia: mass, first moments (h enters as h x v in the angular part and
+// -(h x w) in the linear one), moments xx yy zz, products xy xz yz.
 __device__ __forceinline__ double inertia_grad_comp(const double* yb, const double* x, int e) {
-  const double w0 = x[0], w1 = x[1], w2 = x[2], v0 = x[3], v1 = x[4], v2 = x[5];
-  switch (e) {
-    case 0: return yb[3] * v0 + yb[4] * v1 + yb[5] * v2;
-    case 1: return (v1 * yb[2] - v2 * yb[1]) - (w1 * yb[5] - w2 * yb[4]);
-    case 2: return (v2 * yb[0] - v0 * yb[2]) - (w2 * yb[3] - w0 * yb[5]);
-    case 3: return (v0 * yb[1] - v1 * yb[0]) - (w0 * yb[4] - w1 * yb[3]);
-    case 4: return yb[0] * w0;
-    case 5: return yb[1] * w1;
-    case 6: return yb[2] * w2;
-    case 7: return yb[0] * w1 + yb[1] * w0;
-    case 8: return yb[0] * w2 + yb[2] * w0;
-    default: return yb[1] * w2 + yb[2] * w1;
+  if (e == 0) return yb[3] * x[3] + yb[4] * x[4] + yb[5] * x[5];
+  if (e < 4) {
+    const int k1 = nxt3(e - 1), k2 = prv3(e - 1);
+    return (x[3 + k1] * yb[k2] - x[3 + k2] * yb[k1]) - (x[k1] * yb[3 + k2] - x[k2] * yb[3 + k1]);
   }
+  if (e < 7) return yb[e - 4] * x[e - 4];
+  const int i = e == 9 ? 1 : 0, j = e == 7 ? 1 : 2;
+  return yb[i] * x[j] + yb[j] * x[i];
 }
-// c = a x b (motion): abar, bbar += from cbar.  a = (w; v), b = (w2; v2).
-__device__ __forceinline__ void crm6_vjp(const double* a, const double* b, const double* cb, double* ab, double* bb) {
-  acc_cross(b, cb, ab);            // w2 x cw
-  acc_cross(b + 3, cb + 3, ab);    // v2 x cv
-  acc_cross(b, cb + 3, ab + 3);    // w2 x cv
-  acc_cross(cb, a, bb);            // cw x w
-  acc_cross(cb + 3, a + 3, bb);    // cv x v
-  acc_cross(cb + 3, a, bb + 3);    // cv x w
-}
-// c = a x* b (force): a = (w; v), b = (n; f).
-__device__ __forceinline__ void crf6_vjp(const double* a, const double* b, const double* cb, double* ab, double* bb) {
-  acc_cross(b, cb, ab);            // n x cn
-  acc_cross(b + 3, cb + 3, ab);    // f x cf
-  acc_cross(b + 3, cb, ab + 3);    // f x cn
-  acc_cross(cb, a, bb);            // cn x w
-  acc_cross(cb, a + 3, bb + 3);    // cn x v
-  acc_cross(cb + 3, a, bb + 3);    // cf x w
+// Task t of 10 n tasks (n spatial inertias): first moments of all, then
+// products, moments, masses.
+__device__ __forceinline__ Comp6 comp10(int t, int n) {
+  if (t < 6 * n) {
+    const int h = t < 3 * n ? t : t - 3 * n, i = h / 3;
+    return {i, h - 3 * i + (t < 3 * n ? 1 : 7)};
+  }
+  if (t < 9 * n) {
+    const int h = t - 6 * n, i = h / 3;
+    return {i, h - 3 * i + 4};
+  }
+  return {t - 9 * n, 0};
 }
 // qbar += (d R / d q)^T Rbar for R = quat_to_mat(q) = 1 + s P(q), s = 2 / |q|^2.
 __device__ __forceinline__ void quat_to_mat_vjp(const double* q, const double* Rb, double* qb) {
@@ -102,17 +89,6 @@ __device__ __forceinline__ void quat_to_mat_vjp(const double* q, const double* R
   const double c = -2.0 * sb * s / n2;   // ds/dq = -(s / n2) 2 q
   qb[0] += s * gw + c * w; qb[1] += s * gx + c * x; qb[2] += s * gy + c * y; qb[3] += s * gz + c * z;
 }
-// Rodrigues rotation about the unit axis a by theta and its theta-derivative.
-__device__ __forceinline__ void rodrigues(const double* a, double sn, double cs, double* Rj, double* dR) {
-  const double c1 = 1.0 - cs;
-  Rj[0] = cs + c1 * a[0] * a[0];        Rj[1] = c1 * a[0] * a[1] - sn * a[2]; Rj[2] = c1 * a[0] * a[2] + sn * a[1];
-  Rj[3] = c1 * a[0] * a[1] + sn * a[2]; Rj[4] = cs + c1 * a[1] * a[1];        Rj[5] = c1 * a[1] * a[2] - sn * a[0];
-  Rj[6] = c1 * a[0] * a[2] - sn * a[1]; Rj[7] = c1 * a[1] * a[2] + sn * a[0]; Rj[8] = cs + c1 * a[2] * a[2];
-  dR[0] = -sn + sn * a[0] * a[0];       dR[1] = sn * a[0] * a[1] - cs * a[2]; dR[2] = sn * a[0] * a[2] + cs * a[1];
-  dR[3] = sn * a[0] * a[1] + cs * a[2]; dR[4] = -sn + sn * a[1] * a[1];       dR[5] = sn * a[1] * a[2] - cs * a[0];
-  dR[6] = sn * a[0] * a[2] - cs * a[1]; dR[7] = sn * a[1] * a[2] + cs * a[0]; dR[8] = -sn + sn * a[2] * a[2];
-}
-
 // Value and derivative of the solimp spline shape on x in [0, 1].
 __device__ __forceinline__ double spline_shape_d(double x, double mid, double pw, double* dy) {
   if (x <= mid && mid > 0) {
@@ -441,12 +417,18 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   const double* an = w.at(L.an); const double* J = w.xJ ? w.xJ : w.at(L.J); const double* Dr = w.at(L.Dr);
   const double* z = w.at(L.z); const double* CT = w.xct ? w.xct : w.at(L.ct);
   double* Rb = b.at(LB.R); double* pb = b.at(LB.p); double* cR = b.at(LB.cR); double* cp = b.at(LB.cp);
-  double* Sb = b.at(LB.S); double* Fd = b.at(LB.F); double* Ibb = b.at(LB.Ib); double* Icb = b.at(LB.Ic);
+  double* Sb = b.at(LB.S); double* Fd = b.at(LB.F); double* Icb = b.at(LB.Ic);
   double* Vbb = b.at(LB.V); double* Abb = b.at(LB.A); double* Fbb = b.at(LB.Fb); double* SB = b.at(LB.slot);
   double* y = b.at(LB.y); double* jy = b.at(LB.jy); double* cz = b.at(LB.cz); double* cj = b.at(LB.cj);
   double* qb = b.at(LB.q); double* vb = b.at(LB.v); double* ub = b.at(LB.u);
-  for (int k = g.lane; k < LB.qn - LB.R; k += G) Rb[k] = 0.0;   // every right-hand-side cotangent
-  for (int i = g.lane; i < nv; i += G) y[i] = abar[i];
+  unsigned incl = 0u;                                   // included slots
+  for (int s0 = 0; s0 < m.nslot; s0 += G) {
+    const int s = s0 + g.lane;
+    incl |= g.ballot(s < m.nslot && slotrow[s] >= 0) << s0;
+  }
+  for (int i = g.lane; i < nv; i += G) { y[i] = abar[i]; vb[i] = 0.0; }
+  for (int i = g.lane; i < nq; i += G) qb[i] = 0.0;
+  for (int a = g.lane; a < m.nu; a += G) ub[a] = 0.0;
   g.sync();
   // ---- constraint solve: y = H_A^-1 abar with the factor of the final set
   chol_solve(g, w.at(L.H), w.at(L.tmp2), y, nv);
@@ -458,39 +440,52 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     cz[r] = mask_has(am, rowid[r]) ? Dr[r] * z[r] : 0.0;
     cj[r] = Dr[r] * t;
   }
+  // ---- mass matrix: -(y an^T) folded to the lower triangle, W_kj = -(y_k an_j + y_j an_k),
+  // over the Newton factor, which is done with
+  double* W = w.at(L.H);
+  for (int t = g.lane; t < nv * (nv + 1) / 2; t += G) {
+    const Tri ij = tri(t);
+    const int i = ij.i, j = ij.j;
+    W[i * nv + j] = (i == j) ? -y[i] * an[i] : -(y[i] * an[j] + y[j] * an[i]);
+  }
   g.sync();
-  // ---- per dof: a_ref's J v term, damping, bias force, CRBA products, contact Jacobians
+  // M_kj = S_j . F_k for j <= k with dof j's body an ancestor of dof k's body;
+  // bias force c_i = S_i . Fb; one component per task
+  for (int t = g.lane; t < 6 * nv; t += G) {
+    const int i = t / 6, e = t - 6 * i;
+    const int bi = m.dof_body[i];
+    double fd = 0.0;
+    for (unsigned ms = m.dof_anc[i]; ms; ms &= ms - 1u) {      // dofs j <= i of ancestor bodies
+      const int j = __ffs(ms) - 1;
+      fd += W[i * nv + j] * S[6 * j + e];
+    }
+    Fd[t] = fd;
+    double sb = 0.0;
+    sb -= y[i] * Fb[6 * bi + e];
+    for (unsigned ms = m.dof_desc[i]; ms; ms &= ms - 1u) {     // dofs k >= i of descendant bodies
+      const int k = __ffs(ms) - 1;
+      sb += W[k * nv + i] * F[6 * k + e];
+    }
+    Sb[t] = sb;
+  }
+  g.sync();
+  // ---- per dof: a_ref's J v term, damping, contact Jacobians
   for (int i = g.lane; i < nv; i += G) {
     const int bi = m.dof_body[i];
     double acc = -m.b_damping[bi] * y[i];
     for (int r = 0; r < nr; ++r) acc -= m.bcoef * cj[r] * J[r * nv + i];
     vb[i] += acc;
     double* sbi = Sb + 6 * i;
-    const double* fb = Fb + 6 * bi;
-    for (int e = 0; e < 6; ++e) sbi[e] -= y[i] * fb[e];
-    // M_kj = S_j . F_k for j <= k with dof j's body an ancestor of dof k's body
-    double fd[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = 0; j <= i; ++j) {
-      if (!((m.b_anc[bi] >> m.dof_body[j]) & 1u)) continue;
-      const double wij = (i == j) ? -y[i] * an[i] : -(y[i] * an[j] + y[j] * an[i]);
-      for (int e = 0; e < 6; ++e) fd[e] += wij * S[6 * j + e];
-    }
-    for (int e = 0; e < 6; ++e) Fd[6 * i + e] = fd[e];
-    for (int k = i; k < nv; ++k) {
-      if (!((m.b_anc[m.dof_body[k]] >> bi) & 1u)) continue;
-      const double wki = (i == k) ? -y[i] * an[i] : -(y[k] * an[i] + y[i] * an[k]);
-      for (int e = 0; e < 6; ++e) sbi[e] += wki * F[6 * k + e];
-    }
     const double yai = an[i] + m.bcoef * v[i];
-    for (int s = 0; s < m.nslot; ++s) {
+    for (unsigned ms = incl; ms; ms &= ms - 1u) {
+      const int s = __ffs(ms) - 1;
       const int r0 = slotrow[s];
-      if (r0 < 0) continue;
       const int p = m.s_pair[s];
       const double* ct = CT + 16 * s;
       double pvb[3];
       if (m.p_g2[p] < 0) {
         // ground plane: frame (z, x, y) of the world, the dof moves the geom's body or nothing
-        if (!((m.b_anc[m.g_body[m.p_g1[p]]] >> bi) & 1u)) continue;
+        if (!((m.s_move[s] >> bi) & 1u)) continue;
         double jb[3];
         slot_rows_bar(m, b, p, r0, y[i], yai, jb);
         pvb[0] = jb[1]; pvb[1] = jb[2]; pvb[2] = jb[0];
@@ -510,11 +505,11 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     const double* ct = CT + 16 * s;
     double* sb = SB + m.s_barofs[s];
     const int p = m.s_pair[s];
-    const int nrow = m.p_condim[p] == 1 ? 1 : 4;
+    const int nrow = m.s_rows[s];
     double cb[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (m.p_g2[p] < 0) {
       // ground plane: the frame is fixed (no frame cotangents), pvb in the world frame
-      const unsigned anc = m.b_anc[m.g_body[m.p_g1[p]]];
+      const unsigned anc = m.s_move[s];
       for (int i = 0; i < nv; ++i) {
         if (!((anc >> m.dof_body[i]) & 1u)) continue;
         double jb[3];
@@ -541,10 +536,11 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     for (int e = 0; e < nrow; ++e) { b14 += cj[r0 + e]; b15 -= jy[r0 + e] * z[r0 + e]; }
     const double r = ct[0];
     if (r < thr) {
-      const double ahat = m.p_condim[p] == 1 ? m.p_ahat[p] : m.p_ahat_edge[p];
+      const double ahat = nrow == 1 ? m.p_ahat[p] : m.p_ahat_edge[p];
       cb[0] += impedance_terms_vjp(m, r, cfd, ahat, b14, b15);
     }
     double* b1 = sb; double* b2 = sb + 12;
+    for (int k = 0; k < (m.p_g2[p] < 0 ? 12 : 24); ++k) sb[k] = 0.0;
     const int g1 = m.p_g1[p];
     if (m.p_g2[p] >= 0) {
       const double* st = w.at(L.csv) + 2 * s;
@@ -572,12 +568,11 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   double* GB = b.at(LB.gb);
   for (int t = g.lane; t < 12 * m.ngeom; t += G) {
     const int gi = t / 12, c = t - 12 * gi;
+    const unsigned m1 = m.g_slots1[gi];
     double acc = 0.0;
-    for (int s = 0; s < m.nslot; ++s) {
-      if (slotrow[s] < 0) continue;
-      const int p = m.s_pair[s];
-      if (m.p_g1[p] == gi) acc += SB[m.s_barofs[s] + c];
-      else if (m.p_g2[p] == gi) acc += SB[m.s_barofs[s] + 12 + c];
+    for (unsigned ms = incl & (m1 | m.g_slots2[gi]); ms; ms &= ms - 1u) {
+      const int s = __ffs(ms) - 1;
+      acc += SB[m.s_barofs[s] + (((m1 >> s) & 1u) ? 0 : 12) + c];
     }
     GB[t] = acc;
   }
@@ -585,75 +580,67 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // ---- per body: geom poses -> body pose (gR = R_b Roff, gp = p_b + R_b gpos), one
   // entry per task; per dof and body component: bias-force (c_i = S_i . Fb) and
   // CRBA (F_i = Ic S_i) cotangents
-  {
-    const int n1 = 12 * nb, n2 = n1 + 6 * nv, n3 = n2 + 6 * nb, n4 = n3 + 10 * nb;
-    for (int t = g.lane; t < n4; t += G) {
-      if (t < n1) {
-        const int bb = t / 12, c = t - 12 * bb;
-        double acc = 0.0;
-        for (int gi = 0; gi < m.ngeom; ++gi) {
-          if (m.g_body[gi] != bb) continue;
-          const double* gb = GB + 12 * gi;
-          if (c < 9) {
-            const int i = c / 3, j = c - 3 * (c / 3);
-            const double* Ro = m.g_Roff[gi];
-            acc += gb[3 * i] * Ro[3 * j] + gb[3 * i + 1] * Ro[3 * j + 1] + gb[3 * i + 2] * Ro[3 * j + 2] +
-                   gb[9 + i] * m.g_pos[gi][j];
-          } else {
-            acc += gb[c];
-          }
-        }
-        if (c < 9) Rb[9 * bb + c] += acc; else pb[3 * bb + c - 9] += acc;
-      } else if (t < n2) {
-        const int k = t - n1, i = k / 6, e = k - 6 * (k / 6);
-        Sb[6 * i + e] += inertia_comp(Ic + 10 * m.dof_body[i], Fd + 6 * i, e);
-      } else if (t < n3) {
-        const int k = t - n2, bb = k / 6, e = k - 6 * (k / 6);
-        double acc = 0.0;
-        for (int d = 0; d < m.b_nv[bb]; ++d) { const int i = m.b_vadr[bb] + d; acc += y[i] * S[6 * i + e]; }
-        Fbb[6 * bb + e] -= acc;
+  for (int t = g.lane; t < 12 * nb; t += G) {
+    const int bb = t / 12, c = t - 12 * bb;
+    double acc = 0.0;
+    for (unsigned ms = m.b_geoms[bb]; ms; ms &= ms - 1u) {
+      const int gi = __ffs(ms) - 1;
+      const double* gb = GB + 12 * gi;
+      if (c < 9) {
+        const int i = c / 3, j = c - 3 * (c / 3);
+        const double* Ro = m.g_Roff[gi];
+        acc += gb[3 * i] * Ro[3 * j] + gb[3 * i + 1] * Ro[3 * j + 1] + gb[3 * i + 2] * Ro[3 * j + 2] +
+               gb[9 + i] * m.g_pos[gi][j];
       } else {
-        const int k = t - n3, bb = k / 10, e = k - 10 * (k / 10);
-        double acc = 0.0;
-        for (int d = 0; d < m.b_nv[bb]; ++d) {
-          const int i = m.b_vadr[bb] + d;
-          acc += inertia_grad_comp(Fd + 6 * i, S + 6 * i, e);
-        }
-        Icb[10 * bb + e] += acc;
+        acc += gb[c];
       }
     }
+    if (c < 9) Rb[9 * bb + c] = acc; else pb[3 * bb + c - 9] = acc;
+  }
+  for (int t = g.lane; t < 6 * nv; t += G) {
+    const Comp6 c = comp6(t, nv);
+    Sb[6 * c.i + c.e] += inertia_comp(Ic + 10 * m.dof_body[c.i], Fd + 6 * c.i, c.e);
+  }
+  for (int t = g.lane; t < 6 * nb; t += G) {
+    const int bb = t / 6, e = t - 6 * bb;
+    double acc = 0.0;
+    for (int d = 0; d < m.b_nv[bb]; ++d) { const int i = m.b_vadr[bb] + d; acc += y[i] * S[6 * i + e]; }
+    Fbb[t] = -acc;
+  }
+  for (int t = g.lane; t < 10 * nb; t += G) {
+    const Comp6 c = comp10(t, nb);
+    double acc = 0.0;
+    for (int d = 0; d < m.b_nv[c.i]; ++d) {
+      const int i = m.b_vadr[c.i] + d;
+      acc += inertia_grad_comp(Fd + 6 * i, S + 6 * i, c.e);
+    }
+    Icb[10 * c.i + c.e] = acc;
   }
   g.sync();
-  // accumulated forces and composite inertias: cotangents flow from parents to children
-  for (int lev = 0; lev < m.nlevel; ++lev) {
-    for (int k = m.level_start[lev] + g.lane; k < m.level_start[lev + 1]; k += G) {
-      const int bb = m.level_list[k];
-      const int par = m.b_parent[bb];
-      if (par >= 0) {
-        for (int e = 0; e < 6; ++e) Fbb[6 * bb + e] += Fbb[6 * par + e];
-        for (int e = 0; e < 10; ++e) Icb[10 * bb + e] += Icb[10 * par + e];
-      }
-      for (int e = 0; e < 10; ++e) Ibb[10 * bb + e] += Icb[10 * bb + e];
-    }
-    g.sync();
-  }
+  // accumulated forces and composite inertias: cotangents flow from parents to
+  // children; a body's inertia is a term of its own composite one, so Icb goes
+  // on as the inertia cotangent
+  tree_down<6>(g, m, Fbb);
+  tree_down<10>(g, m, Icb);
+  double* Ibb = Icb;
   // ---- recursive Newton-Euler (forward: V = V_parent + S v, A = A_parent + (V x S) v,
   // F = I A + V x* (I V)), reversed with the same split: per-body work for all
-  // bodies at once, sums along the tree level by level
+  // bodies at once, sums along the tree
   // F's cotangent -> A, V (own terms), one body component per task:
   //   f1 = I A:          Abar = I fbar,  Ibar += grad(fbar, A)
   //   f2 = V x* (I V):   Vbar and (I V)bar from the force cross product, then
   //                      Vbar += I (I V)bar,  Ibar += grad((I V)bar, V)
   double* IV = b.at(LB.iv); double* IVB = b.at(LB.ivb);
   for (int t = g.lane; t < 6 * nb; t += G) {
-    const int bb = t / 6, e = t - 6 * (t / 6);
-    const double* I = Ib + 10 * bb;
-    Abb[t] = inertia_comp(I, Fbb + 6 * bb, e);
-    IV[t] = inertia_comp(I, V + 6 * bb, e);
+    const Comp6 c = comp6(t, nb);
+    const double* I = Ib + 10 * c.i;
+    Abb[6 * c.i + c.e] = inertia_comp(I, Fbb + 6 * c.i, c.e);
+    IV[6 * c.i + c.e] = inertia_comp(I, V + 6 * c.i, c.e);
   }
   g.sync();
   for (int t = g.lane; t < 6 * nb; t += G) {
-    const int bb = t / 6, e = t - 6 * (t / 6);
+    const Comp6 ce = comp6(t, nb);
+    const int bb = ce.i, e = ce.e;
     const double* a = V + 6 * bb; const double* iv = IV + 6 * bb; const double* fbar = Fbb + 6 * bb;
     const int k = e < 3 ? e : e - 3, k1 = nxt3(k), k2 = prv3(k);
     // c = a x* iv with a = (w; v), iv = (n; f): c_n = w x n + v x f, c_f = w x f
@@ -665,107 +652,83 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
       vb_e = iv[3 + k1] * fbar[k2] - iv[3 + k2] * fbar[k1];
       ivb_e = (fbar[k1] * a[3 + k2] - fbar[k2] * a[3 + k1]) + (fbar[3 + k1] * a[k2] - fbar[3 + k2] * a[k1]);
     }
-    Vbb[t] = vb_e;
-    IVB[t] = ivb_e;
+    Vbb[6 * bb + e] = vb_e;
+    IVB[6 * bb + e] = ivb_e;
   }
   g.sync();
-  for (int t = g.lane; t < 16 * nb; t += G) {
-    if (t < 6 * nb) {
-      const int bb = t / 6, e = t - 6 * (t / 6);
-      Vbb[t] += inertia_comp(Ib + 10 * bb, IVB + 6 * bb, e);
-    } else {
-      const int k = t - 6 * nb, bb = k / 10, e = k - 10 * (k / 10);
-      Ibb[10 * bb + e] += inertia_grad_comp(Fbb + 6 * bb, A + 6 * bb, e) + inertia_grad_comp(IVB + 6 * bb, V + 6 * bb, e);
-    }
+  for (int t = g.lane; t < 6 * nb; t += G) {
+    const Comp6 c = comp6(t, nb);
+    Vbb[6 * c.i + c.e] += inertia_comp(Ib + 10 * c.i, IVB + 6 * c.i, c.e);
+  }
+  for (int t = g.lane; t < 10 * nb; t += G) {
+    const Comp6 c = comp10(t, nb);
+    Ibb[10 * c.i + c.e] += inertia_grad_comp(Fbb + 6 * c.i, A + 6 * c.i, c.e) +
+                           inertia_grad_comp(IVB + 6 * c.i, V + 6 * c.i, c.e);
   }
   g.sync();
-  for (int lev = m.nlevel - 1; lev >= 1; --lev) {   // A_child = A_parent + ...: gather into parents
-    for (int k = m.level_start[lev - 1] + g.lane; k < m.level_start[lev]; k += G) {
-      const int bb = m.level_list[k];
-      for (int c = 0; c < m.child_count[bb]; ++c) {
-        const int ch = m.child_list[m.child_start[bb] + c];
-        for (int e = 0; e < 6; ++e) Abb[6 * bb + e] += Abb[6 * ch + e];
-      }
-    }
-    g.sync();
-  }
+  tree_up<6>(g, m, Abb);             // A_child = A_parent + ...: gather into parents
   // A's own term (V x S_d) v_d (d past the free joint's translations):
   //   vbar_d += Abar . (V x S_d);  with cb = Abar v_d:  Vbar_w += S_w x cb_w + S_v x cb_v,
   //   Vbar_v += S_w x cb_v;  Sbar_w += cb_w x V_w + cb_v x V_v,  Sbar_v += cb_v x V_w
-  {
-    const int n1 = nv, n2 = n1 + 6 * nv, n3 = n2 + 6 * nb;
-    for (int t = g.lane; t < n3; t += G) {
-      if (t < n1) {
-        const int i = t, bb = m.dof_body[i];
-        if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
-        const double* vbv = V + 6 * bb; const double* sd = S + 6 * i; const double* ab6 = Abb + 6 * bb;
-        double s1 = 0.0;
-        for (int e = 0; e < 6; ++e) s1 += ab6[e] * crm_comp(vbv, sd, e);
-        vb[i] += s1;
-      } else if (t < n2) {
-        const int k = t - n1, i = k / 6, e = k - 6 * (k / 6), bb = m.dof_body[i];
-        if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
-        const double* a = V + 6 * bb; const double* ab6 = Abb + 6 * bb;
-        const double vd = v[i];
-        const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
-        double r;
-        if (e < 3)
-          r = vd * ((ab6[c1] * a[c2] - ab6[c2] * a[c1]) + (ab6[3 + c1] * a[3 + c2] - ab6[3 + c2] * a[3 + c1]));
-        else
-          r = vd * (ab6[3 + c1] * a[c2] - ab6[3 + c2] * a[c1]);
-        Sb[6 * i + e] += r;
-      } else {
-        const int k = t - n2, bb = k / 6, e = k - 6 * (k / 6);
-        const double* ab6 = Abb + 6 * bb;
-        const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
-        const int va = m.b_vadr[bb], nd = m.b_nv[bb];
-        const int d0 = (m.b_jtype[bb] == JNT_FREE) ? 3 : 0;
-        double acc = 0.0;
-        for (int d = d0; d < nd; ++d) {
-          const double* sd = S + 6 * (va + d);
-          const double vd = v[va + d];
-          if (e < 3)
-            acc += vd * ((sd[c1] * ab6[c2] - sd[c2] * ab6[c1]) + (sd[3 + c1] * ab6[3 + c2] - sd[3 + c2] * ab6[3 + c1]));
-          else
-            acc += vd * (sd[c1] * ab6[3 + c2] - sd[c2] * ab6[3 + c1]);
-        }
-        Vbb[6 * bb + e] += acc;
-      }
+  for (int i = g.lane; i < nv; i += G) {
+    const int bb = m.dof_body[i];
+    if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
+    const double* vbv = V + 6 * bb; const double* sd = S + 6 * i; const double* ab6 = Abb + 6 * bb;
+    double s1 = 0.0;
+    for (int e = 0; e < 6; ++e) s1 += ab6[e] * crm_comp(vbv, sd, e);
+    vb[i] += s1;
+  }
+  for (int t = g.lane; t < 6 * nv; t += G) {
+    const Comp6 ce = comp6(t, nv);
+    const int i = ce.i, e = ce.e, bb = m.dof_body[i];
+    if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
+    const double* a = V + 6 * bb; const double* ab6 = Abb + 6 * bb;
+    const double vd = v[i];
+    const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
+    double r;
+    if (e < 3)
+      r = vd * ((ab6[c1] * a[c2] - ab6[c2] * a[c1]) + (ab6[3 + c1] * a[3 + c2] - ab6[3 + c2] * a[3 + c1]));
+    else
+      r = vd * (ab6[3 + c1] * a[c2] - ab6[3 + c2] * a[c1]);
+    Sb[6 * i + e] += r;
+  }
+  for (int t = g.lane; t < 6 * nb; t += G) {
+    const Comp6 ce = comp6(t, nb);
+    const int bb = ce.i, e = ce.e;
+    const double* ab6 = Abb + 6 * bb;
+    const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
+    const int va = m.b_vadr[bb], nd = m.b_nv[bb];
+    const int d0 = (m.b_jtype[bb] == JNT_FREE) ? 3 : 0;
+    double acc = 0.0;
+    for (int d = d0; d < nd; ++d) {
+      const double* sd = S + 6 * (va + d);
+      const double vd = v[va + d];
+      if (e < 3)
+        acc += vd * ((sd[c1] * ab6[c2] - sd[c2] * ab6[c1]) + (sd[3 + c1] * ab6[3 + c2] - sd[3 + c2] * ab6[3 + c1]));
+      else
+        acc += vd * (sd[c1] * ab6[3 + c2] - sd[c2] * ab6[3 + c1]);
     }
+    Vbb[6 * bb + e] += acc;
   }
   g.sync();
-  for (int lev = m.nlevel - 1; lev >= 1; --lev) {   // V_child = V_parent + ...
-    for (int k = m.level_start[lev - 1] + g.lane; k < m.level_start[lev]; k += G) {
-      const int bb = m.level_list[k];
-      for (int c = 0; c < m.child_count[bb]; ++c) {
-        const int ch = m.child_list[m.child_start[bb] + c];
-        for (int e = 0; e < 6; ++e) Vbb[6 * bb + e] += Vbb[6 * ch + e];
-      }
-    }
-    g.sync();
-  }
+  tree_up<6>(g, m, Vbb);             // V_child = V_parent + ...
   // V's own term S_d v_d: vbar_d += Vbar . S_d, Sbar_d += Vbar v_d (per dof, per dof component)
-  for (int t = g.lane; t < 7 * nv; t += G) {
-    if (t < nv) {
-      const int i = t;
-      const double* vbar6 = Vbb + 6 * m.dof_body[i]; const double* sd = S + 6 * i;
-      double s1 = 0.0;
-      for (int e = 0; e < 6; ++e) s1 += vbar6[e] * sd[e];
-      vb[i] += s1;
-    } else {
-      const int k = t - nv, i = k / 6, e = k - 6 * (k / 6);
-      Sb[6 * i + e] += Vbb[6 * m.dof_body[i] + e] * v[i];
-    }
+  for (int i = g.lane; i < nv; i += G) {
+    const double* vbar6 = Vbb + 6 * m.dof_body[i]; const double* sd = S + 6 * i;
+    double s1 = 0.0;
+    for (int e = 0; e < 6; ++e) s1 += vbar6[e] * sd[e];
+    vb[i] += s1;
   }
-  g.sync();
+  for (int k = g.lane; k < 6 * nv; k += G) {
+    const int i = k / 6, e = k - 6 * i;
+    Sb[6 * i + e] += Vbb[6 * m.dof_body[i] + e] * v[i];
+  }
   // actuators: motor tau += gear u; position servo tau += kp (u - q) - kd v
-  if (g.lane == 0) {
-    for (int a = 0; a < m.nact; ++a) {
-      const int vi = m.a_vadr[a];
-      if (m.a_type[a] == ACT_MOTOR) ub[a] += m.a_gear[a] * y[vi];
-      else { ub[a] += m.a_kp[a] * y[vi]; qb[m.a_qadr[a]] -= m.a_kp[a] * y[vi]; vb[vi] -= m.a_kd[a] * y[vi]; }
+  for (int i = g.lane; i < nv; i += G)
+    for (int a = m.dof_act[i]; a >= 0; a = m.act_next[a]) {
+      if (m.a_type[a] == ACT_MOTOR) ub[a] += m.a_gear[a] * y[i];
+      else { ub[a] += m.a_kp[a] * y[i]; qb[m.a_qadr[a]] -= m.a_kp[a] * y[i]; vb[i] -= m.a_kd[a] * y[i]; }
     }
-  }
   // ---- kinematics (forward: local rotation Rl = Roff Rj(theta) or the free joint's
   // pose; R = R_parent Rl, p = p_parent + R_parent b_pos; then COMs, inertias,
   // motion vectors and geoms from (R, p)).  Own terms of every body first, split
@@ -774,89 +737,88 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // one pose entry per task (inertia, COM and motion-vector terms) and one
   // local-rotation entry per task for the composition.
   double* SCb = b.at(LB.sc); double* TK = b.at(LB.tk);
-  for (int t = g.lane; t < 4 * nb; t += G) {
-    if (t < nb) {
-      if (m.b_jtype[t] == JNT_HINGE) ::sincos(q[m.b_qadr[t]], &SCb[2 * t], &SCb[2 * t + 1]);
-    } else {
-      const int k = t - nb, bb = k / 3, r = k - 3 * (k / 3);
-      const double ms = m.b_mass[bb];
-      const double* ib = Ibb + 10 * bb; const double* c = C + 3 * bb;
-      // Ibar as a symmetric matrix B (diagonal ib[4..6], (0,1) ib[7], (0,2) ib[8], (1,2) ib[9])
-      const double Br[3] = {r == 0 ? 2.0 * ib[4] : (r == 1 ? ib[7] : ib[8]),
-                            r == 0 ? ib[7] : (r == 1 ? 2.0 * ib[5] : ib[9]),
-                            r == 0 ? ib[8] : (r == 1 ? ib[9] : 2.0 * ib[6])};
-      const double tr = ib[4] + ib[5] + ib[6];
-      cp[k] = ms * (ib[1 + r] + 2.0 * c[r] * tr - (Br[0] * c[0] + Br[1] * c[1] + Br[2] * c[2]));
-    }
+  for (int t = g.lane; t < nb; t += G)
+    if (m.b_jtype[t] == JNT_HINGE) ::sincos(q[m.b_qadr[t]], &SCb[2 * t], &SCb[2 * t + 1]);
+  for (int k = g.lane; k < 3 * nb; k += G) {
+    const int bb = k / 3, r = k - 3 * (k / 3);
+    const double ms = m.b_mass[bb];
+    const double* ib = Ibb + 10 * bb; const double* c = C + 3 * bb;
+    // Ibar as a symmetric matrix B (diagonal ib[4..6], (0,1) ib[7], (0,2) ib[8], (1,2) ib[9])
+    const double Br[3] = {r == 0 ? 2.0 * ib[4] : (r == 1 ? ib[7] : ib[8]),
+                          r == 0 ? ib[7] : (r == 1 ? 2.0 * ib[5] : ib[9]),
+                          r == 0 ? ib[8] : (r == 1 ? ib[9] : 2.0 * ib[6])};
+    const double tr = ib[4] + ib[5] + ib[6];
+    cp[k] = ms * (ib[1 + r] + 2.0 * c[r] * tr - (Br[0] * c[0] + Br[1] * c[1] + Br[2] * c[2]));
   }
   g.sync();
-  for (int t = g.lane; t < 21 * nb; t += G) {
-    if (t < 12 * nb) {
-      const int bb = t / 12, comp = t - 12 * (t / 12);
-      const double* Rv = R + 9 * bb; const double* pv = P + 3 * bb;
-      const double* cb3 = cp + 3 * bb;
-      const int va = m.b_vadr[bb];
-      const bool fr = m.b_jtype[bb] == JNT_FREE;
-      if (comp < 9) {
-        const int r = comp / 3, kk = comp - 3 * (comp / 3);
-        const double* ib = Ibb + 10 * bb;
-        const double Br[3] = {r == 0 ? 2.0 * ib[4] : (r == 1 ? ib[7] : ib[8]),
-                              r == 0 ? ib[7] : (r == 1 ? 2.0 * ib[5] : ib[9]),
-                              r == 0 ? ib[8] : (r == 1 ? ib[9] : 2.0 * ib[6])};
-        double val = m.b_inertia[bb][kk] * (Br[0] * Rv[kk] + Br[1] * Rv[3 + kk] + Br[2] * Rv[6 + kk]);
-        val += cb3[r] * m.b_com[bb][kk];
-        // motion vectors: free angular dof kk = column kk of R (lin = p x col);
-        // hinge: sh = R axis (lin = p x sh)
-        const double* sbd = Sb + 6 * (fr ? va + 3 + kk : va);
-        const int r1 = nxt3(r), r2 = prv3(r);
-        const double wb = sbd[r] + (sbd[3 + r1] * pv[r2] - sbd[3 + r2] * pv[r1]);
-        val += fr ? wb : wb * m.b_axis[bb][kk];
-        Rb[9 * bb + comp] += val;
-      } else {
-        const int r = comp - 9, r1 = nxt3(r), r2 = prv3(r);
-        double val = cb3[r];
-        if (fr) {
-          for (int d = 0; d < 3; ++d) {
-            const double* sv = Sb + 6 * (va + 3 + d) + 3;
-            val += Rv[3 * r1 + d] * sv[r2] - Rv[3 * r2 + d] * sv[r1];
-          }
-        } else {
-          const double* sv = Sb + 6 * va + 3;
-          const double* ax = m.b_axis[bb];
-          const double sh1 = Rv[3 * r1] * ax[0] + Rv[3 * r1 + 1] * ax[1] + Rv[3 * r1 + 2] * ax[2];
-          const double sh2 = Rv[3 * r2] * ax[0] + Rv[3 * r2 + 1] * ax[1] + Rv[3 * r2 + 2] * ax[2];
-          val += sh1 * sv[r2] - sh2 * sv[r1];
-        }
-        pb[3 * bb + r] += val;
+  for (int t = g.lane; t < 9 * nb; t += G) {
+    const int bb = t / 9, comp = t - 9 * bb;
+    const double* Rv = R + 9 * bb; const double* pv = P + 3 * bb;
+    const double* cb3 = cp + 3 * bb;
+    const int va = m.b_vadr[bb];
+    const bool fr = m.b_jtype[bb] == JNT_FREE;
+    const int r = comp / 3, kk = comp - 3 * (comp / 3);
+    const double* ib = Ibb + 10 * bb;
+    const double Br[3] = {r == 0 ? 2.0 * ib[4] : (r == 1 ? ib[7] : ib[8]),
+                          r == 0 ? ib[7] : (r == 1 ? 2.0 * ib[5] : ib[9]),
+                          r == 0 ? ib[8] : (r == 1 ? ib[9] : 2.0 * ib[6])};
+    double val = m.b_inertia[bb][kk] * (Br[0] * Rv[kk] + Br[1] * Rv[3 + kk] + Br[2] * Rv[6 + kk]);
+    val += cb3[r] * m.b_com[bb][kk];
+    // motion vectors: free angular dof kk = column kk of R (lin = p x col);
+    // hinge: sh = R axis (lin = p x sh)
+    const double* sbd = Sb + 6 * (fr ? va + 3 + kk : va);
+    const int r1 = nxt3(r), r2 = prv3(r);
+    const double wb = sbd[r] + (sbd[3 + r1] * pv[r2] - sbd[3 + r2] * pv[r1]);
+    val += fr ? wb : wb * m.b_axis[bb][kk];
+    Rb[9 * bb + comp] += val;
+  }
+  for (int t = g.lane; t < 3 * nb; t += G) {
+    const int bb = t / 3, r = t - 3 * bb, r1 = nxt3(r), r2 = prv3(r);
+    const double* Rv = R + 9 * bb;
+    const int va = m.b_vadr[bb];
+    double val = cp[t];
+    if (m.b_jtype[bb] == JNT_FREE) {
+      for (int d = 0; d < 3; ++d) {
+        const double* sv = Sb + 6 * (va + 3 + d) + 3;
+        val += Rv[3 * r1 + d] * sv[r2] - Rv[3 * r2 + d] * sv[r1];
       }
     } else {
-      const int k = t - 12 * nb, bb = k / 9, e = k - 9 * (k / 9);
-      if (m.b_jtype[bb] != JNT_HINGE) continue;
-      const int i = e / 3, j = e - 3 * (e / 3);
-      const double sn = SCb[2 * bb], cs = SCb[2 * bb + 1];
+      const double* sv = Sb + 6 * va + 3;
       const double* ax = m.b_axis[bb];
-      double val;
-      if (m.b_ident[bb]) {
-        val = hinge_entry(ax, sn, cs, i, j);
-      } else {
-        const double* Ro = m.b_Roff[bb];
-        val = Ro[3 * i] * hinge_entry(ax, sn, cs, 0, j) + Ro[3 * i + 1] * hinge_entry(ax, sn, cs, 1, j) +
-              Ro[3 * i + 2] * hinge_entry(ax, sn, cs, 2, j);
-      }
-      cR[9 * bb + e] = val;
+      const double sh1 = Rv[3 * r1] * ax[0] + Rv[3 * r1 + 1] * ax[1] + Rv[3 * r1 + 2] * ax[2];
+      const double sh2 = Rv[3 * r2] * ax[0] + Rv[3 * r2 + 1] * ax[1] + Rv[3 * r2 + 2] * ax[2];
+      val += sh1 * sv[r2] - sh2 * sv[r1];
     }
+    pb[t] += val;
+  }
+  for (int k = g.lane; k < 9 * nb; k += G) {
+    const int bb = k / 9, e = k - 9 * (k / 9);
+    if (m.b_jtype[bb] != JNT_HINGE) continue;
+    const int i = e / 3, j = e - 3 * (e / 3);
+    const double sn = SCb[2 * bb], cs = SCb[2 * bb + 1];
+    const double* ax = m.b_axis[bb];
+    double val;
+    if (m.b_ident[bb]) {
+      val = hinge_entry(ax, sn, cs, i, j);
+    } else {
+      const double* Ro = m.b_Roff[bb];
+      val = Ro[3 * i] * hinge_entry(ax, sn, cs, 0, j) + Ro[3 * i + 1] * hinge_entry(ax, sn, cs, 1, j) +
+            Ro[3 * i + 2] * hinge_entry(ax, sn, cs, 2, j);
+    }
+    cR[9 * bb + e] = val;
   }
   g.sync();
   // composition, leaves to root: R_parent gets Rbar Rl^T + pbar b_pos^T, p_parent gets pbar
   // (one parent entry per task)
   for (int lev = m.nlevel - 1; lev >= 1; --lev) {
-    for (int t = 12 * m.level_start[lev - 1] + g.lane; t < 12 * m.level_start[lev]; t += G) {
+    const int k0 = m.level_start[lev - 1], n = 12 * (m.level_start[lev] - k0);
+    for (int t = g.lane; t < n; t += G) {
       const int kb = t / 12, comp = t - 12 * (t / 12);
-      const int bb = m.level_list[kb];
+      const int bb = m.lv_pack[k0 + kb] & 255;
+      const int c0 = m.child_start[bb], nc = m.child_count[bb];
       double acc = 0.0;
-      for (int c = 0; c < m.child_count[bb]; ++c) {
-        const int ch = m.child_list[m.child_start[bb] + c];
-        if (m.b_jtype[ch] == JNT_FREE) continue;
+      for (int c = 0; c < nc; ++c) {
+        const int ch = m.child_list[c0 + c];
         const double* rc = Rb + 9 * ch; const double* pc = pb + 3 * ch;
         if (comp < 9) {
           const int i = comp / 3, j = comp - 3 * (comp / 3);
@@ -867,40 +829,40 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
           acc += pc[comp - 9];
         }
       }
-      if (comp < 9) Rb[9 * bb + comp] += acc; else pb[3 * bb + comp - 9] += acc;
+      if (nc > 0) {
+        if (comp < 9) Rb[9 * bb + comp] += acc; else pb[3 * bb + comp - 9] += acc;
+      }
     }
     g.sync();
   }
   // joint coordinates: free joints (translation, quaternion), one task per body;
   // hinges: theta bar = <Roff^T R_parent^T Rbar, dRj/dtheta>, one entry per task
-  for (int t = g.lane; t < 10 * nb; t += G) {
-    if (t < nb) {
-      const int bb = t;
-      if (m.b_jtype[bb] != JNT_FREE) continue;
-      const double* rb = Rb + 9 * bb; const double* pbv = pb + 3 * bb;
-      const int qa = m.b_qadr[bb];
-      qb[qa] += pbv[0]; qb[qa + 1] += pbv[1]; qb[qa + 2] += pbv[2];
-      quat_to_mat_vjp(q + qa + 3, rb, qb + qa + 3);
-    } else {
-      const int k = t - nb, bb = k / 9, e = k - 9 * (k / 9);
-      if (m.b_jtype[bb] != JNT_HINGE) continue;
-      const int i = e / 3, j = e - 3 * (e / 3);
-      const double* rb = Rb + 9 * bb;
-      const int par = m.b_parent[bb];
-      double rl[3];   // column j of R_parent^T Rbar
-      for (int kk = 0; kk < 3; ++kk)
-        rl[kk] = par >= 0 ? R[9 * par + kk] * rb[j] + R[9 * par + 3 + kk] * rb[3 + j] + R[9 * par + 6 + kk] * rb[6 + j]
-                          : rb[3 * kk + j];
-      const double* Ro = m.b_Roff[bb];
-      const double rjb = Ro[i] * rl[0] + Ro[3 + i] * rl[1] + Ro[6 + i] * rl[2];
-      // dRj/dtheta (i, j) = sin (a_i a_j - delta_ij) + cos K_ij, K = [a]x
-      const double* ax = m.b_axis[bb];
-      const double sn = SCb[2 * bb], cs = SCb[2 * bb + 1];
-      double dr = sn * ax[i] * ax[j];
-      if (i == j) dr -= sn;
-      else dr += (j == nxt3(i)) ? -cs * ax[3 - i - j] : cs * ax[3 - i - j];
-      TK[k] = rjb * dr;
-    }
+  for (int bb = g.lane; bb < nb; bb += G) {
+    if (m.b_jtype[bb] != JNT_FREE) continue;
+    const double* rb = Rb + 9 * bb; const double* pbv = pb + 3 * bb;
+    const int qa = m.b_qadr[bb];
+    qb[qa] += pbv[0]; qb[qa + 1] += pbv[1]; qb[qa + 2] += pbv[2];
+    quat_to_mat_vjp(q + qa + 3, rb, qb + qa + 3);
+  }
+  for (int k = g.lane; k < 9 * nb; k += G) {
+    const int bb = k / 9, e = k - 9 * (k / 9);
+    if (m.b_jtype[bb] != JNT_HINGE) continue;
+    const int i = e / 3, j = e - 3 * (e / 3);
+    const double* rb = Rb + 9 * bb;
+    const int par = m.b_parent[bb];
+    double rl[3];   // column j of R_parent^T Rbar
+    for (int kk = 0; kk < 3; ++kk)
+      rl[kk] = par >= 0 ? R[9 * par + kk] * rb[j] + R[9 * par + 3 + kk] * rb[3 + j] + R[9 * par + 6 + kk] * rb[6 + j]
+                        : rb[3 * kk + j];
+    const double* Ro = m.b_Roff[bb];
+    const double rjb = Ro[i] * rl[0] + Ro[3 + i] * rl[1] + Ro[6 + i] * rl[2];
+    // dRj/dtheta (i, j) = sin (a_i a_j - delta_ij) + cos K_ij, K = [a]x
+    const double* ax = m.b_axis[bb];
+    const double sn = SCb[2 * bb], cs = SCb[2 * bb + 1];
+    double dr = sn * ax[i] * ax[j];
+    if (i == j) dr -= sn;
+    else dr += (j == nxt3(i)) ? -cs * ax[3 - i - j] : cs * ax[3 - i - j];
+    TK[k] = rjb * dr;
   }
   g.sync();
   for (int bb = g.lane; bb < nb; bb += G) {
