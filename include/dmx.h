@@ -197,9 +197,10 @@ dmx_status dmx_model_params(const dmx_model* m, int32_t* np, double* values);
  * derivative with respect to the masses and box sides).  p_bar [np][B] receives
  * it per environment; p_bar_sum [np] (may be NULL) the sum over the
  * environments (a fixed-order reduction: the batch's gradient when every
- * environment shares the model).  Computed by the forward-mode adjoint kernel
- * (one derivative direction per lane: the states, controls and parameters),
- * whatever dmx_set_adjoint selects.  Device pointers, ordered on `stream`. */
+ * environment shares the model).  Computed by the kernel that dmx_set_adjoint
+ * selects: the reverse-mode one collects the parameters' cotangents of every
+ * right-hand side beside the states' (8, 16 or 32 lanes), the tangent one runs
+ * a derivative direction per parameter.  Device pointers, ordered on `stream`. */
 dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* tape, int32_t cfd, const double* xT_bar,
                                    const double* xb_bar, double* x0_bar, double* ctrl_bar, double* p_bar,
                                    double* p_bar_sum, void* stream);

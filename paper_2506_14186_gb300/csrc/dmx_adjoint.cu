@@ -24,8 +24,8 @@
 #include "dmx_device.cuh"
 
 namespace dmx {
-template <int G> cudaError_t launch_adjoint_rev_g(const AdjParams&, int, int, size_t, cudaStream_t);
-template <int G> int occupancy_adjoint_rev_g(int, size_t);
+template <int G, bool PAR> cudaError_t launch_adjoint_rev_g(const AdjParams&, int, int, size_t, cudaStream_t);
+template <int G, bool PAR> int occupancy_adjoint_rev_g(int, size_t);
 template <int G>
 cudaError_t launch_eval_rhs_vjp_g(const AdjParams&, const double*, const double*, const double*, const double*, double*,
                                   double*, double*, int*, int, size_t, cudaStream_t);
@@ -295,22 +295,23 @@ int adjoint_workspace_limit() { return ADJ_WS; }
 int adjoint_int_limit() { return ADJ_WI; }
 
 cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
+  const bool par = P.p_bar != nullptr;
   switch (G) {
-    case 2: return launch_adjoint_rev_g<2>(P, blocks, threads, smem, st);
-    case 4: return launch_adjoint_rev_g<4>(P, blocks, threads, smem, st);
-    case 8: return launch_adjoint_rev_g<8>(P, blocks, threads, smem, st);
-    case 16: return launch_adjoint_rev_g<16>(P, blocks, threads, smem, st);
-    case 32: return launch_adjoint_rev_g<32>(P, blocks, threads, smem, st);
+    case 2: return par ? cudaErrorInvalidValue : launch_adjoint_rev_g<2, false>(P, blocks, threads, smem, st);
+    case 4: return par ? cudaErrorInvalidValue : launch_adjoint_rev_g<4, false>(P, blocks, threads, smem, st);
+    case 8: return par ? launch_adjoint_rev_g<8, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<8, false>(P, blocks, threads, smem, st);
+    case 16: return par ? launch_adjoint_rev_g<16, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<16, false>(P, blocks, threads, smem, st);
+    case 32: return par ? launch_adjoint_rev_g<32, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<32, false>(P, blocks, threads, smem, st);
   }
   return cudaErrorInvalidValue;
 }
-int adjoint_rev_occupancy(int G, int threads, size_t smem) {
+int adjoint_rev_occupancy(int G, bool par, int threads, size_t smem) {
   switch (G) {
-    case 2: return occupancy_adjoint_rev_g<2>(threads, smem);
-    case 4: return occupancy_adjoint_rev_g<4>(threads, smem);
-    case 8: return occupancy_adjoint_rev_g<8>(threads, smem);
-    case 16: return occupancy_adjoint_rev_g<16>(threads, smem);
-    case 32: return occupancy_adjoint_rev_g<32>(threads, smem);
+    case 2: return occupancy_adjoint_rev_g<2, false>(threads, smem);
+    case 4: return occupancy_adjoint_rev_g<4, false>(threads, smem);
+    case 8: return par ? occupancy_adjoint_rev_g<8, true>(threads, smem) : occupancy_adjoint_rev_g<8, false>(threads, smem);
+    case 16: return par ? occupancy_adjoint_rev_g<16, true>(threads, smem) : occupancy_adjoint_rev_g<16, false>(threads, smem);
+    case 32: return par ? occupancy_adjoint_rev_g<32, true>(threads, smem) : occupancy_adjoint_rev_g<32, false>(threads, smem);
   }
   return 0;
 }

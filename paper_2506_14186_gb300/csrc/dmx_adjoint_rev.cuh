@@ -109,7 +109,7 @@ __device__ __forceinline__ Ws snap_view(const DevModel& m, const Ws& w, const do
 // b.vst.  Qb and Vb are consumed (left zero).  snaps: the step's S - 1 stage
 // snapshots (SN doubles each), or null to evaluate each stage's right-hand
 // side.  Returns the worst right-hand-side status.
-template <int G>
+template <int G, bool PAR>
 __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const WsB& b, const double* u,
                            double h, int mt, bool cfd, const double* snaps, int SN) {
   const Layout& L = *w.L;
@@ -146,7 +146,8 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
       const double* sn = snaps ? snaps + (size_t)s * SN : nullptr;
       const int r = sn ? snap_restore(g, m, w, sn) : rhs(g, m, w, (const double*)Qs, Vs, u, cfd, w.at(L.ka));
       if (r > st) st = r;
-      rhs_vjp(g, m, sn ? snap_view(m, w, sn) : w, b, Qs, Vs, u, cfd, r, kab + s * nv, Qb, Vb, ub);
+      rhs_vjp<G, PAR>(g, m, sn ? snap_view(m, w, sn) : w, b, Qs, Vs, u, cfd, r, kab + s * nv, Qb, Vb, ub,
+                      PAR ? b.at(LB.pa) : nullptr);
       for (int i = g.lane; i < nv; i += G) Vb[i] += kvb[s * nv + i];   // V_s in the later stages' positions
       g.sync();
     }
@@ -173,7 +174,8 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
   return st;
 }
 
-template <int G>
+// PAR: with the model-parameter gradients (p_bar).
+template <int G, bool PAR>
 __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
   extern __shared__ double smem[];
   __shared__ Layout sL;
@@ -207,6 +209,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
     for (int i = g.lane; i < nx; i += G) xbar[i] = P.xT_bar[(size_t)i * P.B + env];
     if (P.ctrl_bar)
       for (int i = g.lane; i < P.NI * nu; i += G) P.ctrl_bar[(size_t)i * P.B + env] = 0.0;
+    if constexpr (PAR)
+      for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] = 0.0;
     if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
     g.sync();
     int worst = 0;
@@ -259,6 +263,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
       // ---- reverse sweep over the segment's steps
       double* bq = b.at(sB.qn); double* bv = b.at(sB.vst);
       double* Qb = b.at(sB.Qb); double* Vb = b.at(sB.Vb);
+      if constexpr (PAR)               // the segment's sums live in the cotangent workspace
+        for (int k = g.lane; k < P.np; k += G) b.at(sB.pa)[k] = 0.0;
       for (int n = n1 - 1; n >= n0; --n) {
         const double* row = seg + (size_t)(n - n0) * RW;
         const double tn0 = row[nq + 7 * nv];
@@ -275,7 +281,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
         for (int i = g.lane; i < nq; i += G) Qb[i] = xbar[i];
         for (int i = g.lane; i < nv; i += G) Vb[i] = xbar[nq + i];
         g.sync();
-        const int st = rk_step_vjp(g, m, w, b, (const double*)u, h, mt, P.cfd != 0,
+        const int st = rk_step_vjp<G, PAR>(g, m, w, b, (const double*)u, h, mt, P.cfd != 0,
                                    use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr, SN);
         if (st > worst) worst = st;
         const double* qnb = b.at(sB.qnb); const double* vnb = b.at(sB.vnb); const double* ub = b.at(sB.ub);
@@ -285,6 +291,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
           for (int a = g.lane; a < nu; a += G) P.ctrl_bar[((size_t)kn * nu + a) * P.B + env] += ub[a];
         g.sync();
       }
+      if constexpr (PAR)
+        for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] += b.at(sB.pa)[k];
       g.sync();
     }
     if (P.xb_bar)
@@ -293,6 +301,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
     // a right-hand side whose rows overflowed the workspace has no derivative: mark the result
     const double bad = (worst == ENV_ROW_OVERFLOW) ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
     for (int i = g.lane; i < nx; i += G) P.x0_bar[(size_t)i * P.B + env] = xbar[i] + bad;
+    if constexpr (PAR)
+      for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] += bad;
     g.sync();
   }
 }
@@ -301,7 +311,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
 // u [nu][B], abar [nv][B]) into qbar [nq][B], vbar [nv][B], ubar [nu][B]
 // (ubar only when nu > 0); status [B] = rhs status.
 template <int G>
-__global__ void __launch_bounds__(32) k_eval_rhs_vjp(AdjParams P, const double* q, const double* v, const double* u,
+__global__ void __launch_bounds__(32, 1) k_eval_rhs_vjp(AdjParams P, const double* q, const double* v, const double* u,
                                                       const double* abar, double* qbar, double* vbar, double* ubar,
                                                       int* status) {
   extern __shared__ double smem[];
@@ -346,17 +356,17 @@ cudaError_t launch_eval_rhs_vjp_g(const AdjParams& P, const double* q, const dou
   return cudaGetLastError();
 }
 
-template <int G>
+template <int G, bool PAR>
 cudaError_t launch_adjoint_rev_g(const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
-  auto k = k_adjoint_rev<G>;
+  auto k = k_adjoint_rev<G, PAR>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k<<<blocks, threads, smem, st>>>(P);
   return cudaGetLastError();
 }
-template <int G>
+template <int G, bool PAR>
 int occupancy_adjoint_rev_g(int threads, size_t smem) {
-  auto k = k_adjoint_rev<G>;
+  auto k = k_adjoint_rev<G, PAR>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;

@@ -198,11 +198,12 @@ struct LayoutBar {
   int gb, iv, ivb;                   // geom pose cotangents, I V and its cotangent per body
   int sc, tk;                        // hinge sine and cosine, theta-cotangent terms per body
   int qn, vst, dq, dqb, Qs, kab, kvb, Qb, Vb, qnb, vnb, ub, xb;            // one step
+  int pr, pd, pa;                    // model parameters: slot records (8 each), bcoef terms per dof, sums
   int nd;                            // doubles per environment (padded to even)
 };
 constexpr int SLOTBAR = 24;          // at most per slot: pose cotangents of its two geoms (R 9 + p 3 each)
 
-DMX_HD inline LayoutBar make_bar_layout(const DevModel& m, int rcap) {
+DMX_HD inline LayoutBar make_bar_layout(const DevModel& m, int rcap, bool params = false) {
   LayoutBar B{};
   int o = 0;
   const int nq = m.nq, nv = m.nv, nb = m.nbody, ns = m.nslot > 0 ? m.nslot : 1, nu = m.nu > 0 ? m.nu : 1;
@@ -218,6 +219,8 @@ DMX_HD inline LayoutBar make_bar_layout(const DevModel& m, int rcap) {
   B.qn = take(nq); B.vst = take(7 * nv); B.dq = take(nv); B.dqb = take(nv); B.Qs = take(nq);
   B.kab = take(6 * nv); B.kvb = take(6 * nv); B.Qb = take(nq); B.Vb = take(nv);
   B.qnb = take(nq); B.vnb = take(nv); B.ub = take(nu); B.xb = take(nq + nv);
+  B.pr = B.pd = B.pa = o;
+  if (params) { B.pr = take(8 * ns); B.pd = take(nv); B.pa = take(PAR_MU0 + m.npair + m.nbody + m.nbox); }
   B.nd = (o + 1) & ~1;
   return B;
 }

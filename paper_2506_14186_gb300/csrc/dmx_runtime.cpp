@@ -708,54 +708,16 @@ extern "C" dmx_status dmx_model_params(const dmx_model* m, int32_t* np, double* 
   return DMX_OK;
 }
 
-extern "C" dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* t, int32_t cfd, const double* xT_bar,
-                                              const double* xb_bar, double* x0_bar, double* ctrl_bar, double* p_bar,
-                                              double* p_bar_sum, void* stream) {
-  if (!m || !t) return dmx_fail(DMX_ERR_INVALID, "null model or tape");
-  if (t->model != m) return dmx_fail(DMX_ERR_INVALID, "tape belongs to another model");
-  if (!p_bar) return dmx_fail(DMX_ERR_INVALID, "p_bar is required");
-  const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int np = model_nparams(m);
-  if (t->B == 0) {
-    if (p_bar_sum) CK(cudaMemsetAsync(p_bar_sum, 0, sizeof(double) * np, st));
-    return DMX_OK;
-  }
-  if (!xT_bar || !x0_bar) return dmx_fail(DMX_ERR_INVALID, "xT_bar and x0_bar are required");
-  if (m->host.nu > 0 && !ctrl_bar) return dmx_fail(DMX_ERR_INVALID, "ctrl_bar is required when the model has actuators");
-  dmx::AdjParams P{};
-  P.model = m->dev; P.L = layout_for(m, cfd); P.B = t->B; P.NI = t->NI; P.K = t->K; P.cfd = cfd; P.method = t->method;
-  P.ckpt = t->ckpt; P.hlog = t->hlog; P.tape_n = t->n; P.ctrl = t->ctrl; P.T = t->T;
-  P.xT_bar = xT_bar; P.xb_bar = xb_bar; P.x0_bar = x0_bar; P.ctrl_bar = m->host.nu ? ctrl_bar : nullptr;
-  P.p_bar = p_bar; P.np = np;
-  const dmx_status s = run_tangent_adjoint(m, t, P, st);
-  if (s != DMX_OK) return s;
-  if (p_bar_sum) CK(dmx::launch_row_sums(p_bar, np, t->B, p_bar_sum, st));
-  return DMX_OK;
-}
-
-extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, const double* xT_bar,
-                                       const double* xb_bar, double* x0_bar, double* ctrl_bar, void* stream) {
-  if (!m || !t) return dmx_fail(DMX_ERR_INVALID, "null model or tape");
-  if (t->model != m) return dmx_fail(DMX_ERR_INVALID, "tape belongs to another model");
-  if (t->B == 0) return DMX_OK;
-  if (!xT_bar || !x0_bar) return dmx_fail(DMX_ERR_INVALID, "xT_bar and x0_bar are required");
-  if (m->host.nu > 0 && !ctrl_bar) return dmx_fail(DMX_ERR_INVALID, "ctrl_bar is required when the model has actuators");
-  const cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int nx = t->nx;
-  int mode;
-  {
-    std::lock_guard<std::mutex> lk(m->mu);
-    mode = m->adj_mode;
-  }
-  dmx::AdjParams P{};
-  const dmx::Layout& L = layout_for(m, cfd);
-  P.model = m->dev; P.L = L; P.B = t->B; P.NI = t->NI; P.K = t->K; P.cfd = cfd; P.method = t->method;
-  P.ckpt = t->ckpt; P.hlog = t->hlog; P.tape_n = t->n; P.ctrl = t->ctrl; P.T = t->T;
-  P.xT_bar = xT_bar; P.xb_bar = xb_bar; P.x0_bar = x0_bar; P.ctrl_bar = m->host.nu ? ctrl_bar : nullptr;
-  if (mode == DMX_ADJ_TANGENT) return run_tangent_adjoint(m, t, P, st);
-  const int G = adjoint_lanes(m, t->B, L, true);
-  P.LB = dmx::make_bar_layout(m->host, L.rcap);
-  const int gpb = 32 / G, threads = 32;
+// The reverse-mode adjoint kernel (with the model-parameter gradients when
+// P.p_bar is set); L: layout of its right-hand side.
+static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams& P, const dmx::Layout& L, int mode,
+                                      cudaStream_t st) {
+  const int cfd = P.cfd;
+  const bool par = P.p_bar != nullptr;
+  int G = adjoint_lanes(m, t->B, L, true);
+  if (par && G < 8) G = 8;             // compiled lane counts
+  P.LB = dmx::make_bar_layout(m->host, L.rcap, par);
+  const int threads = 32;
   const int RW = dmx::rev_row_doubles(m->host);
   const int nsnap = t->method == DMX_METHOD_EULER ? 1 : 6;   // stage right-hand sides per step
   // Launch plan for a workspace layout: doubles per environment, the cotangent
@@ -766,13 +728,14 @@ extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, c
     size_t smem = 0, seg = 0;
   };
   auto plan = [&](const dmx::Layout& Lx, bool overlay, Plan& out) {
+    const int gpb = 32 / G;
     out.L = Lx;
     out.per = overlay ? std::max(Lx.nd, Lx.ovl + P.LB.nd) : Lx.nd + P.LB.nd;
     out.per = (out.per + 1) & ~1;
     out.barofs = overlay ? Lx.ovl : Lx.nd;
     out.smem = (size_t)gpb * ((size_t)out.per * 8 + (size_t)Lx.ni * 4);
     if ((int)out.smem > m->smem_max - 2048) return false;
-    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, threads, out.smem));
+    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, par, threads, out.smem));
     out.blocks = std::min((t->B + gpb - 1) / gpb, m->nsm * occ);
     out.seg = sizeof(double) * (size_t)out.blocks * gpb * t->K * RW;
     return true;
@@ -783,6 +746,9 @@ extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, c
   // recompute uses (dmx::make_layout_adj): fewer bytes per environment, more
   // resident warps.  Otherwise every stage is evaluated again in the sweep.
   Plan pl;
+  if (par)                             // its workspace is larger than the lane choice assumed
+    while (G < 32 && !plan(L, false, pl)) G <<= 1;
+  const int gpb = 32 / G;
   size_t snap_bytes = 0;
   if (mode == DMX_ADJ_REVERSE && !cfd && plan(dmx::make_layout_adj(m->host, L.rcap), true, pl)) {
     P.SN = dmx::snap_offsets(m->host, pl.L).size;
@@ -807,6 +773,59 @@ extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, c
   CK(dmx::launch_adjoint_rev(G, P, blocks, threads, smem, st));
   CK(cudaFreeAsync(scratch, st));
   return DMX_OK;
+}
+
+extern "C" dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* t, int32_t cfd, const double* xT_bar,
+                                              const double* xb_bar, double* x0_bar, double* ctrl_bar, double* p_bar,
+                                              double* p_bar_sum, void* stream) {
+  if (!m || !t) return dmx_fail(DMX_ERR_INVALID, "null model or tape");
+  if (t->model != m) return dmx_fail(DMX_ERR_INVALID, "tape belongs to another model");
+  if (!p_bar) return dmx_fail(DMX_ERR_INVALID, "p_bar is required");
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const int np = model_nparams(m);
+  if (t->B == 0) {
+    if (p_bar_sum) CK(cudaMemsetAsync(p_bar_sum, 0, sizeof(double) * np, st));
+    return DMX_OK;
+  }
+  if (!xT_bar || !x0_bar) return dmx_fail(DMX_ERR_INVALID, "xT_bar and x0_bar are required");
+  if (m->host.nu > 0 && !ctrl_bar) return dmx_fail(DMX_ERR_INVALID, "ctrl_bar is required when the model has actuators");
+  dmx::AdjParams P{};
+  P.model = m->dev; P.L = layout_for(m, cfd); P.B = t->B; P.NI = t->NI; P.K = t->K; P.cfd = cfd; P.method = t->method;
+  P.ckpt = t->ckpt; P.hlog = t->hlog; P.tape_n = t->n; P.ctrl = t->ctrl; P.T = t->T;
+  P.xT_bar = xT_bar; P.xb_bar = xb_bar; P.x0_bar = x0_bar; P.ctrl_bar = m->host.nu ? ctrl_bar : nullptr;
+  P.p_bar = p_bar; P.np = np;
+  int mode;
+  {
+    std::lock_guard<std::mutex> lk(m->mu);
+    mode = m->adj_mode;
+  }
+  const dmx_status s = mode == DMX_ADJ_TANGENT ? run_tangent_adjoint(m, t, P, st)
+                                               : run_reverse_adjoint(m, t, P, layout_for(m, cfd), mode, st);
+  if (s != DMX_OK) return s;
+  if (p_bar_sum) CK(dmx::launch_row_sums(p_bar, np, t->B, p_bar_sum, st));
+  return DMX_OK;
+}
+
+extern "C" dmx_status dmx_rollout_grad(dmx_model* m, dmx_tape* t, int32_t cfd, const double* xT_bar,
+                                       const double* xb_bar, double* x0_bar, double* ctrl_bar, void* stream) {
+  if (!m || !t) return dmx_fail(DMX_ERR_INVALID, "null model or tape");
+  if (t->model != m) return dmx_fail(DMX_ERR_INVALID, "tape belongs to another model");
+  if (t->B == 0) return DMX_OK;
+  if (!xT_bar || !x0_bar) return dmx_fail(DMX_ERR_INVALID, "xT_bar and x0_bar are required");
+  if (m->host.nu > 0 && !ctrl_bar) return dmx_fail(DMX_ERR_INVALID, "ctrl_bar is required when the model has actuators");
+  const cudaStream_t st = static_cast<cudaStream_t>(stream);
+  int mode;
+  {
+    std::lock_guard<std::mutex> lk(m->mu);
+    mode = m->adj_mode;
+  }
+  dmx::AdjParams P{};
+  const dmx::Layout& L = layout_for(m, cfd);
+  P.model = m->dev; P.L = L; P.B = t->B; P.NI = t->NI; P.K = t->K; P.cfd = cfd; P.method = t->method;
+  P.ckpt = t->ckpt; P.hlog = t->hlog; P.tape_n = t->n; P.ctrl = t->ctrl; P.T = t->T;
+  P.xT_bar = xT_bar; P.xb_bar = xb_bar; P.x0_bar = x0_bar; P.ctrl_bar = m->host.nu ? ctrl_bar : nullptr;
+  if (mode == DMX_ADJ_TANGENT) return run_tangent_adjoint(m, t, P, st);
+  return run_reverse_adjoint(m, t, P, L, mode, st);
 }
 
 extern "C" dmx_status dmx_eval_rhs_vjp(dmx_model* m, int32_t B, const double* q, const double* v, const double* u,

@@ -133,6 +133,42 @@ __device__ __forceinline__ double impedance_d(const DevModel& m, double r, bool 
   *dd = dr;
   return d;
 }
+// Parameter cotangents of a slot's impedance terms (impedance_terms_vjp):
+// out[0..4] += those of kcoef, d_o, d_w, width, midpoint (the last four through
+// d(r); nothing on the clamped pieces and on the CFD continuation), out[5] that
+// of A_hat.
+__device__ __forceinline__ double softplus_d(double x, double* ds);
+__device__ __forceinline__ void impedance_par_vjp(const DevModel& m, double r, bool cfd, double ahat, double b14,
+                                                  double b15, double* out) {
+  double dd;
+  const double d = impedance_d(m, r, cfd, &dd), om = 1.0 - d;
+  double db;
+  if (cfd) {
+    double sg;
+    const double sp = m.softplus * softplus_d(-r / m.softplus, &sg);
+    out[0] += b14 * d * sp;
+    db = b14 * m.kcoef * sp;
+  } else {
+    out[0] -= b14 * d * r;
+    db = -b14 * m.kcoef * r;
+  }
+  db += b15 / (ahat * om * om);
+  out[5] -= b15 * d / (ahat * ahat * om);
+  if (cfd && r >= 0) return;
+  const double width = m.solimp[2], mid = m.solimp[3], pw = m.solimp[4], span = m.solimp[1] - m.solimp[0];
+  double x = fabs(r) / width, dx = -x / width;
+  if (x > 1.0) { x = 1.0; dx = 0.0; }
+  double dy;
+  const double y = spline_shape_d(x, mid, pw, &dy);
+  const double raw = m.solimp[0] + span * y;
+  if (raw < 0.0 || raw > 0.9999) return;
+  // y = x^p / mid^(p-1), or 1 - (1 - x)^p / (1 - mid)^(p-1)
+  const double dm = (x <= mid && mid > 0) ? -(pw - 1.0) * y / mid : (mid < 1 ? -(pw - 1.0) * (1.0 - y) / (1.0 - mid) : 0.0);
+  out[1] += db * (1.0 - y);
+  out[2] += db * y;
+  out[3] += db * span * dy * dx;
+  out[4] += db * span * dm;
+}
 // softplus and its derivative (the logistic function), both branches as in softplus().
 __device__ __forceinline__ double softplus_d(double x, double* ds) {
   if (x > 0) {
@@ -271,7 +307,7 @@ static __device__ void seg_seg_vjp(const DevModel& m, const double* gR, const do
 }
 
 static __device__ void capsule_box_vjp(const DevModel& m, const double* gR, const double* gp, int g1, int g2,
-                                       double sv, const double* cb, double* b1, double* b2) {
+                                       double sv, const double* cb, double* b1, double* b2, double* hb = nullptr) {
   const double rc = m.g_size[g1][0], Lh = m.g_size[g1][1];
   const double* h = m.g_size[g2];
   const double* R1 = gR + 9 * g1; const double* R2 = gR + 9 * g2;
@@ -328,6 +364,8 @@ static __device__ void capsule_box_vjp(const DevModel& m, const double* gR, cons
     const double c = -sb / phi2;
     for (int i = 0; i < 3; ++i) { y0b[i] += c * a[i]; wvb[i] += c * (gv[i] + sv * a[i]); }
   }
+  if (hb)   // the field depends on |y| - h: half-size cotangents mirror those of y0
+    for (int i = 0; i < 3; ++i) hb[i] = y[i] < 0 ? y0b[i] : -y0b[i];
   double dcb[3];                              // y0 = R2^T dc, wv = R2^T u
   matvec3(R2, y0b, dcb);
   double uw[3];
@@ -397,10 +435,11 @@ __device__ __forceinline__ bool slot_jbar(const DevModel& m, const Ws& w, const 
 
 // qbar, vbar, ubar += (dF/d(q, v, u))^T abar at the inputs of the rhs() call
 // that immediately precedes this one (same q, v, u, cfd; st = its status).
-template <int G>
+// PAR: pacc[k] += the cotangent of model parameter k (owned by lane k mod G).
+template <int G, bool PAR = false>
 __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const WsB& b, const double* q,
                         const double* v, const double* u, bool cfd, int st, const double* abar, double* qbar,
-                        double* vbar, double* ubar) {
+                        double* vbar, double* ubar, double* pacc = nullptr) {
   const Layout& L = *w.L;
   const LayoutBar& LB = *b.L;
   const int nq = m.nq, nv = m.nv, nb = m.nbody;
@@ -475,6 +514,11 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     double acc = -m.b_damping[bi] * y[i];
     for (int r = 0; r < nr; ++r) acc -= m.bcoef * cj[r] * J[r * nv + i];
     vb[i] += acc;
+    if constexpr (PAR) {               // bcoef: a_ref = -bcoef J v + ...
+      double jc = 0.0;
+      for (int r = 0; r < nr; ++r) jc += cj[r] * J[r * nv + i];
+      b.at(LB.pd)[i] = -jc * v[i];
+    }
     double* sbi = Sb + 6 * i;
     const double yai = an[i] + m.bcoef * v[i];
     for (unsigned ms = incl; ms; ms &= ms - 1u) {
@@ -507,6 +551,21 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     const int p = m.s_pair[s];
     const int nrow = m.s_rows[s];
     double cb[13] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    // PAR record: kcoef, d_o, d_w, width, midpoint, A_hat, mu, half size of the slot's box
+    double pr[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if constexpr (PAR) {
+      if (nrow != 1)                   // edge rows n +- mu t
+        for (int i = 0; i < nv; ++i) {
+          double jb[3], pv[3], sg;
+          const double yai = an[i] + m.bcoef * v[i];
+          if (!slot_jbar(m, w, b, s, r0, i, y[i], yai, jb, pv, &sg)) continue;
+          const bool pl = m.p_g2[p] < 0;
+          const double j1 = sg * (pl ? pv[0] : dot3(ct + 7, pv)), j2 = sg * (pl ? pv[1] : dot3(ct + 10, pv));
+          double e[4];
+          for (int k = 0; k < 4; ++k) e[k] = -(cz[r0 + k] * y[i] + cj[r0 + k] * yai);
+          pr[6] += (e[0] - e[1]) * j1 + (e[2] - e[3]) * j2;
+        }
+    }
     if (m.p_g2[p] < 0) {
       // ground plane: the frame is fixed (no frame cotangents), pvb in the world frame
       const unsigned anc = m.s_move[s];
@@ -538,14 +597,19 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     if (r < thr) {
       const double ahat = nrow == 1 ? m.p_ahat[p] : m.p_ahat_edge[p];
       cb[0] += impedance_terms_vjp(m, r, cfd, ahat, b14, b15);
+      if constexpr (PAR) impedance_par_vjp(m, r, cfd, ahat, b14, b15, pr);
     }
     double* b1 = sb; double* b2 = sb + 12;
     for (int k = 0; k < (m.p_g2[p] < 0 ? 12 : 24); ++k) sb[k] = 0.0;
     const int g1 = m.p_g1[p];
     if (m.p_g2[p] >= 0) {
       const double* st = w.at(L.csv) + 2 * s;
-      if (m.g_type[m.p_g2[p]] == GEOM_BOX) capsule_box_vjp(m, gR, gp, g1, m.p_g2[p], st[0], cb, b1, b2);
-      else seg_seg_vjp(m, gR, gp, g1, m.p_g2[p], st[0], st[1], cb, b1, b2);
+      if (m.g_type[m.p_g2[p]] == GEOM_BOX) {
+        double hb[3];
+        capsule_box_vjp(m, gR, gp, g1, m.p_g2[p], st[0], cb, b1, b2, PAR ? hb : nullptr);
+        const double* h = m.g_size[m.p_g2[p]];
+        if constexpr (PAR) pr[7] = (hb[0] * h[0] + hb[1] * h[1] + hb[2] * h[2]) / (2.0 * h[0]);   // all scale with the side
+      } else seg_seg_vjp(m, gR, gp, g1, m.p_g2[p], st[0], st[1], cb, b1, b2);
     } else {
       // r = pt_z - rad, pos = (pt_x, pt_y, pt_z - rad - r / 2); fixed frame
       const double ptb[3] = {cb[1], cb[2], cb[0] + 0.5 * cb[3]};
@@ -560,8 +624,15 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
                               (j & 4) ? m.g_size[g1][2] : -m.g_size[g1][2]};
         for (int a = 0; a < 3; ++a)
           for (int c = 0; c < 3; ++c) b1[3 * a + c] += ptb[a] * ex[c];
+        if constexpr (PAR) {
+          double t[3];
+          matvec3(gR + 9 * g1, ex, t);
+          pr[7] = dot3(ptb, t) / (2.0 * m.g_size[g1][0]);
+        }
       }
     }
+    if constexpr (PAR)
+      for (int k = 0; k < 8; ++k) b.at(LB.pr)[8 * s + k] = pr[k];
   }
   g.sync();
   // ---- per geom: pose cotangents gathered from its slots (one component per task)
@@ -729,6 +800,67 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
       if (m.a_type[a] == ACT_MOTOR) ub[a] += m.a_gear[a] * y[i];
       else { ub[a] += m.a_kp[a] * y[i]; qb[m.a_qadr[a]] -= m.a_kp[a] * y[i]; vb[i] -= m.a_kd[a] * y[i]; }
     }
+  if constexpr (PAR) {
+    // model parameters, one per task: slot records, the per-dof bcoef terms,
+    // spatial inertias (proportional to the mass; rotational part of a body
+    // that is one box proportional to its side squared) and A_hat's dependence
+    // on masses and sides
+    const int np = PAR_MU0 + m.npair + m.nbody + m.nbox;
+    const double* PR = b.at(LB.pr);
+    for (int k = g.lane; k < np; k += G) {
+      double acc = 0.0;
+      if (k < PAR_MU0) {
+        const double dk = k == PAR_TC ? -2.0 * m.kcoef / m.solref[0]
+                        : k == PAR_DAMP ? -2.0 * m.kcoef / m.solref[1]
+                        : k == PAR_DW ? -2.0 * m.kcoef / m.solimp[1] : 0.0;
+        for (unsigned ms = incl; ms; ms &= ms - 1u) {
+          const double* pr = PR + 8 * (__ffs(ms) - 1);
+          acc += dk * pr[0];
+          if (k >= PAR_DO) acc += pr[k - PAR_DO + 1];
+        }
+        const double db = k == PAR_TC ? -m.bcoef / m.solref[0] : k == PAR_DW ? -m.bcoef / m.solimp[1] : 0.0;
+        if (db != 0.0) {
+          double t = 0.0;
+          for (int i = 0; i < nv; ++i) t += b.at(LB.pd)[i];
+          acc += db * t;
+        }
+      } else {
+        const int p0 = k - PAR_MU0, b0 = p0 - m.npair, j0 = b0 - m.nbody;
+        for (unsigned ms = incl; ms; ms &= ms - 1u) {
+          const int s = __ffs(ms) - 1, p = m.s_pair[s];
+          const double* pr = PR + 8 * s;
+          const double mu = m.p_mu[p];
+          const bool edge = m.s_rows[s] != 1;
+          if (b0 < 0) {
+            if (p == p0 && edge) acc += pr[6] + pr[5] * (2.0 * mu * m.p_ahat[p]);
+          } else {
+            acc += pr[5] * (m.p_dahat[p][b0] * (edge ? 1.0 + mu * mu : 1.0));
+            const int gb = m.p_g2[p] < 0 ? m.p_g1[p] : m.p_g2[p];
+            if (j0 >= 0 && m.g_box[gb] == j0) acc += pr[7];
+          }
+        }
+        if (b0 >= 0 && j0 < 0) {
+          double t = 0.0;
+          for (int e = 0; e < 10; ++e) t += Ibb[10 * b0 + e] * Ib[10 * b0 + e];
+          acc += t / m.b_mass[b0];
+        } else if (j0 >= 0) {
+          for (int bb = 0; bb < nb; ++bb) {
+            const int gs = m.b_solebox[bb];
+            if (gs < 0 || m.g_box[gs] != j0) continue;
+            const double* Rv = R + 9 * bb; const double* In = m.b_inertia[bb];
+            double t = 0.0;
+            for (int e = 0; e < 6; ++e) {
+              const int i = e < 3 ? e : (e == 5 ? 1 : 0), j = e < 3 ? e : (e == 3 ? 1 : 2);
+              t += Ibb[10 * bb + 4 + e] * (Rv[3 * i] * Rv[3 * j] * In[0] + Rv[3 * i + 1] * Rv[3 * j + 1] * In[1] +
+                                           Rv[3 * i + 2] * Rv[3 * j + 2] * In[2]);
+            }
+            acc += 2.0 * t / (2.0 * m.g_size[gs][0]);
+          }
+        }
+      }
+      pacc[k] += acc;
+    }
+  }
   // ---- kinematics (forward: local rotation Rl = Roff Rj(theta) or the free joint's
   // pose; R = R_parent Rl, p = p_parent + R_parent b_pos; then COMs, inertias,
   // motion vectors and geoms from (R, p)).  Own terms of every body first, split
