@@ -176,12 +176,10 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
 
 // PAR: with the model-parameter gradients (p_bar).
 template <int G, bool PAR>
-__global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
+__global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ AdjParams P) {
   extern __shared__ double smem[];
-  __shared__ Layout sL;
-  __shared__ LayoutBar sB;
-  if (threadIdx.x == 0) { sL = P.L; sB = P.LB; }
-  __syncthreads();
+  const Layout& sL = P.L;
+  const LayoutBar& sB = P.LB;
   const DevModel& m = *P.model;
   Grp<G> g;
   const int ngb = blockDim.x / G, gib = threadIdx.x / G;
@@ -311,14 +309,12 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(AdjParams P) {
 // u [nu][B], abar [nv][B]) into qbar [nq][B], vbar [nv][B], ubar [nu][B]
 // (ubar only when nu > 0); status [B] = rhs status.
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_eval_rhs_vjp(AdjParams P, const double* q, const double* v, const double* u,
+__global__ void __launch_bounds__(32, 1) k_eval_rhs_vjp(const __grid_constant__ AdjParams P, const double* q, const double* v, const double* u,
                                                       const double* abar, double* qbar, double* vbar, double* ubar,
                                                       int* status) {
   extern __shared__ double smem[];
-  __shared__ Layout sL;
-  __shared__ LayoutBar sB;
-  if (threadIdx.x == 0) { sL = P.L; sB = P.LB; }
-  __syncthreads();
+  const Layout& sL = P.L;
+  const LayoutBar& sB = P.LB;
   const DevModel& m = *P.model;
   Grp<G> g;
   const int ngb = blockDim.x / G, gib = threadIdx.x / G;

@@ -188,10 +188,8 @@ __device__ Ws group_workspace(const RolloutParams& P, const Layout* L) {
 
 // Persistent form: loop { take next env; integrate it to T }.
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_rollout_persistent(RolloutParams P) {
-  __shared__ Layout sL;
-  if (threadIdx.x == 0) sL = P.L;
-  __syncthreads();
+__global__ void __launch_bounds__(32, 1) k_rollout_persistent(const __grid_constant__ RolloutParams P) {
+  const Layout& sL = P.L;
   const DevModel& m = *P.model;
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
@@ -221,10 +219,8 @@ __global__ void __launch_bounds__(32, 1) k_rollout_persistent(RolloutParams P) {
 
 // Plain form, initialisation launch: state of every environment into HBM.
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_step_init(RolloutParams P, StepState S) {
-  __shared__ Layout sL;
-  if (threadIdx.x == 0) sL = P.L;
-  __syncthreads();
+__global__ void __launch_bounds__(32, 1) k_step_init(const __grid_constant__ RolloutParams P, StepState S) {
+  const Layout& sL = P.L;
   const DevModel& m = *P.model;
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
@@ -241,10 +237,8 @@ __global__ void __launch_bounds__(32, 1) k_step_init(RolloutParams P, StepState 
 
 // Plain form, one attempt of every unfinished environment.
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_step(RolloutParams P, StepState S) {
-  __shared__ Layout sL;
-  if (threadIdx.x == 0) sL = P.L;
-  __syncthreads();
+__global__ void __launch_bounds__(32, 1) k_step(const __grid_constant__ RolloutParams P, StepState S) {
+  const Layout& sL = P.L;
   const DevModel& m = *P.model;
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
@@ -264,11 +258,9 @@ __global__ void __launch_bounds__(32, 1) k_step(RolloutParams P, StepState S) {
 // Right-hand side of a batch of states (q [nq][B], v [nv][B], u [nu][B]) into
 // a [nv][B]; info [4][B]: status, rows, active rows, Newton solves.
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_eval_rhs(RolloutParams P, const double* q, const double* v, const double* u,
+__global__ void __launch_bounds__(32, 1) k_eval_rhs(const __grid_constant__ RolloutParams P, const double* q, const double* v, const double* u,
                                                   int cfd, double* a, int* info) {
-  __shared__ Layout sL;
-  if (threadIdx.x == 0) sL = P.L;
-  __syncthreads();
+  const Layout& sL = P.L;
   const DevModel& m = *P.model;
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);

@@ -103,12 +103,10 @@ __device__ int otd_stage(const Grp<G>& g, const DevModel& m, const Ws& w, const 
 }
 
 template <int G>
-__global__ void __launch_bounds__(32, 1) k_adjoint_otd(OtdParams P) {
+__global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ OtdParams P) {
   extern __shared__ double smem[];
-  __shared__ Layout sL;
-  __shared__ LayoutBar sB;
-  if (threadIdx.x == 0) { sL = P.L; sB = P.LB; }
-  __syncthreads();
+  const Layout& sL = P.L;
+  const LayoutBar& sB = P.LB;
   const DevModel& m = *P.model;
   Grp<G> g;
   const int ngb = blockDim.x / G, gib = threadIdx.x / G;
