@@ -59,11 +59,7 @@ struct Grp {
     const unsigned b = __ballot_sync(mask, p);
     return G == 32 ? b : (b >> base) & ((1u << G) - 1u);
   }
-  __device__ unsigned ior(unsigned x) const {
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) x |= __shfl_xor_sync(mask, x, o);
-    return x;
-  }
+  __device__ unsigned ior(unsigned x) const { return G == 1 ? x : __reduce_or_sync(mask, x); }
   __device__ void sync() const {
     if (G > 1) __syncwarp(mask);
   }
@@ -106,6 +102,34 @@ __device__ __forceinline__ Tri tri(int t) {
 }
 
 // ------------------------------------------------------------------ small helpers
+// Comparisons on the bits of a double (an FP64 comparison takes 106 cycles of
+// the FP64 unit's path, an fmax 210; integer ones about 15).  NaN compares
+// false, as with the floating-point operators.
+constexpr long long kInfBits = 0x7ff0000000000000ll;
+__device__ __forceinline__ bool is_neg(double x) {            // x < 0
+  const long long b = __double_as_longlong(x);
+  return b < 0 && (unsigned long long)(b & 0x7fffffffffffffffll) - 1ull < (unsigned long long)kInfBits;
+}
+__device__ __forceinline__ bool is_pos(double x) {            // x > 0
+  return (unsigned long long)__double_as_longlong(x) - 1ull < (unsigned long long)kInfBits;
+}
+__device__ __forceinline__ bool above(double x, double c) {   // x > c, c >= 0
+  const long long b = __double_as_longlong(x);
+  return b > __double_as_longlong(c) && b <= kInfBits;
+}
+__device__ __forceinline__ bool below(double x, double c) {   // x < c, x >= 0 or NaN, c > 0
+  return __double_as_longlong(x) < __double_as_longlong(c);
+}
+// the larger of two numbers >= 0 (NaN if one is)
+__device__ __forceinline__ double max_pos(double a, double b) {
+  const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+  return __longlong_as_double(x > y ? x : y);
+}
+// x times sg = +-1
+__device__ __forceinline__ double flip(double x, bool minus) {
+  return __longlong_as_double(__double_as_longlong(x) ^ (minus ? (1ll << 63) : 0ll));
+}
+__device__ __forceinline__ Dual flip(const Dual& x, bool minus) { return minus ? -x : x; }
 // Templated on the scalar types so that the same code runs on doubles (the
 // forward path) and on derivative scalars (the adjoint); model constants
 // stay double.
@@ -570,7 +594,9 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
     const int b = t / 6, e = t - 6 * b;
     const int va = m.b_vadr[b], nd = m.b_nv[b];
     T x = 0.0;
-    for (int d = 0; d < nd; ++d) x += S[6 * (va + d) + e] * v[va + d];
+    int d = 0;
+    if (nd == 6) { d = 3; if (e >= 3) x = v[va + e - 3]; }   // unit translation vectors
+    for (; d < nd; ++d) x += S[6 * (va + d) + e] * v[va + d];
     V[t] = x;
   }
   g.sync();
@@ -859,15 +885,15 @@ __device__ __forceinline__ double div_const(double a, double b, double rb) {
 // divisions by the width and the midpoint done by div_const.
 __device__ __forceinline__ double impedance_quadratic(const DevModel& m, double r) {
   const double width = m.solimp[2], mid = m.solimp[3], a = fabs(r);
-  const double x = a < width ? div_const(a, width, m.imp_rwidth) : 1.0;
-  const bool low = x <= mid && mid > 0;
+  const double x = below(a, width) ? div_const(a, width, m.imp_rwidth) : 1.0;
+  const bool low = is_pos(mid) && !above(x, mid);
   const double y = low ? x : 1.0 - x, den = low ? mid : 1.0 - mid;
   const double num = y * y;
-  double sh = den > 0 ? div_const(num, den, low ? m.imp_rmid : m.imp_rmid1) : num / den;
+  double sh = is_pos(den) ? div_const(num, den, low ? m.imp_rmid : m.imp_rmid1) : num / den;
   if (!low) sh = 1.0 - sh;
   const double d = m.solimp[0] + (m.solimp[1] - m.solimp[0]) * sh;
-  if (d < 0.0) return 0.0;
-  if (d > 0.9999) return 0.9999;
+  if (is_neg(d)) return 0.0;
+  if (above(d, 0.9999)) return 0.9999;
   return d;
 }
 // The same shape with a derivative-scalar midpoint (parameter tangents).
@@ -947,7 +973,7 @@ __device__ void collide(const Grp<G>& g, const DevModel& m, const WsT<T>& w, boo
       ct[4] = 0.0; ct[5] = 0.0; ct[6] = 1.0; ct[7] = 1.0; ct[8] = 0.0; ct[9] = 0.0; ct[10] = 0.0; ct[11] = 1.0;
       ct[12] = 0.0;
     }
-    const bool inc = value(ct[0]) < thr;
+    const bool inc = cfd ? value(ct[0]) < thr : is_neg(value(ct[0]));
     w.i[L.sinc + s] = inc ? 1 : 0;
     if (inc) {
       const T r = ct[0];
@@ -1014,11 +1040,10 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
       T pv[3];
       cross3(sv, ct + 1, pv);
       pv[0] += sv[3]; pv[1] += sv[4]; pv[2] += sv[5];
-      const double sg = mA ? 1.0 : -1.0;
       if (bB < 0) {   // ground plane: the frame is the world's (z, x, y)
-        jn = sg * pv[2]; j1 = sg * pv[0]; j2 = sg * pv[1];
+        jn = pv[2]; j1 = pv[0]; j2 = pv[1];
       } else {
-        jn = sg * dot3(ct + 4, pv); j1 = sg * dot3(ct + 7, pv); j2 = sg * dot3(ct + 10, pv);
+        jn = flip(dot3(ct + 4, pv), mB); j1 = flip(dot3(ct + 7, pv), mB); j2 = flip(dot3(ct + 10, pv), mB);
       }
     }
     if (m.p_condim[p] == 1) {
@@ -1057,16 +1082,20 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
 template <int G, class T>
 __device__ bool cholesky(const Grp<G>& g, T* H, T* invd, int n, int rows) {
   bool ok = true;
+  const Tri t0 = tri(g.lane);          // this lane's first entry of every trailing block
+  const int e0 = t0.i * n + 1 + t0.j, r0 = t0.i * n, c0 = t0.j * n;
   for (int k = 0; k < n; ++k) {
     const T hkk = H[k * n + k];
-    ok = ok && (value(hkk) > 0);
+    ok = ok && is_pos(value(hkk));
     const T il = rsqrt_t(hkk);   // the diagonal of the factor is kept as its reciprocal
     for (int i = k + 1 + g.lane; i < rows; i += G) H[i * n + k] *= il;
     if (g.lane == 0) invd[k] = il;
     g.sync();
     const int nt = rows - k - 1, cnt = nt * (nt + 1) / 2 - (rows - n);
     T* Hk = H + (k + 1) * n + k;   // column k below the diagonal
-    for (int t = g.lane; t < cnt; t += G) {   // lower triangle of the trailing block
+    // lower triangle of the trailing block
+    if (g.lane < cnt) Hk[e0] -= Hk[r0] * Hk[c0];
+    for (int t = g.lane + G; t < cnt; t += G) {
       const Tri ij = tri(t);
       Hk[ij.i * n + 1 + ij.j] -= Hk[ij.i * n] * Hk[ij.j * n];
     }
@@ -1203,9 +1232,13 @@ __device__ void residual_set(const Grp<G>& g, const DevModel& m, const WsT<T>& w
     for (int i = 0; i < nv; ++i) t += J[r * nv + i] * a[i];
     const T zr = t - aref[r];
     z[r] = zr;
-    if (value(zr) < 0) bits[rowid[r] >> 5] |= 1u << (rowid[r] & 31);
+    const int id = rowid[r];
+    const unsigned bit = is_neg(value(zr)) ? 1u << (id & 31) : 0u;
+#pragma unroll
+    for (int k = 0; k < MASKW; ++k) bits[k] |= (id >> 5) == k ? bit : 0u;
   }
-  for (int k = 0; k < MASKW; ++k) newmask[k] = (int)g.ior(bits[k]);
+#pragma unroll
+  for (int k = 0; k < MASKW; ++k) newmask[k] = 32 * k < m.nrowid ? (int)g.ior(bits[k]) : 0;
   g.sync();
 }
 
@@ -1244,14 +1277,14 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
   }
   double slope0 = g.sum(c0) + g.sum(s0), slope1 = g.sum(c1) + g.sum(s1);
   // sweep the breakpoints below the current root (each row toggles at most once)
-  unsigned tog[MASKW] = {0u, 0u, 0u, 0u};
+  unsigned long long tog0 = 0ull, tog1 = 0ull;
   for (int iter = 0; iter <= nr; ++iter) {
     // candidate rows: active ones leaving (s > 0) or inactive ones entering (s < 0, z > 0)
     // with breakpoint -z/s below the root -slope0/slope1 (slope1 > 0)
     int best = -1;
     double bz = 0, bs = 1;
     for (int r = g.lane; r < nr; r += G) {
-      if ((tog[r >> 5] >> (r & 31)) & 1u) continue;
+      if (((r < 64 ? tog0 : tog1) >> (r & 63)) & 1ull) continue;
       const double zr = value(z[r]), sr = value(s[r]);
       const bool act = zr < 0 || (zr == 0 && sr < 0);
       const bool cand = act ? (sr > 0) : (sr < 0 && zr > 0);
@@ -1286,7 +1319,7 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
     const bool act = zb < 0 || (zb == 0 && sb < 0);
     const double dz = db * zb * sb, ds = db * sb * sb;
     if (act) { slope0 -= dz; slope1 -= ds; } else { slope0 += dz; slope1 += ds; }
-    tog[best >> 5] |= 1u << (best & 31);
+    if (best < 64) tog0 |= 1ull << best; else tog1 |= 1ull << (best - 64);
   }
   const double alpha = -slope0 / slope1;
   return alpha < 0 ? 0.0 : alpha;
@@ -1457,8 +1490,60 @@ __device__ __forceinline__ void rot_exp(const T& th2, T& cw, T& sk) {   // cos(t
     sk = sn / th;
   }
 }
+// A free joint's quaternion takes four lanes, one component each: a lane
+// evaluates one of the two series, the products of its component and the
+// (shared) normalisation, 25 FP64 instructions on the longest path instead of
+// 46 on one lane.
+template <int G>
+__device__ void integrate_pos_lanes(const Grp<G>& g, const DevModel& m, const double* q, const double* dq,
+                                    double* out) {
+  for (int t0 = 0; t0 < 4 * m.nbody; t0 += G) {
+    const int t = t0 + g.lane, b = min(t >> 2, m.nbody - 1), c = t & 3;
+    const bool live = t < 4 * m.nbody;
+    const int qa = m.b_qadr[b], va = m.b_vadr[b];
+    if (m.b_jtype[b] == JNT_HINGE) {
+      if (live && c == 0) out[qa] = q[qa] + dq[va];
+    } else if (live && c < 3) {
+      out[qa + c] = q[qa + c] + dq[va + c];
+    }
+    const bool fr = live && m.b_jtype[b] == JNT_FREE;
+    if (!g.ballot(fr)) continue;
+    double cw = 1.0, sk = 0.5, d[3] = {0.0, 0.0, 0.0}, x[4] = {1.0, 0.0, 0.0, 0.0};
+    if (fr) {
+      for (int k = 0; k < 3; ++k) d[k] = dq[va + 3 + k];
+      for (int k = 0; k < 4; ++k) x[k] = q[qa + 3 + k];
+    }
+    const double th2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+    const bool small = below(th2, 1e-2);
+    // |dq| < 0.1 rad: the Taylor series of rot_exp, cos on even lanes, sine on odd ones
+    const bool od = c & 1;
+    const double k4 = od ? 1.0 / 185794560.0 : 1.0 / 10321920.0, k3 = od ? -1.0 / 645120.0 : -1.0 / 46080.0;
+    const double k2 = od ? 1.0 / 3840.0 : 1.0 / 384.0, k1 = od ? -1.0 / 48.0 : -1.0 / 8.0, k0 = od ? 0.5 : 1.0;
+    const double sr = k0 + th2 * (k1 + th2 * (k2 + th2 * (k3 + th2 * k4)));
+    const double so = __shfl_xor_sync(g.mask, sr, 1);
+    cw = od ? so : sr;
+    sk = od ? sr : so;
+    if (fr && !small) rot_exp(th2, cw, sk);
+    const double e[4] = {cw, sk * d[0], sk * d[1], sk * d[2]};
+    // component c of x (x) e: x0 e_c then the pairs (k, c ^ k), minus for k = c and along the cycle
+    const double E0 = c == 0 ? e[0] : c == 1 ? e[1] : c == 2 ? e[2] : e[3];
+    const double E1 = flip(c == 0 ? e[1] : c == 1 ? e[0] : c == 2 ? e[3] : e[2], c == 0 || c == 2);
+    const double E2 = flip(c == 0 ? e[2] : c == 1 ? e[3] : c == 2 ? e[0] : e[1], c == 0 || c == 3);
+    const double E3 = flip(c == 0 ? e[3] : c == 1 ? e[2] : c == 2 ? e[1] : e[0], c < 2);
+    const double r = x[0] * E0 + x[1] * E1 + x[2] * E2 + x[3] * E3;
+    const double rw = __shfl_sync(g.mask, r, 0, 4), rx = __shfl_sync(g.mask, r, 1, 4);
+    const double ry = __shfl_sync(g.mask, r, 2, 4), rz = __shfl_sync(g.mask, r, 3, 4);
+    const double in = rsqrt_t(rw * rw + rx * rx + ry * ry + rz * rz);
+    if (fr) out[qa + 3 + c] = r * in;
+  }
+  g.sync();
+}
 template <int G, class T>
 __device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, const T* dq, T* out) {
+  if constexpr (G >= 4 && std::is_same<T, double>::value) {
+    integrate_pos_lanes(g, m, q, dq, out);
+    return;
+  }
   for (int b = g.lane; b < m.nbody; b += G) {
     const int qa = m.b_qadr[b], va = m.b_vadr[b];
     if (m.b_jtype[b] == JNT_HINGE) { out[qa] = q[qa] + dq[va]; continue; }
@@ -1575,8 +1660,8 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
       ev += c * ka[j * nv + i];
     }
     ep *= h; ev *= h;
-    const double sp = atol + rtol * fmax(pos_mag(m, qn, i), pos_mag(m, qs, i));
-    const double sv = atol + rtol * fmax(fabs(vn[i]), fabs(vs[i]));
+    const double sp = atol + rtol * max_pos(pos_mag(m, qn, i), pos_mag(m, qs, i));
+    const double sv = atol + rtol * max_pos(fabs(vn[i]), fabs(vs[i]));
     const double r1 = ep / sp, r2 = ev / sv;
     terms[i] = r1 * r1 + r2 * r2;
   }
