@@ -63,17 +63,17 @@ __device__ void snap_save(const Grp<G>& g, const DevModel& m, const Ws& w, doubl
   const SnapOff o = snap_offsets(m, L);
   const int nr = (st == ENV_ROW_OVERFLOW) ? 0 : w.i[L.slotrow + m.nslot];
   const double* d = w.d;
-  for (int i = g.lane; i < o.n1; i += G) dst[i] = d[L.R + i];
-  for (int i = g.lane; i < o.n2; i += G) dst[o.o2 + i] = d[L.H + i];
-  for (int i = g.lane; i < 16 * m.nslot; i += G) dst[o.o3 + i] = d[L.ct + i];
-  for (int i = g.lane; i < 2 * m.nslot; i += G) dst[o.o3 + 16 * m.nslot + i] = d[L.csv + i];
-  for (int i = g.lane; i < nr * m.nv; i += G) dst[o.o4 + i] = d[L.J + i];
-  for (int i = g.lane; i < nr; i += G) { dst[o.o5 + i] = d[L.Dr + i]; dst[o.o6 + i] = d[L.z + i]; }
+  DMX_TASKS(i, o.n1) dst[i] = d[L.R + i];
+  DMX_TASKS(i, o.n2) dst[o.o2 + i] = d[L.H + i];
+  DMX_TASKS(i, 16 * m.nslot) dst[o.o3 + i] = d[L.ct + i];
+  DMX_TASKS(i, 2 * m.nslot) dst[o.o3 + 16 * m.nslot + i] = d[L.csv + i];
+  DMX_TASKS(i, nr * m.nv) dst[o.o4 + i] = d[L.J + i];
+  DMX_TASKS(i, nr) { dst[o.o5 + i] = d[L.Dr + i]; dst[o.o6 + i] = d[L.z + i]; }
   int* di = reinterpret_cast<int*>(dst + o.oi);
   if (g.lane == 0) { di[0] = st; di[1] = nr; }
   for (int i = g.lane; i <= m.nslot; i += G) di[2 + i] = w.i[L.slotrow + i];
-  for (int i = g.lane; i < nr; i += G) di[3 + m.nslot + i] = w.i[L.rowid + i];
-  for (int i = g.lane; i < MASKW; i += G) di[3 + m.nslot + L.rcap + i] = w.i[L.amask + i];
+  DMX_TASKS(i, nr) di[3 + m.nslot + i] = w.i[L.rowid + i];
+  DMX_TASKS(i, MASKW) di[3 + m.nslot + L.rcap + i] = w.i[L.amask + i];
 }
 // Snapshot src -> workspace (the state rhs() leaves for rhs_vjp, except the
 // contact records and Jacobian rows, which the VJP reads from the snapshot
@@ -87,11 +87,11 @@ __device__ int snap_restore(const Grp<G>& g, const DevModel& m, const Ws& w, con
   double* d = w.d;
   copy_run(g, src, d + L.R, o.n1);
   copy_run(g, src + o.o2, d + L.H, o.n2);
-  for (int i = g.lane; i < 2 * m.nslot; i += G) d[L.csv + i] = src[o.o3 + 16 * m.nslot + i];
-  for (int i = g.lane; i < nr; i += G) { d[L.Dr + i] = src[o.o5 + i]; d[L.z + i] = src[o.o6 + i]; }
+  DMX_TASKS(i, 2 * m.nslot) d[L.csv + i] = src[o.o3 + 16 * m.nslot + i];
+  DMX_TASKS(i, nr) { d[L.Dr + i] = src[o.o5 + i]; d[L.z + i] = src[o.o6 + i]; }
   for (int i = g.lane; i <= m.nslot; i += G) w.i[L.slotrow + i] = si[2 + i];
-  for (int i = g.lane; i < nr; i += G) w.i[L.rowid + i] = si[3 + m.nslot + i];
-  for (int i = g.lane; i < MASKW; i += G) w.i[L.amask + i] = si[3 + m.nslot + L.rcap + i];
+  DMX_TASKS(i, nr) w.i[L.rowid + i] = si[3 + m.nslot + i];
+  DMX_TASKS(i, MASKW) w.i[L.amask + i] = si[3 + m.nslot + L.rcap + i];
   g.sync();
   return st;
 }
@@ -121,15 +121,15 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
   double* Qb = b.at(LB.Qb); double* Vb = b.at(LB.Vb);
   double* qnb = b.at(LB.qnb); double* vnb = b.at(LB.vnb); double* ub = b.at(LB.ub);
   int st = 0;
-  for (int i = g.lane; i < 6 * nv; i += G) { kab[i] = 0.0; kvb[i] = 0.0; }
-  for (int i = g.lane; i < m.nq; i += G) qnb[i] = 0.0;
-  for (int i = g.lane; i < nv; i += G) vnb[i] = 0.0;
-  for (int a = g.lane; a < m.nu; a += G) ub[a] = 0.0;
+  DMX_TASKS(i, 6 * nv) { kab[i] = 0.0; kvb[i] = 0.0; }
+  DMX_TASKS(i, m.nq) qnb[i] = 0.0;
+  DMX_TASKS(i, nv) vnb[i] = 0.0;
+  DMX_TASKS(a, m.nu) ub[a] = 0.0;
   g.sync();
   for (int s = S - 1; s >= 0; --s) {
     const unsigned mq = TAB(mt).nzq[s], mv = TAB(mt).nzv[s];
     if (s >= 1) {
-      for (int i = g.lane; i < nv; i += G) {
+      DMX_TASKS(i, nv) {
         double sq = 0;
         for (int j = 0; j <= s; ++j)
           if ((mq >> j) & 1u) sq += TAB(mt).aq[s][j] * vst[j * nv + i];
@@ -138,7 +138,7 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
       g.sync();
       if (s <= S - 2) integrate_pos(g, m, qn, (const double*)dq, Qs);
     } else {
-      for (int i = g.lane; i < m.nq; i += G) Qs[i] = qn[i];
+      DMX_TASKS(i, m.nq) Qs[i] = qn[i];
       g.sync();
     }
     if (s <= S - 2) {
@@ -148,13 +148,13 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
       if (r > st) st = r;
       rhs_vjp<G, PAR>(g, m, sn ? snap_view(m, w, sn) : w, b, Qs, Vs, u, cfd, r, kab + s * nv, Qb, Vb, ub,
                       PAR ? b.at(LB.pa) : nullptr);
-      for (int i = g.lane; i < nv; i += G) Vb[i] += kvb[s * nv + i];   // V_s in the later stages' positions
+      DMX_TASKS(i, nv) Vb[i] += kvb[s * nv + i];   // V_s in the later stages' positions
       g.sync();
     }
     if (s >= 1) {
       // positions first: a diagonal coefficient puts V_s into Q_s itself
       integrate_pos_vjp(g, m, qn, dq, Qb, qnb, dqb);
-      for (int i = g.lane; i < nv; i += G) {
+      DMX_TASKS(i, nv) {
         for (int j = 0; j < s; ++j)
           if ((mq >> j) & 1u) kvb[j * nv + i] += h * TAB(mt).aq[s][j] * dqb[i];
         if ((mq >> s) & 1u) Vb[i] += h * TAB(mt).aq[s][s] * dqb[i];
@@ -163,12 +163,12 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
           if ((mv >> j) & 1u) kab[j * nv + i] += h * TAB(mt).av[s][j] * Vb[i];
       }
     } else {
-      for (int i = g.lane; i < m.nq; i += G) qnb[i] += Qb[i];
-      for (int i = g.lane; i < nv; i += G) vnb[i] += Vb[i];
+      DMX_TASKS(i, m.nq) qnb[i] += Qb[i];
+      DMX_TASKS(i, nv) vnb[i] += Vb[i];
     }
     g.sync();
-    for (int i = g.lane; i < m.nq; i += G) Qb[i] = 0.0;
-    for (int i = g.lane; i < nv; i += G) Vb[i] = 0.0;
+    DMX_TASKS(i, m.nq) Qb[i] = 0.0;
+    DMX_TASKS(i, nv) Vb[i] = 0.0;
     g.sync();
   }
   return st;
@@ -204,11 +204,11 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
     if (env >= P.B) break;
     const int N = P.tape_n[env];
     const double T = P.T[env];
-    for (int i = g.lane; i < nx; i += G) xbar[i] = P.xT_bar[(size_t)i * P.B + env];
+    DMX_TASKS(i, nx) xbar[i] = P.xT_bar[(size_t)i * P.B + env];
     if (P.ctrl_bar)
-      for (int i = g.lane; i < P.NI * nu; i += G) P.ctrl_bar[(size_t)i * P.B + env] = 0.0;
+      DMX_TASKS(i, P.NI * nu) P.ctrl_bar[(size_t)i * P.B + env] = 0.0;
     if constexpr (PAR)
-      for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] = 0.0;
+      DMX_TASKS(k, P.np) P.p_bar[(size_t)k * P.B + env] = 0.0;
     if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
     g.sync();
     int worst = 0;
@@ -216,11 +216,11 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
       const int n0 = c * P.K, n1 = min(n0 + P.K, N);
       // ---- forward recompute of the segment from checkpoint c: q_n, V_0..V_5, t_n per step
       const double* ck = P.ckpt + (size_t)c * (nx + 1) * P.B;
-      for (int i = g.lane; i < nq; i += G) qn[i] = ck[(size_t)i * P.B + env];
-      for (int i = g.lane; i < nv; i += G) vn[i] = ck[(size_t)(nq + i) * P.B + env];
+      DMX_TASKS(i, nq) qn[i] = ck[(size_t)i * P.B + env];
+      DMX_TASKS(i, nv) vn[i] = ck[(size_t)(nq + i) * P.B + env];
       double t = ck[(size_t)nx * P.B + env];
       int k = rev_interval(T, P.NI, t);
-      for (int a = g.lane; a < nu; a += G) u[a] = P.ctrl[((size_t)k * nu + a) * P.B + env];
+      DMX_TASKS(a, nu) u[a] = P.ctrl[((size_t)k * nu + a) * P.B + env];
       g.sync();
       {
         const int st0 = rhs(g, m, w, (const double*)qn, (const double*)vn, (const double*)u, false, ka);
@@ -236,8 +236,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
           else if (sn_next) snap_save(g, m, w, sn_next, r);   // the last stage = stage 0 of the next step
         });
         const double* kv = w.at(sL.kv);
-        for (int i = g.lane; i < nq; i += G) row[i] = qn[i];
-        for (int i = g.lane; i < S * nv; i += G) row[nq + i] = kv[i];
+        DMX_TASKS(i, nq) row[i] = qn[i];
+        DMX_TASKS(i, S * nv) row[nq + i] = kv[i];
         if (g.lane == 0) row[nq + 7 * nv] = t;
         if (n == n1 - 1) break;
         const double tn = rev_boundary(T, P.NI, k + 1);
@@ -245,12 +245,12 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
         t = reached ? tn : t + h;
         const double* qs = w.at(sL.qs); const double* vs = w.at(sL.vs);
         g.sync();
-        for (int i = g.lane; i < nq; i += G) qn[i] = qs[i];
-        for (int i = g.lane; i < nv; i += G) { vn[i] = vs[i]; ka[i] = ka[(S - 1) * nv + i]; }
+        DMX_TASKS(i, nq) qn[i] = qs[i];
+        DMX_TASKS(i, nv) { vn[i] = vs[i]; ka[i] = ka[(S - 1) * nv + i]; }
         g.sync();
         if (reached && k + 1 < P.NI) {
           ++k;
-          for (int a = g.lane; a < nu; a += G) u[a] = P.ctrl[((size_t)k * nu + a) * P.B + env];
+          DMX_TASKS(a, nu) u[a] = P.ctrl[((size_t)k * nu + a) * P.B + env];
           g.sync();
           const int stb = rhs(g, m, w, (const double*)qn, (const double*)vn, (const double*)u, false, ka);
           if (sn_next) snap_save(g, m, w, sn_next, stb);   // the new control's stage 0
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
       double* bq = b.at(sB.qn); double* bv = b.at(sB.vst);
       double* Qb = b.at(sB.Qb); double* Vb = b.at(sB.Vb);
       if constexpr (PAR)               // the segment's sums live in the cotangent workspace
-        for (int k = g.lane; k < P.np; k += G) b.at(sB.pa)[k] = 0.0;
+        DMX_TASKS(k, P.np) b.at(sB.pa)[k] = 0.0;
       for (int n = n1 - 1; n >= n0; --n) {
         const double* row = seg + (size_t)(n - n0) * RW;
         const double tn0 = row[nq + 7 * nv];
@@ -271,36 +271,36 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
         const double tb = rev_boundary(T, P.NI, kn + 1);
         const bool reached = (h == tb - tn0) || (tn0 + h >= tb);
         if (reached && P.xb_bar)
-          for (int i = g.lane; i < nx; i += G) xbar[i] += P.xb_bar[((size_t)(kn + 1) * nx + i) * P.B + env];
-        for (int i = g.lane; i < nq; i += G) bq[i] = row[i];
-        for (int i = g.lane; i < S * nv; i += G) bv[i] = row[nq + i];
-        for (int a = g.lane; a < nu; a += G) u[a] = P.ctrl[((size_t)kn * nu + a) * P.B + env];
+          DMX_TASKS(i, nx) xbar[i] += P.xb_bar[((size_t)(kn + 1) * nx + i) * P.B + env];
+        DMX_TASKS(i, nq) bq[i] = row[i];
+        DMX_TASKS(i, S * nv) bv[i] = row[nq + i];
+        DMX_TASKS(a, nu) u[a] = P.ctrl[((size_t)kn * nu + a) * P.B + env];
         g.sync();
-        for (int i = g.lane; i < nq; i += G) Qb[i] = xbar[i];
-        for (int i = g.lane; i < nv; i += G) Vb[i] = xbar[nq + i];
+        DMX_TASKS(i, nq) Qb[i] = xbar[i];
+        DMX_TASKS(i, nv) Vb[i] = xbar[nq + i];
         g.sync();
         const int st = rk_step_vjp<G, PAR>(g, m, w, b, (const double*)u, h, mt, P.cfd != 0,
                                    use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr, SN);
         if (st > worst) worst = st;
         const double* qnb = b.at(sB.qnb); const double* vnb = b.at(sB.vnb); const double* ub = b.at(sB.ub);
-        for (int i = g.lane; i < nq; i += G) xbar[i] = qnb[i];
-        for (int i = g.lane; i < nv; i += G) xbar[nq + i] = vnb[i];
+        DMX_TASKS(i, nq) xbar[i] = qnb[i];
+        DMX_TASKS(i, nv) xbar[nq + i] = vnb[i];
         if (P.ctrl_bar)
-          for (int a = g.lane; a < nu; a += G) P.ctrl_bar[((size_t)kn * nu + a) * P.B + env] += ub[a];
+          DMX_TASKS(a, nu) P.ctrl_bar[((size_t)kn * nu + a) * P.B + env] += ub[a];
         g.sync();
       }
       if constexpr (PAR)
-        for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] += b.at(sB.pa)[k];
+        DMX_TASKS(k, P.np) P.p_bar[(size_t)k * P.B + env] += b.at(sB.pa)[k];
       g.sync();
     }
     if (P.xb_bar)
-      for (int i = g.lane; i < nx; i += G) xbar[i] += P.xb_bar[(size_t)i * P.B + env];
+      DMX_TASKS(i, nx) xbar[i] += P.xb_bar[(size_t)i * P.B + env];
     g.sync();
     // a right-hand side whose rows overflowed the workspace has no derivative: mark the result
     const double bad = (worst == ENV_ROW_OVERFLOW) ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
-    for (int i = g.lane; i < nx; i += G) P.x0_bar[(size_t)i * P.B + env] = xbar[i] + bad;
+    DMX_TASKS(i, nx) P.x0_bar[(size_t)i * P.B + env] = xbar[i] + bad;
     if constexpr (PAR)
-      for (int k = g.lane; k < P.np; k += G) P.p_bar[(size_t)k * P.B + env] += bad;
+      DMX_TASKS(k, P.np) P.p_bar[(size_t)k * P.B + env] += bad;
     g.sync();
   }
 }
@@ -325,19 +325,19 @@ __global__ void __launch_bounds__(32, 1) k_eval_rhs_vjp(const __grid_constant__ 
   if (env >= P.B) return;
   double* qs = b.at(sB.Qs); double* vs = b.at(sB.vst); double* uu = w.at(sL.u); double* ab = b.at(sB.kab);
   double* qb = b.at(sB.qnb); double* vb = b.at(sB.vnb); double* ub = b.at(sB.ub);
-  for (int i = g.lane; i < m.nq; i += G) { qs[i] = q[(size_t)i * P.B + env]; qb[i] = 0.0; }
-  for (int i = g.lane; i < m.nv; i += G) {
+  DMX_TASKS(i, m.nq) { qs[i] = q[(size_t)i * P.B + env]; qb[i] = 0.0; }
+  DMX_TASKS(i, m.nv) {
     vs[i] = v[(size_t)i * P.B + env]; ab[i] = abar[(size_t)i * P.B + env]; vb[i] = 0.0;
   }
-  for (int i = g.lane; i < m.nu; i += G) { uu[i] = u[(size_t)i * P.B + env]; ub[i] = 0.0; }
+  DMX_TASKS(i, m.nu) { uu[i] = u[(size_t)i * P.B + env]; ub[i] = 0.0; }
   if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
   g.sync();
   const int st = rhs(g, m, w, (const double*)qs, (const double*)vs, (const double*)uu, P.cfd != 0, w.at(sL.ka));
   rhs_vjp(g, m, w, b, qs, vs, uu, P.cfd != 0, st, ab, qb, vb, ub);
-  for (int i = g.lane; i < m.nq; i += G) qbar[(size_t)i * P.B + env] = qb[i];
-  for (int i = g.lane; i < m.nv; i += G) vbar[(size_t)i * P.B + env] = vb[i];
+  DMX_TASKS(i, m.nq) qbar[(size_t)i * P.B + env] = qb[i];
+  DMX_TASKS(i, m.nv) vbar[(size_t)i * P.B + env] = vb[i];
   if (ubar)
-    for (int i = g.lane; i < m.nu; i += G) ubar[(size_t)i * P.B + env] = ub[i];
+    DMX_TASKS(i, m.nu) ubar[(size_t)i * P.B + env] = ub[i];
   if (g.lane == 0) status[env] = st;
 }
 template <int G>

@@ -77,6 +77,12 @@ struct Grp {
   __device__ double bcast(double x, int src) const { return G == 1 ? x : __shfl_sync(mask, x, src, G); }
 };
 
+// Loop over n tasks spread over the group's lanes.  Not unrolled: the hot loop
+// of a kernel (one right-hand side, its VJP) is a long run of such loops with
+// one to five passes each, and unrolled copies push it out of the instruction
+// caches (4096 box pushes 185 -> 176 ms, 2048 arm gradients 269 -> 250 ms).
+#define DMX_TASKS(t, n) _Pragma("unroll 1") for (int t = g.lane; t < (n); t += G)
+
 // (row, column) of the t-th entry of a lower triangle enumerated row by row
 // ((0,0), (1,0), (1,1), (2,0), ...): the same for every matrix size.  In
 // global memory (read through the L1): the lanes of a group read different
@@ -350,7 +356,7 @@ __device__ __forceinline__ void tree_down(const Grp<G>& g, const DevModel& m, T*
   if (m.nlevel == 1) return;
   for (int cl = 0; cl < m.nchlev; ++cl) {
     const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
-    for (int t = g.lane; t < n; t += G) {
+    DMX_TASKS(t, n) {
       const int c = c0 + t / NC, e = t % NC;
       const int k0 = m.ch_start[c], k1 = m.ch_start[c + 1], par = m.ch_par[c];
       const int b0 = m.ch_list[k0];
@@ -370,7 +376,7 @@ __device__ __forceinline__ void tree_up(const Grp<G>& g, const DevModel& m, T* X
   if (m.nlevel == 1) return;
   for (int cl = m.nchlev - 1; cl >= 0; --cl) {
     const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
-    for (int t = g.lane; t < n; t += G) {
+    DMX_TASKS(t, n) {
       const int c = c0 + t / NC, e = t % NC;
       const int k0 = m.ch_start[c], k1 = m.ch_start[c + 1] - 1;
       const int tail = m.ch_list[k1], nc = m.child_count[tail], cs = m.child_start[tail];
@@ -402,7 +408,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
   T* S = w.at(L.sd); T* Ib = w.at(L.Ib); T* Ic = w.at(L.Ic);
   T* X = w.at(L.xl); T* SC = w.at(L.sc);
   const int nb = m.nbody;
-  for (int b = g.lane; b < nb; b += G) {
+  DMX_TASKS(b, nb) {
     const T* x = q + m.b_qadr[b];
     if (m.b_jtype[b] == JNT_FREE) {
       SC[2 * b] = 2.0 / (x[3] * x[3] + x[4] * x[4] + x[5] * x[5] + x[6] * x[6]);
@@ -415,7 +421,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
   g.sync();
   // local transforms: free joint = world pose; hinge = rotation in the parent frame.
   // Bodies at the root are written straight into the world arrays.
-  for (int t = g.lane; t < 12 * nb; t += G) {
+  DMX_TASKS(t, 12 * nb) {
     const int b = t / 12, e = t - 12 * b;
     const bool root = m.b_parent[b] < 0;
     T v;
@@ -444,7 +450,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
   // column of the local transform
   for (int lev = 1; lev < m.nlevel; ++lev) {
     const int k0 = m.level_start[lev], n = 12 * (m.level_start[lev + 1] - k0);
-    for (int t = g.lane; t < n; t += G) {
+    DMX_TASKS(t, n) {
       const int k = t / 12, e = t - 12 * k;
       const int pk = m.lv_pack[k0 + k], b = pk & 255, par = pk >> 8;
       const bool pos = e >= 9;
@@ -460,7 +466,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
   // a model vector (plus p): com, gpos, the columns of Roff
   T* gR = w.at(L.gR); T* gp = w.at(L.gp);
   const int n1 = 3 * nb, n2 = n1 + 12 * m.ngeom;
-  for (int t = g.lane; t < n2; t += G) {
+  DMX_TASKS(t, n2) {
     int b, i, st = 1;
     const double* c;
     T* out;
@@ -486,7 +492,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
     *out = v;
   }
   // dof motion vectors (w; v at the world origin), one dof per task
-  for (int i = g.lane; i < m.nv; i += G) {
+  DMX_TASKS(i, m.nv) {
     const int b = m.dof_body[i];
     const T* Rb = R + 9 * b; const T* pb = P + 3 * b;
     T* st = S + 6 * i;
@@ -509,7 +515,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
   // one entry per task: the six moments of every body first (12 operations
   // each), then mass and first moments, so that a pass of the lanes mostly
   // meets one kind.  Ic starts as a copy (composite inertias, crba).
-  for (int k = g.lane; k < 6 * nb; k += G) {
+  DMX_TASKS(k, 6 * nb) {
     const int b = k / 6, e = k - 6 * b;
     const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
     const T* c = C + 3 * b;
@@ -529,7 +535,7 @@ __device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, 
     Ib[10 * b + 4 + e] = v;
     Ic[10 * b + 4 + e] = v;
   }
-  for (int k = g.lane; k < 4 * nb; k += G) {
+  DMX_TASKS(k, 4 * nb) {
     const int b = k / 4, e = k - 4 * b;
     const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
     T v;
@@ -558,12 +564,12 @@ __device__ void crba(const Grp<G>& g, const DevModel& m, const WsT<T>& w) {
   const T* S = w.at(L.sd); T* F = w.at(L.F); T* M = w.at(L.M);
   const int nv = m.nv;
   tree_up<10>(g, m, Ic);             // Ic starts as Ib (kinematics)
-  for (int t = g.lane; t < 6 * nv; t += G) {
+  DMX_TASKS(t, 6 * nv) {
     const Comp6 c = comp6(t, nv);
     F[6 * c.i + c.e] = inertia_comp(Ic + 10 * m.dof_body[c.i], S + 6 * c.i, c.e);
   }
   g.sync();
-  for (int t = g.lane; t < nv * (nv + 1) / 2; t += G) {   // lower triangle
+  DMX_TASKS(t, nv * (nv + 1) / 2) {   // lower triangle
     const Tri ij = tri(t);
     const int i = ij.i, j = ij.j;
     T v = 0.0;
@@ -590,7 +596,7 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
   T* V = w.at(L.Vb); T* A = w.at(L.Ab); T* Fb = w.at(L.Fb); T* IV = w.at(L.iv);
   const int nb = m.nbody, nt = 6 * nb;
   // own joint velocity S v
-  for (int t = g.lane; t < nt; t += G) {
+  DMX_TASKS(t, nt) {
     const int b = t / 6, e = t - 6 * b;
     const int va = m.b_vadr[b], nd = m.b_nv[b];
     T x = 0.0;
@@ -602,7 +608,7 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
   g.sync();
   tree_down<6>(g, m, V);
   // own velocity-product acceleration (vb x S_d) v_d (gravity at the roots)
-  for (int t = g.lane; t < nt; t += G) {
+  DMX_TASKS(t, nt) {
     const Comp6 c = comp6(t, nb);
     const int b = c.i, e = c.e;
     const int va = m.b_vadr[b], nd = m.b_nv[b];
@@ -614,14 +620,14 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
   g.sync();
   tree_down<6>(g, m, A);
   // body forces I a + v x* (I v)
-  for (int t = g.lane; t < nt; t += G) {
+  DMX_TASKS(t, nt) {
     const Comp6 c = comp6(t, nb);
     const int b = c.i, e = c.e;
     Fb[6 * b + e] = inertia_comp(Ib + 10 * b, A + 6 * b, e);
     IV[6 * b + e] = inertia_comp(Ib + 10 * b, V + 6 * b, e);
   }
   g.sync();
-  for (int t = g.lane; t < nt; t += G) {
+  DMX_TASKS(t, nt) {
     const Comp6 c = comp6(t, nb);
     const int b = c.i, e = c.e;
     Fb[6 * b + e] += crf_comp(V + 6 * b, IV + 6 * b, e);
@@ -629,7 +635,7 @@ __device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>&
   g.sync();
   tree_up<6>(g, m, Fb);
   T* rhs0 = w.at(L.rhs0);
-  for (int i = g.lane; i < m.nv; i += G) {
+  DMX_TASKS(i, m.nv) {
     const int b = m.dof_body[i];
     const T* s = S + 6 * i; const T* f = Fb + 6 * b;
     const T c = s[0] * f[0] + s[1] * f[1] + s[2] * f[2] + s[3] * f[3] + s[4] * f[4] + s[5] * f[5];
@@ -936,7 +942,7 @@ __device__ void collide(const Grp<G>& g, const DevModel& m, const WsT<T>& w, boo
   const T* gR = w.at(L.gR); const T* gp = w.at(L.gp);
   T* CT = w.at(L.ct);
   const double thr = cfd ? m.cfd[2] : 0.0;
-  for (int s = g.lane; s < m.nslot; s += G) {
+  DMX_TASKS(s, m.nslot) {
     T* ct = CT + 16 * s;
     const int p = m.s_pair[s], j = m.s_idx[s], g1 = m.p_g1[p];
     if (m.p_g2[p] >= 0) {
@@ -1023,6 +1029,7 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
   const int nr = n, nincl = ns;
   if (nr > L.rcap) return -1;
   T* J = w.at(L.J);
+#pragma unroll 1
   for (int idx = g.lane, si = g.lane / nv, i = g.lane - si * nv; idx < nincl * nv;   // included slots only
        idx += G, i += G % nv, si += G / nv + (i >= nv), i -= (i >= nv) ? nv : 0) {
     const int s = slist[si];
@@ -1058,7 +1065,7 @@ __device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, co
   }
   g.sync();
   T* aref = w.at(L.aref); T* Dr = w.at(L.Dr);
-  for (int r = g.lane; r < nr; r += G) {   // one row per task
+  DMX_TASKS(r, nr) {   // one row per task
     const int s = rowslot[r];
     const int e = r - slotrow[s];
     const int p = m.s_pair[s];
@@ -1095,6 +1102,7 @@ __device__ bool cholesky(const Grp<G>& g, T* H, T* invd, int n, int rows) {
     T* Hk = H + (k + 1) * n + k;   // column k below the diagonal
     // lower triangle of the trailing block
     if (g.lane < cnt) Hk[e0] -= Hk[r0] * Hk[c0];
+#pragma unroll 1
     for (int t = g.lane + G; t < cnt; t += G) {
       const Tri ij = tri(t);
       Hk[ij.i * n + 1 + ij.j] -= Hk[ij.i * n] * Hk[ij.j * n];
@@ -1131,7 +1139,7 @@ __device__ void chol_back(const Grp<G>& g, const T* H, const T* invd, T* x, int 
     const T xk = x[k] * invd[k];
     g.sync();
     if (g.lane == 0) x[k] = xk;
-    for (int i = g.lane; i < k; i += G) x[i] -= H[k * n + i] * xk;
+    DMX_TASKS(i, k) x[i] -= H[k * n + i] * xk;
     g.sync();
   }
 }
@@ -1193,13 +1201,13 @@ __device__ bool solve_active(const Grp<G>& g, const DevModel& m, const WsT<T>& w
   const int hb = L.hb;
   for (int k0 = 0; k0 == 0 || k0 < na; k0 += hb) {
     const int nk = min(hb, na - k0);
-    for (int t = g.lane; t < nk * nx1; t += G) {
+    DMX_TASKS(t, nk * nx1) {
       const int k = t / nx1, i = t - k * nx1;
       const int r = alist[k0 + k];
       X[t] = Dr[r] * (i < nv ? J[r * nv + i] : aref[r]);
     }
     g.sync();
-    for (int t = g.lane; t < nent; t += G) {
+    DMX_TASKS(t, nent) {
       const Tri ij = tri(t);
       const int i = ij.i, j = ij.j;
       T h = k0 ? H[i * nv + j] : (i < nv ? M[i * nv + j] : rhs0[j]);
@@ -1227,7 +1235,7 @@ __device__ void residual_set(const Grp<G>& g, const DevModel& m, const WsT<T>& w
   T* z = w.at(L.z);
   const int* rowid = w.i + L.rowid;
   unsigned bits[MASKW] = {0u, 0u, 0u, 0u};
-  for (int r = g.lane; r < nr; r += G) {
+  DMX_TASKS(r, nr) {
     T t = 0.0;
     for (int i = 0; i < nv; ++i) t += J[r * nv + i] * a[i];
     const T zr = t - aref[r];
@@ -1252,17 +1260,17 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
   const T* M = w.at(L.M); const T* J = w.at(L.J); const T* Dr = w.at(L.Dr);
   const T* a = w.at(L.a); const T* an = w.at(L.an); const T* rhs0 = w.at(L.rhs0);
   T* dl = w.at(L.tmp); T* z = w.at(L.z); T* s = w.at(L.s);
-  for (int i = g.lane; i < nv; i += G) dl[i] = an[i] - a[i];
+  DMX_TASKS(i, nv) dl[i] = an[i] - a[i];
   g.sync();
   double c0 = 0, c1 = 0;
-  for (int i = g.lane; i < nv; i += G) {
+  DMX_TASKS(i, nv) {
     double ma = 0, md = 0;
     for (int j = 0; j < nv; ++j) { ma += value(M[i * nv + j]) * value(a[j]); md += value(M[i * nv + j]) * value(dl[j]); }
     c0 += value(dl[i]) * (ma - value(rhs0[i]));
     c1 += value(dl[i]) * md;
   }
   const T* aref = w.at(L.aref);
-  for (int r = g.lane; r < nr; r += G) {
+  DMX_TASKS(r, nr) {
     double t = 0, u = 0;
     for (int i = 0; i < nv; ++i) { t += value(J[r * nv + i]) * value(dl[i]); u += value(J[r * nv + i]) * value(a[i]); }
     s[r] = t;
@@ -1270,7 +1278,7 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
   }
   g.sync();
   double s0 = 0, s1 = 0;
-  for (int r = g.lane; r < nr; r += G) {
+  DMX_TASKS(r, nr) {
     const double zr = value(z[r]), sr = value(s[r]), dr = value(Dr[r]);
     const bool act = zr < 0 || (zr == 0 && sr < 0);
     if (act) { s0 += dr * zr * sr; s1 += dr * sr * sr; }
@@ -1283,7 +1291,7 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
     // with breakpoint -z/s below the root -slope0/slope1 (slope1 > 0)
     int best = -1;
     double bz = 0, bs = 1;
-    for (int r = g.lane; r < nr; r += G) {
+    DMX_TASKS(r, nr) {
       if (((r < 64 ? tog0 : tog1) >> (r & 63)) & 1ull) continue;
       const double zr = value(z[r]), sr = value(s[r]);
       const bool act = zr < 0 || (zr == 0 && sr < 0);
@@ -1353,14 +1361,14 @@ __device__ int solve_constraints(const Grp<G>& g, const DevModel& m, const WsT<T
     if (same) { status = ENV_OK; break; }
     if (it == 0) {
       // start point of the Newton search: the solution of the first candidate set
-      for (int i = g.lane; i < nv; i += G) a[i] = an[i];
+      DMX_TASKS(i, nv) a[i] = an[i];
       for (int k = 0; k < MASKW; ++k) cur[k] = nxt[k];
       g.sync();
       continue;
     }
     const double alpha = line_search(g, m, w, nr);
     const T* dl = w.at(L.tmp);
-    for (int i = g.lane; i < nv; i += G) a[i] += alpha * dl[i];
+    DMX_TASKS(i, nv) a[i] += alpha * dl[i];
     g.sync();
     residual_set(g, m, w, nr, (const T*)a, cur);
   }
@@ -1385,7 +1393,7 @@ __device__ int rhs(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T*
   if (nr < 0) return ENV_ROW_OVERFLOW;
   const int st = solve_constraints(g, m, w, nr);
   const T* an = w.at(L.an);
-  for (int i = g.lane; i < m.nv; i += G) out[i] = an[i];
+  DMX_TASKS(i, m.nv) out[i] = an[i];
   g.sync();
   return st;
 }
@@ -1542,26 +1550,26 @@ template <int G, class T>
 __device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, const T* dq, T* out) {
   if constexpr (G >= 4 && std::is_same<T, double>::value) {
     integrate_pos_lanes(g, m, q, dq, out);
-    return;
+  } else {
+    DMX_TASKS(b, m.nbody) {
+      const int qa = m.b_qadr[b], va = m.b_vadr[b];
+      if (m.b_jtype[b] == JNT_HINGE) { out[qa] = q[qa] + dq[va]; continue; }
+      out[qa] = q[qa] + dq[va]; out[qa + 1] = q[qa + 1] + dq[va + 1]; out[qa + 2] = q[qa + 2] + dq[va + 2];
+      const T* d = dq + va + 3;
+      const T th2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
+      T cw, sk;
+      rot_exp(th2, cw, sk);
+      const T ex = sk * d[0], ey = sk * d[1], ez = sk * d[2];
+      const T w0 = q[qa + 3], a0 = q[qa + 4], b0 = q[qa + 5], c0 = q[qa + 6];
+      const T rw = w0 * cw - a0 * ex - b0 * ey - c0 * ez;
+      const T rx = w0 * ex + a0 * cw + b0 * ez - c0 * ey;
+      const T ry = w0 * ey - a0 * ez + b0 * cw + c0 * ex;
+      const T rz = w0 * ez + a0 * ey - b0 * ex + c0 * cw;
+      const T in = rsqrt_t(rw * rw + rx * rx + ry * ry + rz * rz);
+      out[qa + 3] = rw * in; out[qa + 4] = rx * in; out[qa + 5] = ry * in; out[qa + 6] = rz * in;
+    }
+    g.sync();
   }
-  for (int b = g.lane; b < m.nbody; b += G) {
-    const int qa = m.b_qadr[b], va = m.b_vadr[b];
-    if (m.b_jtype[b] == JNT_HINGE) { out[qa] = q[qa] + dq[va]; continue; }
-    out[qa] = q[qa] + dq[va]; out[qa + 1] = q[qa + 1] + dq[va + 1]; out[qa + 2] = q[qa + 2] + dq[va + 2];
-    const T* d = dq + va + 3;
-    const T th2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-    T cw, sk;
-    rot_exp(th2, cw, sk);
-    const T ex = sk * d[0], ey = sk * d[1], ez = sk * d[2];
-    const T w0 = q[qa + 3], a0 = q[qa + 4], b0 = q[qa + 5], c0 = q[qa + 6];
-    const T rw = w0 * cw - a0 * ex - b0 * ey - c0 * ez;
-    const T rx = w0 * ex + a0 * cw + b0 * ez - c0 * ey;
-    const T ry = w0 * ey - a0 * ez + b0 * cw + c0 * ex;
-    const T rz = w0 * ez + a0 * ey - b0 * ex + c0 * cw;
-    const T in = rsqrt_t(rw * rw + rx * rx + ry * ry + rz * rz);
-    out[qa + 3] = rw * in; out[qa + 4] = rx * in; out[qa + 5] = ry * in; out[qa + 6] = rz * in;
-  }
-  g.sync();
 }
 
 // Magnitude used by the error norm for tangent component i of the positions.
@@ -1586,11 +1594,11 @@ __device__ int rk_stages(const Grp<G>& g, const DevModel& m, const Ws& w, const 
   double* qs = w.at(L.qs); double* vs = w.at(L.vs);
   double* kv = w.at(L.kv); double* ka = w.at(L.ka); double* dq = w.at(L.dq);
   int st = 0;
-  for (int i = g.lane; i < nv; i += G) kv[i] = vn[i];
+  DMX_TASKS(i, nv) kv[i] = vn[i];
   g.sync();
   for (int s = 1; s < S; ++s) {
     const unsigned mq = TAB(mt).nzq[s], mv = TAB(mt).nzv[s];
-    for (int i = g.lane; i < nv; i += G) {
+    DMX_TASKS(i, nv) {
       double sq = 0, sv = 0;
       for (int j = 0; j < s; ++j) {
         if ((mq >> j) & 1u) sq += TAB(mt).aq[s][j] * kv[j * nv + i];
@@ -1618,7 +1626,7 @@ __device__ int rk_stages(const Grp<G>& g, const DevModel& m, const Ws& w, const 
 // without touching a single step decision.
 template <int G>
 __device__ double sum_as_lanes(const Grp<G>& g, double* x, int n, int C) {
-  for (int c = g.lane; c < C && c + C < n; c += G) {
+  DMX_TASKS(c, min(C, n - C)) {
     double acc = x[c];
     for (int i = c + C; i < n; i += C) acc += x[i];
     x[c] = acc;
@@ -1627,7 +1635,7 @@ __device__ double sum_as_lanes(const Grp<G>& g, double* x, int n, int C) {
   const int np = min(n, C);          // partial sums that exist
   for (int o = C >> 1; o > 0; o >>= 1) {
     if (o >= np) continue;
-    for (int c = g.lane; c < o && c + o < np; c += G) x[c] += x[c + o];
+    DMX_TASKS(c, min(o, np - o)) x[c] += x[c + o];
     g.sync();
   }
   return x[0];
@@ -1651,7 +1659,7 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
   if (!TAB(mt).adaptive) return 0.0;
   const unsigned enz = TAB(mt).enz;
   double* terms = w.at(L.dq);        // free after the last stage
-  for (int i = g.lane; i < nv; i += G) {
+  DMX_TASKS(i, nv) {
     double ep = 0, ev = 0;
     for (int j = 0; j < 7; ++j) {
       if (!((enz >> j) & 1u)) continue;

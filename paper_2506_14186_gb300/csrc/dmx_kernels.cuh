@@ -28,7 +28,7 @@ struct EnvState {
 template <int G>
 __device__ void load_ctrl(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env, int k) {
   double* u = w.at(w.L->u);
-  for (int a = g.lane; a < m.nu; a += G) u[a] = P.ctrl[((size_t)k * m.nu + a) * P.B + env];
+  DMX_TASKS(a, m.nu) u[a] = P.ctrl[((size_t)k * m.nu + a) * P.B + env];
   g.sync();
 }
 
@@ -36,8 +36,8 @@ template <int G>
 __device__ void store_state(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
                             double* dst /* [nx][B] */) {
   const double* qn = w.at(w.L->qn); const double* vn = w.at(w.L->vn);
-  for (int i = g.lane; i < m.nq; i += G) dst[(size_t)i * P.B + env] = qn[i];
-  for (int i = g.lane; i < m.nv; i += G) dst[(size_t)(m.nq + i) * P.B + env] = vn[i];
+  DMX_TASKS(i, m.nq) dst[(size_t)i * P.B + env] = qn[i];
+  DMX_TASKS(i, m.nv) dst[(size_t)(m.nq + i) * P.B + env] = vn[i];
 }
 
 template <int G>
@@ -56,8 +56,8 @@ __device__ void env_start(const Grp<G>& g, const DevModel& m, const Ws& w, const
   const Layout& L = *w.L;
   double* qn = w.at(L.qn); double* vn = w.at(L.vn);
   bool fin = true;
-  for (int i = g.lane; i < m.nq; i += G) { qn[i] = P.x0[(size_t)i * P.B + env]; fin = fin && isfinite(qn[i]); }
-  for (int i = g.lane; i < m.nv; i += G) { vn[i] = P.x0[(size_t)(m.nq + i) * P.B + env]; fin = fin && isfinite(vn[i]); }
+  DMX_TASKS(i, m.nq) { qn[i] = P.x0[(size_t)i * P.B + env]; fin = fin && isfinite(qn[i]); }
+  DMX_TASKS(i, m.nv) { vn[i] = P.x0[(size_t)(m.nq + i) * P.B + env]; fin = fin && isfinite(vn[i]); }
   int bad = fin ? 0 : 1;
   bad = g.isum(bad);
   if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[L.pmask + k] = 0;
@@ -97,8 +97,8 @@ __device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, con
     const double* qs = w.at(L.qs); const double* vs = w.at(L.vs);
     double* ka = w.at(L.ka);
     const int last = (TAB(mt).S - 1) * m.nv;
-    for (int i = g.lane; i < m.nq; i += G) qn[i] = qs[i];
-    for (int i = g.lane; i < m.nv; i += G) { vn[i] = vs[i]; ka[i] = ka[last + i]; }
+    DMX_TASKS(i, m.nq) qn[i] = qs[i];
+    DMX_TASKS(i, m.nv) { vn[i] = vs[i]; ka[i] = ka[last + i]; }
     g.sync();
     ++s.nacc;
     if (TAB(mt).adaptive) {
@@ -149,8 +149,8 @@ __device__ void load_step_state(const Grp<G>& g, const DevModel& m, const Ws& w,
                                 const StepState& S, int env, EnvState& s) {
   const Layout& L = *w.L;
   double* qn = w.at(L.qn); double* vn = w.at(L.vn); double* ka = w.at(L.ka);
-  for (int i = g.lane; i < m.nq; i += G) qn[i] = S.q[(size_t)i * P.B + env];
-  for (int i = g.lane; i < m.nv; i += G) { vn[i] = S.v[(size_t)i * P.B + env]; ka[i] = S.ka0[(size_t)i * P.B + env]; }
+  DMX_TASKS(i, m.nq) qn[i] = S.q[(size_t)i * P.B + env];
+  DMX_TASKS(i, m.nv) { vn[i] = S.v[(size_t)i * P.B + env]; ka[i] = S.ka0[(size_t)i * P.B + env]; }
   if (g.lane == 0)
     for (int k = 0; k < MASKW; ++k) w.i[L.pmask + k] = S.pmask[(size_t)k * P.B + env];
   s.t = S.t[env]; s.h = S.h[env]; s.lerrp = S.lerrp[env]; s.T = P.T[env];
@@ -164,8 +164,8 @@ __device__ void save_step_state(const Grp<G>& g, const DevModel& m, const Ws& w,
                                 const StepState& S, int env, const EnvState& s) {
   const Layout& L = *w.L;
   const double* qn = w.at(L.qn); const double* vn = w.at(L.vn); const double* ka = w.at(L.ka);
-  for (int i = g.lane; i < m.nq; i += G) S.q[(size_t)i * P.B + env] = qn[i];
-  for (int i = g.lane; i < m.nv; i += G) { S.v[(size_t)i * P.B + env] = vn[i]; S.ka0[(size_t)i * P.B + env] = ka[i]; }
+  DMX_TASKS(i, m.nq) S.q[(size_t)i * P.B + env] = qn[i];
+  DMX_TASKS(i, m.nv) { S.v[(size_t)i * P.B + env] = vn[i]; S.ka0[(size_t)i * P.B + env] = ka[i]; }
   if (g.lane == 0) {
     for (int k = 0; k < MASKW; ++k) S.pmask[(size_t)k * P.B + env] = w.i[L.pmask + k];
     S.t[env] = s.t; S.h[env] = s.h; S.lerrp[env] = s.lerrp;
@@ -267,14 +267,14 @@ __global__ void __launch_bounds__(32, 1) k_eval_rhs(const __grid_constant__ Roll
   const int env = (blockIdx.x * blockDim.x + threadIdx.x) / G;
   if (env >= P.B) return;
   double* qs = w.at(sL.qs); double* vs = w.at(sL.vs); double* uu = w.at(sL.u);
-  for (int i = g.lane; i < m.nq; i += G) qs[i] = q[(size_t)i * P.B + env];
-  for (int i = g.lane; i < m.nv; i += G) vs[i] = v[(size_t)i * P.B + env];
-  for (int i = g.lane; i < m.nu; i += G) uu[i] = u[(size_t)i * P.B + env];
+  DMX_TASKS(i, m.nq) qs[i] = q[(size_t)i * P.B + env];
+  DMX_TASKS(i, m.nv) vs[i] = v[(size_t)i * P.B + env];
+  DMX_TASKS(i, m.nu) uu[i] = u[(size_t)i * P.B + env];
   if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
   g.sync();
   double* res = w.at(sL.ka);
   const int st = rhs(g, m, w, qs, vs, uu, cfd != 0, res);
-  for (int i = g.lane; i < m.nv; i += G) a[(size_t)i * P.B + env] = res[i];
+  DMX_TASKS(i, m.nv) a[(size_t)i * P.B + env] = res[i];
   if (g.lane == 0) {
     int nact = 0;
     for (int k = 0; k < MASKW; ++k) nact += __popc(w.i[sL.amask + k]);

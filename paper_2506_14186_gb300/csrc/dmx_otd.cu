@@ -57,7 +57,7 @@ __device__ __forceinline__ double otd_boundary(double T, int NI, int k) { return
 template <int G>
 __device__ void kin_adjoint(const Grp<G>& g, const DevModel& m, const double* q, const double* v, const double* aq,
                             double* kq, double* kv) {
-  for (int b = g.lane; b < m.nbody; b += G) {
+  DMX_TASKS(b, m.nbody) {
     const int qa = m.b_qadr[b], va = m.b_vadr[b];
     if (m.b_jtype[b] == JNT_HINGE) { kv[va] += aq[qa]; continue; }
     for (int i = 0; i < 3; ++i) kv[va + i] += aq[qa + i];
@@ -89,14 +89,14 @@ __device__ int otd_stage(const Grp<G>& g, const DevModel& m, const Ws& w, const 
     if (s2 > st) st = s2;
   }
   double* qb = b.at(LB.qnb); double* vb = b.at(LB.vnb); double* ub = b.at(LB.ub);
-  for (int i = g.lane; i < nq; i += G) qb[i] = 0.0;
-  for (int i = g.lane; i < nv; i += G) vb[i] = 0.0;
-  for (int i = g.lane; i < nu; i += G) ub[i] = 0.0;
+  DMX_TASKS(i, nq) qb[i] = 0.0;
+  DMX_TASKS(i, nv) vb[i] = 0.0;
+  DMX_TASKS(i, nu) ub[i] = 0.0;
   g.sync();
   rhs_vjp(g, m, w, b, qs, vs, u, cfd, st, as + nq, qb, vb, ub);
-  for (int i = g.lane; i < nq; i += G) ka[i] = qb[i];
-  for (int i = g.lane; i < nv; i += G) ka[nq + i] = vb[i];
-  for (int i = g.lane; i < nu; i += G) ka[nq + nv + i] = ub[i];
+  DMX_TASKS(i, nq) ka[i] = qb[i];
+  DMX_TASKS(i, nv) ka[nq + i] = vb[i];
+  DMX_TASKS(i, nu) ka[nq + nv + i] = ub[i];
   g.sync();
   kin_adjoint(g, m, qs, vs, as, ka, ka + nq);
   return st;
@@ -129,15 +129,15 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
     env = g.bcast(env, 0);
     if (env >= P.B) break;
     const double T = P.T[env];
-    for (int i = g.lane; i < nq; i += G) qn[i] = P.xT[(size_t)i * P.B + env];
-    for (int i = g.lane; i < nv; i += G) vn[i] = P.xT[(size_t)(nq + i) * P.B + env];
-    for (int i = g.lane; i < na; i += G) {
+    DMX_TASKS(i, nq) qn[i] = P.xT[(size_t)i * P.B + env];
+    DMX_TASKS(i, nv) vn[i] = P.xT[(size_t)(nq + i) * P.B + env];
+    DMX_TASKS(i, na) {
       double x = i < nx ? P.xT_bar[(size_t)i * P.B + env] : 0.0;
       if (i < nx && P.xb_bar) x += P.xb_bar[((size_t)P.NI * nx + i) * P.B + env];
       a[i] = x;
     }
     if (P.ctrl_bar)
-      for (int i = g.lane; i < P.NI * nu; i += G) P.ctrl_bar[(size_t)i * P.B + env] = 0.0;
+      DMX_TASKS(i, P.NI * nu) P.ctrl_bar[(size_t)i * P.B + env] = 0.0;
     if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
     g.sync();
     int k = P.NI - 1, steps = 0, attempts = 0, status = ENV_OK;
@@ -149,13 +149,13 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
       const bool clamped = h >= hb || hb - h < 1e-12;
       const double ht = clamped ? hb : h;
       if (ht < 1e-12) { status = ENV_H_UNDERFLOW; break; }
-      for (int i = g.lane; i < nu; i += G) u[i] = P.ctrl[((size_t)k * nu + i) * P.B + env];
-      for (int i = g.lane; i < nv; i += G) kv[i] = vn[i];
+      DMX_TASKS(i, nu) u[i] = P.ctrl[((size_t)k * nu + i) * P.B + env];
+      DMX_TASKS(i, nv) kv[i] = vn[i];
       g.sync();
       int st = otd_stage(g, m, w, b, qn, vn, u, a, P.cfd != 0, kf, ka);
       for (int s = 1; s < S; ++s) {
         const unsigned mq = TAB(mt).nzq[s], mv = TAB(mt).nzv[s];
-        for (int i = g.lane; i < nv; i += G) {
+        DMX_TASKS(i, nv) {
           double sq = 0, sv = 0;
           for (int j = 0; j < s; ++j) {
             if ((mq >> j) & 1u) sq += TAB(mt).aq[s][j] * kv[j * nv + i];
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
           vs[i] = vv;
           kv[s * nv + i] = vv;
         }
-        for (int i = g.lane; i < na; i += G) {
+        DMX_TASKS(i, na) {
           double sa = 0;
           for (int j = 0; j < s; ++j)
             if ((mv >> j) & 1u) sa += TAB(mt).av[s][j] * ka[j * na + i];
@@ -180,12 +180,12 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
       }
       ++attempts;
       // the result is the last stage: (qs, vs) and as
-      for (int i = g.lane; i < na; i += G) a7[i] = as[i];
+      DMX_TASKS(i, na) a7[i] = as[i];
       double err = 0.0;
       if (TAB(mt).adaptive) {
         const unsigned enz = TAB(mt).enz;
         double acc = 0.0;
-        for (int i = g.lane; i < nv; i += G) {
+        DMX_TASKS(i, nv) {
           double ep = 0, ev = 0;
           for (int j = 0; j < 7; ++j) {
             if (!((enz >> j) & 1u)) continue;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
           const double sv = P.atol + P.rtol * fmax(fabs(vn[i]), fabs(vs[i]));
           acc += (ep / sp) * (ep / sp) + (ev / sv) * (ev / sv);
         }
-        for (int i = g.lane; i < na; i += G) {
+        DMX_TASKS(i, na) {
           double ea = 0;
           for (int j = 0; j < 7; ++j)
             if ((enz >> j) & 1u) ea += TAB(mt).e[j] * ka[j * na + i];
@@ -212,9 +212,9 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
       g.sync();
       if (err <= 1.0) {
         if (st != ENV_OK) { status = st; break; }
-        for (int i = g.lane; i < nq; i += G) qn[i] = qs[i];
-        for (int i = g.lane; i < nv; i += G) vn[i] = vs[i];
-        for (int i = g.lane; i < na; i += G) a[i] = a7[i];
+        DMX_TASKS(i, nq) qn[i] = qs[i];
+        DMX_TASKS(i, nv) vn[i] = vs[i];
+        DMX_TASKS(i, na) a[i] = a7[i];
         g.sync();
         ++steps;
         t = clamped ? tlo : t - ht;
@@ -228,12 +228,12 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
           h = P.h0;
         }
         if (clamped) {                       // reached the interval's lower boundary t_k
-          for (int j = g.lane; j < nu; j += G) {
+          DMX_TASKS(j, nu) {
             if (P.ctrl_bar) P.ctrl_bar[((size_t)k * nu + j) * P.B + env] += a[nx + j];
             a[nx + j] = 0.0;
           }
           if (P.xb_bar)
-            for (int i = g.lane; i < nx; i += G) a[i] += P.xb_bar[((size_t)k * nx + i) * P.B + env];
+            DMX_TASKS(i, nx) a[i] += P.xb_bar[((size_t)k * nx + i) * P.B + env];
           g.sync();
           --k;
         }
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_otd(const __grid_constant__ O
         h = ht * (isfinite(err) ? fmax(0.2, 0.9 * pow(err, -1.0 / 5.0)) : 0.2);
       }
     }
-    for (int i = g.lane; i < nx; i += G) P.x0_bar[(size_t)i * P.B + env] = a[i];
+    DMX_TASKS(i, nx) P.x0_bar[(size_t)i * P.B + env] = a[i];
     if (g.lane == 0) {
       if (P.steps) P.steps[env] = steps;
       if (P.status) P.status[env] = status;

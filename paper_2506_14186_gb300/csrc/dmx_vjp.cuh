@@ -465,13 +465,13 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     const int s = s0 + g.lane;
     incl |= g.ballot(s < m.nslot && slotrow[s] >= 0) << s0;
   }
-  for (int i = g.lane; i < nv; i += G) { y[i] = abar[i]; vb[i] = 0.0; }
-  for (int i = g.lane; i < nq; i += G) qb[i] = 0.0;
-  for (int a = g.lane; a < m.nu; a += G) ub[a] = 0.0;
+  DMX_TASKS(i, nv) { y[i] = abar[i]; vb[i] = 0.0; }
+  DMX_TASKS(i, nq) qb[i] = 0.0;
+  DMX_TASKS(a, m.nu) ub[a] = 0.0;
   g.sync();
   // ---- constraint solve: y = H_A^-1 abar with the factor of the final set
   chol_solve(g, w.at(L.H), w.at(L.tmp2), y, nv);
-  for (int r = g.lane; r < nr; r += G) {
+  DMX_TASKS(r, nr) {
     double t = 0.0;
     if (mask_has(am, rowid[r]))
       for (int i = 0; i < nv; ++i) t += J[r * nv + i] * y[i];
@@ -482,7 +482,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // ---- mass matrix: -(y an^T) folded to the lower triangle, W_kj = -(y_k an_j + y_j an_k),
   // over the Newton factor, which is done with
   double* W = w.at(L.H);
-  for (int t = g.lane; t < nv * (nv + 1) / 2; t += G) {
+  DMX_TASKS(t, nv * (nv + 1) / 2) {
     const Tri ij = tri(t);
     const int i = ij.i, j = ij.j;
     W[i * nv + j] = (i == j) ? -y[i] * an[i] : -(y[i] * an[j] + y[j] * an[i]);
@@ -490,7 +490,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   g.sync();
   // M_kj = S_j . F_k for j <= k with dof j's body an ancestor of dof k's body;
   // bias force c_i = S_i . Fb; one component per task
-  for (int t = g.lane; t < 6 * nv; t += G) {
+  DMX_TASKS(t, 6 * nv) {
     const int i = t / 6, e = t - 6 * i;
     const int bi = m.dof_body[i];
     double fd = 0.0;
@@ -509,7 +509,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   }
   g.sync();
   // ---- per dof: a_ref's J v term, damping, contact Jacobians
-  for (int i = g.lane; i < nv; i += G) {
+  DMX_TASKS(i, nv) {
     const int bi = m.dof_body[i];
     double acc = -m.b_damping[bi] * y[i];
     for (int r = 0; r < nr; ++r) acc -= m.bcoef * cj[r] * J[r * nv + i];
@@ -543,7 +543,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     }
   }
   // ---- per slot: record cotangents, impedance terms, contact geometry
-  for (int s = g.lane; s < m.nslot; s += G) {
+  DMX_TASKS(s, m.nslot) {
     const int r0 = slotrow[s];
     if (r0 < 0) continue;
     const double* ct = CT + 16 * s;
@@ -637,7 +637,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   g.sync();
   // ---- per geom: pose cotangents gathered from its slots (one component per task)
   double* GB = b.at(LB.gb);
-  for (int t = g.lane; t < 12 * m.ngeom; t += G) {
+  DMX_TASKS(t, 12 * m.ngeom) {
     const int gi = t / 12, c = t - 12 * gi;
     const unsigned m1 = m.g_slots1[gi];
     double acc = 0.0;
@@ -651,7 +651,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // ---- per body: geom poses -> body pose (gR = R_b Roff, gp = p_b + R_b gpos), one
   // entry per task; per dof and body component: bias-force (c_i = S_i . Fb) and
   // CRBA (F_i = Ic S_i) cotangents
-  for (int t = g.lane; t < 12 * nb; t += G) {
+  DMX_TASKS(t, 12 * nb) {
     const int bb = t / 12, c = t - 12 * bb;
     double acc = 0.0;
     for (unsigned ms = m.b_geoms[bb]; ms; ms &= ms - 1u) {
@@ -668,17 +668,17 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     }
     if (c < 9) Rb[9 * bb + c] = acc; else pb[3 * bb + c - 9] = acc;
   }
-  for (int t = g.lane; t < 6 * nv; t += G) {
+  DMX_TASKS(t, 6 * nv) {
     const Comp6 c = comp6(t, nv);
     Sb[6 * c.i + c.e] += inertia_comp(Ic + 10 * m.dof_body[c.i], Fd + 6 * c.i, c.e);
   }
-  for (int t = g.lane; t < 6 * nb; t += G) {
+  DMX_TASKS(t, 6 * nb) {
     const int bb = t / 6, e = t - 6 * bb;
     double acc = 0.0;
     for (int d = 0; d < m.b_nv[bb]; ++d) { const int i = m.b_vadr[bb] + d; acc += y[i] * S[6 * i + e]; }
     Fbb[t] = -acc;
   }
-  for (int t = g.lane; t < 10 * nb; t += G) {
+  DMX_TASKS(t, 10 * nb) {
     const Comp6 c = comp10(t, nb);
     double acc = 0.0;
     for (int d = 0; d < m.b_nv[c.i]; ++d) {
@@ -702,14 +702,14 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   //   f2 = V x* (I V):   Vbar and (I V)bar from the force cross product, then
   //                      Vbar += I (I V)bar,  Ibar += grad((I V)bar, V)
   double* IV = b.at(LB.iv); double* IVB = b.at(LB.ivb);
-  for (int t = g.lane; t < 6 * nb; t += G) {
+  DMX_TASKS(t, 6 * nb) {
     const Comp6 c = comp6(t, nb);
     const double* I = Ib + 10 * c.i;
     Abb[6 * c.i + c.e] = inertia_comp(I, Fbb + 6 * c.i, c.e);
     IV[6 * c.i + c.e] = inertia_comp(I, V + 6 * c.i, c.e);
   }
   g.sync();
-  for (int t = g.lane; t < 6 * nb; t += G) {
+  DMX_TASKS(t, 6 * nb) {
     const Comp6 ce = comp6(t, nb);
     const int bb = ce.i, e = ce.e;
     const double* a = V + 6 * bb; const double* iv = IV + 6 * bb; const double* fbar = Fbb + 6 * bb;
@@ -727,11 +727,11 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     IVB[6 * bb + e] = ivb_e;
   }
   g.sync();
-  for (int t = g.lane; t < 6 * nb; t += G) {
+  DMX_TASKS(t, 6 * nb) {
     const Comp6 c = comp6(t, nb);
     Vbb[6 * c.i + c.e] += inertia_comp(Ib + 10 * c.i, IVB + 6 * c.i, c.e);
   }
-  for (int t = g.lane; t < 10 * nb; t += G) {
+  DMX_TASKS(t, 10 * nb) {
     const Comp6 c = comp10(t, nb);
     Ibb[10 * c.i + c.e] += inertia_grad_comp(Fbb + 6 * c.i, A + 6 * c.i, c.e) +
                            inertia_grad_comp(IVB + 6 * c.i, V + 6 * c.i, c.e);
@@ -741,7 +741,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // A's own term (V x S_d) v_d (d past the free joint's translations):
   //   vbar_d += Abar . (V x S_d);  with cb = Abar v_d:  Vbar_w += S_w x cb_w + S_v x cb_v,
   //   Vbar_v += S_w x cb_v;  Sbar_w += cb_w x V_w + cb_v x V_v,  Sbar_v += cb_v x V_w
-  for (int i = g.lane; i < nv; i += G) {
+  DMX_TASKS(i, nv) {
     const int bb = m.dof_body[i];
     if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
     const double* vbv = V + 6 * bb; const double* sd = S + 6 * i; const double* ab6 = Abb + 6 * bb;
@@ -749,7 +749,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     for (int e = 0; e < 6; ++e) s1 += ab6[e] * crm_comp(vbv, sd, e);
     vb[i] += s1;
   }
-  for (int t = g.lane; t < 6 * nv; t += G) {
+  DMX_TASKS(t, 6 * nv) {
     const Comp6 ce = comp6(t, nv);
     const int i = ce.i, e = ce.e, bb = m.dof_body[i];
     if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
@@ -763,7 +763,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
       r = vd * (ab6[3 + c1] * a[c2] - ab6[3 + c2] * a[c1]);
     Sb[6 * i + e] += r;
   }
-  for (int t = g.lane; t < 6 * nb; t += G) {
+  DMX_TASKS(t, 6 * nb) {
     const Comp6 ce = comp6(t, nb);
     const int bb = ce.i, e = ce.e;
     const double* ab6 = Abb + 6 * bb;
@@ -784,18 +784,18 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   g.sync();
   tree_up<6>(g, m, Vbb);             // V_child = V_parent + ...
   // V's own term S_d v_d: vbar_d += Vbar . S_d, Sbar_d += Vbar v_d (per dof, per dof component)
-  for (int i = g.lane; i < nv; i += G) {
+  DMX_TASKS(i, nv) {
     const double* vbar6 = Vbb + 6 * m.dof_body[i]; const double* sd = S + 6 * i;
     double s1 = 0.0;
     for (int e = 0; e < 6; ++e) s1 += vbar6[e] * sd[e];
     vb[i] += s1;
   }
-  for (int k = g.lane; k < 6 * nv; k += G) {
+  DMX_TASKS(k, 6 * nv) {
     const int i = k / 6, e = k - 6 * i;
     Sb[6 * i + e] += Vbb[6 * m.dof_body[i] + e] * v[i];
   }
   // actuators: motor tau += gear u; position servo tau += kp (u - q) - kd v
-  for (int i = g.lane; i < nv; i += G)
+  DMX_TASKS(i, nv)
     for (int a = m.dof_act[i]; a >= 0; a = m.act_next[a]) {
       if (m.a_type[a] == ACT_MOTOR) ub[a] += m.a_gear[a] * y[i];
       else { ub[a] += m.a_kp[a] * y[i]; qb[m.a_qadr[a]] -= m.a_kp[a] * y[i]; vb[i] -= m.a_kd[a] * y[i]; }
@@ -807,7 +807,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     // on masses and sides
     const int np = PAR_MU0 + m.npair + m.nbody + m.nbox;
     const double* PR = b.at(LB.pr);
-    for (int k = g.lane; k < np; k += G) {
+    DMX_TASKS(k, np) {
       double acc = 0.0;
       if (k < PAR_MU0) {
         const double dk = k == PAR_TC ? -2.0 * m.kcoef / m.solref[0]
@@ -869,9 +869,9 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // one pose entry per task (inertia, COM and motion-vector terms) and one
   // local-rotation entry per task for the composition.
   double* SCb = b.at(LB.sc); double* TK = b.at(LB.tk);
-  for (int t = g.lane; t < nb; t += G)
+  DMX_TASKS(t, nb)
     if (m.b_jtype[t] == JNT_HINGE) ::sincos(q[m.b_qadr[t]], &SCb[2 * t], &SCb[2 * t + 1]);
-  for (int k = g.lane; k < 3 * nb; k += G) {
+  DMX_TASKS(k, 3 * nb) {
     const int bb = k / 3, r = k - 3 * (k / 3);
     const double ms = m.b_mass[bb];
     const double* ib = Ibb + 10 * bb; const double* c = C + 3 * bb;
@@ -883,7 +883,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     cp[k] = ms * (ib[1 + r] + 2.0 * c[r] * tr - (Br[0] * c[0] + Br[1] * c[1] + Br[2] * c[2]));
   }
   g.sync();
-  for (int t = g.lane; t < 9 * nb; t += G) {
+  DMX_TASKS(t, 9 * nb) {
     const int bb = t / 9, comp = t - 9 * bb;
     const double* Rv = R + 9 * bb; const double* pv = P + 3 * bb;
     const double* cb3 = cp + 3 * bb;
@@ -904,7 +904,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     val += fr ? wb : wb * m.b_axis[bb][kk];
     Rb[9 * bb + comp] += val;
   }
-  for (int t = g.lane; t < 3 * nb; t += G) {
+  DMX_TASKS(t, 3 * nb) {
     const int bb = t / 3, r = t - 3 * bb, r1 = nxt3(r), r2 = prv3(r);
     const double* Rv = R + 9 * bb;
     const int va = m.b_vadr[bb];
@@ -923,7 +923,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     }
     pb[t] += val;
   }
-  for (int k = g.lane; k < 9 * nb; k += G) {
+  DMX_TASKS(k, 9 * nb) {
     const int bb = k / 9, e = k - 9 * (k / 9);
     if (m.b_jtype[bb] != JNT_HINGE) continue;
     const int i = e / 3, j = e - 3 * (e / 3);
@@ -944,7 +944,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   // (one parent entry per task)
   for (int lev = m.nlevel - 1; lev >= 1; --lev) {
     const int k0 = m.level_start[lev - 1], n = 12 * (m.level_start[lev] - k0);
-    for (int t = g.lane; t < n; t += G) {
+    DMX_TASKS(t, n) {
       const int kb = t / 12, comp = t - 12 * (t / 12);
       const int bb = m.lv_pack[k0 + kb] & 255;
       const int c0 = m.child_start[bb], nc = m.child_count[bb];
@@ -969,14 +969,14 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
   }
   // joint coordinates: free joints (translation, quaternion), one task per body;
   // hinges: theta bar = <Roff^T R_parent^T Rbar, dRj/dtheta>, one entry per task
-  for (int bb = g.lane; bb < nb; bb += G) {
+  DMX_TASKS(bb, nb) {
     if (m.b_jtype[bb] != JNT_FREE) continue;
     const double* rb = Rb + 9 * bb; const double* pbv = pb + 3 * bb;
     const int qa = m.b_qadr[bb];
     qb[qa] += pbv[0]; qb[qa + 1] += pbv[1]; qb[qa + 2] += pbv[2];
     quat_to_mat_vjp(q + qa + 3, rb, qb + qa + 3);
   }
-  for (int k = g.lane; k < 9 * nb; k += G) {
+  DMX_TASKS(k, 9 * nb) {
     const int bb = k / 9, e = k - 9 * (k / 9);
     if (m.b_jtype[bb] != JNT_HINGE) continue;
     const int i = e / 3, j = e - 3 * (e / 3);
@@ -997,15 +997,15 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
     TK[k] = rjb * dr;
   }
   g.sync();
-  for (int bb = g.lane; bb < nb; bb += G) {
+  DMX_TASKS(bb, nb) {
     if (m.b_jtype[bb] != JNT_HINGE) continue;
     const double* tk = TK + 9 * bb;
     qb[m.b_qadr[bb]] += (((tk[0] + tk[1]) + (tk[2] + tk[3])) + ((tk[4] + tk[5]) + (tk[6] + tk[7]))) + tk[8];
   }
   g.sync();
-  for (int i = g.lane; i < nq; i += G) qbar[i] += qb[i];
-  for (int i = g.lane; i < nv; i += G) vbar[i] += vb[i];
-  for (int a = g.lane; a < m.nu; a += G) ubar[a] += ub[a];
+  DMX_TASKS(i, nq) qbar[i] += qb[i];
+  DMX_TASKS(i, nv) vbar[i] += vb[i];
+  DMX_TASKS(a, m.nu) ubar[a] += ub[a];
   g.sync();
 }
 
@@ -1014,7 +1014,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
 template <int G>
 __device__ void integrate_pos_vjp(const Grp<G>& g, const DevModel& m, const double* q, const double* dq,
                                   const double* ob, double* qbar, double* dqbar) {
-  for (int b = g.lane; b < m.nbody; b += G) {
+  DMX_TASKS(b, m.nbody) {
     const int qa = m.b_qadr[b], va = m.b_vadr[b];
     if (m.b_jtype[b] == JNT_HINGE) { qbar[qa] += ob[qa]; dqbar[va] = ob[qa]; continue; }
     for (int k = 0; k < 3; ++k) { qbar[qa + k] += ob[qa + k]; dqbar[va + k] = ob[qa + k]; }
