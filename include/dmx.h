@@ -163,7 +163,9 @@ typedef struct {
   int32_t* nrej;              /* out [B] rejected attempts, or NULL */
   int32_t* status;            /* out [B] DMX_ENV_* codes, or NULL */
   dmx_tape** tape;            /* out: tape for dmx_rollout_grad (checkpoints every K accepted
-                                 steps + accepted step sizes), or NULL for forward only */
+                                 steps + accepted step sizes; with the reverse adjoint selected,
+                                 also the steps' stage snapshots, within an eighth of the free
+                                 device memory and 24 GiB), or NULL for forward only */
   int32_t method;             /* DMX_METHOD_*: integration scheme (0 = adaptive Dormand-Prince 5(4)) */
 } dmx_rollout_args;
 
@@ -244,7 +246,8 @@ dmx_status dmx_rollout_grad_otd(dmx_model* m, const dmx_otd_args* a, void* strea
  *     library device memory while a segment between two checkpoints is
  *     recomputed (K steps x 6 stages per resident environment, used when it
  *     fits 1/8 of the free device memory and 8 GiB), so each stage is
- *     evaluated once; otherwise as DMX_ADJ_RECOMPUTE.  An environment whose
+ *     evaluated once; otherwise as DMX_ADJ_RECOMPUTE.  Segments whose steps the
+ *     tape kept with their snapshots are not recomputed at all.  An environment whose
  *     right-hand side overflowed the row workspace during the adjoint gets
  *     NaN in x0_bar.
  *   DMX_ADJ_RECOMPUTE: the same reverse mode, evaluating each stage's

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include "dmx_model.h"
+#include "dmx_record.h"
 
 namespace dmx {
 
@@ -24,38 +25,12 @@ struct AdjParams {
   double* segbuf;         // per warp (tangent) or group (reverse): recomputed steps of a segment
   double* snapbuf;        // reverse mode: per group, K steps x (S - 1) stage snapshots of SN doubles (or null)
   int SN;                 // doubles per snapshot
+  StepRecords rec;        // records of the taped rollout
   int per, barofs;        // reverse mode: doubles per environment, offset of the cotangent workspace
   double* p_bar;          // [np][B] model-parameter gradients, or null
   int np;                 // model parameters differentiated when p_bar is set
   int* queue;             // next environment
 };
-
-// Offsets (doubles) of one stage snapshot: the part of a right-hand-side
-// workspace that its VJP reads (poses .. geom frames, the Cholesky factor of
-// the final Newton system with the solution, contact records, the used
-// Jacobian rows with D and the residuals, then as ints: status, rows,
-// slot->row map, row ids, final active set).
-struct SnapOff {
-  int n1, o2, n2, o3, o4, o5, o6, oi, size;
-};
-__host__ __device__ inline SnapOff snap_offsets(const DevModel& m, const Layout& L) {
-  SnapOff o{};
-  o.n1 = L.gp + 3 * m.ngeom - L.R;
-  o.o2 = o.n1;
-  o.n2 = L.tmp2 + m.nv - L.H;
-  o.o3 = o.o2 + o.n2;
-  o.o4 = o.o3 + 18 * m.nslot;          // contact records, then the closest-point parameters (2 per slot)
-  o.o5 = o.o4 + L.rcap * m.nv;
-  o.o6 = o.o5 + L.rcap;
-  o.oi = o.o6 + L.rcap;
-  const int nints = 3 + m.nslot + L.rcap + MASKW;
-  o.size = (o.oi + (nints + 1) / 2 + 1) & ~1;
-  return o;
-}
-
-// Doubles per recomputed step in the reverse kernel's segment buffer: q_n,
-// the stage velocities V_0..V_6, t_n.
-__host__ __device__ inline int rev_row_doubles(const DevModel& m) { return m.nq + 7 * m.nv + 1; }
 
 cudaError_t launch_adjoint(const AdjParams& P, int blocks, cudaStream_t st);
 // out[k] = sum over e of x[k][e] (k < n, e < B): one block per row, fixed order.

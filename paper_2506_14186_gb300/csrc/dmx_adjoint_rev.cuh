@@ -25,11 +25,13 @@
 // evaluating the right-hand side a second time: device memory traded for
 // FP64 work.  The final active set of a stage does not depend on the
 // warm start of its Newton search, so the restored workspace equals a
-// recomputed one.
+// recomputed one.  Segments whose steps the forward pass kept (dmx_record.h)
+// are not recomputed at all: rows and snapshots are read from the records.
 #pragma once
 #include <cuda_runtime.h>
 
 #include "dmx_adjoint.h"
+#include "dmx_record.cuh"
 #include "dmx_vjp.cuh"
 
 namespace dmx {
@@ -41,40 +43,6 @@ __device__ __forceinline__ int rev_interval(double T, int NI, double t) {
   return k;
 }
 
-// dst[i] = src[i], i < n, eight loads in flight per lane (the snapshots live in
-// device memory: one round trip per eight passes instead of one per pass).
-template <int G>
-__device__ __forceinline__ void copy_run(const Grp<G>& g, const double* __restrict__ src, double* __restrict__ dst,
-                                         int n) {
-  for (int i0 = g.lane; i0 < n; i0 += 8 * G) {
-    double x[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (i0 + k * G < n) x[k] = src[i0 + k * G];
-#pragma unroll
-    for (int k = 0; k < 8; ++k)
-      if (i0 + k * G < n) dst[i0 + k * G] = x[k];
-  }
-}
-// Workspace of the right-hand side just evaluated (status st) -> snapshot dst.
-template <int G>
-__device__ void snap_save(const Grp<G>& g, const DevModel& m, const Ws& w, double* dst, int st) {
-  const Layout& L = *w.L;
-  const SnapOff o = snap_offsets(m, L);
-  const int nr = (st == ENV_ROW_OVERFLOW) ? 0 : w.i[L.slotrow + m.nslot];
-  const double* d = w.d;
-  DMX_TASKS(i, o.n1) dst[i] = d[L.R + i];
-  DMX_TASKS(i, o.n2) dst[o.o2 + i] = d[L.H + i];
-  DMX_TASKS(i, 16 * m.nslot) dst[o.o3 + i] = d[L.ct + i];
-  DMX_TASKS(i, 2 * m.nslot) dst[o.o3 + 16 * m.nslot + i] = d[L.csv + i];
-  DMX_TASKS(i, nr * m.nv) dst[o.o4 + i] = d[L.J + i];
-  DMX_TASKS(i, nr) { dst[o.o5 + i] = d[L.Dr + i]; dst[o.o6 + i] = d[L.z + i]; }
-  int* di = reinterpret_cast<int*>(dst + o.oi);
-  if (g.lane == 0) { di[0] = st; di[1] = nr; }
-  for (int i = g.lane; i <= m.nslot; i += G) di[2 + i] = w.i[L.slotrow + i];
-  DMX_TASKS(i, nr) di[3 + m.nslot + i] = w.i[L.rowid + i];
-  DMX_TASKS(i, MASKW) di[3 + m.nslot + L.rcap + i] = w.i[L.amask + i];
-}
 // Snapshot src -> workspace (the state rhs() leaves for rhs_vjp, except the
 // contact records and Jacobian rows, which the VJP reads from the snapshot
 // itself: see snap_view); returns the status.
@@ -214,6 +182,10 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
     int worst = 0;
     for (int c = N > 0 ? (N - 1) / P.K : -1; c >= 0; --c) {
       const int n0 = c * P.K, n1 = min(n0 + P.K, N);
+      // the forward pass kept this segment's steps: nothing to recompute
+      bool kept = P.rec.mem != nullptr;
+      for (int k = n0 / REC_STEPS; kept && k <= (n1 - 1) / REC_STEPS; ++k) kept = P.rec.chunk[(size_t)env * P.rec.per_env + k] > 0;
+      if (!kept) {
       // ---- forward recompute of the segment from checkpoint c: q_n, V_0..V_5, t_n per step
       const double* ck = P.ckpt + (size_t)c * (nx + 1) * P.B;
       DMX_TASKS(i, nq) qn[i] = ck[(size_t)i * P.B + env];
@@ -258,13 +230,15 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
       }
       __threadfence_block();
       g.sync();
+      }
       // ---- reverse sweep over the segment's steps
       double* bq = b.at(sB.qn); double* bv = b.at(sB.vst);
       double* Qb = b.at(sB.Qb); double* Vb = b.at(sB.Vb);
       if constexpr (PAR)               // the segment's sums live in the cotangent workspace
         DMX_TASKS(k, P.np) b.at(sB.pa)[k] = 0.0;
       for (int n = n1 - 1; n >= n0; --n) {
-        const double* row = seg + (size_t)(n - n0) * RW;
+        const double* srec = kept ? step_record(P.rec, env, n) : nullptr;
+        const double* row = kept ? srec + (S - 1) * P.rec.snap : seg + (size_t)(n - n0) * RW;
         const double tn0 = row[nq + 7 * nv];
         const int kn = rev_interval(T, P.NI, tn0);
         const double h = P.hlog[(size_t)n * P.B + env];
@@ -280,7 +254,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
         DMX_TASKS(i, nv) Vb[i] = xbar[nq + i];
         g.sync();
         const int st = rk_step_vjp<G, PAR>(g, m, w, b, (const double*)u, h, mt, P.cfd != 0,
-                                   use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr, SN);
+                                   P.cfd ? nullptr : kept ? srec : use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr,
+                                   SN);
         if (st > worst) worst = st;
         const double* qnb = b.at(sB.qnb); const double* vnb = b.at(sB.vnb); const double* ub = b.at(sB.ub);
         DMX_TASKS(i, nq) xbar[i] = qnb[i];

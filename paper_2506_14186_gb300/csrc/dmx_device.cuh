@@ -1646,15 +1646,15 @@ __device__ double sum_as_lanes(const Grp<G>& g, double* x, int n, int C) {
 // the RMS error norm of the embedded estimate (NaN-safe: non-finite -> +inf;
 // 0 for a fixed-step scheme; summed in the order of `red` lanes) and the
 // worst stage status.
-template <int G>
+template <int G, class Hook>
 __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
-                             double rtol, double atol, int red, int* st_out) {
+                             double rtol, double atol, int red, int* st_out, Hook&& hook) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   const double* qn = w.at(L.qn); const double* vn = w.at(L.vn);
   const double* qs = w.at(L.qs); const double* vs = w.at(L.vs);
   const double* kv = w.at(L.kv); const double* ka = w.at(L.ka);
-  const int st = rk_stages(g, m, w, u, h, mt, [](int, int) {});
+  const int st = rk_stages(g, m, w, u, h, mt, hook);
   *st_out = st;
   if (!TAB(mt).adaptive) return 0.0;
   const unsigned enz = TAB(mt).enz;
@@ -1680,4 +1680,9 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
   return isfinite(err) ? err : INFINITY;
 }
 
+template <int G>
+__device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
+                             double rtol, double atol, int red, int* st_out) {
+  return rk_attempt(g, m, w, u, h, mt, rtol, atol, red, st_out, [](int, int) {});
+}
 }  // namespace dmx

@@ -15,6 +15,7 @@
 
 #include "dmx_device.cuh"
 #include "dmx_kernels.h"
+#include "dmx_record.cuh"
 
 namespace dmx {
 
@@ -69,6 +70,7 @@ __device__ void env_start(const Grp<G>& g, const DevModel& m, const Ws& w, const
   if (bad) { s.st = ENV_NONFINITE; s.done = 1; return; }
   if (m.nu) load_ctrl(g, m, w, P, env, 0);
   const int st = rhs(g, m, w, qn, vn, w.at(L.u), false, w.at(L.ka));
+  if (double* r = claim_record(g, P.rec, env, 0)) snap_save(g, m, w, r, st);
   if (st != ENV_OK) { s.st = st; s.done = 1; }
 }
 
@@ -86,11 +88,27 @@ __device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, con
   if (ht < 1e-12) { s.st = ENV_H_UNDERFLOW; s.done = 1; return; }
   int stage_st = 0;
   const int mt = P.method;
-  const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, P.red, &stage_st);
+  // records of a taped rollout: stages 1 .. S - 2 belong to this step, the
+  // last one is stage 0 of the next (a rejected attempt's are overwritten)
+  double* rec = claim_record(g, P.rec, env, s.nacc);
+  double* rec1 = rec ? claim_record(g, P.rec, env, s.nacc + 1) : nullptr;
+  const int S = TAB(mt).S;
+  const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, P.red, &stage_st, [&](int st, int r) {
+    double* dst = st <= S - 2 ? (rec ? rec + (size_t)st * P.rec.snap : nullptr) : rec1;
+    if (dst) snap_save(g, m, w, dst, r);
+  });
   ++s.att;
   if (err <= 1.0) {
     if (stage_st != ENV_OK) { s.st = stage_st; s.done = 1; return; }
     if (P.hlog && g.lane == 0) P.hlog[(size_t)s.nacc * P.B + env] = ht;
+    if (rec) {                         // the step's row: q_n, stage velocities, t_n
+      double* row = rec + (size_t)(S - 1) * P.rec.snap;
+      const double* q0 = w.at(L.qn); const double* kv = w.at(L.kv);
+      DMX_TASKS(i, m.nq) row[i] = q0[i];
+      DMX_TASKS(i, S * m.nv) row[m.nq + i] = kv[i];
+      if (g.lane == 0) row[m.nq + 7 * m.nv] = s.t;
+      g.sync();
+    }
     const bool reached = clamped || (s.t + ht >= tn);
     s.t = reached ? tn : s.t + ht;
     double* qn = w.at(L.qn); double* vn = w.at(L.vn);
@@ -120,6 +138,7 @@ __device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, con
       if (s.k < P.NI) {
         if (m.nu) load_ctrl(g, m, w, P, env, s.k);
         const int st = rhs(g, m, w, qn, vn, w.at(L.u), false, ka);
+        if (rec1) snap_save(g, m, w, rec1, st);   // the new control's stage 0
         if (st != ENV_OK) { s.st = st; s.done = 1; return; }
       }
     }

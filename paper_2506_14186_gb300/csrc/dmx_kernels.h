@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include "dmx_model.h"
+#include "dmx_record.h"
 
 namespace dmx {
 
@@ -25,6 +26,7 @@ struct RolloutParams {
   double* hlog;         // [max_steps][B] or null (tape: accepted step sizes)
   int* tape_n;          // [B] or null (tape: accepted steps)
   int* queue;           // persistent form: next environment
+  StepRecords rec;      // tape: step records for the reverse adjoint
 };
 
 // Plain (one launch per attempt) form: integrator state in HBM.

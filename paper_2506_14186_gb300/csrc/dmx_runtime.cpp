@@ -500,13 +500,51 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
   return DMX_OK;
 }
 
+// Step records for a tape: as many chunks as 512 steps of every environment
+// take, within an eighth of the free device memory and 24 GiB; none when that
+// is less than a chunk per environment, or the allocation fails.  With them
+// the adjoint has no segment to recompute (45 % of its time), for the price of
+// the writes (118 KB an arm's step).
+constexpr size_t kRecMaxBytes = size_t(24) << 30;
+static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
+  const int stages = t->method == DMX_METHOD_EULER ? 1 : 6;
+  dmx::StepRecords r{};
+  r.snap = dmx::snap_offsets(m->host, m->L).size;
+  r.stride = (stages * r.snap + dmx::rev_row_doubles(m->host) + 1) & ~1;
+  r.per_env = (t->max_steps + dmx::REC_STEPS) / dmx::REC_STEPS;
+  const size_t chunk = sizeof(double) * dmx::REC_STEPS * (size_t)r.stride;
+  const size_t table = (sizeof(int) * ((size_t)t->B * r.per_env + 1) + 255) & ~size_t(255);
+  const size_t most = (size_t)t->B * std::min(r.per_env, 512 / dmx::REC_STEPS);
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
+  const size_t room = std::min(free_b / 8, kRecMaxBytes);
+  if (table > room / 8) return;
+  const size_t n = std::min(most, (room - table) / chunk);
+  if (n < (size_t)t->B || n > (size_t)INT32_MAX / 2) return;
+  if (cudaMallocAsync(&t->recmem, table + n * chunk, st) != cudaSuccess) {
+    cudaGetLastError();               // not enough memory: the tape does without
+    t->recmem = nullptr;
+    return;
+  }
+  r.chunk = static_cast<int*>(t->recmem);
+  r.next = r.chunk + (size_t)t->B * r.per_env;
+  r.mem = reinterpret_cast<double*>(static_cast<char*>(t->recmem) + table);
+  r.nchunk = (int)n;
+  if (cudaMemsetAsync(t->recmem, 0, table, st) != cudaSuccess) return;
+  t->rec = r;
+}
+
 extern "C" void dmx_tape_free(dmx_tape* t) {
   if (!t) return;
   cudaFreeAsync(t->mem, t->stream);   // ordered after the work queued on the tape's stream
+  if (t->recmem) cudaFreeAsync(t->recmem, t->stream);
   delete t;
 }
 
 extern "C" dmx_status dmx_rollout(dmx_model* m, const dmx_rollout_args* a, void* stream) {
+  return rollout_call(m, a, stream, true);
+}
+dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, bool records) {
   if (!m || !a) return dmx_fail(DMX_ERR_INVALID, "null argument");
   const cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int nq = m->host.nq, nv = m->host.nv, nx = nq + nv, nu = m->host.nu;
@@ -569,6 +607,13 @@ extern "C" dmx_status dmx_rollout(dmx_model* m, const dmx_rollout_args* a, void*
     if (s != DMX_OK) return s;
     tape->G = G;
     P.ckpt = tape->ckpt; P.hlog = tape->hlog; P.tape_n = tape->n;
+    bool reverse;
+    {
+      std::lock_guard<std::mutex> lk(m->mu);
+      reverse = m->adj_mode == DMX_ADJ_REVERSE;
+    }
+    if (records && reverse && a->B > 0) add_records(m, tape, st);
+    P.rec = tape->rec;
   }
   dmx_status s = run_rollout(m, P, a->form, G, st);
   if (s != DMX_OK) { dmx_tape_free(tape); return s; }
@@ -714,6 +759,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
                                       cudaStream_t st) {
   const int cfd = P.cfd;
   const bool par = P.p_bar != nullptr;
+  if (mode == DMX_ADJ_REVERSE) P.rec = t->rec;
   int G = adjoint_lanes(m, t->B, L, true);
   if (par && G < 8) G = 8;             // compiled lane counts
   P.LB = dmx::make_bar_layout(m->host, L.rcap, par);
@@ -749,9 +795,9 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   if (par)                             // its workspace is larger than the lane choice assumed
     while (G < 32 && !plan(L, false, pl)) G <<= 1;
   const int gpb = 32 / G;
+  P.SN = dmx::snap_offsets(m->host, m->L).size;
   size_t snap_bytes = 0;
   if (mode == DMX_ADJ_REVERSE && !cfd && plan(dmx::make_layout_adj(m->host, L.rcap), true, pl)) {
-    P.SN = dmx::snap_offsets(m->host, pl.L).size;
     snap_bytes = sizeof(double) * (size_t)pl.blocks * gpb * t->K * nsnap * (size_t)P.SN;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || snap_bytes > free_b / 8 || snap_bytes > kSnapMaxBytes)

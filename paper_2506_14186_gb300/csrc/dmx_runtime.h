@@ -42,6 +42,8 @@ struct dmx_tape {
   double* ctrl = nullptr;   // [NI][nu][B]
   double* T = nullptr;      // [B]
   int* n = nullptr;         // [B] accepted steps
+  void* recmem = nullptr;   // step records (dmx_record.h), their table and counter, or null
+  dmx::StepRecords rec{};
   cudaStream_t stream = nullptr;   // allocation stream (stream-ordered free)
 };
 
@@ -64,6 +66,9 @@ int reduction_lanes(const dmx_model* m, int B);
 // The recorded lane count of (model, B, grad), else default_lanes; *red (if
 // not null) receives the matching summation order.
 int tuned_lanes(dmx_model* m, int B, int grad, int* red);
+// dmx_rollout; records = false keeps a tape to the checkpoints (a server's
+// requests, whose memory is budgeted).
+dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, bool records);
 dmx_status run_rollout(dmx_model* m, const dmx::RolloutParams& P, int form, int G, cudaStream_t st);
 int model_smem_bytes(const dmx_model* m, int groups);
 // Upper bound of the device scratch that dmx_rollout_grad allocates for B

@@ -193,7 +193,7 @@ static void issue(dmx_server* s, ServerRequest* q, cudaStream_t st) {
   a.host = 0; a.xT = xT; a.xb = nullptr; a.nsteps = nsteps; a.nrej = nullptr; a.status = status;
   dmx_tape* tape = nullptr;
   a.tape = r.grad ? &tape : nullptr;
-  dmx_status e = dmx_rollout(r.model, &a, st);
+  dmx_status e = rollout_call(r.model, &a, st, false);
   if (e == DMX_OK && r.grad) {
     e = dmx_rollout_grad(r.model, tape, r.cfd, xTb, nullptr, x0b, z.nu ? cb : nullptr, st);
     dmx_tape_free(tape);   // stream ordered after the adjoint
