@@ -81,6 +81,7 @@ struct DevModel {
   double p_dahat[MAXP][MAXB + MAXBOX];   // d A_hat / d (mass of each body, then side of each box)
   int s_pair[MAXS], s_idx[MAXS];
   int s_rows[MAXS];                  // constraint rows of the slot (1 or 4)
+  unsigned s_rdofs[MAXS];            // dofs with an angular motion vector that move geom 1 of the slot
   unsigned s_move[MAXS];             // bodies that move geom 1 of the slot (bit mask: its body and its ancestors)
   unsigned g_slots1[MAXG], g_slots2[MAXG];   // bit s: the geom is geom 1 / geom 2 of slot s
   unsigned b_geoms[MAXB];            // bit g: geom g is fixed to the body

@@ -211,6 +211,12 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
   for (int i = 0; i < m.nv; ++i)
     for (int j = 0; j <= i; ++j)
       if ((m.b_anc[m.dof_body[i]] >> m.dof_body[j]) & 1u) { m.dof_anc[i] |= 1u << j; m.dof_desc[j] |= 1u << i; }
+  for (int s = 0; s < m.nslot; ++s)
+    for (int i = 0; i < m.nv; ++i) {
+      const int b = m.dof_body[i];
+      const bool translation = m.b_jtype[b] == DMX_JNT_FREE && i - m.b_vadr[b] < 3;
+      if (!translation && ((m.s_move[s] >> b) & 1u)) m.s_rdofs[s] |= 1u << i;
+    }
   for (int i = 0; i < m.nv; ++i) m.dof_act[i] = -1;
   for (int a = m.nact - 1; a >= 0; --a) {   // in actuator order along each dof's list
     m.act_next[a] = m.dof_act[m.a_vadr[a]];
@@ -516,6 +522,8 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   const size_t table = (sizeof(int) * ((size_t)t->B * r.per_env + 1) + 255) & ~size_t(255);
   const size_t most = (size_t)t->B * std::min(r.per_env, 512 / dmx::REC_STEPS);
   size_t free_b = 0, total_b = 0;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;   // a graph would own the memory for good
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
   const size_t room = std::min(free_b / 8, kRecMaxBytes);
   if (table > room / 8) return;
