@@ -24,8 +24,8 @@
 #include "dmx_device.cuh"
 
 namespace dmx {
-template <int G, bool PAR> cudaError_t launch_adjoint_rev_g(const AdjParams&, int, int, size_t, cudaStream_t);
-template <int G, bool PAR> int occupancy_adjoint_rev_g(int, size_t);
+template <int G, bool PAR, class MD> cudaError_t launch_adjoint_rev_g(const AdjParams&, int, int, size_t, cudaStream_t);
+template <int G, bool PAR, class MD> int occupancy_adjoint_rev_g(int, size_t);
 template <int G>
 cudaError_t launch_eval_rhs_vjp_g(const AdjParams&, const double*, const double*, const double*, const double*, double*,
                                   double*, double*, int*, int, size_t, cudaStream_t);
@@ -294,24 +294,37 @@ int adjoint_warps_per_block() { return ADJ_WARPS; }
 int adjoint_workspace_limit() { return ADJ_WS; }
 int adjoint_int_limit() { return ADJ_WI; }
 
-cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
+template <int G>
+static cudaError_t launch_adjoint_rev_m(const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
   const bool par = P.p_bar != nullptr;
+  if (P.one_body)
+    return par ? launch_adjoint_rev_g<G, true, OneBody>(P, blocks, threads, smem, st)
+               : launch_adjoint_rev_g<G, false, OneBody>(P, blocks, threads, smem, st);
+  return par ? launch_adjoint_rev_g<G, true, DevModel>(P, blocks, threads, smem, st)
+             : launch_adjoint_rev_g<G, false, DevModel>(P, blocks, threads, smem, st);
+}
+cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
   switch (G) {
-    case 2: return par ? cudaErrorInvalidValue : launch_adjoint_rev_g<2, false>(P, blocks, threads, smem, st);
-    case 4: return par ? cudaErrorInvalidValue : launch_adjoint_rev_g<4, false>(P, blocks, threads, smem, st);
-    case 8: return par ? launch_adjoint_rev_g<8, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<8, false>(P, blocks, threads, smem, st);
-    case 16: return par ? launch_adjoint_rev_g<16, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<16, false>(P, blocks, threads, smem, st);
-    case 32: return par ? launch_adjoint_rev_g<32, true>(P, blocks, threads, smem, st) : launch_adjoint_rev_g<32, false>(P, blocks, threads, smem, st);
+    case 2: return P.p_bar ? cudaErrorInvalidValue : launch_adjoint_rev_g<2, false, DevModel>(P, blocks, threads, smem, st);
+    case 4: return P.p_bar ? cudaErrorInvalidValue : launch_adjoint_rev_g<4, false, DevModel>(P, blocks, threads, smem, st);
+    case 8: return launch_adjoint_rev_m<8>(P, blocks, threads, smem, st);
+    case 16: return launch_adjoint_rev_m<16>(P, blocks, threads, smem, st);
+    case 32: return launch_adjoint_rev_m<32>(P, blocks, threads, smem, st);
   }
   return cudaErrorInvalidValue;
 }
-int adjoint_rev_occupancy(int G, bool par, int threads, size_t smem) {
+template <int G>
+static int occupancy_adjoint_rev_m(bool par, bool one_body, int threads, size_t smem) {
+  if (one_body) return par ? occupancy_adjoint_rev_g<G, true, OneBody>(threads, smem) : occupancy_adjoint_rev_g<G, false, OneBody>(threads, smem);
+  return par ? occupancy_adjoint_rev_g<G, true, DevModel>(threads, smem) : occupancy_adjoint_rev_g<G, false, DevModel>(threads, smem);
+}
+int adjoint_rev_occupancy(int G, bool par, bool one_body, int threads, size_t smem) {
   switch (G) {
-    case 2: return occupancy_adjoint_rev_g<2, false>(threads, smem);
-    case 4: return occupancy_adjoint_rev_g<4, false>(threads, smem);
-    case 8: return par ? occupancy_adjoint_rev_g<8, true>(threads, smem) : occupancy_adjoint_rev_g<8, false>(threads, smem);
-    case 16: return par ? occupancy_adjoint_rev_g<16, true>(threads, smem) : occupancy_adjoint_rev_g<16, false>(threads, smem);
-    case 32: return par ? occupancy_adjoint_rev_g<32, true>(threads, smem) : occupancy_adjoint_rev_g<32, false>(threads, smem);
+    case 2: return occupancy_adjoint_rev_g<2, false, DevModel>(threads, smem);
+    case 4: return occupancy_adjoint_rev_g<4, false, DevModel>(threads, smem);
+    case 8: return occupancy_adjoint_rev_m<8>(par, one_body, threads, smem);
+    case 16: return occupancy_adjoint_rev_m<16>(par, one_body, threads, smem);
+    case 32: return occupancy_adjoint_rev_m<32>(par, one_body, threads, smem);
   }
   return 0;
 }

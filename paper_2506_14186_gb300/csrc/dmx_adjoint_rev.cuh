@@ -46,8 +46,8 @@ __device__ __forceinline__ int rev_interval(double T, int NI, double t) {
 // Snapshot src -> workspace (the state rhs() leaves for rhs_vjp, except the
 // contact records and Jacobian rows, which the VJP reads from the snapshot
 // itself: see snap_view); returns the status.
-template <int G>
-__device__ int snap_restore(const Grp<G>& g, const DevModel& m, const Ws& w, const double* src) {
+template <int G, class MD>
+__device__ int snap_restore(const Grp<G>& g, const MD& m, const Ws& w, const double* src) {
   const Layout& L = *w.L;
   const SnapOff o = snap_offsets(m, L);
   const int* si = reinterpret_cast<const int*>(src + o.oi);
@@ -77,8 +77,8 @@ __device__ __forceinline__ Ws snap_view(const DevModel& m, const Ws& w, const do
 // b.vst.  Qb and Vb are consumed (left zero).  snaps: the step's S - 1 stage
 // snapshots (SN doubles each), or null to evaluate each stage's right-hand
 // side.  Returns the worst right-hand-side status.
-template <int G, bool PAR>
-__device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const WsB& b, const double* u,
+template <int G, bool PAR, class MD>
+__device__ int rk_step_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b, const double* u,
                            double h, int mt, bool cfd, const double* snaps, int SN) {
   const Layout& L = *w.L;
   const LayoutBar& LB = *b.L;
@@ -143,12 +143,12 @@ __device__ int rk_step_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, cons
 }
 
 // PAR: with the model-parameter gradients (p_bar).
-template <int G, bool PAR>
+template <int G, bool PAR, class MD>
 __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ AdjParams P) {
   extern __shared__ double smem[];
   const Layout& sL = P.L;
   const LayoutBar& sB = P.LB;
-  const DevModel& m = *P.model;
+  const MD& m = *static_cast<const MD*>(P.model);
   Grp<G> g;
   const int ngb = blockDim.x / G, gib = threadIdx.x / G;
   // doubles per environment and the cotangent workspace's offset in them (with
@@ -327,17 +327,17 @@ cudaError_t launch_eval_rhs_vjp_g(const AdjParams& P, const double* q, const dou
   return cudaGetLastError();
 }
 
-template <int G, bool PAR>
+template <int G, bool PAR, class MD>
 cudaError_t launch_adjoint_rev_g(const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
-  auto k = k_adjoint_rev<G, PAR>;
+  auto k = k_adjoint_rev<G, PAR, MD>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k<<<blocks, threads, smem, st>>>(P);
   return cudaGetLastError();
 }
-template <int G, bool PAR>
+template <int G, bool PAR, class MD>
 int occupancy_adjoint_rev_g(int threads, size_t smem) {
-  auto k = k_adjoint_rev<G, PAR>;
+  auto k = k_adjoint_rev<G, PAR, MD>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;

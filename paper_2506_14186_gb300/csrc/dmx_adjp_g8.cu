@@ -3,6 +3,6 @@
 #include "dmx_adjoint_rev.cuh"
 
 namespace dmx {
-template cudaError_t launch_adjoint_rev_g<8, true>(const AdjParams&, int, int, size_t, cudaStream_t);
-template int occupancy_adjoint_rev_g<8, true>(int, size_t);
+template cudaError_t launch_adjoint_rev_g<8, true, DevModel>(const AdjParams&, int, int, size_t, cudaStream_t);
+template int occupancy_adjoint_rev_g<8, true, DevModel>(int, size_t);
 }  // namespace dmx

@@ -351,8 +351,8 @@ __device__ __forceinline__ T hinge_entry(const double* a, const T& sn, const T& 
 // (parents first), tree_up each body's children into it (children first, in
 // order).  A chain is one loop of dependent additions in a register; the
 // lanes meet once per chain level instead of once per body level.
-template <int NC, int G, class T>
-__device__ __forceinline__ void tree_down(const Grp<G>& g, const DevModel& m, T* X) {
+template <int NC, int G, class T, class MD>
+__device__ __forceinline__ void tree_down(const Grp<G>& g, const MD& m, T* X) {
   if (m.nlevel == 1) return;
   for (int cl = 0; cl < m.nchlev; ++cl) {
     const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
@@ -371,8 +371,8 @@ __device__ __forceinline__ void tree_down(const Grp<G>& g, const DevModel& m, T*
     g.sync();
   }
 }
-template <int NC, int G, class T>
-__device__ __forceinline__ void tree_up(const Grp<G>& g, const DevModel& m, T* X) {
+template <int NC, int G, class T, class MD>
+__device__ __forceinline__ void tree_up(const Grp<G>& g, const MD& m, T* X) {
   if (m.nlevel == 1) return;
   for (int cl = m.nchlev - 1; cl >= 0; --cl) {
     const int c0 = m.chlev_start[cl], n = NC * (m.chlev_start[cl + 1] - c0);
@@ -401,8 +401,8 @@ __device__ __forceinline__ void tree_up(const Grp<G>& g, const DevModel& m, T* X
 // quaternion normalisation), then every entry of every local transform, then
 // the composition along the tree level by level (one entry per task), then
 // COMs, geom poses and dof motion vectors, then spatial inertias.
-template <int G, class T>
-__device__ void kinematics(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* q) {
+template <int G, class T, class MD>
+__device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const T* q) {
   const Layout& L = *w.L;
   T* R = w.at(L.R); T* P = w.at(L.p); T* C = w.at(L.com);
   T* S = w.at(L.sd); T* Ib = w.at(L.Ib); T* Ic = w.at(L.Ic);
@@ -557,8 +557,8 @@ __device__ __forceinline__ Comp6 comp6(int t, int n) {
 }
 
 // Composite-rigid-body algorithm: M (dense, both triangles).
-template <int G, class T>
-__device__ void crba(const Grp<G>& g, const DevModel& m, const WsT<T>& w) {
+template <int G, class T, class MD>
+__device__ void crba(const Grp<G>& g, const MD& m, const WsT<T>& w) {
   const Layout& L = *w.L;
   T* Ic = w.at(L.Ic);
   const T* S = w.at(L.sd); T* F = w.at(L.F); T* M = w.at(L.M);
@@ -588,8 +588,8 @@ __device__ void crba(const Grp<G>& g, const DevModel& m, const WsT<T>& w) {
 // from the root: each body's own joint term is computed for all bodies at
 // once, then added down the tree.  The per-body work is split by component
 // (one body component per task).
-template <int G, class T>
-__device__ void rne_and_forces(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* q, const T* v,
+template <int G, class T, class MD>
+__device__ void rne_and_forces(const Grp<G>& g, const MD& m, const WsT<T>& w, const T* q, const T* v,
                                const T* u) {
   const Layout& L = *w.L;
   const T* Ib = w.at(L.Ib); const T* S = w.at(L.sd);
@@ -936,8 +936,8 @@ __device__ __forceinline__ T softplus(const T& x) { return value(x) > 0 ? x + lo
 
 // All contact slots, then the included ones (r < 0, or r < w_c for F~) and
 // their per-slot impedance terms.
-template <int G, class T>
-__device__ void collide(const Grp<G>& g, const DevModel& m, const WsT<T>& w, bool cfd) {
+template <int G, class T, class MD>
+__device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd) {
   const Layout& L = *w.L;
   const T* gR = w.at(L.gR); const T* gp = w.at(L.gp);
   T* CT = w.at(L.ct);
@@ -999,8 +999,8 @@ __device__ void collide(const Grp<G>& g, const DevModel& m, const WsT<T>& w, boo
 
 // Constraint rows of the included contacts (compacted in slot order).
 // Returns the number of rows, or -1 when they exceed the workspace.
-template <int G, class T>
-__device__ int make_rows(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* v, bool cfd) {
+template <int G, class T, class MD>
+__device__ int make_rows(const Grp<G>& g, const MD& m, const WsT<T>& w, const T* v, bool cfd) {
   const Layout& L = *w.L;
   const T* CT = w.at(L.ct); const T* S = w.at(L.sd);
   int* slotrow = w.i + L.slotrow; int* rowid = w.i + L.rowid; int* slist = w.i + L.slist;
@@ -1173,8 +1173,8 @@ __device__ void chol_solve(const Grp<G>& g, const T* H, const T* invd, T* x, int
 __device__ __forceinline__ bool mask_has(const int* mk, int id) { return (mk[id >> 5] >> (id & 31)) & 1; }
 
 // H = M + J_A^T D_A J_A, b = rhs0 + J_A^T D_A a_ref,A; factor; an = H^-1 b.
-template <int G, class T>
-__device__ bool solve_active(const Grp<G>& g, const DevModel& m, const WsT<T>& w, int nr, const int* act) {
+template <int G, class T, class MD>
+__device__ bool solve_active(const Grp<G>& g, const MD& m, const WsT<T>& w, int nr, const int* act) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   const T* M = w.at(L.M); T* H = w.at(L.H);
@@ -1227,8 +1227,8 @@ __device__ bool solve_active(const Grp<G>& g, const DevModel& m, const WsT<T>& w
 }
 
 // z = J a - a_ref for every row; returns the active set {z < 0} in newmask.
-template <int G, class T>
-__device__ void residual_set(const Grp<G>& g, const DevModel& m, const WsT<T>& w, int nr, const T* a, int* newmask) {
+template <int G, class T, class MD>
+__device__ void residual_set(const Grp<G>& g, const MD& m, const WsT<T>& w, int nr, const T* a, int* newmask) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   const T* J = w.at(L.J); const T* aref = w.at(L.aref);
@@ -1253,8 +1253,8 @@ __device__ void residual_set(const Grp<G>& g, const DevModel& m, const WsT<T>& w
 // Exact line search along d = an - a: minimiser over alpha >= 0 of the convex
 // piecewise quadratic primal cost; breakpoints compared without divisions.
 // The search only selects the next Newton iterate, so it runs on values.
-template <int G, class T>
-__device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& w, int nr) {
+template <int G, class T, class MD>
+__device__ double line_search(const Grp<G>& g, const MD& m, const WsT<T>& w, int nr) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   const T* M = w.at(L.M); const T* J = w.at(L.J); const T* Dr = w.at(L.Dr);
@@ -1343,8 +1343,8 @@ __device__ double line_search(const Grp<G>& g, const DevModel& m, const WsT<T>& 
 // from its solution.  pmask receives the final set.  In derivative scalars the
 // final solve with the final set carries the implicit-function derivative.
 // Returns 0 or an ENV_* code.
-template <int G, class T>
-__device__ int solve_constraints(const Grp<G>& g, const DevModel& m, const WsT<T>& w, int nr) {
+template <int G, class T, class MD>
+__device__ int solve_constraints(const Grp<G>& g, const MD& m, const WsT<T>& w, int nr) {
   const Layout& L = *w.L;
   const int nv = m.nv;
   int* pm = w.i + L.pmask; int* am = w.i + L.amask;
@@ -1381,8 +1381,8 @@ __device__ int solve_constraints(const Grp<G>& g, const DevModel& m, const WsT<T
 }
 
 // v' = F(q, v, u) (or F~ with cfd) into out[nv].  Returns 0 or an ENV_* code.
-template <int G, class T>
-__device__ int rhs(const Grp<G>& g, const DevModel& m, const WsT<T>& w, const T* q, const T* v,
+template <int G, class T, class MD>
+__device__ int rhs(const Grp<G>& g, const MD& m, const WsT<T>& w, const T* q, const T* v,
                                 const T* u, bool cfd, T* out) {
   const Layout& L = *w.L;
   kinematics(g, m, w, q);
@@ -1502,8 +1502,8 @@ __device__ __forceinline__ void rot_exp(const T& th2, T& cw, T& sk) {   // cos(t
 // evaluates one of the two series, the products of its component and the
 // (shared) normalisation, 25 FP64 instructions on the longest path instead of
 // 46 on one lane.
-template <int G>
-__device__ void integrate_pos_lanes(const Grp<G>& g, const DevModel& m, const double* q, const double* dq,
+template <int G, class MD>
+__device__ void integrate_pos_lanes(const Grp<G>& g, const MD& m, const double* q, const double* dq,
                                     double* out) {
   for (int t0 = 0; t0 < 4 * m.nbody; t0 += G) {
     const int t = t0 + g.lane, b = min(t >> 2, m.nbody - 1), c = t & 3;
@@ -1546,8 +1546,8 @@ __device__ void integrate_pos_lanes(const Grp<G>& g, const DevModel& m, const do
   }
   g.sync();
 }
-template <int G, class T>
-__device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, const T* dq, T* out) {
+template <int G, class T, class MD>
+__device__ void integrate_pos(const Grp<G>& g, const MD& m, const T* q, const T* dq, T* out) {
   if constexpr (G >= 4 && std::is_same<T, double>::value) {
     integrate_pos_lanes(g, m, q, dq, out);
   } else {
@@ -1573,7 +1573,8 @@ __device__ void integrate_pos(const Grp<G>& g, const DevModel& m, const T* q, co
 }
 
 // Magnitude used by the error norm for tangent component i of the positions.
-__device__ __forceinline__ double pos_mag(const DevModel& m, const double* q, int i) {
+template <class MD>
+__device__ __forceinline__ double pos_mag(const MD& m, const double* q, int i) {
   const int b = m.dof_body[i];
   if (m.b_jtype[b] == JNT_HINGE) return fabs(q[m.b_qadr[b]]);
   const int d = i - m.b_vadr[b];
@@ -1585,8 +1586,8 @@ __device__ __forceinline__ double pos_mag(const DevModel& m, const double* q, in
 // result in (qs, vs) and its derivative in ka[(S-1) nv].  hook(s, status)
 // runs after the right-hand side of stage s (the workspace then holds that
 // evaluation).  Returns the worst stage status.
-template <int G, class Hook>
-__device__ int rk_stages(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
+template <int G, class Hook, class MD>
+__device__ int rk_stages(const Grp<G>& g, const MD& m, const Ws& w, const double* u, double h, int mt,
                          Hook&& hook) {
   const Layout& L = *w.L;
   const int nv = m.nv, S = TAB(mt).S;
@@ -1646,8 +1647,8 @@ __device__ double sum_as_lanes(const Grp<G>& g, double* x, int n, int C) {
 // the RMS error norm of the embedded estimate (NaN-safe: non-finite -> +inf;
 // 0 for a fixed-step scheme; summed in the order of `red` lanes) and the
 // worst stage status.
-template <int G, class Hook>
-__device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
+template <int G, class Hook, class MD>
+__device__ double rk_attempt(const Grp<G>& g, const MD& m, const Ws& w, const double* u, double h, int mt,
                              double rtol, double atol, int red, int* st_out, Hook&& hook) {
   const Layout& L = *w.L;
   const int nv = m.nv;
@@ -1680,8 +1681,8 @@ __device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, co
   return isfinite(err) ? err : INFINITY;
 }
 
-template <int G>
-__device__ double rk_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const double* u, double h, int mt,
+template <int G, class MD>
+__device__ double rk_attempt(const Grp<G>& g, const MD& m, const Ws& w, const double* u, double h, int mt,
                              double rtol, double atol, int red, int* st_out) {
   return rk_attempt(g, m, w, u, h, mt, rtol, atol, red, st_out, [](int, int) {});
 }

@@ -5,18 +5,24 @@
 
 namespace dmx {
 
+#define DMX_DECLARE_ROLLOUT(G, MD)                                                                                \
+  extern template cudaError_t launch_persistent_g<G, MD>(const RolloutParams&, int, int, size_t, cudaStream_t); \
+  extern template int occupancy_g<G, MD>(int, size_t);
 #define DMX_DECLARE(G)                                                                                   \
-  extern template cudaError_t launch_persistent_g<G>(const RolloutParams&, int, int, size_t, cudaStream_t); \
-  extern template cudaError_t launch_step_g<G>(const RolloutParams&, const StepState&, bool, int, size_t, cudaStream_t); \
-  extern template int occupancy_g<G>(int, size_t); \
-  extern template cudaError_t launch_eval_rhs_g<G>(const RolloutParams&, const double*, const double*, const double*, \
-                                                   int, double*, int*, int, size_t, cudaStream_t);
+  DMX_DECLARE_ROLLOUT(G, DevModel)                                                                       \
+  extern template cudaError_t launch_step_g<G, DevModel>(const RolloutParams&, const StepState&, bool, int, size_t, cudaStream_t); \
+  extern template cudaError_t launch_eval_rhs_g<G, DevModel>(const RolloutParams&, const double*, const double*, \
+                                                             const double*, int, double*, int*, int, size_t, cudaStream_t);
 DMX_DECLARE(1)
 DMX_DECLARE(2)
 DMX_DECLARE(4)
 DMX_DECLARE(8)
 DMX_DECLARE(16)
 DMX_DECLARE(32)
+DMX_DECLARE_ROLLOUT(4, OneBody)
+DMX_DECLARE_ROLLOUT(8, OneBody)
+DMX_DECLARE_ROLLOUT(16, OneBody)
+DMX_DECLARE_ROLLOUT(32, OneBody)
 
 // Model set-up: translational inverse weight of every body at qpos0,
 // trace(Jc M^-1 Jc^T) / 3 (one environment, one lane).
@@ -60,48 +66,60 @@ __global__ void k_body_invweight(const DevModel* mp, const double* qpos0, double
 }
 
 cudaError_t launch_persistent(int G, const RolloutParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
+  if (P.one_body) switch (G) {
+    case 4: return launch_persistent_g<4, OneBody>(P, blocks, threads, smem, st);
+    case 8: return launch_persistent_g<8, OneBody>(P, blocks, threads, smem, st);
+    case 16: return launch_persistent_g<16, OneBody>(P, blocks, threads, smem, st);
+    case 32: return launch_persistent_g<32, OneBody>(P, blocks, threads, smem, st);
+  }
   switch (G) {
-    case 1: return launch_persistent_g<1>(P, blocks, threads, smem, st);
-    case 2: return launch_persistent_g<2>(P, blocks, threads, smem, st);
-    case 4: return launch_persistent_g<4>(P, blocks, threads, smem, st);
-    case 8: return launch_persistent_g<8>(P, blocks, threads, smem, st);
-    case 16: return launch_persistent_g<16>(P, blocks, threads, smem, st);
-    case 32: return launch_persistent_g<32>(P, blocks, threads, smem, st);
+    case 1: return launch_persistent_g<1, DevModel>(P, blocks, threads, smem, st);
+    case 2: return launch_persistent_g<2, DevModel>(P, blocks, threads, smem, st);
+    case 4: return launch_persistent_g<4, DevModel>(P, blocks, threads, smem, st);
+    case 8: return launch_persistent_g<8, DevModel>(P, blocks, threads, smem, st);
+    case 16: return launch_persistent_g<16, DevModel>(P, blocks, threads, smem, st);
+    case 32: return launch_persistent_g<32, DevModel>(P, blocks, threads, smem, st);
   }
   return cudaErrorInvalidValue;
 }
 cudaError_t launch_eval_rhs(int G, const RolloutParams& P, const double* q, const double* v, const double* u, int cfd,
                             double* a, int* info, int threads, size_t smem, cudaStream_t st) {
   switch (G) {
-    case 1: return launch_eval_rhs_g<1>(P, q, v, u, cfd, a, info, threads, smem, st);
-    case 2: return launch_eval_rhs_g<2>(P, q, v, u, cfd, a, info, threads, smem, st);
-    case 4: return launch_eval_rhs_g<4>(P, q, v, u, cfd, a, info, threads, smem, st);
-    case 8: return launch_eval_rhs_g<8>(P, q, v, u, cfd, a, info, threads, smem, st);
-    case 16: return launch_eval_rhs_g<16>(P, q, v, u, cfd, a, info, threads, smem, st);
-    case 32: return launch_eval_rhs_g<32>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 1: return launch_eval_rhs_g<1, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 2: return launch_eval_rhs_g<2, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 4: return launch_eval_rhs_g<4, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 8: return launch_eval_rhs_g<8, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 16: return launch_eval_rhs_g<16, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
+    case 32: return launch_eval_rhs_g<32, DevModel>(P, q, v, u, cfd, a, info, threads, smem, st);
   }
   return cudaErrorInvalidValue;
 }
-int persistent_occupancy(int G, int threads, size_t smem) {
+int persistent_occupancy(int G, bool one_body, int threads, size_t smem) {
+  if (one_body) switch (G) {
+    case 4: return occupancy_g<4, OneBody>(threads, smem);
+    case 8: return occupancy_g<8, OneBody>(threads, smem);
+    case 16: return occupancy_g<16, OneBody>(threads, smem);
+    case 32: return occupancy_g<32, OneBody>(threads, smem);
+  }
   switch (G) {
-    case 1: return occupancy_g<1>(threads, smem);
-    case 2: return occupancy_g<2>(threads, smem);
-    case 4: return occupancy_g<4>(threads, smem);
-    case 8: return occupancy_g<8>(threads, smem);
-    case 16: return occupancy_g<16>(threads, smem);
-    case 32: return occupancy_g<32>(threads, smem);
+    case 1: return occupancy_g<1, DevModel>(threads, smem);
+    case 2: return occupancy_g<2, DevModel>(threads, smem);
+    case 4: return occupancy_g<4, DevModel>(threads, smem);
+    case 8: return occupancy_g<8, DevModel>(threads, smem);
+    case 16: return occupancy_g<16, DevModel>(threads, smem);
+    case 32: return occupancy_g<32, DevModel>(threads, smem);
   }
   return 0;
 }
 cudaError_t launch_step(int G, const RolloutParams& P, const StepState& S, bool init, int threads, size_t smem,
                         cudaStream_t st) {
   switch (G) {
-    case 1: return launch_step_g<1>(P, S, init, threads, smem, st);
-    case 2: return launch_step_g<2>(P, S, init, threads, smem, st);
-    case 4: return launch_step_g<4>(P, S, init, threads, smem, st);
-    case 8: return launch_step_g<8>(P, S, init, threads, smem, st);
-    case 16: return launch_step_g<16>(P, S, init, threads, smem, st);
-    case 32: return launch_step_g<32>(P, S, init, threads, smem, st);
+    case 1: return launch_step_g<1, DevModel>(P, S, init, threads, smem, st);
+    case 2: return launch_step_g<2, DevModel>(P, S, init, threads, smem, st);
+    case 4: return launch_step_g<4, DevModel>(P, S, init, threads, smem, st);
+    case 8: return launch_step_g<8, DevModel>(P, S, init, threads, smem, st);
+    case 16: return launch_step_g<16, DevModel>(P, S, init, threads, smem, st);
+    case 32: return launch_step_g<32, DevModel>(P, S, init, threads, smem, st);
   }
   return cudaErrorInvalidValue;
 }

@@ -26,23 +26,23 @@ struct EnvState {
   int k, nacc, nrej, att, st, done;
 };
 
-template <int G>
-__device__ void load_ctrl(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env, int k) {
+template <int G, class MD>
+__device__ void load_ctrl(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env, int k) {
   double* u = w.at(w.L->u);
   DMX_TASKS(a, m.nu) u[a] = P.ctrl[((size_t)k * m.nu + a) * P.B + env];
   g.sync();
 }
 
-template <int G>
-__device__ void store_state(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
+template <int G, class MD>
+__device__ void store_state(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env,
                             double* dst /* [nx][B] */) {
   const double* qn = w.at(w.L->qn); const double* vn = w.at(w.L->vn);
   DMX_TASKS(i, m.nq) dst[(size_t)i * P.B + env] = qn[i];
   DMX_TASKS(i, m.nv) dst[(size_t)(m.nq + i) * P.B + env] = vn[i];
 }
 
-template <int G>
-__device__ void write_checkpoint(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
+template <int G, class MD>
+__device__ void write_checkpoint(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env,
                                  int c, double t) {
   const int nx = m.nq + m.nv;
   double* ck = P.ckpt + (size_t)c * (nx + 1) * P.B;
@@ -51,8 +51,8 @@ __device__ void write_checkpoint(const Grp<G>& g, const DevModel& m, const Ws& w
 }
 
 // Initial state, first right-hand side; returns the initial environment state.
-template <int G>
-__device__ void env_start(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
+template <int G, class MD>
+__device__ void env_start(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env,
                           EnvState& s) {
   const Layout& L = *w.L;
   double* qn = w.at(L.qn); double* vn = w.at(L.vn);
@@ -75,8 +75,8 @@ __device__ void env_start(const Grp<G>& g, const DevModel& m, const Ws& w, const
 }
 
 // One step attempt with its bookkeeping.
-template <int G>
-__device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
+template <int G, class MD>
+__device__ void env_attempt(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env,
                             EnvState& s) {
   const Layout& L = *w.L;
   if (s.t >= s.T) { s.done = 1; return; }
@@ -150,8 +150,8 @@ __device__ void env_attempt(const Grp<G>& g, const DevModel& m, const Ws& w, con
   }
 }
 
-template <int G>
-__device__ void env_finish(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P, int env,
+template <int G, class MD>
+__device__ void env_finish(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P, int env,
                            const EnvState& s) {
   store_state(g, m, w, P, env, P.xT);
   if (g.lane == 0) {
@@ -163,8 +163,8 @@ __device__ void env_finish(const Grp<G>& g, const DevModel& m, const Ws& w, cons
 }
 
 // Plain form: per-environment integrator state kept in HBM between launches.
-template <int G>
-__device__ void load_step_state(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P,
+template <int G, class MD>
+__device__ void load_step_state(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P,
                                 const StepState& S, int env, EnvState& s) {
   const Layout& L = *w.L;
   double* qn = w.at(L.qn); double* vn = w.at(L.vn); double* ka = w.at(L.ka);
@@ -178,8 +178,8 @@ __device__ void load_step_state(const Grp<G>& g, const DevModel& m, const Ws& w,
   g.sync();
   if (m.nu) load_ctrl(g, m, w, P, env, s.k < P.NI ? s.k : P.NI - 1);
 }
-template <int G>
-__device__ void save_step_state(const Grp<G>& g, const DevModel& m, const Ws& w, const RolloutParams& P,
+template <int G, class MD>
+__device__ void save_step_state(const Grp<G>& g, const MD& m, const Ws& w, const RolloutParams& P,
                                 const StepState& S, int env, const EnvState& s) {
   const Layout& L = *w.L;
   const double* qn = w.at(L.qn); const double* vn = w.at(L.vn); const double* ka = w.at(L.ka);
@@ -206,10 +206,10 @@ __device__ Ws group_workspace(const RolloutParams& P, const Layout* L) {
 }
 
 // Persistent form: loop { take next env; integrate it to T }.
-template <int G>
+template <int G, class MD>
 __global__ void __launch_bounds__(32, 1) k_rollout_persistent(const __grid_constant__ RolloutParams P) {
   const Layout& sL = P.L;
-  const DevModel& m = *P.model;
+  const MD& m = *static_cast<const MD*>(P.model);
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
   // One loop level: every pass makes one step attempt of the group's
@@ -237,10 +237,10 @@ __global__ void __launch_bounds__(32, 1) k_rollout_persistent(const __grid_const
 }
 
 // Plain form, initialisation launch: state of every environment into HBM.
-template <int G>
+template <int G, class MD>
 __global__ void __launch_bounds__(32, 1) k_step_init(const __grid_constant__ RolloutParams P, StepState S) {
   const Layout& sL = P.L;
-  const DevModel& m = *P.model;
+  const MD& m = *static_cast<const MD*>(P.model);
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
   const int env = (blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -255,10 +255,10 @@ __global__ void __launch_bounds__(32, 1) k_step_init(const __grid_constant__ Rol
 }
 
 // Plain form, one attempt of every unfinished environment.
-template <int G>
+template <int G, class MD>
 __global__ void __launch_bounds__(32, 1) k_step(const __grid_constant__ RolloutParams P, StepState S) {
   const Layout& sL = P.L;
-  const DevModel& m = *P.model;
+  const MD& m = *static_cast<const MD*>(P.model);
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
   const int env = (blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -276,11 +276,11 @@ __global__ void __launch_bounds__(32, 1) k_step(const __grid_constant__ RolloutP
 
 // Right-hand side of a batch of states (q [nq][B], v [nv][B], u [nu][B]) into
 // a [nv][B]; info [4][B]: status, rows, active rows, Newton solves.
-template <int G>
+template <int G, class MD>
 __global__ void __launch_bounds__(32, 1) k_eval_rhs(const __grid_constant__ RolloutParams P, const double* q, const double* v, const double* u,
                                                   int cfd, double* a, int* info) {
   const Layout& sL = P.L;
-  const DevModel& m = *P.model;
+  const MD& m = *static_cast<const MD*>(P.model);
   Grp<G> g;
   const Ws w = group_workspace<G>(P, &sL);
   const int env = (blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -304,10 +304,10 @@ __global__ void __launch_bounds__(32, 1) k_eval_rhs(const __grid_constant__ Roll
   }
 }
 
-template <int G>
+template <int G, class MD>
 cudaError_t launch_eval_rhs_g(const RolloutParams& P, const double* q, const double* v, const double* u, int cfd,
                               double* a, int* info, int threads, size_t smem, cudaStream_t st) {
-  auto k = k_eval_rhs<G>;
+  auto k = k_eval_rhs<G, MD>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int blocks = (int)(((size_t)P.B * G + threads - 1) / threads);
@@ -315,33 +315,33 @@ cudaError_t launch_eval_rhs_g(const RolloutParams& P, const double* q, const dou
   return cudaGetLastError();
 }
 
-template <int G>
+template <int G, class MD>
 cudaError_t launch_persistent_g(const RolloutParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
-  auto k = k_rollout_persistent<G>;
+  auto k = k_rollout_persistent<G, MD>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k<<<blocks, threads, smem, st>>>(P);
   return cudaGetLastError();
 }
-template <int G>
+template <int G, class MD>
 int occupancy_g(int threads, size_t smem) {
-  auto k = k_rollout_persistent<G>;
+  auto k = k_rollout_persistent<G, MD>;
   if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem) != cudaSuccess) return 0;
   return n;
 }
-template <int G>
+template <int G, class MD>
 cudaError_t launch_step_g(const RolloutParams& P, const StepState& S, bool init, int threads, size_t smem,
                           cudaStream_t st) {
   const int blocks = (int)(((size_t)P.B * G + threads - 1) / threads);
   if (init) {
-    auto k = k_step_init<G>;
+    auto k = k_step_init<G, MD>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k<<<blocks, threads, smem, st>>>(P, S);
   } else {
-    auto k = k_step<G>;
+    auto k = k_step<G, MD>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k<<<blocks, threads, smem, st>>>(P, S);

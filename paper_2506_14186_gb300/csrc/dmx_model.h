@@ -93,6 +93,32 @@ struct DevModel {
   double a_gear[MAXU], a_kp[MAXU], a_kd[MAXU];
 };
 
+// A model of one free body with ground-plane contacts only (ball, box, toss),
+// as the device code sees it: the same data with the tree, dof and pair tables
+// known to the compiler.  The functions over a model type then lose their
+// loops over bodies and levels, joint types, index reads and geom pairs, and
+// unroll the sums over six dofs (a right-hand side runs 13 instructions per
+// FP64 instruction otherwise).  The table members only hide the base's; they
+// hold no data, and a DevModel is read through this type by a cast.
+template <int V>
+struct ConstTab {
+  DMX_HD constexpr int operator[](int) const { return V; }
+};
+struct OneBody : DevModel {
+  static constexpr int nbody = 1, nlevel = 1, nq = 7, nv = 6, nu = 0, nact = 0;
+  ConstTab<-1> b_parent, p_g2, dof_act;
+  ConstTab<JNT_FREE> b_jtype;
+  ConstTab<0> b_qadr, b_vadr, dof_body, g_body, child_count;
+  ConstTab<6> b_nv;
+  ConstTab<1> b_anc, s_move;
+};
+inline bool is_one_body(const DevModel& m) {
+  if (m.nbody != 1 || m.b_jtype[0] != JNT_FREE || m.nact != 0) return false;
+  for (int p = 0; p < m.npair; ++p)
+    if (m.p_g2[p] >= 0) return false;
+  return true;
+}
+
 // Offsets (in doubles / ints) of one environment's shared-memory workspace.
 struct Layout {
   int qn, vn, qs, vs, kv, ka, dq;

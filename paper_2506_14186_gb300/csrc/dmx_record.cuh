@@ -22,8 +22,8 @@ __device__ __forceinline__ void copy_run(const Grp<G>& g, const double* __restri
   }
 }
 // Workspace of the right-hand side just evaluated (status st) -> snapshot dst.
-template <int G>
-__device__ void snap_save(const Grp<G>& g, const DevModel& m, const Ws& w, double* dst, int st) {
+template <int G, class MD>
+__device__ void snap_save(const Grp<G>& g, const MD& m, const Ws& w, double* dst, int st) {
   const Layout& L = *w.L;
   const SnapOff o = snap_offsets(m, L);
   const int nr = (st == ENV_ROW_OVERFLOW) ? 0 : w.i[L.slotrow + m.nslot];

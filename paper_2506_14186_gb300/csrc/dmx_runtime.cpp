@@ -246,6 +246,7 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   dmx_model* m = new dmx_model();
   std::string err = compile_model(desc, m->host);
   if (!err.empty()) { delete m; return dmx_fail(DMX_ERR_INVALID, err); }
+  m->one_body = dmx::is_one_body(m->host);
   m->rcap = std::max(1, std::min(m->host.nrowid, dmx::ROWCAP));
   m->L = make_layout(m->host, m->rcap);
   m->rcap_c = std::max(1, std::min(m->host.nrowid, dmx::MAXROWID));
@@ -409,7 +410,8 @@ dmx_status run_rollout(dmx_model* m, const RolloutParams& P0, int form, int G, c
     CK(cudaMallocAsync(reinterpret_cast<void**>(&q), sizeof(int), st));
     CK(cudaMemsetAsync(q, 0, sizeof(int), st));
     P.queue = q;
-    int per_sm = persistent_occupancy(G, threads, smem);
+    P.one_body = m->one_body;
+    int per_sm = persistent_occupancy(G, m->one_body, threads, smem);
     if (per_sm < 1) per_sm = 1;
     const long long groups = (long long)m->nsm * per_sm * (threads / G);
     long long blocks = (long long)m->nsm * per_sm;
@@ -768,6 +770,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   const int cfd = P.cfd;
   const bool par = P.p_bar != nullptr;
   if (mode == DMX_ADJ_REVERSE) P.rec = t->rec;
+  P.one_body = m->one_body;
   int G = adjoint_lanes(m, t->B, L, true);
   if (par && G < 8) G = 8;             // compiled lane counts
   P.LB = dmx::make_bar_layout(m->host, L.rcap, par);
@@ -789,7 +792,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
     out.barofs = overlay ? Lx.ovl : Lx.nd;
     out.smem = (size_t)gpb * ((size_t)out.per * 8 + (size_t)Lx.ni * 4);
     if ((int)out.smem > m->smem_max - 2048) return false;
-    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, par, threads, out.smem));
+    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, par, m->one_body, threads, out.smem));
     out.blocks = std::min((t->B + gpb - 1) / gpb, m->nsm * occ);
     out.seg = sizeof(double) * (size_t)out.blocks * gpb * t->K * RW;
     return true;

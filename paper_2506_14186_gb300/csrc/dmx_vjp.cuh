@@ -419,7 +419,8 @@ static __device__ void capsule_box_vjp(const DevModel& m, const double* gR, cons
 // i moves the first geom's body, -1 the second's.  Returns false when the dof
 // moves neither or both (no Jacobian entry).  With ya_i = an_i + bcoef v_i:
 //   Jbar_r,i = -(D_r z_r y_i + D_r (J_r y) ya_i)   (active rows, else 0).
-__device__ __forceinline__ void slot_rows_bar(const DevModel& m, const WsB& b, int p, int r0, double yi, double yai,
+template <class MD>
+__device__ __forceinline__ void slot_rows_bar(const MD& m, const WsB& b, int p, int r0, double yi, double yai,
                                               double* jb) {
   const LayoutBar& LB = *b.L;
   const double* cz = b.at(LB.cz); const double* cj = b.at(LB.cj);
@@ -435,7 +436,8 @@ __device__ __forceinline__ void slot_rows_bar(const DevModel& m, const WsB& b, i
     jb[2] = mu * (e[2] - e[3]);
   }
 }
-__device__ __forceinline__ bool slot_jbar(const DevModel& m, const Ws& w, const WsB& b, int s, int r0, int i,
+template <class MD>
+__device__ __forceinline__ bool slot_jbar(const MD& m, const Ws& w, const WsB& b, int s, int r0, int i,
                                           double yi, double yai, double* jb, double* pv, double* sg) {
   const Layout& L = *w.L;
   const LayoutBar& LB = *b.L;
@@ -469,8 +471,8 @@ __device__ __forceinline__ bool slot_jbar(const DevModel& m, const Ws& w, const 
 // qbar, vbar, ubar += (dF/d(q, v, u))^T abar at the inputs of the rhs() call
 // that immediately precedes this one (same q, v, u, cfd; st = its status).
 // PAR: pacc[k] += the cotangent of model parameter k (owned by lane k mod G).
-template <int G, bool PAR = false>
-__device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const WsB& b, const double* q,
+template <int G, bool PAR = false, class MD>
+__device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b, const double* q,
                         const double* v, const double* u, bool cfd, int st, const double* abar, double* qbar,
                         double* vbar, double* ubar, double* pacc = nullptr) {
   const Layout& L = *w.L;
@@ -1044,8 +1046,8 @@ __device__ void rhs_vjp(const Grp<G>& g, const DevModel& m, const Ws& w, const W
 
 // ------------------------------------------------------------------ integrator VJPs
 // out = q (+) dq (integrate_pos): qbar += and dqbar = from outbar.
-template <int G>
-__device__ void integrate_pos_vjp(const Grp<G>& g, const DevModel& m, const double* q, const double* dq,
+template <int G, class MD>
+__device__ void integrate_pos_vjp(const Grp<G>& g, const MD& m, const double* q, const double* dq,
                                   const double* ob, double* qbar, double* dqbar) {
   DMX_TASKS(b, m.nbody) {
     const int qa = m.b_qadr[b], va = m.b_vadr[b];
