@@ -297,9 +297,11 @@ int adjoint_int_limit() { return ADJ_WI; }
 template <int G>
 static cudaError_t launch_adjoint_rev_m(const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
   const bool par = P.p_bar != nullptr;
-  if (P.one_body)
+  if (P.kind == MODEL_ONE_BODY)
     return par ? launch_adjoint_rev_g<G, true, OneBody>(P, blocks, threads, smem, st)
                : launch_adjoint_rev_g<G, false, OneBody>(P, blocks, threads, smem, st);
+  if constexpr (G >= 16)
+    if (P.kind == MODEL_PLANE_ONLY && !par) return launch_adjoint_rev_g<G, false, PlaneOnly>(P, blocks, threads, smem, st);
   return par ? launch_adjoint_rev_g<G, true, DevModel>(P, blocks, threads, smem, st)
              : launch_adjoint_rev_g<G, false, DevModel>(P, blocks, threads, smem, st);
 }
@@ -314,17 +316,19 @@ cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int thread
   return cudaErrorInvalidValue;
 }
 template <int G>
-static int occupancy_adjoint_rev_m(bool par, bool one_body, int threads, size_t smem) {
-  if (one_body) return par ? occupancy_adjoint_rev_g<G, true, OneBody>(threads, smem) : occupancy_adjoint_rev_g<G, false, OneBody>(threads, smem);
+static int occupancy_adjoint_rev_m(bool par, int kind, int threads, size_t smem) {
+  if (kind == MODEL_ONE_BODY) return par ? occupancy_adjoint_rev_g<G, true, OneBody>(threads, smem) : occupancy_adjoint_rev_g<G, false, OneBody>(threads, smem);
+  if constexpr (G >= 16)
+    if (kind == MODEL_PLANE_ONLY && !par) return occupancy_adjoint_rev_g<G, false, PlaneOnly>(threads, smem);
   return par ? occupancy_adjoint_rev_g<G, true, DevModel>(threads, smem) : occupancy_adjoint_rev_g<G, false, DevModel>(threads, smem);
 }
-int adjoint_rev_occupancy(int G, bool par, bool one_body, int threads, size_t smem) {
+int adjoint_rev_occupancy(int G, bool par, int kind, int threads, size_t smem) {
   switch (G) {
     case 2: return occupancy_adjoint_rev_g<2, false, DevModel>(threads, smem);
     case 4: return occupancy_adjoint_rev_g<4, false, DevModel>(threads, smem);
-    case 8: return occupancy_adjoint_rev_m<8>(par, one_body, threads, smem);
-    case 16: return occupancy_adjoint_rev_m<16>(par, one_body, threads, smem);
-    case 32: return occupancy_adjoint_rev_m<32>(par, one_body, threads, smem);
+    case 8: return occupancy_adjoint_rev_m<8>(par, kind, threads, smem);
+    case 16: return occupancy_adjoint_rev_m<16>(par, kind, threads, smem);
+    case 32: return occupancy_adjoint_rev_m<32>(par, kind, threads, smem);
   }
   return 0;
 }

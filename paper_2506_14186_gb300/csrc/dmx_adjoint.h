@@ -26,7 +26,7 @@ struct AdjParams {
   double* snapbuf;        // reverse mode: per group, K steps x (S - 1) stage snapshots of SN doubles (or null)
   int SN;                 // doubles per snapshot
   StepRecords rec;        // records of the taped rollout
-  int one_body;           // the model is a OneBody (8, 16, 32 lanes)
+  int kind;               // MODEL_* type of the kernels (OneBody: 8, 16, 32 lanes, PlaneOnly: 16, 32)
   int per, barofs;        // reverse mode: doubles per environment, offset of the cotangent workspace
   double* p_bar;          // [np][B] model-parameter gradients, or null
   int np;                 // model parameters differentiated when p_bar is set
@@ -44,7 +44,7 @@ cudaError_t launch_body_invweight_tangent(const DevModel* m, const double* qpos0
 // reverse-mode kernel, G lanes per environment (G = 2, 4, 8, 16, 32; with model
 // parameters, P.p_bar set / par: 8, 16, 32)
 cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st);
-int adjoint_rev_occupancy(int G, bool par, bool one_body, int threads, size_t smem);
+int adjoint_rev_occupancy(int G, bool par, int kind, int threads, size_t smem);
 cudaError_t launch_eval_rhs_vjp(int G, const AdjParams& P, const double* q, const double* v, const double* u,
                                 const double* abar, double* qbar, double* vbar, double* ubar, int* status, int threads,
                                 size_t smem, cudaStream_t st);

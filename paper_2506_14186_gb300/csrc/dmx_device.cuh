@@ -409,8 +409,9 @@ __device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const 
   T* X = w.at(L.xl); T* SC = w.at(L.sc);
   const int nb = m.nbody;
   DMX_TASKS(b, nb) {
-    const T* x = q + m.b_qadr[b];
-    if (m.b_jtype[b] == JNT_FREE) {
+    const BodyInfo bi = body_info(m, b);
+    const T* x = q + bi.qadr;
+    if (bi.jtype == JNT_FREE) {
       SC[2 * b] = 2.0 / (x[3] * x[3] + x[4] * x[4] + x[5] * x[5] + x[6] * x[6]);
     } else {
       T sn, cs;
@@ -423,17 +424,18 @@ __device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const 
   // Bodies at the root are written straight into the world arrays.
   DMX_TASKS(t, 12 * nb) {
     const int b = t / 12, e = t - 12 * b;
-    const bool root = m.b_parent[b] < 0;
+    const BodyInfo bi = body_info(m, b);
+    const bool root = bi.parent < 0;
     T v;
-    if (m.b_jtype[b] == JNT_FREE) {
-      const T* x = q + m.b_qadr[b];
+    if (bi.jtype == JNT_FREE) {
+      const T* x = q + bi.qadr;
       v = e < 9 ? quat_entry(x + 3, SC[2 * b], e) : x[e - 9];
     } else if (e >= 9) {
       v = m.b_pos[b][e - 9];
     } else {
       const int i = e / 3, j = e - 3 * (e / 3);
       const T sn = SC[2 * b], cs = SC[2 * b + 1];
-      if (m.b_ident[b]) {
+      if (bi.ident) {
         v = hinge_entry(m.b_axis[b], sn, cs, i, j);
       } else {
         const double* Ro = m.b_Roff[b];
@@ -493,11 +495,12 @@ __device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const 
   }
   // dof motion vectors (w; v at the world origin), one dof per task
   DMX_TASKS(i, m.nv) {
-    const int b = m.dof_body[i];
+    const DofInfo di = dof_info(m, i);
+    const int b = di.body;
     const T* Rb = R + 9 * b; const T* pb = P + 3 * b;
     T* st = S + 6 * i;
-    if (m.b_jtype[b] == JNT_FREE) {
-      const int d = i - m.b_vadr[b];
+    if (di.free) {
+      const int d = di.k;
       if (d < 3) {
         st[0] = 0.0; st[1] = 0.0; st[2] = 0.0; st[3] = d == 0 ? 1.0 : 0.0; st[4] = d == 1 ? 1.0 : 0.0;
         st[5] = d == 2 ? 1.0 : 0.0;
@@ -598,7 +601,8 @@ __device__ void rne_and_forces(const Grp<G>& g, const MD& m, const WsT<T>& w, co
   // own joint velocity S v
   DMX_TASKS(t, nt) {
     const int b = t / 6, e = t - 6 * b;
-    const int va = m.b_vadr[b], nd = m.b_nv[b];
+    const BodyInfo bi = body_info(m, b);
+    const int va = bi.vadr, nd = bi.nv;
     T x = 0.0;
     int d = 0;
     if (nd == 6) { d = 3; if (e >= 3) x = v[va + e - 3]; }   // unit translation vectors
@@ -611,9 +615,10 @@ __device__ void rne_and_forces(const Grp<G>& g, const MD& m, const WsT<T>& w, co
   DMX_TASKS(t, nt) {
     const Comp6 c = comp6(t, nb);
     const int b = c.i, e = c.e;
-    const int va = m.b_vadr[b], nd = m.b_nv[b];
-    T x = (m.b_parent[b] < 0 && e >= 3) ? T(-m.grav[e - 3]) : T(0.0);
-    const int d0 = (m.b_jtype[b] == JNT_FREE) ? 3 : 0;   // world-fixed translation axes
+    const BodyInfo bi = body_info(m, b);
+    const int va = bi.vadr, nd = bi.nv;
+    T x = (bi.parent < 0 && e >= 3) ? T(-m.grav[e - 3]) : T(0.0);
+    const int d0 = (bi.jtype == JNT_FREE) ? 3 : 0;   // world-fixed translation axes
     for (int d = d0; d < nd; ++d) x += crm_comp(V + 6 * b, S + 6 * (va + d), e) * v[va + d];
     A[6 * b + e] = x;
   }
@@ -944,10 +949,11 @@ __device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd)
   const double thr = cfd ? m.cfd[2] : 0.0;
   DMX_TASKS(s, m.nslot) {
     T* ct = CT + 16 * s;
-    const int p = m.s_pair[s], j = m.s_idx[s], g1 = m.p_g1[p];
-    if (m.p_g2[p] >= 0) {
-      if (m.g_type[m.p_g2[p]] == GEOM_BOX) capsule_box(m, gR, gp, g1, m.p_g2[p], thr, ct, w.at(L.csv) + 2 * s, w.pdir);
-      else seg_seg(m, gR, gp, g1, m.p_g2[p], thr, ct, w.at(L.csv) + 2 * s);
+    const SlotInfo si = slot_info(m, s);
+    const int j = si.idx, g1 = si.g1;
+    if (si.g2 >= 0) {
+      if (m.g_type[si.g2] == GEOM_BOX) capsule_box(m, gR, gp, g1, si.g2, thr, ct, w.at(L.csv) + 2 * s, w.pdir);
+      else seg_seg(m, gR, gp, g1, si.g2, thr, ct, w.at(L.csv) + 2 * s);
     } else {
       const T* Rg = gR + 9 * g1; const T* cg = gp + 3 * g1;
       T pt[3];
@@ -986,8 +992,8 @@ __device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd)
       T d;
       if constexpr (std::is_same<T, double>::value) d = (!cfd && m.solimp[4] == 2.0) ? impedance_quadratic(m, r) : impedance(m, r, cfd);
       else d = impedance(m, r, cfd, w.pdir);
-      const int pr = m.s_pair[s];
-      const auto ahat = m.p_condim[pr] == 1 ? Par<T>::ahat(m, w.pdir, pr) : Par<T>::ahat_edge(m, w.pdir, pr);
+      const int pr = si.pair;
+      const auto ahat = m.s_rows[s] == 1 ? Par<T>::ahat(m, w.pdir, pr) : Par<T>::ahat_edge(m, w.pdir, pr);
       const auto kc = Par<T>::kcoef(m, w.pdir);
       ct[13] = d;
       ct[14] = cfd ? kc * d * (m.softplus * softplus(-r / m.softplus)) : -(kc * d * r);
@@ -1036,24 +1042,22 @@ __device__ int make_rows(const Grp<G>& g, const MD& m, const WsT<T>& w, const T*
     const int r0 = slotrow[s];
     const T* ct = CT + 16 * s;
     const int p = m.s_pair[s];
-    const int bA = m.g_body[m.p_g1[p]];
-    const int bB = m.p_g2[p] >= 0 ? m.g_body[m.p_g2[p]] : -1;
-    const int bi = m.dof_body[i];
-    const bool mA = (m.b_anc[bA] >> bi) & 1u;
-    const bool mB = bB >= 0 && ((m.b_anc[bB] >> bi) & 1u);
+    const unsigned mv2 = slot_move2(m, s);
+    const int bi = dof_info(m, i).body;
+    const bool mA = (m.s_move[s] >> bi) & 1u, mB = (mv2 >> bi) & 1u;
     T jn = 0.0, j1 = 0.0, j2 = 0.0;
     if (mA != mB) {
       const T* sv = S + 6 * i;
       T pv[3];
       cross3(sv, ct + 1, pv);
       pv[0] += sv[3]; pv[1] += sv[4]; pv[2] += sv[5];
-      if (bB < 0) {   // ground plane: the frame is the world's (z, x, y)
+      if (mv2 == 0u) {   // ground plane: the frame is the world's (z, x, y)
         jn = pv[2]; j1 = pv[0]; j2 = pv[1];
       } else {
         jn = flip(dot3(ct + 4, pv), mB); j1 = flip(dot3(ct + 7, pv), mB); j2 = flip(dot3(ct + 10, pv), mB);
       }
     }
-    if (m.p_condim[p] == 1) {
+    if (m.s_rows[s] == 1) {
       J[r0 * nv + i] = jn;
     } else {
       const auto mu = Par<T>::get(w.pdir, PAR_MU0 + p, m.p_mu[p]);
@@ -1069,7 +1073,7 @@ __device__ int make_rows(const Grp<G>& g, const MD& m, const WsT<T>& w, const T*
     const int s = rowslot[r];
     const int e = r - slotrow[s];
     const int p = m.s_pair[s];
-    const int nrow = m.p_condim[p] == 1 ? 1 : 4;
+    const int nrow = m.s_rows[s];
     const T* ct = CT + 16 * s;
     T jv = 0.0;
     for (int i = 0; i < nv; ++i) jv += J[r * nv + i] * v[i];
@@ -1508,13 +1512,14 @@ __device__ void integrate_pos_lanes(const Grp<G>& g, const MD& m, const double* 
   for (int t0 = 0; t0 < 4 * m.nbody; t0 += G) {
     const int t = t0 + g.lane, b = min(t >> 2, m.nbody - 1), c = t & 3;
     const bool live = t < 4 * m.nbody;
-    const int qa = m.b_qadr[b], va = m.b_vadr[b];
-    if (m.b_jtype[b] == JNT_HINGE) {
+    const BodyInfo bi = body_info(m, b);
+    const int qa = bi.qadr, va = bi.vadr;
+    if (bi.jtype == JNT_HINGE) {
       if (live && c == 0) out[qa] = q[qa] + dq[va];
     } else if (live && c < 3) {
       out[qa + c] = q[qa + c] + dq[va + c];
     }
-    const bool fr = live && m.b_jtype[b] == JNT_FREE;
+    const bool fr = live && bi.jtype == JNT_FREE;
     if (!g.ballot(fr)) continue;
     double cw = 1.0, sk = 0.5, d[3] = {0.0, 0.0, 0.0}, x[4] = {1.0, 0.0, 0.0, 0.0};
     if (fr) {

@@ -23,6 +23,8 @@ DMX_DECLARE_ROLLOUT(4, OneBody)
 DMX_DECLARE_ROLLOUT(8, OneBody)
 DMX_DECLARE_ROLLOUT(16, OneBody)
 DMX_DECLARE_ROLLOUT(32, OneBody)
+DMX_DECLARE_ROLLOUT(16, PlaneOnly)
+DMX_DECLARE_ROLLOUT(32, PlaneOnly)
 
 // Model set-up: translational inverse weight of every body at qpos0,
 // trace(Jc M^-1 Jc^T) / 3 (one environment, one lane).
@@ -66,11 +68,15 @@ __global__ void k_body_invweight(const DevModel* mp, const double* qpos0, double
 }
 
 cudaError_t launch_persistent(int G, const RolloutParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
-  if (P.one_body) switch (G) {
+  if (P.kind == MODEL_ONE_BODY) switch (G) {
     case 4: return launch_persistent_g<4, OneBody>(P, blocks, threads, smem, st);
     case 8: return launch_persistent_g<8, OneBody>(P, blocks, threads, smem, st);
     case 16: return launch_persistent_g<16, OneBody>(P, blocks, threads, smem, st);
     case 32: return launch_persistent_g<32, OneBody>(P, blocks, threads, smem, st);
+  }
+  if (P.kind == MODEL_PLANE_ONLY) switch (G) {
+    case 16: return launch_persistent_g<16, PlaneOnly>(P, blocks, threads, smem, st);
+    case 32: return launch_persistent_g<32, PlaneOnly>(P, blocks, threads, smem, st);
   }
   switch (G) {
     case 1: return launch_persistent_g<1, DevModel>(P, blocks, threads, smem, st);
@@ -94,12 +100,16 @@ cudaError_t launch_eval_rhs(int G, const RolloutParams& P, const double* q, cons
   }
   return cudaErrorInvalidValue;
 }
-int persistent_occupancy(int G, bool one_body, int threads, size_t smem) {
-  if (one_body) switch (G) {
+int persistent_occupancy(int G, int kind, int threads, size_t smem) {
+  if (kind == MODEL_ONE_BODY) switch (G) {
     case 4: return occupancy_g<4, OneBody>(threads, smem);
     case 8: return occupancy_g<8, OneBody>(threads, smem);
     case 16: return occupancy_g<16, OneBody>(threads, smem);
     case 32: return occupancy_g<32, OneBody>(threads, smem);
+  }
+  if (kind == MODEL_PLANE_ONLY) switch (G) {
+    case 16: return occupancy_g<16, PlaneOnly>(threads, smem);
+    case 32: return occupancy_g<32, PlaneOnly>(threads, smem);
   }
   switch (G) {
     case 1: return occupancy_g<1, DevModel>(threads, smem);

@@ -27,7 +27,7 @@ struct RolloutParams {
   int* tape_n;          // [B] or null (tape: accepted steps)
   int* queue;           // persistent form: next environment
   StepRecords rec;      // tape: step records for the reverse adjoint
-  int one_body;         // the model is a OneBody (persistent form)
+  int kind;             // MODEL_* type of the kernels (persistent form)
 };
 
 // Plain (one launch per attempt) form: integrator state in HBM.

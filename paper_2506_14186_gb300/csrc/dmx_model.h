@@ -65,6 +65,11 @@ struct DevModel {
   // down or up a whole run without meeting the others.
   int nchlev, chlev_start[MAXLEV + 1];                 // chain levels: ranges of chains
   int ch_start[MAXB + 1], ch_list[MAXB], ch_par[MAXB]; // bodies of each chain (head first), parent of its head (-1 = world)
+  // the same tables packed, one read each (BodyInfo, DofInfo, SlotInfo)
+  unsigned long long b_pack[MAXB];   // bytes: parent (255 = world), joint, qadr, vadr, nv, ident
+  unsigned dof_pack[MAXV];           // bytes: body, index within its joint, joint
+  unsigned s_pack[MAXS];             // bytes: pair, index within the pair, geom 1, geom 2 (255 = plane)
+  unsigned s_move2[MAXS];            // bodies that move geom 2 of the slot (0: plane)
   int lv_pack[MAXB];                 // k-th body in level order: body | parent << 8 (parent 255 = world)
   int dof_act[MAXV], act_next[MAXU]; // first actuator on a dof (-1 = none), next one on the same dof
   // geoms
@@ -112,11 +117,69 @@ struct OneBody : DevModel {
   ConstTab<6> b_nv;
   ConstTab<1> b_anc, s_move;
 };
-inline bool is_one_body(const DevModel& m) {
-  if (m.nbody != 1 || m.b_jtype[0] != JNT_FREE || m.nact != 0) return false;
+// A model without geom pairs (the quadruped): the device code loses the
+// capsule-box and segment-pair contacts.
+struct PlaneOnly : DevModel {
+  ConstTab<-1> p_g2;
+};
+enum { MODEL_GENERAL = 0, MODEL_ONE_BODY = 1, MODEL_PLANE_ONLY = 2 };   // DevModel, OneBody, PlaneOnly
+template <class MD>
+constexpr bool plane_only_v = false;
+template <>
+constexpr bool plane_only_v<OneBody> = true;
+template <>
+constexpr bool plane_only_v<PlaneOnly> = true;
+template <class MD>
+constexpr bool one_body_v = false;
+template <>
+constexpr bool one_body_v<OneBody> = true;
+struct BodyInfo {
+  int parent, jtype, qadr, vadr, nv, ident;
+};
+template <class MD>
+DMX_HD inline BodyInfo body_info(const MD& m, int b) {
+  if constexpr (one_body_v<MD>) return {-1, JNT_FREE, 0, 0, 6, 1};
+  else {
+    const unsigned long long x = m.b_pack[b];
+    const int par = (int)(x & 255u);
+    return {par == 255 ? -1 : par, (int)(x >> 8 & 255u), (int)(x >> 16 & 255u), (int)(x >> 24 & 255u),
+            (int)(x >> 32 & 255u), (int)(x >> 40 & 255u)};
+  }
+}
+struct DofInfo {
+  int body, k;                       // its body and its index within the joint
+  bool free, translation;            // of a free joint; one of its translations
+};
+template <class MD>
+DMX_HD inline DofInfo dof_info(const MD& m, int i) {
+  if constexpr (one_body_v<MD>) return {0, i, true, i < 3};
+  else {
+    const unsigned x = m.dof_pack[i];
+    const int k = (int)(x >> 8 & 255u);
+    const bool fr = (x >> 16 & 255u) == (unsigned)JNT_FREE;
+    return {(int)(x & 255u), k, fr, fr && k < 3};
+  }
+}
+struct SlotInfo {
+  int pair, idx, g1, g2;             // g2 = -1: ground plane
+};
+template <class MD>
+DMX_HD inline SlotInfo slot_info(const MD& m, int s) {
+  const unsigned x = m.s_pack[s];
+  const int g2 = (int)(x >> 24);
+  return {(int)(x & 255u), (int)(x >> 8 & 255u), (int)(x >> 16 & 255u), plane_only_v<MD> || g2 == 255 ? -1 : g2};
+}
+template <class MD>
+DMX_HD inline unsigned slot_move2(const MD& m, int s) {
+  return plane_only_v<MD> ? 0u : m.s_move2[s];
+}
+inline bool is_plane_only(const DevModel& m) {
   for (int p = 0; p < m.npair; ++p)
     if (m.p_g2[p] >= 0) return false;
   return true;
+}
+inline bool is_one_body(const DevModel& m) {
+  return m.nbody == 1 && m.b_jtype[0] == JNT_FREE && m.nact == 0 && is_plane_only(m);
 }
 
 // Offsets (in doubles / ints) of one environment's shared-memory workspace.

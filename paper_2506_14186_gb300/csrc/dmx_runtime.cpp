@@ -211,6 +211,21 @@ static std::string compile_model(const dmx_model_desc* d, DevModel& m) {
   for (int i = 0; i < m.nv; ++i)
     for (int j = 0; j <= i; ++j)
       if ((m.b_anc[m.dof_body[i]] >> m.dof_body[j]) & 1u) { m.dof_anc[i] |= 1u << j; m.dof_desc[j] |= 1u << i; }
+  for (int b = 0; b < m.nbody; ++b) {
+    const unsigned long long f[6] = {(unsigned long long)(m.b_parent[b] < 0 ? 255 : m.b_parent[b]), (unsigned long long)m.b_jtype[b],
+                                     (unsigned long long)m.b_qadr[b], (unsigned long long)m.b_vadr[b],
+                                     (unsigned long long)m.b_nv[b], (unsigned long long)m.b_ident[b]};
+    for (int k = 0; k < 6; ++k) m.b_pack[b] |= f[k] << (8 * k);
+  }
+  for (int i = 0; i < m.nv; ++i) {
+    const int b = m.dof_body[i];
+    m.dof_pack[i] = (unsigned)b | (unsigned)(i - m.b_vadr[b]) << 8 | (unsigned)m.b_jtype[b] << 16;
+  }
+  for (int s = 0; s < m.nslot; ++s) {
+    const int p = m.s_pair[s], g2 = m.p_g2[p];
+    m.s_pack[s] = (unsigned)p | (unsigned)m.s_idx[s] << 8 | (unsigned)m.p_g1[p] << 16 | (unsigned)(g2 < 0 ? 255 : g2) << 24;
+    m.s_move2[s] = g2 < 0 ? 0u : m.b_anc[m.g_body[g2]];
+  }
   for (int s = 0; s < m.nslot; ++s)
     for (int i = 0; i < m.nv; ++i) {
       const int b = m.dof_body[i];
@@ -246,7 +261,7 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   dmx_model* m = new dmx_model();
   std::string err = compile_model(desc, m->host);
   if (!err.empty()) { delete m; return dmx_fail(DMX_ERR_INVALID, err); }
-  m->one_body = dmx::is_one_body(m->host);
+  m->kind = dmx::is_one_body(m->host) ? dmx::MODEL_ONE_BODY : dmx::is_plane_only(m->host) ? dmx::MODEL_PLANE_ONLY : dmx::MODEL_GENERAL;
   m->rcap = std::max(1, std::min(m->host.nrowid, dmx::ROWCAP));
   m->L = make_layout(m->host, m->rcap);
   m->rcap_c = std::max(1, std::min(m->host.nrowid, dmx::MAXROWID));
@@ -410,8 +425,8 @@ dmx_status run_rollout(dmx_model* m, const RolloutParams& P0, int form, int G, c
     CK(cudaMallocAsync(reinterpret_cast<void**>(&q), sizeof(int), st));
     CK(cudaMemsetAsync(q, 0, sizeof(int), st));
     P.queue = q;
-    P.one_body = m->one_body;
-    int per_sm = persistent_occupancy(G, m->one_body, threads, smem);
+    P.kind = m->kind;
+    int per_sm = persistent_occupancy(G, m->kind, threads, smem);
     if (per_sm < 1) per_sm = 1;
     const long long groups = (long long)m->nsm * per_sm * (threads / G);
     long long blocks = (long long)m->nsm * per_sm;
@@ -770,7 +785,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   const int cfd = P.cfd;
   const bool par = P.p_bar != nullptr;
   if (mode == DMX_ADJ_REVERSE) P.rec = t->rec;
-  P.one_body = m->one_body;
+  P.kind = m->kind;
   int G = adjoint_lanes(m, t->B, L, true);
   if (par && G < 8) G = 8;             // compiled lane counts
   P.LB = dmx::make_bar_layout(m->host, L.rcap, par);
@@ -792,7 +807,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
     out.barofs = overlay ? Lx.ovl : Lx.nd;
     out.smem = (size_t)gpb * ((size_t)out.per * 8 + (size_t)Lx.ni * 4);
     if ((int)out.smem > m->smem_max - 2048) return false;
-    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, par, m->one_body, threads, out.smem));
+    const int occ = std::max(1, dmx::adjoint_rev_occupancy(G, par, m->kind, threads, out.smem));
     out.blocks = std::min((t->B + gpb - 1) / gpb, m->nsm * occ);
     out.seg = sizeof(double) * (size_t)out.blocks * gpb * t->K * RW;
     return true;

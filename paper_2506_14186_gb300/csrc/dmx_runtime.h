@@ -24,7 +24,7 @@ struct dmx_model {
   dmx::Layout L;                              // workspace of the forward right-hand side (rows: rcap)
   dmx::Layout Lc;                             // workspace of the CFD right-hand side F~ (rows: rcap_c)
   int device = 0, nsm = 0, smem_max = 0, rcap = 0, rcap_c = 0;
-  bool one_body = false;                      // one free body, plane contacts only: kernels of dmx::OneBody
+  int kind = 0;                               // model type of its kernels (dmx::MODEL_*)
   double invw[dmx::MAXB];
   std::mutex mu;
   std::map<std::pair<int, int>, int> tuned;   // (B, kind) -> lanes per environment
@@ -78,5 +78,5 @@ int model_smem_bytes(const dmx_model* m, int groups);
 size_t adjoint_scratch_bound(dmx_model* m, int B, int K, int cfd);
 
 namespace dmx {
-int persistent_occupancy(int G, bool one_body, int threads, size_t smem);
+int persistent_occupancy(int G, int kind, int threads, size_t smem);
 }

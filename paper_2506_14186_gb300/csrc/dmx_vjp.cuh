@@ -442,11 +442,8 @@ __device__ __forceinline__ bool slot_jbar(const MD& m, const Ws& w, const WsB& b
   const Layout& L = *w.L;
   const LayoutBar& LB = *b.L;
   const int p = m.s_pair[s];
-  const int bA = m.g_body[m.p_g1[p]];
-  const int bB = m.p_g2[p] >= 0 ? m.g_body[m.p_g2[p]] : -1;
-  const int bi = m.dof_body[i];
-  const bool mA = (m.b_anc[bA] >> bi) & 1u;
-  const bool mB = bB >= 0 && ((m.b_anc[bB] >> bi) & 1u);
+  const int bi = dof_info(m, i).body;
+  const bool mA = (m.s_move[s] >> bi) & 1u, mB = (slot_move2(m, s) >> bi) & 1u;
   if (mA == mB) return false;
   const double* ct = (w.xct ? w.xct : w.at(L.ct)) + 16 * s;
   const double* sv = w.at(L.sd) + 6 * i;
@@ -778,7 +775,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b,
   //   Vbar_v += S_w x cb_v;  Sbar_w += cb_w x V_w + cb_v x V_v,  Sbar_v += cb_v x V_w
   DMX_TASKS(i, nv) {
     const int bb = m.dof_body[i];
-    if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
+    if (dof_info(m, i).translation) continue;
     const double* vbv = V + 6 * bb; const double* sd = S + 6 * i; const double* ab6 = Abb + 6 * bb;
     double s1 = 0.0;
     for (int e = 0; e < 6; ++e) s1 += ab6[e] * crm_comp(vbv, sd, e);
@@ -787,7 +784,7 @@ __device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b,
   DMX_TASKS(t, 6 * nv) {
     const Comp6 ce = comp6(t, nv);
     const int i = ce.i, e = ce.e, bb = m.dof_body[i];
-    if (m.b_jtype[bb] == JNT_FREE && i - m.b_vadr[bb] < 3) continue;
+    if (dof_info(m, i).translation) continue;
     const double* a = V + 6 * bb; const double* ab6 = Abb + 6 * bb;
     const double vd = v[i];
     const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
@@ -803,8 +800,9 @@ __device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b,
     const int bb = ce.i, e = ce.e;
     const double* ab6 = Abb + 6 * bb;
     const int c = e < 3 ? e : e - 3, c1 = nxt3(c), c2 = prv3(c);
-    const int va = m.b_vadr[bb], nd = m.b_nv[bb];
-    const int d0 = (m.b_jtype[bb] == JNT_FREE) ? 3 : 0;
+    const BodyInfo bi = body_info(m, bb);
+    const int va = bi.vadr, nd = bi.nv;
+    const int d0 = (bi.jtype == JNT_FREE) ? 3 : 0;
     double acc = 0.0;
     for (int d = d0; d < nd; ++d) {
       const double* sd = S + 6 * (va + d);
@@ -922,8 +920,9 @@ __device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b,
     const int bb = t / 9, comp = t - 9 * bb;
     const double* Rv = R + 9 * bb; const double* pv = P + 3 * bb;
     const double* cb3 = cp + 3 * bb;
-    const int va = m.b_vadr[bb];
-    const bool fr = m.b_jtype[bb] == JNT_FREE;
+    const BodyInfo bi = body_info(m, bb);
+    const int va = bi.vadr;
+    const bool fr = bi.jtype == JNT_FREE;
     const int r = comp / 3, kk = comp - 3 * (comp / 3);
     const double* ib = Ibb + 10 * bb;
     const double Br[3] = {r == 0 ? 2.0 * ib[4] : (r == 1 ? ib[7] : ib[8]),
@@ -942,9 +941,10 @@ __device__ void rhs_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB& b,
   DMX_TASKS(t, 3 * nb) {
     const int bb = t / 3, r = t - 3 * bb, r1 = nxt3(r), r2 = prv3(r);
     const double* Rv = R + 9 * bb;
-    const int va = m.b_vadr[bb];
+    const BodyInfo bi = body_info(m, bb);
+    const int va = bi.vadr;
     double val = cp[t];
-    if (m.b_jtype[bb] == JNT_FREE) {
+    if (bi.jtype == JNT_FREE) {
       for (int d = 0; d < 3; ++d) {
         const double* sv = Sb + 6 * (va + 3 + d) + 3;
         val += Rv[3 * r1 + d] * sv[r2] - Rv[3 * r2 + d] * sv[r1];
