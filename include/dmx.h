@@ -201,8 +201,10 @@ dmx_status dmx_model_params(const dmx_model* m, int32_t* np, double* values);
  * environments (a fixed-order reduction: the batch's gradient when every
  * environment shares the model).  Computed by the kernel that dmx_set_adjoint
  * selects: the reverse-mode one collects the parameters' cotangents of every
- * right-hand side beside the states' (8, 16 or 32 lanes), the tangent one runs
- * a derivative direction per parameter.  Device pointers, ordered on `stream`. */
+ * right-hand side beside the states' (8, 16 or 32 lanes; without cfd it leaves
+ * the environments that met no contact to the tangent one), the tangent one
+ * runs a derivative direction per parameter.  A model that does not fit the
+ * tangent kernel is refused.  Device pointers, ordered on `stream`. */
 dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* tape, int32_t cfd, const double* xT_bar,
                                    const double* xb_bar, double* x0_bar, double* ctrl_bar, double* p_bar,
                                    double* p_bar_sum, void* stream);

@@ -21,7 +21,7 @@
 #include <cuda_runtime.h>
 
 #include "dmx_adjoint.h"
-#include "dmx_device.cuh"
+#include "dmx_plain.cuh"
 
 namespace dmx {
 template <int G, bool PAR, class MD> cudaError_t launch_adjoint_rev_g(const AdjParams&, int, int, size_t, cudaStream_t);
@@ -32,6 +32,7 @@ cudaError_t launch_eval_rhs_vjp_g(const AdjParams&, const double*, const double*
 }  // namespace dmx
 
 namespace dmx {
+using namespace plain;
 
 constexpr int ADJ_WARPS = 2;          // warps (environments) per block
 constexpr int ADJ_WS = 4096;          // per-lane workspace (derivative scalars)
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS) k_adjoint(AdjParams P) {
     if (lane == 0) env = atomicAdd(P.queue, 1);
     env = __shfl_sync(full, env, 0);
     if (env >= P.B) break;
+    if (P.touched && P.touched[env]) continue;     // left to the reverse-mode kernel
     const int N = P.tape_n[env];
     const double T = P.T[env];
     for (int i = lane; i < nx; i += 32) xbar[i] = P.xT_bar[(size_t)i * P.B + env];
@@ -148,7 +150,7 @@ __global__ void __launch_bounds__(32 * ADJ_WARPS) k_adjoint(AdjParams P) {
         if (n == n1 - 1) break;
         const double h = P.hlog[(size_t)n * P.B + env];
         int st;
-        rk_attempt(g, m, wp, (const double*)u, h, P.method, 1.0, 1.0, 1, &st);
+        rk_attempt(g, m, wp, (const double*)u, h, P.method, 1.0, 1.0, &st);
         const double tn = adj_boundary(T, P.NI, k + 1);
         const bool reached = (h == tn - t) || (t + h >= tn);
         t = reached ? tn : t + h;
@@ -256,7 +258,7 @@ __global__ void k_body_invweight_tangent(const DevModel* mp, const double* qpos0
   crba(g, m, w);
   Dual* H = w.at(sL.H); const Dual* M = w.at(sL.M);
   for (int i = 0; i < m.nv * m.nv; ++i) H[i] = M[i];
-  cholesky(g, H, w.at(sL.tmp2), m.nv, m.nv);
+  cholesky(g, H, w.at(sL.tmp2), m.nv);
   const Dual* S = w.at(sL.sd); const Dual* C = w.at(sL.com);
   for (int b = 0; b < m.nbody; ++b) {
     Dual tr = 0.0;

@@ -30,6 +30,8 @@ struct AdjParams {
   int per, barofs;        // reverse mode: doubles per environment, offset of the cotangent workspace
   double* p_bar;          // [np][B] model-parameter gradients, or null
   int np;                 // model parameters differentiated when p_bar is set
+  const int* touched;     // [B] or null (every environment): the reverse-mode kernel takes the environments whose
+                          // taped steps met a contact, the tangent kernel the others
   int* queue;             // next environment
 };
 

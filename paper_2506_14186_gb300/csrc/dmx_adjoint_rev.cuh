@@ -170,6 +170,8 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
     if (g.lane == 0) env = atomicAdd(P.queue, 1);
     env = g.bcast(env, 0);
     if (env >= P.B) break;
+    if constexpr (PAR)
+      if (P.touched && !P.touched[env]) continue;
     const int N = P.tape_n[env];
     const double T = P.T[env];
     DMX_TASKS(i, nx) xbar[i] = P.xT_bar[(size_t)i * P.B + env];

@@ -71,6 +71,7 @@ __device__ void env_start(const Grp<G>& g, const MD& m, const Ws& w, const Rollo
   if (m.nu) load_ctrl(g, m, w, P, env, 0);
   const int st = rhs(g, m, w, qn, vn, w.at(L.u), false, w.at(L.ka));
   if (double* r = claim_record(g, P.rec, env, 0)) snap_save(g, m, w, r, st);
+  if (P.touched && g.lane == 0) P.touched[env] = w.i[L.slotrow + m.nslot] > 0;
   if (st != ENV_OK) { s.st = st; s.done = 1; }
 }
 
@@ -93,14 +94,17 @@ __device__ void env_attempt(const Grp<G>& g, const MD& m, const Ws& w, const Rol
   double* rec = claim_record(g, P.rec, env, s.nacc);
   double* rec1 = rec ? claim_record(g, P.rec, env, s.nacc + 1) : nullptr;
   const int S = TAB(mt).S;
+  bool contact = false;                // some stage includes a contact
   const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, P.red, &stage_st, [&](int st, int r) {
     double* dst = st <= S - 2 ? (rec ? rec + (size_t)st * P.rec.snap : nullptr) : rec1;
     if (dst) snap_save(g, m, w, dst, r);
+    if (P.touched) contact = contact || w.i[L.slotrow + m.nslot] > 0;
   });
   ++s.att;
   if (err <= 1.0) {
     if (stage_st != ENV_OK) { s.st = stage_st; s.done = 1; return; }
     if (P.hlog && g.lane == 0) P.hlog[(size_t)s.nacc * P.B + env] = ht;
+    if (contact && g.lane == 0) P.touched[env] = 1;
     if (rec) {                         // the step's row: q_n, stage velocities, t_n
       double* row = rec + (size_t)(S - 1) * P.rec.snap;
       const double* q0 = w.at(L.qn); const double* kv = w.at(L.kv);

@@ -26,6 +26,7 @@ struct RolloutParams {
   double* hlog;         // [max_steps][B] or null (tape: accepted step sizes)
   int* tape_n;          // [B] or null (tape: accepted steps)
   int* queue;           // persistent form: next environment
+  int* touched;         // [B] or null (tape: 1 where an accepted step met a contact)
   StepRecords rec;      // tape: step records for the reverse adjoint
   int kind;             // MODEL_* type of the kernels (persistent form)
 };

@@ -507,7 +507,7 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
   t->rtol = a->rtol; t->atol = a->atol; t->h0 = a->h0; t->method = a->method;
   const size_t B = a->B;
   const size_t bytes = sizeof(double) * ((size_t)t->ncheck * (t->nx + 1) * B + (size_t)a->max_steps * B +
-                                         (size_t)a->NI * t->nu * B + B) + sizeof(int) * B;
+                                         (size_t)a->NI * t->nu * B + B) + sizeof(int) * 2 * B;
   if (cudaMallocAsync(&t->mem, bytes, st) != cudaSuccess) { delete t; return dmx_fail(DMX_ERR_OOM, "tape allocation of " + std::to_string(bytes) + " bytes"); }
   t->stream = st;
   t->bytes = bytes;
@@ -517,6 +517,8 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
   t->ctrl = p; p += (size_t)a->NI * t->nu * B;
   t->T = p; p += B;
   t->n = reinterpret_cast<int*>(p);
+  t->touched = t->n + B;
+  CK(cudaMemsetAsync(t->touched, 0, sizeof(int) * B, st));
   if (t->nu && ctrl) CK(cudaMemcpyAsync(t->ctrl, ctrl, sizeof(double) * a->NI * t->nu * B, cudaMemcpyDeviceToDevice, st));
   CK(cudaMemcpyAsync(t->T, T, sizeof(double) * B, cudaMemcpyDeviceToDevice, st));
   *out = t;
@@ -631,7 +633,7 @@ dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, b
     dmx_status s = make_tape(m, a, a->ctrl, a->T, st, &tape);
     if (s != DMX_OK) return s;
     tape->G = G;
-    P.ckpt = tape->ckpt; P.hlog = tape->hlog; P.tape_n = tape->n;
+    P.ckpt = tape->ckpt; P.hlog = tape->hlog; P.tape_n = tape->n; P.touched = tape->touched;
     bool reverse;
     {
       std::lock_guard<std::mutex> lk(m->mu);
@@ -871,8 +873,19 @@ extern "C" dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* t, int32_t
     std::lock_guard<std::mutex> lk(m->mu);
     mode = m->adj_mode;
   }
-  const dmx_status s = mode == DMX_ADJ_TANGENT ? run_tangent_adjoint(m, t, P, st)
-                                               : run_reverse_adjoint(m, t, P, layout_for(m, cfd), mode, st);
+  // An environment that met no contact has no parameter gradient but for
+  // rounding (mass and sides cancel in free flight), which is the tangent
+  // kernel's, as it was; its few long steps cost that kernel little.  The
+  // flags know F's contacts only, so with cfd the reverse kernel takes all.
+  const dmx::Layout& L = layout_for(m, cfd);
+  if (L.nd > dmx::adjoint_workspace_limit() || L.ni > dmx::adjoint_int_limit())
+    return dmx_fail(DMX_ERR_INVALID, "model workspace exceeds the tangent adjoint kernel's per-lane limit");
+  dmx_status s = DMX_OK;
+  if (!cfd || mode == DMX_ADJ_TANGENT) {
+    P.touched = mode == DMX_ADJ_TANGENT ? nullptr : t->touched;
+    s = run_tangent_adjoint(m, t, P, st);
+  }
+  if (s == DMX_OK && mode != DMX_ADJ_TANGENT) s = run_reverse_adjoint(m, t, P, L, mode, st);
   if (s != DMX_OK) return s;
   if (p_bar_sum) CK(dmx::launch_row_sums(p_bar, np, t->B, p_bar_sum, st));
   return DMX_OK;

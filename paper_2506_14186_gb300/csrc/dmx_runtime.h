@@ -43,6 +43,7 @@ struct dmx_tape {
   double* ctrl = nullptr;   // [NI][nu][B]
   double* T = nullptr;      // [B]
   int* n = nullptr;         // [B] accepted steps
+  int* touched = nullptr;   // [B] an accepted step met a contact
   void* recmem = nullptr;   // step records (dmx_record.h), their table and counter, or null
   dmx::StepRecords rec{};
   cudaStream_t stream = nullptr;   // allocation stream (stream-ordered free)
