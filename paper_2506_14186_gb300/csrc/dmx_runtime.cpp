@@ -695,11 +695,12 @@ static bool adj_launch_config(const dmx_model* m, const dmx::Layout& L, const dm
 
 // Lanes of the reverse-mode kernels: the recorded choice, else by fill_lanes.
 // `sweep`: the adjoint of a tape, whose groups stay resident (0: one VJP per
-// environment).  Larger models run their sweep on 32 lanes; a single body's
-// has 8 tasks in its longest phase (the vertices), so one warp per
-// sub-partition of 8-lane groups is the better use (tosses, 2048 for 0.25 s,
-// forward and adjoint: 270 ms with 16 lanes, 192 with 8).  Single VJPs keep
-// one warp per sub-partition, too (arms, 16384: 17.0 -> 10.8 ms).
+// environment).  Larger models run their sweep on 32 lanes (arms, 2048 for
+// 0.1 s: 71 ms with 32, 73 with 16, 116 with 8); a single body's has 8 tasks in
+// its longest phase (the vertices), and two warps per sub-partition fill it
+// (box pushes, 4096 for 0.03 s: 52 ms with 8 lanes, 73 with 16, 111 with 32;
+// tosses, 2048 for 0.25 s: 63, 57, 79; 300: 41, 32, 29).  Single VJPs keep about
+// one warp per sub-partition (arms, 16384: 17.0 -> 10.8 ms).
 static int adjoint_lanes(dmx_model* m, int B, const dmx::Layout& L, bool sweep) {
   const dmx::LayoutBar LB = dmx::make_bar_layout(m->host, L.rcap);
   int t; size_t s;
@@ -710,7 +711,7 @@ static int adjoint_lanes(dmx_model* m, int B, const dmx::Layout& L, bool sweep) 
       return it->second;
   }
   const size_t per = (size_t)(L.nd + LB.nd) * 8 + (size_t)L.ni * 4;
-  int G = fill_lanes(m, B, per, sweep ? (m->host.nv > 8 ? 16 : 4) : 5, 8);
+  int G = fill_lanes(m, B, per, sweep ? (m->host.nv > 8 ? 16 : 8) : 5, 8);
   while (G < 32 && !adj_launch_config(m, L, LB, G, &t, &s)) G <<= 1;
   return G;
 }
