@@ -35,9 +35,6 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
-#include <type_traits>
-
-#include "dmx_dual.cuh"
 #include "dmx_model.h"
 
 namespace dmx {
@@ -135,10 +132,6 @@ __device__ __forceinline__ double max_pos(double a, double b) {
 __device__ __forceinline__ double flip(double x, bool minus) {
   return __longlong_as_double(__double_as_longlong(x) ^ (minus ? (1ll << 63) : 0ll));
 }
-__device__ __forceinline__ Dual flip(const Dual& x, bool minus) { return minus ? -x : x; }
-// Templated on the scalar types so that the same code runs on doubles (the
-// forward path) and on derivative scalars (the adjoint); model constants
-// stay double.
 template <class A, class B, class C>
 __device__ __forceinline__ void cross3(const A* a, const B* b, C* c) {
   c[0] = a[1] * b[2] - a[2] * b[1];
@@ -147,13 +140,6 @@ __device__ __forceinline__ void cross3(const A* a, const B* b, C* c) {
 }
 template <class A, class B>
 __device__ __forceinline__ auto dot3(const A* a, const B* b) { return a[0] * b[0] + a[1] * b[1] + a[2] * b[2]; }
-template <class A, class B, class C>
-__device__ __forceinline__ void matmul3(const A* M, const B* N, C* P) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) P[3 * i + j] = M[3 * i] * N[j] + M[3 * i + 1] * N[3 + j] + M[3 * i + 2] * N[6 + j];
-}
 template <class A, class B, class C>
 __device__ __forceinline__ void matvec3(const A* M, const B* x, C* y) {
   y[0] = M[0] * x[0] + M[1] * x[1] + M[2] * x[2];
@@ -166,51 +152,6 @@ __device__ __forceinline__ void matTvec3(const A* M, const B* x, C* y) {
   y[1] = M[1] * x[0] + M[4] * x[1] + M[7] * x[2];
   y[2] = M[2] * x[0] + M[5] * x[1] + M[8] * x[2];
 }
-// rotation matrix of the normalised quaternion (w, x, y, z)
-template <class T>
-__device__ __forceinline__ void quat_to_mat(const T* q, T* R) {
-  const T n2 = q[0] * q[0] + q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
-  const T s = 2.0 / n2;   // 2 / |q|^2 folds the normalisation into the products
-  const T w = q[0], x = q[1], y = q[2], z = q[3];
-  const T xx = s * x * x, yy = s * y * y, zz = s * z * z;
-  const T xy = s * x * y, xz = s * x * z, yz = s * y * z;
-  const T wx = s * w * x, wy = s * w * y, wz = s * w * z;
-  R[0] = 1.0 - (yy + zz); R[1] = xy - wz; R[2] = xz + wy;
-  R[3] = xy + wz; R[4] = 1.0 - (xx + zz); R[5] = yz - wx;
-  R[6] = xz - wy; R[7] = yz + wx; R[8] = 1.0 - (xx + yy);
-}
-// spatial inertia (10 numbers: m, h = m c, I_O xx yy zz xy xz yz about the world
-// origin) applied to a motion vector (w; v): (I_O w + h x v; m v - h x w)
-template <class T>
-__device__ __forceinline__ void inertia_apply(const T* I, const T* x, T* y) {
-  const T m = I[0], h0 = I[1], h1 = I[2], h2 = I[3];
-  const T w0 = x[0], w1 = x[1], w2 = x[2], v0 = x[3], v1 = x[4], v2 = x[5];
-  y[0] = I[4] * w0 + I[7] * w1 + I[8] * w2 + (h1 * v2 - h2 * v1);
-  y[1] = I[7] * w0 + I[5] * w1 + I[9] * w2 + (h2 * v0 - h0 * v2);
-  y[2] = I[8] * w0 + I[9] * w1 + I[6] * w2 + (h0 * v1 - h1 * v0);
-  y[3] = m * v0 - (h1 * w2 - h2 * w1);
-  y[4] = m * v1 - (h2 * w0 - h0 * w2);
-  y[5] = m * v2 - (h0 * w1 - h1 * w0);
-}
-// motion cross product (w; v) x (w2; v2) = (w x w2; w x v2 + v x w2)
-template <class T>
-__device__ __forceinline__ void crm6(const T* a, const T* b, T* c) {
-  T t[3];
-  cross3(a, b, c);
-  cross3(a, b + 3, c + 3);
-  cross3(a + 3, b, t);
-  c[3] += t[0]; c[4] += t[1]; c[5] += t[2];
-}
-// force cross product (w; v) x* (n; f) = (w x n + v x f; w x f)
-template <class T>
-__device__ __forceinline__ void crf6(const T* a, const T* b, T* c) {
-  T t[3];
-  cross3(a, b, c);
-  cross3(a + 3, b + 3, t);
-  c[0] += t[0]; c[1] += t[1]; c[2] += t[2];
-  cross3(a, b + 3, c + 3);
-}
-
 // Single components (e = 0..5) of the spatial products above, so that the
 // six components of a body's vector can go to six lanes.
 __device__ __forceinline__ int nxt3(int k) { return k == 2 ? 0 : k + 1; }
@@ -250,71 +191,9 @@ struct WsT {
   // when set (a stage snapshot in device memory), else from the workspace
   const double* xct = nullptr;
   const double* xJ = nullptr;
-  // derivative scalars: the model parameter (PAR_*) whose tangent this
-  // evaluation carries, -1 for none
-  int pdir = -1;
   __device__ T* at(int off) const { return d + off; }
 };
 
-// Value v of model parameter k; a derivative scalar carries a unit tangent
-// when k is the direction pdir being differentiated.
-// Parameter order: PAR_TC .. PAR_MID, mu of every pair, then the mass of
-// every body (rotational inertia scaled in proportion).
-__device__ __forceinline__ int par_mass(const DevModel& m, int b) { return PAR_MU0 + m.npair + b; }
-// then the side length of every box geom (its edge along the geom's x axis;
-// the half sizes scale together; the inertia of a body whose only geom is the
-// box scales with the square)
-__device__ __forceinline__ int par_side(const DevModel& m, int j) { return PAR_MU0 + m.npair + m.nbody + j; }
-template <class T>
-struct Par {
-  static __device__ __forceinline__ double get(int, int, double v) { return v; }
-  static __device__ __forceinline__ double bcoef(const DevModel& m, int) { return m.bcoef; }
-  static __device__ __forceinline__ double kcoef(const DevModel& m, int) { return m.kcoef; }
-  static __device__ __forceinline__ double ahat(const DevModel& m, int, int p) { return m.p_ahat[p]; }
-  static __device__ __forceinline__ double ahat_edge(const DevModel& m, int, int p) { return m.p_ahat_edge[p]; }
-  static __device__ __forceinline__ bool mass_dir(const DevModel&, int, int) { return false; }
-  static __device__ __forceinline__ bool side_dir(const DevModel&, int, int) { return false; }
-  static __device__ __forceinline__ double half(const DevModel& m, int, int g, int i) { return m.g_size[g][i]; }
-};
-template <>
-struct Par<Dual> {
-  static __device__ __forceinline__ Dual get(int pdir, int k, double v) { return Dual(v, pdir == k ? 1.0 : 0.0); }
-  // bcoef = 2 / (d_w t_c), kcoef = 1 / (d_w^2 t_c^2 phi_d^2): values as
-  // compiled, tangents by their logarithmic derivatives
-  static __device__ __forceinline__ Dual bcoef(const DevModel& m, int pdir) {
-    const double b = m.bcoef;
-    return Dual(b, pdir == PAR_TC ? -b / m.solref[0] : pdir == PAR_DW ? -b / m.solimp[1] : 0.0);
-  }
-  static __device__ __forceinline__ Dual kcoef(const DevModel& m, int pdir) {
-    const double k = m.kcoef;
-    return Dual(k, pdir == PAR_TC ? -2.0 * k / m.solref[0]
-                 : pdir == PAR_DAMP ? -2.0 * k / m.solref[1]
-                 : pdir == PAR_DW ? -2.0 * k / m.solimp[1] : 0.0);
-  }
-  // d A_hat / d theta: non-zero for the body masses and box sides only
-  static __device__ __forceinline__ double dahat(const DevModel& m, int pdir, int p) {
-    const int b = pdir - par_mass(m, 0);
-    return (b >= 0 && b < m.nbody + m.nbox) ? m.p_dahat[p][b] : 0.0;
-  }
-  static __device__ __forceinline__ Dual ahat(const DevModel& m, int pdir, int p) {
-    return Dual(m.p_ahat[p], dahat(m, pdir, p));
-  }
-  // A_hat (1 + mu^2) of a pyramid-edge row
-  static __device__ __forceinline__ Dual ahat_edge(const DevModel& m, int pdir, int p) {
-    const double mu = m.p_mu[p];
-    return Dual(m.p_ahat_edge[p], (pdir == PAR_MU0 + p ? 2.0 * mu * m.p_ahat[p] : 0.0) +
-                                      dahat(m, pdir, p) * (1.0 + mu * mu));
-  }
-  static __device__ __forceinline__ bool mass_dir(const DevModel& m, int pdir, int b) { return pdir == par_mass(m, b); }
-  static __device__ __forceinline__ bool side_dir(const DevModel& m, int pdir, int b) {
-    return m.b_solebox[b] >= 0 && pdir == par_side(m, m.g_box[m.b_solebox[b]]);
-  }
-  // half size i of geom g: a box's carries dh_i/dl = h_i / (2 h_0) along its side l
-  static __device__ __forceinline__ Dual half(const DevModel& m, int pdir, int g, int i) {
-    const double h = m.g_size[g][i];
-    return Dual(h, (m.g_box[g] >= 0 && pdir == par_side(m, m.g_box[g])) ? h / (2.0 * m.g_size[g][0]) : 0.0);
-  }
-};
 using Ws = WsT<double>;
 
 // Entry e (row-major) of the rotation of the quaternion x (w, x, y, z) with
@@ -323,7 +202,6 @@ using Ws = WsT<double>;
 // e, so that the nine lanes of a body run one instruction sequence: a switch
 // over e costs the sum of its nine sides.
 __device__ __forceinline__ double mul_add(double a, double b, double c) { return __fma_rn(a, b, c); }
-__device__ __forceinline__ Dual mul_add(const Dual& a, const Dual& b, const Dual& c) { return a * b + c; }
 template <class T>
 __device__ __forceinline__ T quat_entry(const T* x, const T& s, int e) {
   // per entry 8 bits: u1, u3, u2, u4 (2 bits each, lowest first; 0 = w)
@@ -520,19 +398,12 @@ __device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const 
   // meets one kind.  Ic starts as a copy (composite inertias, crba).
   DMX_TASKS(k, 6 * nb) {
     const int b = k / 6, e = k - 6 * b;
-    const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
+    const double ms = m.b_mass[b];
     const T* c = C + 3 * b;
     const int i = e < 3 ? e : (e == 5 ? 1 : 0), j = e < 3 ? e : (e == 3 ? 1 : 2);   // xx yy zz xy xz yz
     const T* Rb = R + 9 * b;
     const double* In = m.b_inertia[b];
     T v = Rb[3 * i] * Rb[3 * j] * In[0] + Rb[3 * i + 1] * Rb[3 * j + 1] * In[1] + Rb[3 * i + 2] * Rb[3 * j + 2] * In[2];
-    if (Par<T>::mass_dir(m, w.pdir, b)) v = v * (ms / m.b_mass[b]);   // inertia proportional to the mass
-    if (Par<T>::side_dir(m, w.pdir, b)) {                             // ... and to the side squared
-      const int gs = m.b_solebox[b];
-      const double l0 = 2.0 * m.g_size[gs][0];
-      const auto lam = Par<T>::get(w.pdir, par_side(m, m.g_box[gs]), l0) / l0;
-      v = v * (lam * lam);
-    }
     const T cc = c[0] * c[0] + c[1] * c[1] + c[2] * c[2];
     v += ms * ((i == j ? cc : T(0.0)) - c[i] * c[j]);
     Ib[10 * b + 4 + e] = v;
@@ -540,7 +411,7 @@ __device__ void kinematics(const Grp<G>& g, const MD& m, const WsT<T>& w, const 
   }
   DMX_TASKS(k, 4 * nb) {
     const int b = k / 4, e = k - 4 * b;
-    const auto ms = Par<T>::get(w.pdir, par_mass(m, b), m.b_mass[b]);
+    const double ms = m.b_mass[b];
     T v;
     if (e == 0) v = ms; else v = ms * C[3 * b + e - 1];
     Ib[10 * b + e] = v;
@@ -661,22 +532,22 @@ template <class T, class H>
 __device__ __forceinline__ T box_sdf(const T* y, const H* h, T* grad) {
   T qd[3];
   bool out = false;
-  for (int i = 0; i < 3; ++i) { qd[i] = fabs(y[i]) - h[i]; out = out || value(qd[i]) > 0; }
+  for (int i = 0; i < 3; ++i) { qd[i] = fabs(y[i]) - h[i]; out = out || qd[i] > 0; }
   if (out) {
     T ss = 0.0;
-    for (int i = 0; i < 3; ++i) if (value(qd[i]) > 0) ss += qd[i] * qd[i];
+    for (int i = 0; i < 3; ++i) if (qd[i] > 0) ss += qd[i] * qd[i];
     const T d = sqrt(ss), inv = 1.0 / d;
     for (int i = 0; i < 3; ++i) {
-      const T gg = value(qd[i]) > 0 ? qd[i] * inv : T(0.0);
-      grad[i] = value(y[i]) < 0 ? -gg : gg;
+      const T gg = qd[i] > 0 ? qd[i] * inv : T(0.0);
+      grad[i] = y[i] < 0 ? -gg : gg;
     }
     return d;
   }
   int k = 0;
-  if (value(qd[1]) > value(qd[k])) k = 1;
-  if (value(qd[2]) > value(qd[k])) k = 2;
+  if (qd[1] > qd[k]) k = 1;
+  if (qd[2] > qd[k]) k = 2;
   grad[0] = 0.0; grad[1] = 0.0; grad[2] = 0.0;
-  grad[k] = value(y[k]) < 0 ? -1.0 : 1.0;
+  grad[k] = y[k] < 0 ? -1.0 : 1.0;
   return qd[k];
 }
 // A number with the sign of the slope of the box distance field along
@@ -732,46 +603,28 @@ __device__ __forceinline__ double capsule_box_curv(const double* y0v, const doub
 
 // Capsule (geom g1) against box (geom g2): minimum over the capsule axis of
 // the box distance field (convex along the axis; bisection on its slope, in
-// values).  In derivative scalars the minimiser s carries ds/dtheta from the
-// implicit function theorem (slope = 0 at an interior minimum of the smooth
-// outside field: ds = -d(slope) / (d slope / ds)); elsewhere s is constant.
+// values).
 template <class T>
 __device__ void capsule_box(const DevModel& m, const T* gR, const T* gp, int g1, int g2, double thr, T* ct,
-                            T* s_out, int pdir = -1) {
+                            T* s_out) {
   const double rc = m.g_size[g1][0], Lh = m.g_size[g1][1];
   const double* h = m.g_size[g2];
-  // the box half sizes as the evaluation's scalars (a side-length tangent in derivative scalars)
-  T hd[3];
-  if constexpr (!std::is_same<T, double>::value)
-    for (int i = 0; i < 3; ++i) hd[i] = Par<T>::half(m, pdir, g2, i);
-  const auto* hT = [&]() {
-    if constexpr (std::is_same<T, double>::value) return h; else return static_cast<const T*>(hd);
-  }();
   const T* R1 = gR + 9 * g1; const T* R2 = gR + 9 * g2;
   const T* c1 = gp + 3 * g1; const T* c2 = gp + 3 * g2;
   T dc[3] = {c1[0] - c2[0], c1[1] - c2[1], c1[2] - c2[2]};
   const double reach = m.g_bound[g1] + m.g_bound[g2] + (thr > 0 ? thr : 0.0);
-  const double dd = value(dc[0]) * value(dc[0]) + value(dc[1]) * value(dc[1]) + value(dc[2]) * value(dc[2]);
+  const double dd = dc[0] * dc[0] + dc[1] * dc[1] + dc[2] * dc[2];
   if (dd > reach * reach) { ct[0] = 1e30; return; }   // cannot be within the threshold
   const T u[3] = {R1[0], R1[3], R1[6]};
   T y0[3], wv[3];
   matTvec3(R2, dc, y0);
   matTvec3(R2, u, wv);
-  const double y0v[3] = {value(y0[0]), value(y0[1]), value(y0[2])}, wvv[3] = {value(wv[0]), value(wv[1]), value(wv[2])};
+  const double y0v[3] = {y0[0], y0[1], y0[2]}, wvv[3] = {wv[0], wv[1], wv[2]};
   const double sv = capsule_box_s(y0v, wvv, Lh, h);
   *s_out = T(sv);
   T s = sv;
-  if constexpr (!std::is_same<T, double>::value) {
-    const double phi2 = capsule_box_curv(y0v, wvv, sv, Lh, h);
-    if (phi2 > 0) {
-      T yT[3] = {y0[0] + sv * wv[0], y0[1] + sv * wv[1], y0[2] + sv * wv[2]}, gT[3];
-      box_sdf(yT, hT, gT);
-      const T slope = gT[0] * wv[0] + gT[1] * wv[1] + gT[2] * wv[2];
-      s = T(sv, -slope.d / phi2);
-    }
-  }
   T y[3] = {y0[0] + s * wv[0], y0[1] + s * wv[1], y0[2] + s * wv[2]}, gr[3], n[3];
-  const T dist = box_sdf(y, hT, gr);
+  const T dist = box_sdf(y, h, gr);
   matvec3(R2, gr, n);
   const T r = dist - rc;
   ct[0] = r;
@@ -779,26 +632,23 @@ __device__ void capsule_box(const DevModel& m, const T* gR, const T* gp, int g1,
   for (int i = 0; i < 3; ++i) { ct[1 + i] = c1[i] + s * u[i] - off * n[i]; ct[4 + i] = n[i]; }
   // tangent frame: t1 perpendicular to n and world z (world x when n is near z)
   double ref[3] = {0, 0, 1};
-  if (fabs(value(n[2])) >= 0.5) { ref[0] = 1; ref[2] = 0; }
+  if (fabs(n[2]) >= 0.5) { ref[0] = 1; ref[2] = 0; }
   T t1[3], t2[3];
   cross3(n, ref, t1);
-  const T il = rsqrt_t(dot3(t1, t1));
+  const T il = rsqrt(dot3(t1, t1));
   t1[0] *= il; t1[1] *= il; t1[2] *= il;
   cross3(n, t1, t2);
   for (int i = 0; i < 3; ++i) { ct[7 + i] = t1[i]; ct[10 + i] = t2[i]; }
 }
 
-// Spline of the solimp shape on x in [0, 1] (midpoint mid, power pw).
 // Sphere / capsule pair (the billiard's ball-ball contact of Sec. 4, capsule
 // pairs of App. C.1): geom g is the segment c + s u, |s| <= L along its local
 // x (L = 0 for a sphere), radius rad.  Closest points: the least of the
 // candidates of the box-constrained optimality conditions of
 // |D + s ua - t ub|^2 (D = ca - cb): the interior point (non-parallel axes)
-// and each edge with the other parameter clamped.  Decisions on values; with
-// derivative scalars the free parameters are re-solved from the reduced
-// optimality conditions (Du + s - c t = 0, -Dv - c s + t = 0), carrying
-// ds/dtheta, dt/dtheta.  n from geom 2 to geom 1, r = |d| - ra - rb,
-// pos = pa - (ra + r/2) n; tangent frame as for capsule-box.  st_out: s, t.
+// and each edge with the other parameter clamped.  n from geom 2 to geom 1,
+// r = |d| - ra - rb, pos = pa - (ra + r/2) n; tangent frame as for
+// capsule-box.  st_out: s, t.
 __device__ __forceinline__ double seg_half(const DevModel& m, int g) {
   return m.g_type[g] == GEOM_CAPSULE ? m.g_size[g][1] : 0.0;
 }
@@ -833,28 +683,16 @@ __device__ void seg_seg(const DevModel& m, const T* gR, const T* gp, int g1, int
   const T* c1 = gp + 3 * g1; const T* c2 = gp + 3 * g2;
   const T D[3] = {c1[0] - c2[0], c1[1] - c2[1], c1[2] - c2[2]};
   const double reach = m.g_bound[g1] + m.g_bound[g2] + (thr > 0 ? thr : 0.0);
-  const double Dv0[3] = {value(D[0]), value(D[1]), value(D[2])};
+  const double Dv0[3] = {D[0], D[1], D[2]};
   if (Dv0[0] * Dv0[0] + Dv0[1] * Dv0[1] + Dv0[2] * Dv0[2] > reach * reach) { ct[0] = 1e30; return; }
   const T ua[3] = {R1[0], R1[3], R1[6]}, ub[3] = {R2[0], R2[3], R2[6]};
-  const double uav[3] = {value(ua[0]), value(ua[1]), value(ua[2])}, ubv[3] = {value(ub[0]), value(ub[1]), value(ub[2])};
+  const double uav[3] = {ua[0], ua[1], ua[2]}, ubv[3] = {ub[0], ub[1], ub[2]};
   const double cv = dot3(uav, ubv), Duv = dot3(Dv0, uav), Dvv = dot3(Dv0, ubv);
   double sv, tv;
   seg_closest(cv, Duv, Dvv, La, Lb, Dv0, uav, ubv, &sv, &tv);
   st_out[0] = T(sv);
   st_out[1] = T(tv);
   T s = sv, t = tv;
-  if constexpr (!std::is_same<T, double>::value) {
-    const bool sf = fabs(sv) < La, tf = fabs(tv) < Lb;
-    const T c = dot3(ua, ub), Du = dot3(D, ua), Dv = dot3(D, ub);
-    if (sf && tf) {
-      s = (c * Dv - Du) / (1.0 - c * c);
-      t = Dv + c * s;
-    } else if (sf) {
-      s = tv * c - Du;
-    } else if (tf) {
-      t = Dv + sv * c;
-    }
-  }
   T d[3], n[3];
   for (int i = 0; i < 3; ++i) d[i] = D[i] + s * ua[i] - t * ub[i];
   const T rho = sqrt(dot3(d, d));
@@ -865,18 +703,19 @@ __device__ void seg_seg(const DevModel& m, const T* gR, const T* gp, int g1, int
   const T off = ra + 0.5 * r;
   for (int i = 0; i < 3; ++i) { ct[1 + i] = c1[i] + s * ua[i] - off * n[i]; ct[4 + i] = n[i]; }
   double ref[3] = {0, 0, 1};
-  if (fabs(value(n[2])) >= 0.5) { ref[0] = 1; ref[2] = 0; }
+  if (fabs(n[2]) >= 0.5) { ref[0] = 1; ref[2] = 0; }
   T t1[3], t2[3];
   cross3(n, ref, t1);
-  const T il = rsqrt_t(dot3(t1, t1));
+  const T il = rsqrt(dot3(t1, t1));
   t1[0] *= il; t1[1] *= il; t1[2] *= il;
   cross3(n, t1, t2);
   for (int i = 0; i < 3; ++i) { ct[7 + i] = t1[i]; ct[10 + i] = t2[i]; }
 }
 
+// Spline of the solimp shape on x in [0, 1] (midpoint mid, power pw).
 template <class T>
 __device__ __forceinline__ T spline_shape(const T& x, double mid, double pw) {
-  if (value(x) <= mid && mid > 0) {
+  if (x <= mid && mid > 0) {
     const T num = (pw == 2.0) ? x * x : (pw == 4.0 ? (x * x) * (x * x) : pow(x, pw));
     return num / ((pw == 2.0) ? mid : ::pow(mid, pw - 1.0));
   }
@@ -886,7 +725,8 @@ __device__ __forceinline__ T spline_shape(const T& x, double mid, double pw) {
 }
 // a / b for a model constant b > 0 whose reciprocal rb was rounded on the host
 // and 0 <= a <= 2 b: the quotient estimate a rb corrected by its exact
-// remainder, three FP64 instructions instead of nine.
+// remainder (Markstein 1990: with rb correctly rounded this is the rounded
+// quotient).  Three FP64 instructions.
 __device__ __forceinline__ double div_const(double a, double b, double rb) {
   const double q = a * rb;
   return __fma_rn(__fma_rn(-b, q, a), rb, q);
@@ -907,37 +747,25 @@ __device__ __forceinline__ double impedance_quadratic(const DevModel& m, double 
   if (above(d, 0.9999)) return 0.9999;
   return d;
 }
-// The same shape with a derivative-scalar midpoint (parameter tangents).
-__device__ __forceinline__ Dual spline_shape(const Dual& x, const Dual& mid, double pw) {
-  if (value(x) <= value(mid) && value(mid) > 0) {
-    const Dual num = (pw == 2.0) ? x * x : (pw == 4.0 ? (x * x) * (x * x) : pow(x, pw));
-    return num / ((pw == 2.0) ? mid : pow(mid, pw - 1.0));
-  }
-  const Dual y = 1.0 - x;
-  const Dual num = (pw == 2.0) ? y * y : (pw == 4.0 ? (y * y) * (y * y) : pow(y, pw));
-  const Dual om = 1.0 - mid;
-  return 1.0 - num / ((pw == 2.0) ? om : pow(om, pw - 1.0));
-}
 template <class T>
-__device__ __forceinline__ T impedance(const DevModel& m, const T& r, bool cfd, int pdir = -1) {
+__device__ __forceinline__ T impedance(const DevModel& m, const T& r, bool cfd) {
   T d;
-  if (cfd && value(r) >= 0) {
+  if (cfd && r >= 0) {
     T x = 1.0 - r / m.cfd[2];
-    if (value(x) < 0) x = 0.0;
+    if (x < 0) x = 0.0;
     d = m.cfd[0] + (m.cfd[1] - m.cfd[0]) * spline_shape(x, m.cfd[3], m.cfd[4]);
   } else {
-    const auto d_o = Par<T>::get(pdir, PAR_DO, m.solimp[0]), d_w = Par<T>::get(pdir, PAR_DW, m.solimp[1]);
-    const auto width = Par<T>::get(pdir, PAR_WIDTH, m.solimp[2]), mid = Par<T>::get(pdir, PAR_MID, m.solimp[3]);
+    const double d_o = m.solimp[0], d_w = m.solimp[1], width = m.solimp[2], mid = m.solimp[3];
     T x = fabs(r) / width;
-    if (value(x) > 1.0) x = 1.0;
+    if (x > 1.0) x = 1.0;
     d = d_o + (d_w - d_o) * spline_shape(x, mid, m.solimp[4]);
   }
-  if (value(d) < 0.0) return T(0.0);
-  if (value(d) > 0.9999) return T(0.9999);
+  if (d < 0.0) return T(0.0);
+  if (d > 0.9999) return T(0.9999);
   return d;
 }
 template <class T>
-__device__ __forceinline__ T softplus(const T& x) { return value(x) > 0 ? x + log1p(exp(-x)) : log1p(exp(x)); }
+__device__ __forceinline__ T softplus(const T& x) { return x > 0 ? x + log1p(exp(-x)) : log1p(exp(x)); }
 
 // All contact slots, then the included ones (r < 0, or r < w_c for F~) and
 // their per-slot impedance terms.
@@ -952,7 +780,7 @@ __device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd)
     const SlotInfo si = slot_info(m, s);
     const int j = si.idx, g1 = si.g1;
     if (si.g2 >= 0) {
-      if (m.g_type[si.g2] == GEOM_BOX) capsule_box(m, gR, gp, g1, si.g2, thr, ct, w.at(L.csv) + 2 * s, w.pdir);
+      if (m.g_type[si.g2] == GEOM_BOX) capsule_box(m, gR, gp, g1, si.g2, thr, ct, w.at(L.csv) + 2 * s);
       else seg_seg(m, gR, gp, g1, si.g2, thr, ct, w.at(L.csv) + 2 * s);
     } else {
       const T* Rg = gR + 9 * g1; const T* cg = gp + 3 * g1;
@@ -966,17 +794,10 @@ __device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd)
         rad = m.g_size[g1][0];
       } else {
         T t[3];
-        if constexpr (std::is_same<T, double>::value) {
-          const double ex[3] = {(j & 1) ? m.g_size[g1][0] : -m.g_size[g1][0],
-                                (j & 2) ? m.g_size[g1][1] : -m.g_size[g1][1],
-                                (j & 4) ? m.g_size[g1][2] : -m.g_size[g1][2]};
-          matvec3(Rg, ex, t);
-        } else {   // derivative scalars: the half sizes carry a side-length tangent
-          const T h0 = Par<T>::half(m, w.pdir, g1, 0), h1 = Par<T>::half(m, w.pdir, g1, 1);
-          const T h2 = Par<T>::half(m, w.pdir, g1, 2);
-          const T ex[3] = {(j & 1) ? h0 : -h0, (j & 2) ? h1 : -h1, (j & 4) ? h2 : -h2};
-          matvec3(Rg, ex, t);
-        }
+        const double ex[3] = {(j & 1) ? m.g_size[g1][0] : -m.g_size[g1][0],
+                              (j & 2) ? m.g_size[g1][1] : -m.g_size[g1][1],
+                              (j & 4) ? m.g_size[g1][2] : -m.g_size[g1][2]};
+        matvec3(Rg, ex, t);
         pt[0] = cg[0] + t[0]; pt[1] = cg[1] + t[1]; pt[2] = cg[2] + t[2];
       }
       const T r = pt[2] - rad;
@@ -985,16 +806,14 @@ __device__ void collide(const Grp<G>& g, const MD& m, const WsT<T>& w, bool cfd)
       ct[4] = 0.0; ct[5] = 0.0; ct[6] = 1.0; ct[7] = 1.0; ct[8] = 0.0; ct[9] = 0.0; ct[10] = 0.0; ct[11] = 1.0;
       ct[12] = 0.0;
     }
-    const bool inc = cfd ? value(ct[0]) < thr : is_neg(value(ct[0]));
+    const bool inc = cfd ? ct[0] < thr : is_neg(ct[0]);
     w.i[L.sinc + s] = inc ? 1 : 0;
     if (inc) {
       const T r = ct[0];
-      T d;
-      if constexpr (std::is_same<T, double>::value) d = (!cfd && m.solimp[4] == 2.0) ? impedance_quadratic(m, r) : impedance(m, r, cfd);
-      else d = impedance(m, r, cfd, w.pdir);
+      const T d = (!cfd && m.solimp[4] == 2.0) ? impedance_quadratic(m, r) : impedance(m, r, cfd);
       const int pr = si.pair;
-      const auto ahat = m.s_rows[s] == 1 ? Par<T>::ahat(m, w.pdir, pr) : Par<T>::ahat_edge(m, w.pdir, pr);
-      const auto kc = Par<T>::kcoef(m, w.pdir);
+      const double ahat = m.s_rows[s] == 1 ? m.p_ahat[pr] : m.p_ahat_edge[pr];
+      const double kc = m.kcoef;
       ct[13] = d;
       ct[14] = cfd ? kc * d * (m.softplus * softplus(-r / m.softplus)) : -(kc * d * r);
       ct[15] = d / (ahat * (1.0 - d));
@@ -1060,7 +879,7 @@ __device__ int make_rows(const Grp<G>& g, const MD& m, const WsT<T>& w, const T*
     if (m.s_rows[s] == 1) {
       J[r0 * nv + i] = jn;
     } else {
-      const auto mu = Par<T>::get(w.pdir, PAR_MU0 + p, m.p_mu[p]);
+      const double mu = m.p_mu[p];
       J[r0 * nv + i] = jn + mu * j1;
       J[(r0 + 1) * nv + i] = jn - mu * j1;
       J[(r0 + 2) * nv + i] = jn + mu * j2;
@@ -1077,7 +896,7 @@ __device__ int make_rows(const Grp<G>& g, const MD& m, const WsT<T>& w, const T*
     const T* ct = CT + 16 * s;
     T jv = 0.0;
     for (int i = 0; i < nv; ++i) jv += J[r * nv + i] * v[i];
-    aref[r] = -(Par<T>::bcoef(m, w.pdir) * jv) + ct[14];
+    aref[r] = -(m.bcoef * jv) + ct[14];
     Dr[r] = ct[15];
     rowid[r] = m.p_row0[p] + m.s_idx[s] * nrow + e;
   }
@@ -1097,8 +916,8 @@ __device__ bool cholesky(const Grp<G>& g, T* H, T* invd, int n, int rows) {
   const int e0 = t0.i * n + 1 + t0.j, r0 = t0.i * n, c0 = t0.j * n;
   for (int k = 0; k < n; ++k) {
     const T hkk = H[k * n + k];
-    ok = ok && is_pos(value(hkk));
-    const T il = rsqrt_t(hkk);   // the diagonal of the factor is kept as its reciprocal
+    ok = ok && is_pos(hkk);
+    const T il = rsqrt(hkk);   // the diagonal of the factor is kept as its reciprocal
     for (int i = k + 1 + g.lane; i < rows; i += G) H[i * n + k] *= il;
     if (g.lane == 0) invd[k] = il;
     g.sync();
@@ -1131,7 +950,7 @@ __device__ __forceinline__ double chol_back_lanes(const Grp<G>& g, const double*
 }
 template <int G, class T>
 __device__ void chol_back(const Grp<G>& g, const T* H, const T* invd, T* x, int n) {
-  if constexpr (G > 1 && std::is_same<T, double>::value) {
+  if constexpr (G > 1) {
     if (n <= G) {
       const double xi = chol_back_lanes(g, H, invd, g.lane < n ? x[g.lane] : 0.0, n);
       if (g.lane < n) x[g.lane] = xi;
@@ -1150,7 +969,7 @@ __device__ void chol_back(const Grp<G>& g, const T* H, const T* invd, T* x, int 
 // x <- H^-1 x with the factor from cholesky().
 template <int G, class T>
 __device__ void chol_solve(const Grp<G>& g, const T* H, const T* invd, T* x, int n) {
-  if constexpr (G > 1 && std::is_same<T, double>::value) {
+  if constexpr (G > 1) {
     if (n <= G) {
       double xi = g.lane < n ? x[g.lane] : 0.0;
       for (int k = 0; k < n; ++k) {
@@ -1245,7 +1064,7 @@ __device__ void residual_set(const Grp<G>& g, const MD& m, const WsT<T>& w, int 
     const T zr = t - aref[r];
     z[r] = zr;
     const int id = rowid[r];
-    const unsigned bit = is_neg(value(zr)) ? 1u << (id & 31) : 0u;
+    const unsigned bit = is_neg(zr) ? 1u << (id & 31) : 0u;
 #pragma unroll
     for (int k = 0; k < MASKW; ++k) bits[k] |= (id >> 5) == k ? bit : 0u;
   }
@@ -1269,21 +1088,21 @@ __device__ double line_search(const Grp<G>& g, const MD& m, const WsT<T>& w, int
   double c0 = 0, c1 = 0;
   DMX_TASKS(i, nv) {
     double ma = 0, md = 0;
-    for (int j = 0; j < nv; ++j) { ma += value(M[i * nv + j]) * value(a[j]); md += value(M[i * nv + j]) * value(dl[j]); }
-    c0 += value(dl[i]) * (ma - value(rhs0[i]));
-    c1 += value(dl[i]) * md;
+    for (int j = 0; j < nv; ++j) { ma += M[i * nv + j] * a[j]; md += M[i * nv + j] * dl[j]; }
+    c0 += dl[i] * (ma - rhs0[i]);
+    c1 += dl[i] * md;
   }
   const T* aref = w.at(L.aref);
   DMX_TASKS(r, nr) {
     double t = 0, u = 0;
-    for (int i = 0; i < nv; ++i) { t += value(J[r * nv + i]) * value(dl[i]); u += value(J[r * nv + i]) * value(a[i]); }
+    for (int i = 0; i < nv; ++i) { t += J[r * nv + i] * dl[i]; u += J[r * nv + i] * a[i]; }
     s[r] = t;
-    z[r] = u - value(aref[r]);
+    z[r] = u - aref[r];
   }
   g.sync();
   double s0 = 0, s1 = 0;
   DMX_TASKS(r, nr) {
-    const double zr = value(z[r]), sr = value(s[r]), dr = value(Dr[r]);
+    const double zr = z[r], sr = s[r], dr = Dr[r];
     const bool act = zr < 0 || (zr == 0 && sr < 0);
     if (act) { s0 += dr * zr * sr; s1 += dr * sr * sr; }
   }
@@ -1297,7 +1116,7 @@ __device__ double line_search(const Grp<G>& g, const MD& m, const WsT<T>& w, int
     double bz = 0, bs = 1;
     DMX_TASKS(r, nr) {
       if (((r < 64 ? tog0 : tog1) >> (r & 63)) & 1ull) continue;
-      const double zr = value(z[r]), sr = value(s[r]);
+      const double zr = z[r], sr = s[r];
       const bool act = zr < 0 || (zr == 0 && sr < 0);
       const bool cand = act ? (sr > 0) : (sr < 0 && zr > 0);
       if (!cand) continue;
@@ -1327,7 +1146,7 @@ __device__ double line_search(const Grp<G>& g, const MD& m, const WsT<T>& w, int
       }
     }
     if (best < 0) break;
-    const double zb = value(z[best]), sb = value(s[best]), db = value(Dr[best]);
+    const double zb = z[best], sb = s[best], db = Dr[best];
     const bool act = zb < 0 || (zb == 0 && sb < 0);
     const double dz = db * zb * sb, ds = db * sb * sb;
     if (act) { slope0 -= dz; slope1 -= ds; } else { slope0 += dz; slope1 += ds; }
@@ -1344,8 +1163,7 @@ __device__ double line_search(const Grp<G>& g, const MD& m, const WsT<T>& w, int
 // minimum between the iterate and an.  The first candidate set is the final
 // set of the previous right-hand side of this environment (pmask): when it is
 // still right, one factorisation finishes the solve; when not, Newton starts
-// from its solution.  pmask receives the final set.  In derivative scalars the
-// final solve with the final set carries the implicit-function derivative.
+// from its solution.  pmask receives the final set.
 // Returns 0 or an ENV_* code.
 template <int G, class T, class MD>
 __device__ int solve_constraints(const Grp<G>& g, const MD& m, const WsT<T>& w, int nr) {
@@ -1489,7 +1307,7 @@ static __constant__ TabSet c_tabs = make_tabs();
 // q (+) dq for every joint (free: translation + body-frame rotation exponential).
 template <class T>
 __device__ __forceinline__ void rot_exp(const T& th2, T& cw, T& sk) {   // cos(th / 2), sin(th / 2) / th
-  if (value(th2) < 1e-2) {
+  if (th2 < 1e-2) {
     // |dq| < 0.1 rad: Taylor series of cos(th/2) and sin(th/2)/th in th^2
     // (the next terms are below 3e-20): no square root, sine or division
     cw = 1.0 + th2 * (-1.0 / 8.0 + th2 * (1.0 / 384.0 + th2 * (-1.0 / 46080.0 + th2 * (1.0 / 10321920.0))));
@@ -1546,14 +1364,14 @@ __device__ void integrate_pos_lanes(const Grp<G>& g, const MD& m, const double* 
     const double r = x[0] * E0 + x[1] * E1 + x[2] * E2 + x[3] * E3;
     const double rw = __shfl_sync(g.mask, r, 0, 4), rx = __shfl_sync(g.mask, r, 1, 4);
     const double ry = __shfl_sync(g.mask, r, 2, 4), rz = __shfl_sync(g.mask, r, 3, 4);
-    const double in = rsqrt_t(rw * rw + rx * rx + ry * ry + rz * rz);
+    const double in = rsqrt(rw * rw + rx * rx + ry * ry + rz * rz);
     if (fr) out[qa + 3 + c] = r * in;
   }
   g.sync();
 }
 template <int G, class T, class MD>
 __device__ void integrate_pos(const Grp<G>& g, const MD& m, const T* q, const T* dq, T* out) {
-  if constexpr (G >= 4 && std::is_same<T, double>::value) {
+  if constexpr (G >= 4) {
     integrate_pos_lanes(g, m, q, dq, out);
   } else {
     DMX_TASKS(b, m.nbody) {
@@ -1570,7 +1388,7 @@ __device__ void integrate_pos(const Grp<G>& g, const MD& m, const T* q, const T*
       const T rx = w0 * ex + a0 * cw + b0 * ez - c0 * ey;
       const T ry = w0 * ey - a0 * ez + b0 * cw + c0 * ex;
       const T rz = w0 * ez + a0 * ey - b0 * ex + c0 * cw;
-      const T in = rsqrt_t(rw * rw + rx * rx + ry * ry + rz * rz);
+      const T in = rsqrt(rw * rw + rx * rx + ry * ry + rz * rz);
       out[qa + 3] = rw * in; out[qa + 4] = rx * in; out[qa + 5] = ry * in; out[qa + 6] = rz * in;
     }
     g.sync();

@@ -287,7 +287,7 @@ static __device__ void seg_seg_vjp(const DevModel& m, const double* gR, const do
   if (fabs(n[2]) >= 0.5) { ref[0] = 1; ref[2] = 0; }
   double t1r[3], t1[3];
   cross3(n, ref, t1r);
-  const double il = rsqrt_t(dot3(t1r, t1r));
+  const double il = rsqrt(dot3(t1r, t1r));
   for (int i = 0; i < 3; ++i) t1[i] = t1r[i] * il;
   // reverse: frame, position, distance
   double nb[3] = {cb[4], cb[5], cb[6]}, t1b[3] = {cb[7], cb[8], cb[9]};
@@ -360,7 +360,7 @@ static __device__ void capsule_box_vjp(const DevModel& m, const double* gR, cons
   if (fabs(n[2]) >= 0.5) { ref[0] = 1; ref[2] = 0; }
   double t1r[3], t1[3];
   cross3(n, ref, t1r);
-  const double il = rsqrt_t(dot3(t1r, t1r));
+  const double il = rsqrt(dot3(t1r, t1r));
   for (int i = 0; i < 3; ++i) t1[i] = t1r[i] * il;
   // reverse
   double nb[3] = {cb[4], cb[5], cb[6]}, t1b[3] = {cb[7], cb[8], cb[9]};
@@ -1077,7 +1077,7 @@ __device__ void integrate_pos_vjp(const Grp<G>& g, const MD& m, const double* q,
     r[1] = qq[0] * e[1] + qq[1] * e[0] + qq[2] * e[3] - qq[3] * e[2];
     r[2] = qq[0] * e[2] - qq[1] * e[3] + qq[2] * e[0] + qq[3] * e[1];
     r[3] = qq[0] * e[3] + qq[1] * e[2] - qq[2] * e[1] + qq[3] * e[0];
-    const double in = rsqrt_t(r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3]);
+    const double in = rsqrt(r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3]);
     const double* o4 = ob + qa + 3;
     double oo = 0.0;
     for (int k = 0; k < 4; ++k) oo += r[k] * in * o4[k];

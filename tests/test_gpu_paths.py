@@ -78,8 +78,9 @@ def test_parameter_gradients_without_contact(dmx, name, B):
     import torch
     sc = W.box_scene(solref=(0.005, 1.0)) if name == "toss" else W.SCENES[name]()
     inp = W.INPUTS[name](B, T=0.05)
-    z = inp["x0"][:, 2]
-    z[:] = np.where(np.arange(B) % 2 == 0, 2.0 + 0.01 * np.arange(B), 0.1)   # every other one starts at the ground
+    ground = np.arange(B) % 2 == 1        # every other one falls onto the plane from below its rest height
+    inp["x0"][:, 2] = np.where(ground, 0.045 if name == "toss" else 0.095, 2.0 + 0.01 * np.arange(B))
+    inp["x0"][:, 9] = np.where(ground, -0.5, 0.0)
     model = dmx.Model(sc)
     bar = _dev(np.random.default_rng(4).normal(size=(model.nx, B)))
     out = _call(dmx, model, inp, tape=True, K=8)
