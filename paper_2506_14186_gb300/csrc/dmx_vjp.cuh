@@ -43,21 +43,6 @@ struct WsB {
 };
 
 // ------------------------------------------------------------------ small VJP helpers
-// a / b: the hardware's 20-bit reciprocal estimate y of b, refined by the
-// first two terms of 1 / (1 - e) = 1 + e + e^2 + ... (e = 1 - b y, the third
-// is below 2^-60), then the quotient corrected by its exact remainder
-// (Markstein): six FP64 instructions, against nine of the operator.  Operands
-// whose exponents are far out take the operator.
-__device__ __forceinline__ double quotient(double a, double b) {
-  const unsigned ea = (unsigned)(__double2hiint(a) >> 20) & 0x7ffu, eb = (unsigned)(__double2hiint(b) >> 20) & 0x7ffu;
-  if (eb - 523u >= 1000u || (ea - 523u >= 1000u && a != 0.0)) return a / b;
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
-  const double e = __fma_rn(-b, y, 1.0);
-  y = __fma_rn(y, __fma_rn(e, e, e), y);
-  const double q = __dmul_rn(a, y);
-  return __fma_rn(__fma_rn(-b, q, a), y, q);
-}
 __device__ __forceinline__ void acc_cross(const double* a, const double* b, double* out) {
   out[0] += a[1] * b[2] - a[2] * b[1];
   out[1] += a[2] * b[0] - a[0] * b[2];
@@ -231,7 +216,7 @@ __device__ __forceinline__ double impedance_terms_vjp(const DevModel& m, double 
     rb -= b14 * m.kcoef * d;
   }
   const double om = 1.0 - d;
-  db += quotient(b15, ahat * om * om);
+  db += b15 / (ahat * om * om);
   return rb + db * dd;
 }
 
