@@ -942,7 +942,11 @@ extern "C" dmx_status dmx_eval_rhs(dmx_model* m, int32_t B, const double* q, con
   if (!valid_lanes(G)) return dmx_fail(DMX_ERR_INVALID, "lanes must be 0, 1, 2, 4, 8, 16 or 32");
   int threads; size_t smem;
   const dmx::Layout& L = layout_for(m, cfd);
-  if (!launch_config_layout(m, L, G, &threads, &smem)) return dmx_fail(DMX_ERR_INVALID, "workspace does not fit");
+  // the default stands for the rollout's group of that batch (reduction_lanes): where F~'s rows
+  // do not fit that one, the caller has to choose the lanes
+  if ((!lanes && !launch_config_layout(m, L, reduction_lanes(m, B), &threads, &smem)) ||
+      !launch_config_layout(m, L, G, &threads, &smem))
+    return dmx_fail(DMX_ERR_INVALID, "workspace does not fit");
   RolloutParams P{};
   P.model = m->dev; P.L = L; P.B = B;
   CK(launch_eval_rhs(G, P, q, v, m->host.nu ? u : q, cfd, a, info, threads, smem, static_cast<cudaStream_t>(stream)));
