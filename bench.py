@@ -177,14 +177,16 @@ def reduce_sum(x, world, device=None):
 
 
 # sources of the forward rollout kernel (the ncu record is valid while they are unchanged)
-FORWARD_SOURCES = ("dmx_device.cuh", "dmx_dual.cuh", "dmx_kernels.cuh", "dmx_kernels.h", "dmx_model.h",
-                   "dmx_inst_g1.cu", "dmx_inst_g2.cu", "dmx_inst_g4.cu", "dmx_inst_g8.cu", "dmx_inst_g16.cu",
-                   "dmx_inst_g32.cu")
+FORWARD_SOURCES = ("dmx_device.cuh", "dmx_kernels.cuh", "dmx_kernels.h", "dmx_model.h", "dmx_record.h",
+                   "dmx_record.cuh", "dmx_inst_g1.cu", "dmx_inst_g2.cu", "dmx_inst_g4.cu", "dmx_inst_g8.cu",
+                   "dmx_inst_g16.cu", "dmx_inst_g32.cu", "dmx_one_g4.cu", "dmx_one_g8.cu", "dmx_one_g16.cu",
+                   "dmx_one_g32.cu", "dmx_plane_g16.cu", "dmx_plane_g32.cu")
 
 
 # sources of the reverse adjoint kernel (its FP64 counter record is valid while they are unchanged)
 ADJOINT_SOURCES = FORWARD_SOURCES + ("dmx_adjoint.h", "dmx_adjoint_rev.cuh", "dmx_vjp.cuh", "dmx_adj_g2.cu",
-                                     "dmx_adj_g4.cu", "dmx_adj_g8.cu", "dmx_adj_g16.cu", "dmx_adj_g32.cu")
+                                     "dmx_adj_g4.cu", "dmx_adj_g8.cu", "dmx_adj_g16.cu", "dmx_adj_g32.cu",
+                                     "dmx_adjp_g8.cu", "dmx_adjp_g16.cu", "dmx_adjp_g32.cu")
 
 
 def _sources_sha(files):
