@@ -26,13 +26,15 @@ struct AdjParams {
   double* snapbuf;        // reverse mode: per group, K steps x (S - 1) stage snapshots of SN doubles (or null)
   int SN;                 // doubles per snapshot
   StepRecords rec;        // records of the taped rollout
+  double* cfdsnap;        // with cfd: snapshots of F~ at the recorded stage states ([ncfd] chunks), or null
+  int ncfd;
   int kind;               // MODEL_* type of the kernels (OneBody: 8, 16, 32 lanes, PlaneOnly: 16, 32)
   int per, barofs;        // reverse mode: doubles per environment, offset of the cotangent workspace
   double* p_bar;          // [np][B] model-parameter gradients, or null
   int np;                 // model parameters differentiated when p_bar is set
   const int* touched;     // [B] or null (every environment): the reverse-mode kernel takes the environments whose
                           // taped steps met a contact, the tangent kernel the others
-  int* queue;             // next environment
+  int* queue;             // [2] next environment, next recorded step (cfd)
 };
 
 cudaError_t launch_adjoint(const AdjParams& P, int blocks, cudaStream_t st);

@@ -27,6 +27,13 @@
 // warm start of its Newton search, so the restored workspace equals a
 // recomputed one.  Segments whose steps the forward pass kept (dmx_record.h)
 // are not recomputed at all: rows and snapshots are read from the records.
+//
+// Bound by the chain of a stage (restore, VJP, stage cotangents): about 160 k
+// cycles for the arm on 32 lanes, with one to four warps on a sub-partition.
+// 2048 arms with their
+// gradient (0.2 s) went from 413 to 165 ms, 2048 tosses from 269 to 97 ms, 300
+// quadrupeds with cfd from 545 to 248 ms, parameter gradients of 256 tosses
+// (PAR, against the forward-mode kernel) from 314 to 63 ms.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -140,6 +147,68 @@ __device__ int rk_step_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB&
     g.sync();
   }
   return st;
+}
+
+// Snapshots of F~ at the stage states of step n (k_cfd_stages), or null.
+__device__ __forceinline__ const double* cfd_snaps(const AdjParams& P, int env, int n, int stages) {
+  const int k = n / REC_STEPS, c = P.rec.chunk[(size_t)env * P.rec.per_env + k] - 1;
+  return c >= 0 && c < P.ncfd ? P.cfdsnap + ((size_t)c * REC_STEPS + (n - k * REC_STEPS)) * stages * P.SN : nullptr;
+}
+
+// F~ at the stage states of every recorded step, one step per group at a time:
+// nothing here depends on the cotangents, so the steps of all environments run
+// at once instead of one after the other inside the sweeps (a third of a cfd
+// sweep's chain, on as many warps as there are environments).  Bound by the
+// FP64 unit.  Forward and cfd adjoint, bitwise the same gradients: 300 quadrupeds
+// 288 -> 248 ms, 300 arms 88 -> 71, 1500 tosses 168 -> 141, 1500 quadrupeds 348 ->
+// 319.
+template <int G, class MD>
+__global__ void __launch_bounds__(32, 1) k_cfd_stages(const __grid_constant__ AdjParams P) {
+  extern __shared__ double smem[];
+  const Layout& sL = P.L;
+  const MD& m = *static_cast<const MD*>(P.model);
+  Grp<G> g;
+  const int ngb = blockDim.x / G, gib = threadIdx.x / G;
+  const Ws w{smem + (size_t)gib * sL.nd, reinterpret_cast<int*>(smem + (size_t)ngb * sL.nd) + (size_t)gib * sL.ni, &sL};
+  const int nq = m.nq, nv = m.nv, nu = m.nu, mt = P.method, S = TAB(mt).S;
+  double* qs = w.at(sL.qs); double* vs = w.at(sL.vs); double* qn = w.at(sL.qn); double* dq = w.at(sL.dq);
+  double* u = w.at(sL.u);
+  const int total = min(*P.rec.next, P.ncfd) * REC_STEPS;
+  if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
+  g.sync();
+  for (;;) {
+    int it = 0;
+    if (g.lane == 0) it = atomicAdd(P.queue + 1, 1);
+    it = g.bcast(it, 0);
+    if (it >= total) break;
+    const int c = it / REC_STEPS, env = P.rec.owner[2 * c];
+    const int n = P.rec.owner[2 * c + 1] * REC_STEPS + (it - c * REC_STEPS);
+    if (n >= P.tape_n[env]) continue;
+    const double* row = P.rec.mem + (size_t)it * P.rec.stride + (S - 1) * P.rec.snap;
+    const double* vst = row + nq;
+    const double h = P.hlog[(size_t)n * P.B + env];
+    const int kn = rev_interval(P.T[env], P.NI, row[nq + 7 * nv]);
+    DMX_TASKS(i, nq) qn[i] = row[i];
+    DMX_TASKS(a, nu) u[a] = P.ctrl[((size_t)kn * nu + a) * P.B + env];
+    g.sync();
+    for (int s = 0; s <= S - 2; ++s) {
+      const unsigned mq = TAB(mt).nzq[s];
+      DMX_TASKS(i, nv) {
+        double sq = 0;
+        for (int j = 0; j <= s; ++j)
+          if ((mq >> j) & 1u) sq += TAB(mt).aq[s][j] * vst[j * nv + i];
+        dq[i] = h * sq;
+        vs[i] = vst[s * nv + i];
+      }
+      if (s == 0)
+        DMX_TASKS(i, nq) qs[i] = qn[i];
+      g.sync();
+      if (s >= 1) integrate_pos(g, m, (const double*)qn, (const double*)dq, qs);
+      const int r = rhs(g, m, w, (const double*)qs, (const double*)vs, (const double*)u, true, w.at(sL.ka));
+      snap_save(g, m, w, P.cfdsnap + ((size_t)it * (S - 1) + s) * P.SN, r);
+      g.sync();
+    }
+  }
 }
 
 // PAR: with the model-parameter gradients (p_bar).
@@ -256,7 +325,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
         DMX_TASKS(i, nv) Vb[i] = xbar[nq + i];
         g.sync();
         const int st = rk_step_vjp<G, PAR>(g, m, w, b, (const double*)u, h, mt, P.cfd != 0,
-                                   P.cfd ? nullptr : kept ? srec : use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr,
+                                   P.cfd ? (kept ? cfd_snaps(P, env, n, S - 1) : nullptr) : kept ? srec : use_snap ? snb + (size_t)(n - n0) * (S - 1) * SN : nullptr,
                                    SN);
         if (st > worst) worst = st;
         const double* qnb = b.at(sB.qnb); const double* vnb = b.at(sB.vnb); const double* ub = b.at(sB.ub);
@@ -331,6 +400,20 @@ cudaError_t launch_eval_rhs_vjp_g(const AdjParams& P, const double* q, const dou
 
 template <int G, bool PAR, class MD>
 cudaError_t launch_adjoint_rev_g(const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
+  if constexpr (!PAR)
+    if (P.cfdsnap) {
+      auto ks = k_cfd_stages<G, MD>;
+      const size_t sm = (size_t)(32 / G) * ((size_t)P.L.nd * 8 + (size_t)P.L.ni * 4);
+      cudaError_t e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      if (e != cudaSuccess) return e;
+      int dev = 0, nsm = 0, occ = 0;
+      if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+          (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+          (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ks, threads, sm)) != cudaSuccess)
+        return e;
+      ks<<<nsm * (occ > 0 ? occ : 1), threads, sm, st>>>(P);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
   auto k = k_adjoint_rev<G, PAR, MD>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -61,6 +61,7 @@ __device__ double* claim_record(const Grp<G>& g, const StepRecords& r, int env, 
       c = atomicAdd(r.next, 1);
       c = c < r.nchunk ? c + 1 : -1;
       *p = c;
+      if (c > 0) { r.owner[2 * (c - 1)] = env; r.owner[2 * (c - 1) + 1] = k; }
     }
   }
   c = g.bcast(c, 0);

@@ -41,6 +41,7 @@ struct StepRecords {
   double* mem;              // [nchunk][REC_STEPS][stride], or null: no records
   int* chunk;               // [B][per_env]: 0 not asked for, -1 none left, else chunk index + 1
   int* next;                // chunks handed out
+  int* owner;               // [nchunk][2]: environment and place (step / REC_STEPS) of a chunk
   int nchunk, per_env, stride, snap;   // capacity, table width, doubles per step, per snapshot
 };
 

@@ -385,10 +385,10 @@ int reduction_lanes(const dmx_model* m, int B) {
 // least) that leave an SM at most `warps` warps of the environments it holds
 // (its share of the batch, or what its shared memory takes).  Fewer lanes leave
 // an SM's few environments on too few warps to cover their dependent reads
-// (quadruped rollouts, 3000 for 0.1 s: 172 ms with 32 lanes, 197 with 16, 358
+// (quadruped rollouts, 3000 for 0.1 s: 158 ms with 32 lanes, 188 with 16, 365
 // with 8); more lanes spread the same FP64 instructions thinner once the FP64
-// unit is busy (box pushes, 4096 for 0.05 s: 55 ms with 8 lanes, 63 with 16,
-// 94 with 32; tosses, 20001 for 0.2 s: 250, 287, 385).
+// unit is busy (box pushes, 4096 for 0.1 s: 76 ms with 8 lanes, 104 with 16,
+// 133 with 32; tosses, 20001 for 0.2 s: 171, 225, 303).
 int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
   const long long share = ((long long)B + m->nsm - 1) / m->nsm;
   const long long fit = (long long)((size_t)(m->smem_max + 1024) / (per + 256));
@@ -399,8 +399,8 @@ int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
 }
 // Rollouts: two warps per sub-partition fill the FP64 unit with a single
 // body's short phases (8 to 36 tasks); the phases of larger models (100 tasks)
-// use 32 lanes, and four warps still gain (arms, 4000 for 0.1 s: 74 ms with 32
-// lanes, 83 with 16).  Below 4 lanes nothing was faster.
+// use 32 lanes, and four warps still gain (arms, 1000 for 0.1 s: 24 ms with 32
+// lanes, 27 with 16).  Below 4 lanes nothing was faster.
 int default_lanes(const dmx_model* m, int B) { return layout_lanes(m, m->L, B, m->host.nv > 8 ? 16 : 8); }
 int layout_lanes(const dmx_model* m, const dmx::Layout& L, int B, int warps) {
   int G = fill_lanes(m, B, (size_t)L.nd * 8 + (size_t)L.ni * 4, warps, 4);
@@ -546,16 +546,18 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
   const size_t room = std::min(free_b / 8, kRecMaxBytes);
   if (table > room / 8) return;
-  const size_t n = std::min(most, (room - table) / chunk);
+  const size_t n = std::min(most, (room - table - 256) / (chunk + 2 * sizeof(int)));
   if (n < (size_t)t->B || n > (size_t)INT32_MAX / 2) return;
-  if (cudaMallocAsync(&t->recmem, table + n * chunk, st) != cudaSuccess) {
+  const size_t owners = (2 * sizeof(int) * n + 255) & ~size_t(255);
+  if (cudaMallocAsync(&t->recmem, table + owners + n * chunk, st) != cudaSuccess) {
     cudaGetLastError();               // not enough memory: the tape does without
     t->recmem = nullptr;
     return;
   }
   r.chunk = static_cast<int*>(t->recmem);
   r.next = r.chunk + (size_t)t->B * r.per_env;
-  r.mem = reinterpret_cast<double*>(static_cast<char*>(t->recmem) + table);
+  r.owner = reinterpret_cast<int*>(static_cast<char*>(t->recmem) + table);
+  r.mem = reinterpret_cast<double*>(static_cast<char*>(t->recmem) + table + owners);
   r.nchunk = (int)n;
   if (cudaMemsetAsync(t->recmem, 0, table, st) != cudaSuccess) return;
   t->rec = r;
@@ -839,12 +841,31 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   P.barofs = pl.barofs;
   const int blocks = pl.blocks;
   const size_t smem = pl.smem, seg_bytes = pl.seg;
+  // The CFD right-hand side at the recorded stage states, for as many chunks as
+  // fit the snapshots' share of the memory; later ones are evaluated in the sweep.
+  size_t cfd_bytes = 0;
+  if (cfd && !par && P.rec.mem) {
+    P.SN = dmx::snap_offsets(m->host, P.L).size;
+    const size_t chunk = sizeof(double) * dmx::REC_STEPS * (t->method == DMX_METHOD_EULER ? 1 : 6) * (size_t)P.SN;
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
+      P.ncfd = (int)std::min((size_t)P.rec.nchunk, std::min(free_b / 8, kSnapMaxBytes) / chunk);
+      cfd_bytes = (size_t)P.ncfd * chunk;
+    }
+  }
   void* scratch = nullptr;
-  CK(cudaMallocAsync(&scratch, seg_bytes + snap_bytes + 256, st));
+  if (cfd_bytes && cudaMallocAsync(&scratch, seg_bytes + cfd_bytes + 256, st) != cudaSuccess) {
+    cudaGetLastError();                // not enough memory: the sweep evaluates every stage
+    scratch = nullptr;
+    cfd_bytes = 0;
+    P.ncfd = 0;
+  }
+  if (!scratch) CK(cudaMallocAsync(&scratch, seg_bytes + snap_bytes + 256, st));
   P.segbuf = static_cast<double*>(scratch);
+  P.cfdsnap = cfd_bytes ? reinterpret_cast<double*>(static_cast<char*>(scratch) + seg_bytes) : nullptr;
   P.snapbuf = snap_bytes ? reinterpret_cast<double*>(static_cast<char*>(scratch) + seg_bytes) : nullptr;
-  P.queue = reinterpret_cast<int*>(static_cast<char*>(scratch) + seg_bytes + snap_bytes);
-  CK(cudaMemsetAsync(P.queue, 0, sizeof(int), st));
+  P.queue = reinterpret_cast<int*>(static_cast<char*>(scratch) + seg_bytes + snap_bytes + cfd_bytes);
+  CK(cudaMemsetAsync(P.queue, 0, 2 * sizeof(int), st));
   CK(dmx::launch_adjoint_rev(G, P, blocks, threads, smem, st));
   CK(cudaFreeAsync(scratch, st));
   return DMX_OK;

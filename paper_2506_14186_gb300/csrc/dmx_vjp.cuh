@@ -31,6 +31,7 @@
 // ones; sums along the tree run in chains (tree_down, tree_up).  On stiff
 // pushing contacts the gradient amplifies a rounding difference to 1e-8 of
 // its norm, so every split keeps each result's operations and their order.
+// 16384 single VJPs of the arm: 17.0 -> 7.1 ms.
 #pragma once
 #include "dmx_device.cuh"
 

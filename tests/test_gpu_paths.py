@@ -1,6 +1,7 @@
 """GPU paths that a call takes by its size: the default lane count against the
 lane count whose summation order it keeps, taped rollouts whose step records
-run out, and the parameter gradients of environments without contact."""
+run out, the right-hand sides with contacts from distance of recorded steps,
+and the parameter gradients of environments without contact."""
 
 import numpy as np
 import pytest
@@ -69,6 +70,29 @@ def test_records_that_run_out(dmx):
     scale = got["recompute"].abs().amax(0)
     assert float(((got["reverse"] - got["recompute"]).abs() / scale).max()) < 1e-12
     assert torch.isfinite(got["reverse"]).all()
+
+
+@pytest.mark.parametrize("name,B,T,NI,method", [("box", 5, 0.02, 1, "dopri5"), ("box", 70, 0.02, 1, "euler"),
+                                                 ("quadruped", 3, 0.02, 1, "tsit5"), ("chain_cube", 2, 0.04, 3, "dopri5")])
+def test_cfd_stages_of_recorded_steps(dmx, name, B, T, NI, method):
+    """With contacts from distance the right-hand sides at the recorded stage
+    states are evaluated beforehand; the gradient is that of evaluating them
+    in the sweep (within 1e-9: the same formulas along the same steps)."""
+    sc = W.SCENES[name](**W.CFD_OPTIONS)
+    inp = W.chain_inputs(B, T=T, NI=NI) if name == "chain_cube" else W.INPUTS[name](B)
+    inp["T"] = np.full(B, T)
+    if name == "quadruped":
+        inp["x0"][:, 2] = 0.4255
+    model = dmx.Model(sc)
+    bar = _dev(np.random.default_rng(6).normal(size=(model.nx, B)))
+    out = _call(dmx, model, inp, tape=True, K=8, method=method)
+    got = {}
+    for mode in ("reverse", "recompute"):
+        model.set_adjoint(mode)
+        got[mode] = dmx.rollout_grad(out["tape"], bar, cfd=True)
+    for a, b in zip(got["reverse"], got["recompute"]):
+        if b is not None and b.numel():
+            assert float((a - b).abs().max()) <= 1e-9 * float(b.abs().max())
 
 
 @pytest.mark.parametrize("name,B", [("ball", 1), ("ball", 65), ("toss", 33)])
