@@ -103,7 +103,8 @@ struct DevModel {
 // known to the compiler.  The functions over a model type then lose their
 // loops over bodies and levels, joint types, index reads and geom pairs, and
 // unroll the sums over six dofs (a right-hand side runs 13 instructions per
-// FP64 instruction otherwise).  The table members only hide the base's; they
+// FP64 instruction otherwise): 4096 box pushes 180 -> 135 ms, 20001 tosses 212 ->
+// 155, 2048 toss gradients 127 -> 102.  The table members only hide the base's; they
 // hold no data, and a DevModel is read through this type by a cast.
 template <int V>
 struct ConstTab {
@@ -118,7 +119,7 @@ struct OneBody : DevModel {
   ConstTab<1> b_anc, s_move;
 };
 // A model without geom pairs (the quadruped): the device code loses the
-// capsule-box and segment-pair contacts.
+// capsule-box and segment-pair contacts (3000 quadrupeds 283 -> 278 ms).
 struct PlaneOnly : DevModel {
   ConstTab<-1> p_g2;
 };
