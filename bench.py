@@ -521,7 +521,8 @@ def sysid_leg(dmx, dev, world=1, rank=0, B=4096, parity_envs=(0, 1)):
             "envs_per_gpu": B, "params": ["t_c", "phi_d", "d_o", "d_w", "width", "midpoint", "mu", "mass", "side"],
             "grad_rollouts_per_s": B * world / t, "s": t, "env_steps": int(out["nsteps"].sum().item()),
             "p_bar_sum": ps.cpu().numpy().tolist(), "reduction": "in-library row sums, all-reduce over ranks",
-            "kernel": "k_adjoint_rev (with parameter cotangents); k_adjoint where no contact was met", "parity_vs_oracle": parity}
+            "kernel": "k_adjoint_rev (with parameter cotangents); k_adjoint where no contact was met",
+            "parity_vs_oracle": parity}
 
 
 def _grad_parity(m, out, xT_bar, gx, gu, inp, scene, envs):

@@ -249,7 +249,9 @@ dmx_status dmx_rollout_grad_otd(dmx_model* m, const dmx_otd_args* a, void* strea
  *     recomputed (K steps x 6 stages per resident environment, used when it
  *     fits 1/8 of the free device memory and 8 GiB), so each stage is
  *     evaluated once; otherwise as DMX_ADJ_RECOMPUTE.  Segments whose steps the
- *     tape kept with their snapshots are not recomputed at all.  An environment whose
+ *     tape kept with their snapshots are not recomputed at all.  With
+ *     cfd their F~ is evaluated for all recorded steps before the sweep (its
+ *     snapshots within the same 1/8 and 8 GiB).  An environment whose
  *     right-hand side overflowed the row workspace during the adjoint gets
  *     NaN in x0_bar.
  *   DMX_ADJ_RECOMPUTE: the same reverse mode, evaluating each stage's
