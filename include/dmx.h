@@ -271,10 +271,13 @@ void dmx_tape_free(dmx_tape* t);
 dmx_status dmx_tape_read(const dmx_tape* t, double* hlog, int32_t* nsteps, double* ckpt, int32_t* dims,
                          void* stream);
 
-/* Lanes per environment used for (model, B, forward/gradient) when
- * dmx_rollout_args.lanes == 0: the value recorded by dmx_set_lanes (the
- * autotuner's choice), else a default that gives every SM sub-partition a
- * warp of FP64 work.  `stream` is unused (may be NULL). */
+/* Lanes per environment whose results a call with dmx_rollout_args.lanes == 0
+ * has for (model, B, forward/gradient), bit for bit: the value recorded by
+ * dmx_set_lanes (the autotuner's choice), which such a call also runs on, else
+ * the fewest that give every SM sub-partition a warp of FP64 work.  Without a
+ * recorded value the call sums its error norms in the order of these lanes but
+ * runs on as many as an SM's shared memory and registers hold to advantage;
+ * naming them runs on them.  `stream` is unused (may be NULL). */
 dmx_status dmx_autotune(dmx_model* m, int32_t B, int32_t grad, int32_t* lanes, void* stream);
 /* Records the lanes per environment for (model, B, kind): kind 0 = forward
  * rollout, 1 = taped rollout, 2 = reverse-mode adjoint kernel; lanes in

@@ -663,10 +663,15 @@ int tuned_lanes(dmx_model* m, int B, int grad, int* red) {
   return default_lanes(m, B);
 }
 
+// The lane count that, named in a call, gives the bits of a call that names
+// none: the recorded one, else the one whose summation order it follows (the
+// lanes it runs on, default_lanes, would sum the error norm in another order).
 extern "C" dmx_status dmx_autotune(dmx_model* m, int32_t B, int32_t grad, int32_t* lanes, void* stream) {
   (void)stream;
   if (!m || B < 0) return dmx_fail(DMX_ERR_INVALID, "bad argument");
-  if (lanes) *lanes = tuned_lanes(m, B, grad, nullptr);
+  int red;
+  tuned_lanes(m, B, grad, &red);
+  if (lanes) *lanes = red;
   return DMX_OK;
 }
 
