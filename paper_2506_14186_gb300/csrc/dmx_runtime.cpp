@@ -498,6 +498,21 @@ dmx_status run_rollout(dmx_model* m, const RolloutParams& P0, int form, int G, c
 }
 
 
+// Device memory that an allocation here can have: what the device reports as
+// free and what the stream-ordered pool holds unused (kept for the next call,
+// so the same call gets the same shares whatever ran before it).
+static size_t free_memory(const dmx_model* m) {
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
+  cudaMemPool_t pool;
+  uint64_t reserved = 0, used = 0;
+  if (cudaDeviceGetMemPool(&pool, m->device) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && reserved > used)
+    free_b += (size_t)(reserved - used);
+  return free_b;
+}
+
 static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const double* ctrl, const double* T,
                             cudaStream_t st, dmx_tape** out) {
   dmx_tape* t = new dmx_tape();
@@ -541,11 +556,9 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   const size_t chunk = sizeof(double) * dmx::REC_STEPS * (size_t)r.stride;
   const size_t table = (sizeof(int) * ((size_t)t->B * r.per_env + 1) + 255) & ~size_t(255);
   const size_t most = (size_t)t->B * std::min(r.per_env, 512 / dmx::REC_STEPS);
-  size_t free_b = 0, total_b = 0;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;   // a graph would own the memory for good
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return;
-  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return;
-  const size_t room = std::min(free_b / 8, kRecMaxBytes);
+  const size_t room = std::min(free_memory(m) / 8, kRecMaxBytes);
   if (table > room / 8) return;
   const size_t n = std::min(most, (room - table - 256) / (chunk + 2 * sizeof(int)));
   if (n < (size_t)t->B || n > (size_t)INT32_MAX / 2) return;
@@ -836,9 +849,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   size_t snap_bytes = 0;
   if (mode == DMX_ADJ_REVERSE && !cfd && plan(dmx::make_layout_adj(m->host, L.rcap), true, pl)) {
     snap_bytes = sizeof(double) * (size_t)pl.blocks * gpb * t->K * nsnap * (size_t)P.SN;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || snap_bytes > free_b / 8 || snap_bytes > kSnapMaxBytes)
-      snap_bytes = 0;
+    if (snap_bytes > std::min(free_memory(m) / 8, kSnapMaxBytes)) snap_bytes = 0;
   }
   if (snap_bytes == 0 && !plan(L, false, pl))
     return dmx_fail(DMX_ERR_INVALID, "adjoint workspace of " + std::to_string(G) + " lanes/env does not fit shared memory");
@@ -853,11 +864,8 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   if (cfd && !par && P.rec.mem) {
     P.SN = dmx::snap_offsets(m->host, P.L).size;
     const size_t chunk = sizeof(double) * dmx::REC_STEPS * (t->method == DMX_METHOD_EULER ? 1 : 6) * (size_t)P.SN;
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess) {
-      P.ncfd = (int)std::min((size_t)P.rec.nchunk, std::min(free_b / 8, kSnapMaxBytes) / chunk);
-      cfd_bytes = (size_t)P.ncfd * chunk;
-    }
+    P.ncfd = (int)std::min((size_t)P.rec.nchunk, std::min(free_memory(m) / 8, kSnapMaxBytes) / chunk);
+    cfd_bytes = (size_t)P.ncfd * chunk;
   }
   void* scratch = nullptr;
   if (cfd_bytes && cudaMallocAsync(&scratch, seg_bytes + cfd_bytes + 256, st) != cudaSuccess) {

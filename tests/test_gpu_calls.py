@@ -56,3 +56,63 @@ def test_the_lanes_a_model_names_give_the_same_bits(dmx, name, B, T, recorded):
     b = _call(dmx, model, inp, lanes=model.lanes(B))
     for k in ("xT", "nsteps", "nrej", "status"):
         assert torch.equal(a[k], b[k]), k
+
+
+# ------------------------------------------------------------------ step records: memory
+_MEMORY = r'''
+import ctypes, gc, re, sys
+import numpy as np, torch
+from paper_2506_14186_gb300 import workloads as W
+import paper_2506_14186_gb300 as dmx
+
+rt = ctypes.CDLL(next(l.split()[-1] for l in open("/proc/self/maps") if re.search(r"libcudart\.so", l)))
+torch.zeros(1, device="cuda")
+pool = ctypes.c_void_p()
+assert rt.cudaDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+
+def used():                                     # bytes of the device's default pool in use (attribute 7)
+    torch.cuda.synchronize()
+    v = ctypes.c_uint64()
+    assert rt.cudaMemPoolGetAttribute(pool, 7, ctypes.byref(v)) == 0
+    return v.value
+
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+def dev(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+def tape(model, inp, T, **kw):
+    B = len(inp["x0"])
+    ctrl = None if inp["ctrl"] is None else dev(np.transpose(inp["ctrl"], (1, 2, 0)))
+    return dmx.rollout(model, dev(inp["x0"].T), dev(np.full(B, T)), ctrl=ctrl, NI=inp["NI"], max_steps=2000,
+                       tape=True, **kw)["tape"]
+
+GiB = 1 << 30
+'''
+
+
+def _run(code):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _MEMORY + code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
+
+
+def test_records_do_not_depend_on_what_the_pool_keeps_unused(dmx):
+    """With little memory free, a tape gets the same room as the one freed before
+    it: the pool's unused bytes count as free."""
+    _run(r'''
+model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(20000)
+filler = torch.empty(free() - 80 * GiB, dtype=torch.uint8, device="cuda")
+sizes = []
+for _ in range(3):
+    t = tape(model, inp, 0.001)
+    sizes.append(used())
+    del t; gc.collect()
+    assert used() < GiB
+assert max(sizes) - min(sizes) < GiB // 8, sizes
+''')
