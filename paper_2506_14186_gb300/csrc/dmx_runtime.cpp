@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -547,6 +548,18 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
 // the writes (118 KB an arm's step): forward and adjoint of 2048 arms 249 -> 171
 // ms, of 2048 tosses 167 -> 133.
 constexpr size_t kRecMaxBytes = size_t(24) << 30;
+// All live tapes of a device together hold twice that at most (a loop's next
+// rollout runs while the previous tape is still alive); further ones go without.
+// Counted on the host: a freed tape's bytes are given up in stream order.
+constexpr size_t kRecLiveBytes = 2 * kRecMaxBytes;
+constexpr int kMaxDevices = 64;
+static std::atomic<size_t> g_rec_live[kMaxDevices];
+static void free_records(dmx_tape* t) {
+  if (!t->recmem) return;
+  cudaFreeAsync(t->recmem, t->stream);
+  g_rec_live[t->model_device] -= t->recbytes;
+  t->recmem = nullptr;
+}
 static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   const int stages = t->method == DMX_METHOD_EULER ? 1 : 6;
   dmx::StepRecords r{};
@@ -558,13 +571,22 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   const size_t most = (size_t)t->B * std::min(r.per_env, 512 / dmx::REC_STEPS);
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;   // a graph would own the memory for good
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return;
-  const size_t room = std::min(free_memory(m) / 8, kRecMaxBytes);
+  if (m->device < 0 || m->device >= kMaxDevices) return;
+  const size_t live = g_rec_live[m->device];
+  const size_t room = std::min({free_memory(m) / 8, kRecMaxBytes, kRecLiveBytes - std::min(live, kRecLiveBytes)});
   if (table > room / 8) return;
   const size_t n = std::min(most, (room - table - 256) / (chunk + 2 * sizeof(int)));
   if (n < (size_t)t->B || n > (size_t)INT32_MAX / 2) return;
   const size_t owners = (2 * sizeof(int) * n + 255) & ~size_t(255);
-  if (cudaMallocAsync(&t->recmem, table + owners + n * chunk, st) != cudaSuccess) {
+  t->recbytes = table + owners + n * chunk;
+  t->model_device = m->device;
+  if ((g_rec_live[m->device] += t->recbytes) > kRecLiveBytes) {   // another thread's tape took the room meanwhile
+    g_rec_live[m->device] -= t->recbytes;
+    return;
+  }
+  if (cudaMallocAsync(&t->recmem, t->recbytes, st) != cudaSuccess) {
     cudaGetLastError();               // not enough memory: the tape does without
+    g_rec_live[m->device] -= t->recbytes;
     t->recmem = nullptr;
     return;
   }
@@ -580,7 +602,7 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
 extern "C" void dmx_tape_free(dmx_tape* t) {
   if (!t) return;
   cudaFreeAsync(t->mem, t->stream);   // ordered after the work queued on the tape's stream
-  if (t->recmem) cudaFreeAsync(t->recmem, t->stream);
+  free_records(t);
   delete t;
 }
 

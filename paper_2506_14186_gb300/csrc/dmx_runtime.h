@@ -45,6 +45,8 @@ struct dmx_tape {
   int* n = nullptr;         // [B] accepted steps
   int* touched = nullptr;   // [B] an accepted step met a contact
   void* recmem = nullptr;   // step records (dmx_record.h), their table and counter, or null
+  size_t recbytes = 0;
+  int model_device = 0;
   dmx::StepRecords rec{};
   cudaStream_t stream = nullptr;   // allocation stream (stream-ordered free)
 };

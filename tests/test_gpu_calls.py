@@ -116,3 +116,16 @@ for _ in range(3):
     assert used() < GiB
 assert max(sizes) - min(sizes) < GiB // 8, sizes
 ''')
+
+
+def test_live_tapes_hold_a_bounded_amount_of_records(dmx):
+    """Tapes that want 24 GiB of step records each hold 48 GiB together at most
+    (a tape's own arrays: below 1 GiB here)."""
+    _run(r'''
+model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(20000)
+tapes = [tape(model, inp, 0.001) for _ in range(4)]
+assert used() < (48 + 4) * GiB, used() / GiB
+del tapes[0]; gc.collect()
+tapes.append(tape(model, inp, 0.001))           # the room of a freed tape can be had again
+assert 46 * GiB < used() < (48 + 4) * GiB, used() / GiB
+''')
