@@ -542,11 +542,13 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
 }
 
 // Step records for a tape: as many chunks as 512 steps of every environment
-// take, within an eighth of the free device memory and 24 GiB; none when that
-// is less than a chunk per environment, or the allocation fails.  With them
-// the adjoint has no segment to recompute (45 % of its time), for the price of
-// the writes (118 KB an arm's step): forward and adjoint of 2048 arms 249 -> 171
-// ms, of 2048 tosses 167 -> 133.
+// take, within an eighth of the free device memory and 24 GiB; none when they
+// could not hold a segment of every environment in flight (chunks go out as the
+// environments proceed, and a segment is used only if all of its chunks came;
+// of longer segments, as short rollouts have them, 64 steps), or the allocation
+// fails.  With them the adjoint has no segment to recompute (45 % of its time),
+// for the price of the writes (118 KB an arm's step): forward and adjoint of
+// 2048 arms 249 -> 171 ms, of 2048 tosses 167 -> 133.
 constexpr size_t kRecMaxBytes = size_t(24) << 30;
 // All live tapes of a device together hold twice that at most (a loop's next
 // rollout runs while the previous tape is still alive); further ones go without.
@@ -576,7 +578,10 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   const size_t room = std::min({free_memory(m) / 8, kRecMaxBytes, kRecLiveBytes - std::min(live, kRecLiveBytes)});
   if (table > room / 8) return;
   const size_t n = std::min(most, (room - table - 256) / (chunk + 2 * sizeof(int)));
-  if (n < (size_t)t->B || n > (size_t)INT32_MAX / 2) return;
+  const int K = std::min(t->K, 64);
+  const size_t segment = std::min(r.per_env, (K + dmx::REC_STEPS - 1) / dmx::REC_STEPS);
+  const size_t fit = (size_t)(m->smem_max + 1024) / ((size_t)m->L.nd * 8 + (size_t)m->L.ni * 4 + 256);
+  if (n < std::min((size_t)t->B, m->nsm * fit) * segment || n > (size_t)INT32_MAX / 2) return;
   const size_t owners = (2 * sizeof(int) * n + 255) & ~size_t(255);
   t->recbytes = table + owners + n * chunk;
   t->model_device = m->device;

@@ -129,3 +129,18 @@ del tapes[0]; gc.collect()
 tapes.append(tape(model, inp, 0.001))           # the room of a freed tape can be had again
 assert 46 * GiB < used() < (48 + 4) * GiB, used() / GiB
 ''')
+
+
+def test_no_records_that_complete_no_segment(dmx):
+    """Records that could not hold one segment of every environment in flight are
+    not kept (2048 arms, 2.5 GiB: 2800 chunks of 8 steps, 1368 in flight with
+    segments of 8 chunks)."""
+    _run(r'''
+model, inp = dmx.Model(W.SCENES["chain_cube"]()), W.chain_inputs(2048, T=0.001)
+filler = torch.empty(free() - 20 * GiB, dtype=torch.uint8, device="cuda")
+t = tape(model, inp, 0.001, K=64)
+assert used() < GiB // 2, used() / GiB
+del t; gc.collect()
+t = tape(model, inp, 0.001, K=8)                # one chunk a segment: kept
+assert used() > 2 * GiB, used() / GiB
+''')
