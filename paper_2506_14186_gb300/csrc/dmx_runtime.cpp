@@ -53,6 +53,24 @@ cudaError_t DevBuf::ensure(size_t n) {
   return e;
 }
 
+// Models of each device come and go (by = +-1).  While there are some, the
+// stream-ordered scratch of a call stays cached in the device's default pool for
+// the next one (the driver hands it to any allocation of this process that finds
+// too little free).  With the last model it goes back to the device: what is
+// freed by then at once, the rest when the device is next waited for.
+constexpr int kMaxDevices = 64;
+static void count_models(int device, int by) {
+  static std::mutex mu;
+  static int n[kMaxDevices] = {};
+  cudaMemPool_t pool;
+  if (device >= kMaxDevices || cudaDeviceGetDefaultMemPool(&pool, device) != cudaSuccess) return;
+  std::lock_guard<std::mutex> lk(mu);
+  n[device] += by;
+  uint64_t keep = n[device] > 0 ? ~0ull : 0ull;
+  cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+  if (!keep) cudaMemPoolTrimTo(pool, 0);
+}
+
 // ------------------------------------------------------------------ model compiler
 static void quat_mat(const double* q0, double* R) {
   double n = std::sqrt(q0[0] * q0[0] + q0[1] * q0[1] + q0[2] * q0[2] + q0[3] * q0[3]);
@@ -271,14 +289,6 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   cudaDeviceProp prop;
   CK(cudaGetDeviceProperties(&prop, m->device));
   m->nsm = prop.multiProcessorCount;
-  {
-    // keep stream-ordered per-call scratch cached in the device's default pool
-    cudaMemPool_t pool;
-    if (cudaDeviceGetDefaultMemPool(&pool, m->device) == cudaSuccess) {
-      uint64_t thr = ~0ull;
-      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
-    }
-  }
   m->smem_max = (int)prop.sharedMemPerBlockOptin;
   if (cudaMalloc(&m->dev, sizeof(DevModel)) != cudaSuccess) { delete m; return dmx_fail(DMX_ERR_OOM, "model upload"); }
   CK(cudaMemcpy(m->dev, &m->host, sizeof(DevModel), cudaMemcpyHostToDevice));
@@ -320,6 +330,7 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   }
   for (int b = 0; b < m->host.nbody; ++b) m->invw[b] = invw[b];
   CK(cudaMemcpy(m->dev, &m->host, sizeof(DevModel), cudaMemcpyHostToDevice));
+  count_models(m->device, 1);
   *out = m;
   return DMX_OK;
 }
@@ -330,6 +341,7 @@ extern "C" void dmx_destroy_model(dmx_model* m) {
   cudaGetDevice(&cur);
   cudaSetDevice(m->device);
   cudaFree(m->dev);
+  count_models(m->device, -1);
   cudaSetDevice(cur);
   delete m;
 }
@@ -554,7 +566,6 @@ constexpr size_t kRecMaxBytes = size_t(24) << 30;
 // rollout runs while the previous tape is still alive); further ones go without.
 // Counted on the host: a freed tape's bytes are given up in stream order.
 constexpr size_t kRecLiveBytes = 2 * kRecMaxBytes;
-constexpr int kMaxDevices = 64;
 static std::atomic<size_t> g_rec_live[kMaxDevices];
 static void free_records(dmx_tape* t) {
   if (!t->recmem) return;

@@ -144,3 +144,17 @@ del t; gc.collect()
 t = tape(model, inp, 0.001, K=8)                # one chunk a segment: kept
 assert used() > 2 * GiB, used() / GiB
 ''')
+
+
+def test_the_last_model_gives_back_the_memory(dmx):
+    """What the pool keeps of freed tapes goes back to the device with the last model."""
+    _run(r'''
+before = free()
+model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(20000)
+other = dmx.Model(W.SCENES["ball"]())
+t = tape(model, inp, 0.001)
+assert before - free() > 16 * GiB
+del t, model; gc.collect()
+del other; gc.collect()
+assert before - free() < GiB, (before - free()) / GiB
+''')
