@@ -307,7 +307,37 @@ static cudaError_t launch_adjoint_rev_m(const AdjParams& P, int blocks, int thre
   return par ? launch_adjoint_rev_g<G, true, DevModel>(P, blocks, threads, smem, st)
              : launch_adjoint_rev_g<G, false, DevModel>(P, blocks, threads, smem, st);
 }
+// cfdofs[e] = steps of kept segments (those that end within the records) over the
+// environments before e, cfdofs[B] of all: the recorded steps of k_cfd_stages
+// without gaps, whatever their spread over the environments.  One block.
+__global__ void __launch_bounds__(1024) k_cfd_offsets(const __grid_constant__ AdjParams P) {
+  __shared__ int part[1024];
+  const int t = threadIdx.x, per = (P.B + 1023) / 1024;
+  const int e0 = min(t * per, P.B), e1 = min(e0 + per, P.B);
+  auto kept = [&](int e) {
+    const int N = P.tape_n[e];
+    return N <= P.rec.steps ? N : P.rec.steps - P.rec.steps % P.K;
+  };
+  int s = 0;
+  for (int e = e0; e < e1; ++e) s += kept(e);
+  part[t] = s;
+  __syncthreads();
+  for (int o = 1; o < 1024; o <<= 1) {
+    const int x = t >= o ? part[t - o] : 0;
+    __syncthreads();
+    part[t] += x;
+    __syncthreads();
+  }
+  int at = part[t] - s;
+  for (int e = e0; e < e1; ++e) { P.cfdofs[e] = at; at += kept(e); }
+  if (t == 1023) P.cfdofs[P.B] = part[t];
+}
 cudaError_t launch_adjoint_rev(int G, const AdjParams& P, int blocks, int threads, size_t smem, cudaStream_t st) {
+  if (P.cfdsnap) {
+    k_cfd_offsets<<<1, 1024, 0, st>>>(P);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   switch (G) {
     case 2: return P.p_bar ? cudaErrorInvalidValue : launch_adjoint_rev_g<2, false, DevModel>(P, blocks, threads, smem, st);
     case 4: return P.p_bar ? cudaErrorInvalidValue : launch_adjoint_rev_g<4, false, DevModel>(P, blocks, threads, smem, st);

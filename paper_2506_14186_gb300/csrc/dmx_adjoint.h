@@ -26,8 +26,9 @@ struct AdjParams {
   double* snapbuf;        // reverse mode: per group, K steps x (S - 1) stage snapshots of SN doubles (or null)
   int SN;                 // doubles per snapshot
   StepRecords rec;        // records of the taped rollout
-  double* cfdsnap;        // with cfd: snapshots of F~ at the recorded stage states ([ncfd] chunks), or null
+  double* cfdsnap;        // with cfd: snapshots of F~ at the stage states of ncfd recorded steps, or null
   int ncfd;
+  int* cfdofs;            // [B + 1] first of an environment's steps among them (k_cfd_offsets)
   int kind;               // MODEL_* type of the kernels (OneBody: 8, 16, 32 lanes, PlaneOnly: 16, 32)
   int per, barofs;        // reverse mode: doubles per environment, offset of the cotangent workspace
   double* p_bar;          // [np][B] model-parameter gradients, or null

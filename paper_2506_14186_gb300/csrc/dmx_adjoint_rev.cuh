@@ -149,10 +149,12 @@ __device__ int rk_step_vjp(const Grp<G>& g, const MD& m, const Ws& w, const WsB&
   return st;
 }
 
-// Snapshots of F~ at the stage states of step n (k_cfd_stages), or null.
+// Snapshots of F~ at the stage states of step n of a kept segment (k_cfd_stages),
+// or null.
 __device__ __forceinline__ const double* cfd_snaps(const AdjParams& P, int env, int n, int stages) {
-  const int k = n / REC_STEPS, c = P.rec.chunk[(size_t)env * P.rec.per_env + k] - 1;
-  return c >= 0 && c < P.ncfd ? P.cfdsnap + ((size_t)c * REC_STEPS + (n - k * REC_STEPS)) * stages * P.SN : nullptr;
+  if (!P.cfdsnap) return nullptr;
+  const int i = P.cfdofs[env] + n;
+  return i < P.ncfd ? P.cfdsnap + (size_t)i * stages * P.SN : nullptr;
 }
 
 // F~ at the stage states of every recorded step, one step per group at a time:
@@ -173,23 +175,28 @@ __global__ void __launch_bounds__(32, 1) k_cfd_stages(const __grid_constant__ Ad
   const int nq = m.nq, nv = m.nv, nu = m.nu, mt = P.method, S = TAB(mt).S;
   double* qs = w.at(sL.qs); double* vs = w.at(sL.vs); double* qn = w.at(sL.qn); double* dq = w.at(sL.dq);
   double* u = w.at(sL.u);
-  const int total = min(*P.rec.next, P.ncfd) * REC_STEPS;
-  if (g.lane == 0) for (int k = 0; k < MASKW; ++k) w.i[sL.pmask + k] = 0;
-  g.sync();
+  const int total = min(P.cfdofs[P.B], P.ncfd);
   for (;;) {
     int it = 0;
     if (g.lane == 0) it = atomicAdd(P.queue + 1, 1);
     it = g.bcast(it, 0);
     if (it >= total) break;
-    const int c = it / REC_STEPS, env = P.rec.owner[2 * c];
-    const int n = P.rec.owner[2 * c + 1] * REC_STEPS + (it - c * REC_STEPS);
-    if (n >= P.tape_n[env]) continue;
-    const double* row = P.rec.mem + (size_t)it * P.rec.stride + (S - 1) * P.rec.snap;
+    int env = 0, hi = P.B;             // the environment with cfdofs[env] <= it < cfdofs[env + 1]
+    while (hi - env > 1) {
+      const int mid = (env + hi) >> 1;
+      if (P.cfdofs[mid] <= it) env = mid; else hi = mid;
+    }
+    const int n = it - P.cfdofs[env];
+    const double* rec = step_record(P.rec, env, n);
+    const double* row = rec + (S - 1) * P.rec.snap;
     const double* vst = row + nq;
     const double h = P.hlog[(size_t)n * P.B + env];
     const int kn = rev_interval(P.T[env], P.NI, row[nq + 7 * nv]);
     DMX_TASKS(i, nq) qn[i] = row[i];
     DMX_TASKS(a, nu) u[a] = P.ctrl[((size_t)kn * nu + a) * P.B + env];
+    // each step's Newton searches start from F's recorded active set, not from
+    // what the group evaluated before: a function of the step alone
+    DMX_TASKS(k, MASKW) w.i[sL.pmask + k] = reinterpret_cast<const int*>(rec)[P.rec.active + k];
     g.sync();
     for (int s = 0; s <= S - 2; ++s) {
       const unsigned mq = TAB(mt).nzq[s];
@@ -254,8 +261,7 @@ __global__ void __launch_bounds__(32, 1) k_adjoint_rev(const __grid_constant__ A
     for (int c = N > 0 ? (N - 1) / P.K : -1; c >= 0; --c) {
       const int n0 = c * P.K, n1 = min(n0 + P.K, N);
       // the forward pass kept this segment's steps: nothing to recompute
-      bool kept = P.rec.mem != nullptr;
-      for (int k = n0 / REC_STEPS; kept && k <= (n1 - 1) / REC_STEPS; ++k) kept = P.rec.chunk[(size_t)env * P.rec.per_env + k] > 0;
+      const bool kept = n1 <= P.rec.steps;
       if (!kept) {
       // ---- forward recompute of the segment from checkpoint c: q_n, V_0..V_5, t_n per step
       const double* ck = P.ckpt + (size_t)c * (nx + 1) * P.B;

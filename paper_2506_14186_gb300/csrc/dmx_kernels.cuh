@@ -70,7 +70,7 @@ __device__ void env_start(const Grp<G>& g, const MD& m, const Ws& w, const Rollo
   if (bad) { s.st = ENV_NONFINITE; s.done = 1; return; }
   if (m.nu) load_ctrl(g, m, w, P, env, 0);
   const int st = rhs(g, m, w, qn, vn, w.at(L.u), false, w.at(L.ka));
-  if (double* r = claim_record(g, P.rec, env, 0)) snap_save(g, m, w, r, st);
+  if (double* r = step_record(P.rec, env, 0)) snap_save(g, m, w, r, st);
   if (P.touched && g.lane == 0) P.touched[env] = w.i[L.slotrow + m.nslot] > 0;
   if (st != ENV_OK) { s.st = st; s.done = 1; }
 }
@@ -91,8 +91,8 @@ __device__ void env_attempt(const Grp<G>& g, const MD& m, const Ws& w, const Rol
   const int mt = P.method;
   // records of a taped rollout: stages 1 .. S - 2 belong to this step, the
   // last one is stage 0 of the next (a rejected attempt's are overwritten)
-  double* rec = claim_record(g, P.rec, env, s.nacc);
-  double* rec1 = rec ? claim_record(g, P.rec, env, s.nacc + 1) : nullptr;
+  double* rec = step_record(P.rec, env, s.nacc);
+  double* rec1 = step_record(P.rec, env, s.nacc + 1);
   const int S = TAB(mt).S;
   bool contact = false;                // some stage includes a contact
   const double err = rk_attempt(g, m, w, w.at(L.u), ht, mt, P.rtol, P.atol, P.red, &stage_st, [&](int st, int r) {

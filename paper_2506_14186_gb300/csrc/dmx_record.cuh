@@ -40,32 +40,11 @@ __device__ void snap_save(const Grp<G>& g, const MD& m, const Ws& w, double* dst
   DMX_TASKS(i, nr) di[3 + m.nslot + i] = w.i[L.rowid + i];
   DMX_TASKS(i, MASKW) di[3 + m.nslot + L.rcap + i] = w.i[L.amask + i];
 }
-// Record of step n of an environment, null when there is none.
+// Record of step n of an environment, null when there is none.  A step's
+// records of all environments lie side by side: environments proceed at about
+// the same pace, so what is written at a time spans few pages.
 __device__ __forceinline__ double* step_record(const StepRecords& r, int env, int n) {
-  const int k = n / REC_STEPS;
-  const int c = k < r.per_env ? r.chunk[(size_t)env * r.per_env + k] : 0;
-  return c > 0 ? r.mem + ((size_t)(c - 1) * REC_STEPS + (n - k * REC_STEPS)) * r.stride : nullptr;
-}
-// The same while the rollout runs: the first request for a chunk takes the
-// next free one.
-template <int G>
-__device__ double* claim_record(const Grp<G>& g, const StepRecords& r, int env, int n) {
-  if (!r.mem) return nullptr;
-  const int k = n / REC_STEPS;
-  if (k >= r.per_env) return nullptr;
-  int c = 0;
-  if (g.lane == 0) {
-    int* p = r.chunk + (size_t)env * r.per_env + k;
-    c = *p;
-    if (c == 0) {
-      c = atomicAdd(r.next, 1);
-      c = c < r.nchunk ? c + 1 : -1;
-      *p = c;
-      if (c > 0) { r.owner[2 * (c - 1)] = env; r.owner[2 * (c - 1) + 1] = k; }
-    }
-  }
-  c = g.bcast(c, 0);
-  return c > 0 ? r.mem + ((size_t)(c - 1) * REC_STEPS + (n - k * REC_STEPS)) * r.stride : nullptr;
+  return n < r.steps ? r.mem + ((size_t)n * r.B + env) * r.stride : nullptr;
 }
 
 }  // namespace dmx

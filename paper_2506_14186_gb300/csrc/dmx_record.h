@@ -2,15 +2,15 @@
 // would otherwise evaluate again.  One record per accepted step: the snapshots
 // of its S - 1 stage right-hand sides (the part of the workspace that the VJP
 // reads), then the step's row (q_n, the stage velocities V_0..V_6, t_n).
-// Records come in chunks of REC_STEPS steps, handed out while the rollout runs
-// (the accepted steps are not known before); an environment that finds none
-// left goes on without, and the adjoint recomputes those segments.
+// Every environment has records for its first `steps` steps; the adjoint
+// recomputes the segments beyond.  A kept and a recomputed segment differ in the
+// last bits where a contact row lies at the edge of the active set (the start of
+// the Newton search decides there), so which ones are kept depends on the step
+// and the size of the buffer alone, never on the order in which environments run.
 #pragma once
 #include "dmx_model.h"
 
 namespace dmx {
-
-constexpr int REC_STEPS = 8;
 
 // Offsets (doubles) of one stage snapshot: the part of a right-hand-side
 // workspace that its VJP reads (poses .. geom frames, the Cholesky factor of
@@ -34,15 +34,18 @@ DMX_HD inline SnapOff snap_offsets(const DevModel& m, const Layout& L) {
   o.size = (o.oi + (nints + 1) / 2 + 1) & ~1;
   return o;
 }
+// Offset (ints) of the final active set in a snapshot.
+DMX_HD inline int snap_active(const DevModel& m, const Layout& L) {
+  return 2 * snap_offsets(m, L).oi + 3 + m.nslot + L.rcap;
+}
 // Doubles of a step's row: q_n, the stage velocities V_0..V_6, t_n.
 DMX_HD inline int rev_row_doubles(const DevModel& m) { return m.nq + 7 * m.nv + 1; }
 
 struct StepRecords {
-  double* mem;              // [nchunk][REC_STEPS][stride], or null: no records
-  int* chunk;               // [B][per_env]: 0 not asked for, -1 none left, else chunk index + 1
-  int* next;                // chunks handed out
-  int* owner;               // [nchunk][2]: environment and place (step / REC_STEPS) of a chunk
-  int nchunk, per_env, stride, snap;   // capacity, table width, doubles per step, per snapshot
+  double* mem;              // [steps][B][stride], or null: no records
+  int steps, B;             // steps of every environment that have a record
+  int stride, snap;         // doubles per step, per snapshot
+  int active;               // offset (ints) of the final active set in a snapshot
 };
 
 }  // namespace dmx

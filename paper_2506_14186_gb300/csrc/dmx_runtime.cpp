@@ -553,14 +553,13 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
   return DMX_OK;
 }
 
-// Step records for a tape: as many chunks as 512 steps of every environment
-// take, within an eighth of the free device memory and 24 GiB; none when they
-// could not hold a segment of every environment in flight (chunks go out as the
-// environments proceed, and a segment is used only if all of its chunks came;
-// of longer segments, as short rollouts have them, 64 steps), or the allocation
-// fails.  With them the adjoint has no segment to recompute (45 % of its time),
-// for the price of the writes (118 KB an arm's step): forward and adjoint of
-// 2048 arms 249 -> 171 ms, of 2048 tosses 167 -> 133.
+// Step records for a tape: the first 512 steps of every environment (or as
+// many as it may take), within an eighth of the free device memory and 24 GiB;
+// whole segments where that is less, and none when not even one fits (longer
+// segments than 64 steps serve short rollouts only, and count as 64), or the
+// allocation fails.  With them the adjoint has no segment to recompute (45 % of
+// its time), for the price of the writes (118 KB an arm's step): forward and
+// adjoint of 2048 arms 249 -> 171 ms, of 2048 tosses 167 -> 133.
 constexpr size_t kRecMaxBytes = size_t(24) << 30;
 // All live tapes of a device together hold twice that at most (a loop's next
 // rollout runs while the previous tape is still alive); further ones go without.
@@ -578,23 +577,18 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   dmx::StepRecords r{};
   r.snap = dmx::snap_offsets(m->host, m->L).size;
   r.stride = (stages * r.snap + dmx::rev_row_doubles(m->host) + 1) & ~1;
-  r.per_env = (t->max_steps + dmx::REC_STEPS) / dmx::REC_STEPS;
-  const size_t chunk = sizeof(double) * dmx::REC_STEPS * (size_t)r.stride;
-  const size_t table = (sizeof(int) * ((size_t)t->B * r.per_env + 1) + 255) & ~size_t(255);
-  const size_t most = (size_t)t->B * std::min(r.per_env, 512 / dmx::REC_STEPS);
+  r.B = t->B;
+  const size_t step = sizeof(double) * (size_t)r.stride * t->B;   // of every environment
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;   // a graph would own the memory for good
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return;
   if (m->device < 0 || m->device >= kMaxDevices) return;
   const size_t live = g_rec_live[m->device];
   const size_t room = std::min({free_memory(m) / 8, kRecMaxBytes, kRecLiveBytes - std::min(live, kRecLiveBytes)});
-  if (table > room / 8) return;
-  const size_t n = std::min(most, (room - table - 256) / (chunk + 2 * sizeof(int)));
-  const int K = std::min(t->K, 64);
-  const size_t segment = std::min(r.per_env, (K + dmx::REC_STEPS - 1) / dmx::REC_STEPS);
-  const size_t fit = (size_t)(m->smem_max + 1024) / ((size_t)m->L.nd * 8 + (size_t)m->L.ni * 4 + 256);
-  if (n < std::min((size_t)t->B, m->nsm * fit) * segment || n > (size_t)INT32_MAX / 2) return;
-  const size_t owners = (2 * sizeof(int) * n + 255) & ~size_t(255);
-  t->recbytes = table + owners + n * chunk;
+  const int want = std::min(t->max_steps, 512);
+  r.steps = (int)std::min((size_t)want, room / step);
+  if (r.steps < want && t->K <= 64) r.steps -= r.steps % t->K;
+  if (r.steps < std::min({t->K, 64, want})) return;
+  t->recbytes = r.steps * step;
   t->model_device = m->device;
   if ((g_rec_live[m->device] += t->recbytes) > kRecLiveBytes) {   // another thread's tape took the room meanwhile
     g_rec_live[m->device] -= t->recbytes;
@@ -606,12 +600,7 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
     t->recmem = nullptr;
     return;
   }
-  r.chunk = static_cast<int*>(t->recmem);
-  r.next = r.chunk + (size_t)t->B * r.per_env;
-  r.owner = reinterpret_cast<int*>(static_cast<char*>(t->recmem) + table);
-  r.mem = reinterpret_cast<double*>(static_cast<char*>(t->recmem) + table + owners);
-  r.nchunk = (int)n;
-  if (cudaMemsetAsync(t->recmem, 0, table, st) != cudaSuccess) return;
+  r.mem = static_cast<double*>(t->recmem);
   t->rec = r;
 }
 
@@ -896,14 +885,14 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   P.barofs = pl.barofs;
   const int blocks = pl.blocks;
   const size_t smem = pl.smem, seg_bytes = pl.seg;
-  // The CFD right-hand side at the recorded stage states, for as many chunks as
+  // The CFD right-hand side at the recorded stage states, for as many steps as
   // fit the snapshots' share of the memory; later ones are evaluated in the sweep.
   size_t cfd_bytes = 0;
   if (cfd && !par && P.rec.mem) {
     P.SN = dmx::snap_offsets(m->host, P.L).size;
-    const size_t chunk = sizeof(double) * dmx::REC_STEPS * (t->method == DMX_METHOD_EULER ? 1 : 6) * (size_t)P.SN;
-    P.ncfd = (int)std::min((size_t)P.rec.nchunk, std::min(free_memory(m) / 8, kSnapMaxBytes) / chunk);
-    cfd_bytes = (size_t)P.ncfd * chunk;
+    const size_t step = sizeof(double) * nsnap * (size_t)P.SN;
+    P.ncfd = (int)std::min((size_t)t->B * P.rec.steps, std::min(free_memory(m) / 8, kSnapMaxBytes) / step);
+    cfd_bytes = P.ncfd ? P.ncfd * step + sizeof(int) * ((size_t)t->B + 1) : 0;
   }
   void* scratch = nullptr;
   if (cfd_bytes && cudaMallocAsync(&scratch, seg_bytes + cfd_bytes + 256, st) != cudaSuccess) {
@@ -915,6 +904,7 @@ static dmx_status run_reverse_adjoint(dmx_model* m, dmx_tape* t, dmx::AdjParams&
   if (!scratch) CK(cudaMallocAsync(&scratch, seg_bytes + snap_bytes + 256, st));
   P.segbuf = static_cast<double*>(scratch);
   P.cfdsnap = cfd_bytes ? reinterpret_cast<double*>(static_cast<char*>(scratch) + seg_bytes) : nullptr;
+  if (cfd_bytes) P.cfdofs = reinterpret_cast<int*>(P.cfdsnap + (size_t)P.ncfd * nsnap * P.SN);
   P.snapbuf = snap_bytes ? reinterpret_cast<double*>(static_cast<char*>(scratch) + seg_bytes) : nullptr;
   P.queue = reinterpret_cast<int*>(static_cast<char*>(scratch) + seg_bytes + snap_bytes + cfd_bytes);
   CK(cudaMemsetAsync(P.queue, 0, 2 * sizeof(int), st));

@@ -44,7 +44,7 @@ struct dmx_tape {
   double* T = nullptr;      // [B]
   int* n = nullptr;         // [B] accepted steps
   int* touched = nullptr;   // [B] an accepted step met a contact
-  void* recmem = nullptr;   // step records (dmx_record.h), their table and counter, or null
+  void* recmem = nullptr;   // step records (dmx_record.h), or null
   size_t recbytes = 0;
   int model_device = 0;
   dmx::StepRecords rec{};

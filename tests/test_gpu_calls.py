@@ -110,7 +110,8 @@ model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(20000)
 filler = torch.empty(free() - 80 * GiB, dtype=torch.uint8, device="cuda")
 sizes = []
 for _ in range(3):
-    t = tape(model, inp, 0.001)
+    t = tape(model, inp, 0.001, K=8)
+    assert used() > 6 * GiB, used() / GiB
     sizes.append(used())
     del t; gc.collect()
     assert used() < GiB
@@ -124,25 +125,26 @@ def test_live_tapes_hold_a_bounded_amount_of_records(dmx):
     _run(r'''
 model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(20000)
 tapes = [tape(model, inp, 0.001) for _ in range(4)]
-assert used() < (48 + 4) * GiB, used() / GiB
+full = used()
+assert 24 * GiB < full < (48 + 4) * GiB, full / GiB
 del tapes[0]; gc.collect()
+assert used() < full - 12 * GiB
 tapes.append(tape(model, inp, 0.001))           # the room of a freed tape can be had again
-assert 46 * GiB < used() < (48 + 4) * GiB, used() / GiB
+assert abs(used() - full) < GiB, (used() / GiB, full / GiB)
 ''')
 
 
 def test_no_records_that_complete_no_segment(dmx):
-    """Records that could not hold one segment of every environment in flight are
-    not kept (2048 arms, 2.5 GiB: 2800 chunks of 8 steps, 1368 in flight with
-    segments of 8 chunks)."""
+    """Records that could not hold one segment of every environment are
+    not kept (2048 arms, 2.5 GiB: 11 steps of 118 KB an arm)."""
     _run(r'''
 model, inp = dmx.Model(W.SCENES["chain_cube"]()), W.chain_inputs(2048, T=0.001)
 filler = torch.empty(free() - 20 * GiB, dtype=torch.uint8, device="cuda")
 t = tape(model, inp, 0.001, K=64)
 assert used() < GiB // 2, used() / GiB
 del t; gc.collect()
-t = tape(model, inp, 0.001, K=8)                # one chunk a segment: kept
-assert used() > 2 * GiB, used() / GiB
+t = tape(model, inp, 0.001, K=8)                # the first segment: kept
+assert used() > GiB, used() / GiB
 ''')
 
 
@@ -158,3 +160,51 @@ del t, model; gc.collect()
 del other; gc.collect()
 assert before - free() < GiB, (before - free()) / GiB
 ''')
+
+
+# ------------------------------------------------------------------ step records: results
+@pytest.mark.parametrize("cfd", [False, True])
+def test_repeated_calls_with_too_few_records(dmx, cfd):
+    """Capsules resting with contact rows at the edge of the active set: where the
+    Newton search starts decides their last bits, so a kept and a recomputed
+    segment differ there.  Which segments are kept when there is little memory
+    must not depend on scheduling: the same call gives the same bits again."""
+    _run(r'''
+cfd = %r
+model, inp = dmx.Model(W.SCENES["capsules"](**(W.CFD_OPTIONS if cfd else {}))), W.INPUTS["capsules"](2000)
+bar = dev(np.random.default_rng(8).normal(size=(model.nx, 2000)))
+filler = torch.empty(free() - 24 * GiB, dtype=torch.uint8, device="cuda")
+first = None
+for k in range(5):
+    t = tape(model, inp, 0.1, K=8, rtol=inp["rtol"], atol=inp["atol"], h0=inp["h0"])
+    n = t.read()[1]
+    g = dmx.rollout_grad(t, bar, cfd=cfd)[0]
+    assert used() > 2 * GiB and int(n.max()) > 64   # records, and more steps than they hold
+    del t; gc.collect()
+    assert torch.isfinite(g).all()
+    first = g if first is None else first
+    assert torch.equal(first, g), (k, int((first != g).any(0).sum()))
+''' % cfd)
+
+
+@pytest.mark.parametrize("B", [1, 3, 1500])
+def test_cfd_stages_over_uneven_step_counts(dmx, B):
+    """The recorded steps that are evaluated beforehand are numbered without gaps
+    over environments with many, few and no steps (a state that is not finite
+    takes none: its cotangent passes through)."""
+    import torch
+    model = dmx.Model(W.box_scene(**W.CFD_OPTIONS))
+    inp = W.box_push_inputs(B, seed=3, T=0.01)
+    inp["T"] = 0.012 * (1 + np.arange(B) % 7) / 7.0
+    if B > 1:
+        inp["x0"][1::5, 0] = np.nan
+    bar = _dev(np.random.default_rng(6).normal(size=(model.nx, B)))
+    out = _call(dmx, model, inp, tape=True, K=4)
+    got = {}
+    for mode in ("reverse", "recompute"):
+        model.set_adjoint(mode)
+        got[mode] = dmx.rollout_grad(out["tape"], bar, cfd=True)[0]
+    a, b = got["reverse"], got["recompute"]
+    assert torch.isfinite(b).all() and float((a - b).abs().max()) <= 1e-9 * float(b.abs().max())
+    if B > 1:
+        assert torch.equal(a[:, 1::5], bar[:, 1::5])
