@@ -330,6 +330,12 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   }
   for (int b = 0; b < m->host.nbody; ++b) m->invw[b] = invw[b];
   CK(cudaMemcpy(m->dev, &m->host, sizeof(DevModel), cudaMemcpyHostToDevice));
+  int threads;
+  size_t smem;
+  if (launch_config(m, 32, &threads, &smem)) {
+    const int warps = persistent_occupancy(32, m->kind, threads, smem);
+    if (warps > 0 && warps < (int)(prop.sharedMemPerMultiprocessor / (smem + prop.reservedSharedMemPerBlock))) m->warps = warps;
+  }
   count_models(m->device, 1);
   *out = m;
   return DMX_OK;
@@ -394,6 +400,8 @@ int reduction_lanes(const dmx_model* m, int B) {
   return G;
 }
 
+// Environments of `per` bytes of workspace that an SM's shared memory holds.
+static int sm_environments(const dmx_model* m, size_t per) { return (int)((size_t)(m->smem_max + 1024) / (per + 256)); }
 // Lanes for `per` bytes of workspace per environment: the most lanes (gmin at
 // least) that leave an SM at most `warps` warps of the environments it holds
 // (its share of the batch, or what its shared memory takes).  Fewer lanes leave
@@ -404,8 +412,7 @@ int reduction_lanes(const dmx_model* m, int B) {
 // 133 with 32; tosses, 20001 for 0.2 s: 171, 225, 303).
 int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
   const long long share = ((long long)B + m->nsm - 1) / m->nsm;
-  const long long fit = (long long)((size_t)(m->smem_max + 1024) / (per + 256));
-  const long long e = std::max(1LL, std::min(share, fit));
+  const long long e = std::max(1LL, std::min(share, (long long)sm_environments(m, per)));
   int G = 32;
   while (G > gmin && e * G > warps * 32) G >>= 1;
   return G;
@@ -414,7 +421,22 @@ int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
 // body's short phases (8 to 36 tasks); the phases of larger models (100 tasks)
 // use 32 lanes, and four warps still gain (arms, 1000 for 0.1 s: 24 ms with 32
 // lanes, 27 with 16).  Below 4 lanes nothing was faster.
-int default_lanes(const dmx_model* m, int B) { return layout_lanes(m, m->L, B, m->host.nv > 8 ? 16 : 8); }
+// `even`: environments of equal step counts (a fixed-step scheme).  They end
+// together, so what an SM has no registers for waits a whole round: fewer lanes
+// where that saves a round (billiards over 0.3 s: 2000 8.1 ms with 16 lanes, 15.6
+// with 32; 4096 11.9 with 8, 19.3 with 16; 16384 46.8, 55.9; capsules, 4096 over
+// 0.1 s: 10.8 with 16, 15.7 with 32; without a round saved, 10000 billiards, 34.6
+// with 8, 33.8 with 16).  Uneven environments refill the gaps and prefer the
+// lanes (2000 capsules with adaptive steps: 49 ms with 32, 63 with 16).
+int default_lanes(const dmx_model* m, int B, bool even) {
+  int G = layout_lanes(m, m->L, B, m->host.nv > 8 ? 16 : 8);
+  if (!even) return G;
+  const int share = (B + m->nsm - 1) / m->nsm, fit = sm_environments(m, (size_t)m->L.nd * 8 + (size_t)m->L.ni * 4);
+  auto rounds = [&](int g) { const int e = std::max(1, std::min(fit, m->warps * (32 / g))); return (share + e - 1) / e; };
+  int t; size_t s;
+  while (G > 4 && rounds(G / 2) < rounds(G) && launch_config(m, G / 2, &t, &s)) G >>= 1;
+  return G;
+}
 int layout_lanes(const dmx_model* m, const dmx::Layout& L, int B, int warps) {
   int G = fill_lanes(m, B, (size_t)L.nd * 8 + (size_t)L.ni * 4, warps, 4);
   int t; size_t s;
@@ -633,7 +655,8 @@ dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, b
   CK(cudaGetDevice(&cur));
   if (cur != m->device) return dmx_fail(DMX_ERR_INVALID, "model belongs to another device");
   int red = 0;
-  const int G = a->lanes ? a->lanes : tuned_lanes(m, a->B, 0, &red);
+  const bool even = a->form == DMX_FORM_PERSISTENT && a->method == DMX_METHOD_EULER;
+  const int G = a->lanes ? a->lanes : tuned_lanes(m, a->B, 0, &red, even);
   const size_t B = a->B;
   RolloutParams P{};
   P.model = m->dev; P.L = m->L; P.B = a->B; P.NI = a->NI; P.max_steps = a->max_steps; P.K = a->K > 0 ? a->K : 1;
@@ -692,7 +715,7 @@ dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, b
 }
 
 // ------------------------------------------------------------------ autotuner
-int tuned_lanes(dmx_model* m, int B, int grad, int* red) {
+int tuned_lanes(dmx_model* m, int B, int grad, int* red, bool even) {
   std::lock_guard<std::mutex> lk(m->mu);
   auto it = m->tuned.find({B, grad});
   if (it != m->tuned.end()) {
@@ -700,7 +723,7 @@ int tuned_lanes(dmx_model* m, int B, int grad, int* red) {
     return it->second;
   }
   if (red) *red = reduction_lanes(m, B);
-  return default_lanes(m, B);
+  return default_lanes(m, B, even);
 }
 
 // The lane count that, named in a call, gives the bits of a call that names

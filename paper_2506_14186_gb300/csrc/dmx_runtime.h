@@ -25,6 +25,7 @@ struct dmx_model {
   dmx::Layout Lc;                             // workspace of the CFD right-hand side F~ (rows: rcap_c)
   int device = 0, nsm = 0, smem_max = 0, rcap = 0, rcap_c = 0;
   int kind = 0;                               // model type of its kernels (dmx::MODEL_*)
+  int warps = 64;                             // rollout warps that an SM's registers hold (where shared memory holds more)
   double invw[dmx::MAXB];
   std::mutex mu;
   std::map<std::pair<int, int>, int> tuned;   // (B, kind) -> lanes per environment
@@ -61,7 +62,7 @@ inline const dmx::Layout& layout_for(const dmx_model* m, int cfd) { return cfd ?
 // right-hand-side layout, default_lanes for a rollout.
 int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin);
 int layout_lanes(const dmx_model* m, const dmx::Layout& L, int B, int warps);
-int default_lanes(const dmx_model* m, int B);
+int default_lanes(const dmx_model* m, int B, bool even = false);
 // Lanes whose summation order the error norm follows when the caller names no
 // lane count: the fewest that give every SM sub-partition a warp.  Kept apart
 // from the lanes a call runs on, so that these can follow the hardware while
@@ -69,7 +70,7 @@ int default_lanes(const dmx_model* m, int B);
 int reduction_lanes(const dmx_model* m, int B);
 // The recorded lane count of (model, B, grad), else default_lanes; *red (if
 // not null) receives the matching summation order.
-int tuned_lanes(dmx_model* m, int B, int grad, int* red);
+int tuned_lanes(dmx_model* m, int B, int grad, int* red, bool even = false);
 // dmx_rollout; records = false keeps a tape to the checkpoints (a server's
 // requests, whose memory is budgeted).
 dmx_status rollout_call(dmx_model* m, const dmx_rollout_args* a, void* stream, bool records);

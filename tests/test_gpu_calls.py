@@ -58,6 +58,18 @@ def test_the_lanes_a_model_names_give_the_same_bits(dmx, name, B, T, recorded):
         assert torch.equal(a[k], b[k]), k
 
 
+# fixed steps: batches a little over the warps that an SM's registers hold
+@pytest.mark.parametrize("name,B", [("billiard", 2000), ("billiard", 4096), ("capsules", 1900), ("chain_cube", 1400)])
+def test_lanes_of_fixed_step_rollouts_keep_the_results(dmx, name, B):
+    import torch
+    model = dmx.Model(W.SCENES[name]())
+    inp = _inputs(name, B, 0.02)
+    a = _call(dmx, model, inp, method="euler")
+    b = _call(dmx, model, inp, method="euler", lanes=32)
+    for k in ("xT", "nsteps", "status"):
+        assert torch.equal(a[k], b[k]), k
+
+
 # ------------------------------------------------------------------ step records: memory
 _MEMORY = r'''
 import ctypes, gc, re, sys
