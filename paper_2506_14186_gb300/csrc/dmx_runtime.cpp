@@ -536,7 +536,15 @@ dmx_status run_rollout(dmx_model* m, const RolloutParams& P0, int form, int G, c
 // Device memory that an allocation here can have: what the device reports as
 // free and what the stream-ordered pool holds unused (kept for the next call,
 // so the same call gets the same shares whatever ran before it).
+// The queries are no part of a stream capture that is going on in this or another
+// thread, and must not end it.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 static size_t free_memory(const dmx_model* m) {
+  RelaxedCapture relaxed;
   size_t free_b = 0, total_b = 0;
   if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
   cudaMemPool_t pool;

@@ -220,3 +220,29 @@ def test_cfd_stages_over_uneven_step_counts(dmx, B):
     assert torch.isfinite(b).all() and float((a - b).abs().max()) <= 1e-9 * float(b.abs().max())
     if B > 1:
         assert torch.equal(a[:, 1::5], bar[:, 1::5])
+
+
+@pytest.mark.parametrize("call", ["grad", "grad_cfd", "params", "params_cfd"])
+def test_gradients_can_be_captured(dmx, call):
+    """The gradient of a tape, captured in a graph after a first call, has the bits of
+    the call."""
+    import torch
+    B = 24
+    model, inp = dmx.Model(W.toss_scene()), W.INPUTS["toss"](B, T=0.05)
+    inp["x0"][:, 2] = np.where(np.arange(B) % 2 == 1, 0.055, 3.0)
+    out = _call(dmx, model, inp, tape=True, K=8)
+    bar = _dev(np.random.default_rng(4).normal(size=(model.nx, B)))
+    fn = dmx.rollout_grad_params if call.startswith("params") else dmx.rollout_grad
+
+    def grads():
+        return [x for x in fn(out["tape"], bar, cfd=call.endswith("cfd")) if x is not None]
+
+    want = grads()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        got = grads()
+    g.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
