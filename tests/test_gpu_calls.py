@@ -246,3 +246,27 @@ def test_gradients_can_be_captured(dmx, call):
     torch.cuda.synchronize()
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+def test_parameter_gradients_keep_the_order_of_their_stream(dmx):
+    """The two kernels of a parameter gradient (environments with and without
+    contact) start after what is queued on the call's stream, and what follows on
+    it sees both results."""
+    import torch
+    B = 24
+    model, inp = dmx.Model(W.toss_scene()), W.INPUTS["toss"](B, T=0.05)
+    inp["x0"][:, 2] = np.where(np.arange(B) % 2 == 1, 0.055, 3.0)
+    out = _call(dmx, model, inp, tape=True, K=8)
+    bar = _dev(np.random.default_rng(4).normal(size=(model.nx, B)))
+    want = [x for x in dmx.rollout_grad_params(out["tape"], bar) if x is not None]
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    late = torch.zeros_like(bar)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(20_000_000)              # 10 ms before the cotangents are there
+        late.copy_(bar)
+        got = [2.0 * x for x in dmx.rollout_grad_params(out["tape"], late) if x is not None]
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert torch.equal(a, 2.0 * b)
