@@ -126,7 +126,9 @@ static size_t request_bytes(const dmx_request& r) {
     d += (size_t)(r.max_steps / K + 2) * (nx + 1) * B + (size_t)r.max_steps * B + z.n_u + B;   // tape
   }
   size_t extra = 0;
-  if (r.grad) extra = adjoint_scratch_bound(r.model, r.B, r.K > 0 ? r.K : 32, r.cfd);   // segment buffers, snapshots
+  if (r.grad)
+    extra = adjoint_scratch_bound(r.model, r.B, r.K > 0 ? r.K : 32, r.cfd)   // segment buffers, snapshots
+            + 2 * sizeof(int32_t) * B;                                       // the tape's step counts and contact flags
   return stage_layout(r).bytes + d * sizeof(double) + extra + 4096;
 }
 

@@ -270,3 +270,35 @@ def test_parameter_gradients_keep_the_order_of_their_stream(dmx):
     torch.cuda.synchronize()
     for a, b in zip(got, want):
         assert torch.equal(a, 2.0 * b)
+
+
+def test_a_served_gradient_stays_within_its_admitted_memory(dmx):
+    """What a gradient request takes from the device's pool while it runs is at most
+    what admission counts for it (a batch whose adjoint groups are all resident,
+    so that the count has no slack but its constant)."""
+    _run(r'''
+def high(reset=False):                          # most bytes in use at a time since the last reset (attribute 8)
+    torch.cuda.synchronize()
+    v = ctypes.c_uint64()
+    if reset: assert rt.cudaMemPoolSetAttribute(pool, 8, ctypes.byref(v)) == 0
+    assert rt.cudaMemPoolGetAttribute(pool, 8, ctypes.byref(v)) == 0
+    return v.value
+
+B = 8 * torch.cuda.get_device_properties(0).multi_processor_count
+model, inp = dmx.Model(W.box_scene()), W.box_push_inputs(B, T=0.002)
+req = dict(x0=np.ascontiguousarray(inp["x0"].T), T=inp["T"], grad=True, xT_bar=np.ones((13, B)), K=8, max_steps=200)
+small = dmx.Server(device_bytes=1000, max_inflight=1, nstreams=1)
+try:
+    small.submit(model, **req)
+    raise SystemExit("admitted")
+except dmx.DmxError as e:
+    counted = int(re.search(r"needs (\d+) device bytes", str(e)).group(1))
+small.close()
+srv = dmx.Server(device_bytes=8 << 30, max_inflight=1, nstreams=1)
+base = used()
+high(reset=True)
+srv.wait(srv.submit(model, **req))
+taken = high() - base
+srv.close()
+assert counted - (1 << 20) < taken <= counted, (taken, counted)
+''')
