@@ -302,3 +302,24 @@ taken = high() - base
 srv.close()
 assert counted - (1 << 20) < taken <= counted, (taken, counted)
 ''')
+
+
+@pytest.mark.parametrize("name", ["box", "toss", "chain_cube", "quadruped", "capsules"])
+def test_cfd_parameter_gradients_match_the_oracle(dmx, orc, name):
+    """Parameter gradients with contacts from distance (reverse-mode kernel: friction
+    rows, capsule-box and segment pairs, box sides) against the oracle's along the
+    GPU's steps, within 1e-6: moving x0 by 1e-15 moves the oracle's own by 6e-9 at
+    most on these inputs."""
+    from tests.test_gpu_adjoint import CFD_OPT, assert_grad, gpu_grad_params, param_inputs
+    sc = W.box_scene(solref=(0.005, 1.0), **CFD_OPT) if name == "toss" else W.SCENES[name](**CFD_OPT)
+    inp = (W.INPUTS["toss"](6, T=0.2) if name == "toss" else W.INPUTS[name](8) if name == "capsules" else
+           param_inputs(name))
+    inp.setdefault("max_steps", 20000)
+    m = dmx.Model(sc)
+    xT_bar = np.random.default_rng(17).normal(size=(len(inp["x0"]), m.nx))
+    g = gpu_grad_params(dmx, m, inp, xT_bar, cfd=True)
+    assert np.all(g["status"] == 0)
+    o = orc.OracleModel(sc).batch_replay_grad(inp["x0"], inp["T"], g["hlog"], g["n"], xT_bar, ctrl=inp["ctrl"],
+                                              NI=inp["NI"], cfd=True, params=True)
+    assert_grad(g, o, "p_bar")
+    assert_grad(g, o)
