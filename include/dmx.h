@@ -164,8 +164,7 @@ typedef struct {
   int32_t* status;            /* out [B] DMX_ENV_* codes, or NULL */
   dmx_tape** tape;            /* out: tape for dmx_rollout_grad (checkpoints every K accepted
                                  steps + accepted step sizes; with the reverse adjoint selected,
-                                 also the steps' stage snapshots, within an eighth of the free
-                                 device memory and 24 GiB), or NULL for forward only */
+                                 also step records, see dmx_tape_free), or NULL for forward only */
   int32_t method;             /* DMX_METHOD_*: integration scheme (0 = adaptive Dormand-Prince 5(4)) */
 } dmx_rollout_args;
 
@@ -202,8 +201,8 @@ dmx_status dmx_model_params(const dmx_model* m, int32_t* np, double* values);
  * environment shares the model).  Computed by the kernel that dmx_set_adjoint
  * selects: the reverse-mode one collects the parameters' cotangents of every
  * right-hand side beside the states' (8, 16 or 32 lanes; without cfd it leaves
- * the environments that met no contact to the tangent one), the tangent one
- * runs a derivative direction per parameter.  A model that does not fit the
+ * the environments that met no contact to the tangent one, beside it), the tangent
+ * one runs a derivative direction per parameter.  A model that does not fit the
  * tangent kernel is refused.  Device pointers, ordered on `stream`. */
 dmx_status dmx_rollout_grad_params(dmx_model* m, dmx_tape* tape, int32_t cfd, const double* xT_bar,
                                    const double* xb_bar, double* x0_bar, double* ctrl_bar, double* p_bar,
@@ -261,6 +260,16 @@ dmx_status dmx_rollout_grad_otd(dmx_model* m, const dmx_otd_args* a, void* strea
  *     step, column by column); kept as an independent check.
  * DMX_ERR_INVALID for another mode. */
 dmx_status dmx_set_adjoint(dmx_model* m, int32_t mode);
+/* Frees a tape, ordered after the work queued on the stream of its rollout.
+ * While DMX_ADJ_REVERSE is selected a rollout's tape also keeps step records: the
+ * stage snapshots of the first 512 accepted steps of every environment, or as
+ * many whole segments of K steps as an eighth of the free device memory and
+ * 24 GiB hold; all live tapes of a device together keep 48 GiB at most, further
+ * ones (and batches of which not one segment fits) none.  They belong to the tape
+ * until it is freed; a rollout made while another adjoint is selected keeps none,
+ * and its tape can be differentiated with any.  Freed memory stays cached for the
+ * next call until the device's last model is destroyed; the driver hands it to
+ * other allocations of the process that need it. */
 void dmx_tape_free(dmx_tape* t);
 /* Copies a tape into caller DEVICE buffers (any may be NULL), on `stream`:
  * hlog [max_steps][B] accepted step sizes (entries past nsteps[e] undefined),
@@ -365,8 +374,11 @@ dmx_status dmx_rollout_static(dmx_model* m, const dmx_rollout_args* a, void* str
  * integration): q [nq][B], v [nv][B], u [nu][B] (NULL iff nu == 0) device
  * arrays; cfd = 1 evaluates the CFD right-hand side F~ of Sec. 4.  Writes
  * a [nv][B] and info [4][B] (DMX_ENV_* status, constraint rows, active rows,
- * 0).  The constraint solve starts from an empty active set.  lanes as in
- * dmx_rollout_args (0 = default). */
+ * 0).  The constraint solve starts from an empty active set.  lanes: 1, 2, 4, 8,
+ * 16, 32, or 0 = by what an SM holds; with 0 a batch is refused
+ * (DMX_ERR_INVALID) whose rollout lanes (dmx_autotune) leave no room for the rows
+ * of F~, which models with more than 64 row ids reach in large batches: name the
+ * lanes there. */
 dmx_status dmx_eval_rhs(dmx_model* m, int32_t B, const double* q, const double* v, const double* u, int32_t cfd,
                         int32_t lanes, double* a, int32_t* info, void* stream);
 

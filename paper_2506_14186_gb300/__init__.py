@@ -212,7 +212,8 @@ class Model:
 
     def set_adjoint(self, mode):
         """Adjoint kernel of rollout_grad: "reverse" (default; stage snapshots in
-        device memory when they fit), "recompute" (reverse mode evaluating each
+        device memory when they fit, and step records in the tapes of rollouts made
+        while it is selected), "recompute" (reverse mode evaluating each
         stage's right-hand side again) or "tangent" (forward-mode columns)."""
         _check(lib().dmx_set_adjoint(self.h, ADJOINT_MODES[mode]))
 

@@ -24,9 +24,10 @@
 // (K steps x (S - 1) stages per group) and the reverse sweep restores it instead of
 // evaluating the right-hand side a second time: device memory traded for
 // FP64 work.  The final active set of a stage does not depend on the
-// warm start of its Newton search, so the restored workspace equals a
-// recomputed one.  Segments whose steps the forward pass kept (dmx_record.h)
-// are not recomputed at all: rows and snapshots are read from the records.
+// warm start of its Newton search but where a row lies at the edge of the set to
+// rounding, so the restored workspace equals a recomputed one up to the last bits
+// there.  Segments whose steps the forward pass kept (dmx_record.h) are not
+// recomputed at all: rows and snapshots are read from the records.
 //
 // Bound by the chain of a stage (restore, VJP, stage cotangents): about 160 k
 // cycles for the arm on 32 lanes, with one to four warps on a sub-partition.

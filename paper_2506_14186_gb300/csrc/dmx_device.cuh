@@ -27,10 +27,12 @@
 // tasks of one matrix or vector component (branches inside a task cost the sum
 // of their sides), tree recursions run along chains without meeting the other
 // lanes, and indices come packed or from tables.  Every split keeps the
-// operations of each result and their order, so that results do not depend on
-// the lane count.  The Newton search starts from the active set of
-// the previous right-hand side of the same environment (the minimiser is
-// unique, so the start only changes the number of iterations).
+// operations of each result and their order: for a given final active set the
+// results do not depend on the lane count.  (The line search, which only picks
+// the next set to try, sums its slopes in lane order.)  The Newton search starts
+// from the active set of the previous right-hand side of the same environment:
+// the minimiser is unique, so the start changes the number of iterations, and the
+// last bits where a row lies at the edge of the active set to rounding.
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>

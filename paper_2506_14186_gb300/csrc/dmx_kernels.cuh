@@ -213,8 +213,8 @@ __device__ Ws group_workspace(const RolloutParams& P, const Layout* L) {
 // Bound by the FP64 unit and, below one warp per sub-partition, by the chain of
 // a right-hand side (33 k cycles for a box on 32 lanes, 95 k for a quadruped);
 // no memory traffic but the state.  Splitting the right-hand side into equal
-// one-component tasks, lanes by what an SM holds and the model types took 4096
-// box pushes (0.2 s) from 216 to 135 ms, 20001 tosses from 901 to 154 ms, 3000
+// one-component tasks, lanes by what an SM holds and the model types took (device
+// times) 4096 box pushes (0.2 s) from 216 to 135 ms, 20001 tosses from 901 to 154 ms, 3000
 // quadrupeds from 833 to 274 ms and 1000 arms from 50.5 to 37.7 ms.
 template <int G, class MD>
 __global__ void __launch_bounds__(32, 1) k_rollout_persistent(const __grid_constant__ RolloutParams P) {
