@@ -262,7 +262,7 @@ dmx_status dmx_rollout_grad_otd(dmx_model* m, const dmx_otd_args* a, void* strea
 dmx_status dmx_set_adjoint(dmx_model* m, int32_t mode);
 /* Frees a tape, ordered after the work queued on the stream of its rollout.
  * While DMX_ADJ_REVERSE is selected a rollout's tape also keeps step records: the
- * stage snapshots of the first 512 accepted steps of every environment, or as
+ * stage snapshots of the first 1024 accepted steps of every environment, or as
  * many whole segments of K steps as an eighth of the free device memory and
  * 24 GiB hold; all live tapes of a device together keep 48 GiB at most, further
  * ones (and batches of which not one segment fits) none.  They belong to the tape

@@ -583,11 +583,13 @@ static dmx_status make_tape(dmx_model* m, const dmx_rollout_args* a, const doubl
   return DMX_OK;
 }
 
-// Step records for a tape: the first 512 steps of every environment (or as
-// many as it may take), within an eighth of the free device memory and 24 GiB;
-// whole segments where that is less, and none when not even one fits (longer
-// segments than 64 steps serve short rollouts only, and count as 64), or the
-// allocation fails.  With them the adjoint has no segment to recompute (45 % of
+// Step records for a tape: the first 1024 steps of every environment (or as
+// many as it may take; the longest environments set the adjoint's time, and take
+// twice the steps of the mean: 256 arms over 2 s, 444 to 751 steps, 402 ms with
+// all of them kept, 472 with 512), within an eighth of the free device memory and
+// 24 GiB; whole segments where that is less, and none when not even one fits
+// (longer segments than 64 steps serve short rollouts only, and count as 64), or
+// the allocation fails.  With them the adjoint has no segment to recompute (45 % of
 // its time), for the price of the writes (118 KB an arm's step): forward and
 // adjoint of 2048 arms 249 -> 171 ms, of 2048 tosses 167 -> 133.
 constexpr size_t kRecMaxBytes = size_t(24) << 30;
@@ -614,7 +616,7 @@ static void add_records(dmx_model* m, dmx_tape* t, cudaStream_t st) {
   if (m->device < 0 || m->device >= kMaxDevices) return;
   const size_t live = g_rec_live[m->device];
   const size_t room = std::min({free_memory(m) / 8, kRecMaxBytes, kRecLiveBytes - std::min(live, kRecLiveBytes)});
-  const int want = std::min(t->max_steps, 512);
+  const int want = std::min(t->max_steps, 1024);
   r.steps = (int)std::min((size_t)want, room / step);
   if (r.steps < want && t->K <= 64) r.steps -= r.steps % t->K;
   if (r.steps < std::min({t->K, 64, want})) return;
