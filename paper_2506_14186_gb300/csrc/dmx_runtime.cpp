@@ -330,12 +330,8 @@ extern "C" dmx_status dmx_create_model(const dmx_model_desc* desc, dmx_model** o
   }
   for (int b = 0; b < m->host.nbody; ++b) m->invw[b] = invw[b];
   CK(cudaMemcpy(m->dev, &m->host, sizeof(DevModel), cudaMemcpyHostToDevice));
-  int threads;
-  size_t smem;
-  if (launch_config(m, 32, &threads, &smem)) {
-    const int warps = persistent_occupancy(32, m->kind, threads, smem);
-    if (warps > 0 && warps < (int)(prop.sharedMemPerMultiprocessor / (smem + prop.reservedSharedMemPerBlock))) m->warps = warps;
-  }
+  m->smem_sm = (int)prop.sharedMemPerMultiprocessor;
+  m->smem_reserved = (int)prop.reservedSharedMemPerBlock;
   count_models(m->device, 1);
   *out = m;
   return DMX_OK;
@@ -417,6 +413,18 @@ int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
   while (G > gmin && e * G > warps * 32) G >>= 1;
   return G;
 }
+// Warps of the rollout kernel that an SM's registers hold, 64 where its shared
+// memory is the tighter limit.
+static int register_warps(const dmx_model* m) {
+  int w = m->warps, threads;
+  size_t smem;
+  if (w == 0) {                        // first asked for: an occupancy query loads the kernel
+    w = launch_config(m, 32, &threads, &smem) ? persistent_occupancy(32, m->kind, threads, smem) : 0;
+    if (w <= 0 || w >= m->smem_sm / ((int)smem + m->smem_reserved)) w = 64;   // shared memory is the tighter limit
+    m->warps = w;
+  }
+  return w;
+}
 // Rollouts: two warps per sub-partition fill the FP64 unit with a single
 // body's short phases (8 to 36 tasks); the phases of larger models (100 tasks)
 // use 32 lanes, and four warps still gain (arms, 1000 for 0.1 s: 24 ms with 32
@@ -431,8 +439,9 @@ int fill_lanes(const dmx_model* m, int B, size_t per, int warps, int gmin) {
 int default_lanes(const dmx_model* m, int B, bool even) {
   int G = layout_lanes(m, m->L, B, m->host.nv > 8 ? 16 : 8);
   if (!even) return G;
+  const int warps = register_warps(m);
   const int share = (B + m->nsm - 1) / m->nsm, fit = sm_environments(m, (size_t)m->L.nd * 8 + (size_t)m->L.ni * 4);
-  auto rounds = [&](int g) { const int e = std::max(1, std::min(fit, m->warps * (32 / g))); return (share + e - 1) / e; };
+  auto rounds = [&](int g) { const int e = std::max(1, std::min(fit, warps * (32 / g))); return (share + e - 1) / e; };
   int t; size_t s;
   while (G > 4 && rounds(G / 2) < rounds(G) && launch_config(m, G / 2, &t, &s)) G >>= 1;
   return G;

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <string>
@@ -25,7 +26,8 @@ struct dmx_model {
   dmx::Layout Lc;                             // workspace of the CFD right-hand side F~ (rows: rcap_c)
   int device = 0, nsm = 0, smem_max = 0, rcap = 0, rcap_c = 0;
   int kind = 0;                               // model type of its kernels (dmx::MODEL_*)
-  int warps = 64;                             // rollout warps that an SM's registers hold (where shared memory holds more)
+  int smem_sm = 0, smem_reserved = 0;         // shared memory of an SM, and what it keeps of it per block
+  mutable std::atomic<int> warps{0};          // rollout warps that an SM's registers hold (default_lanes), 0: not asked for yet
   double invw[dmx::MAXB];
   std::mutex mu;
   std::map<std::pair<int, int>, int> tuned;   // (B, kind) -> lanes per environment
