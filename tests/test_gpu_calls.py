@@ -323,3 +323,27 @@ def test_cfd_parameter_gradients_match_the_oracle(dmx, orc, name):
                                               NI=inp["NI"], cfd=True, params=True)
     assert_grad(g, o, "p_bar")
     assert_grad(g, o)
+
+
+@pytest.mark.parametrize("cfd", [False, True])
+def test_records_for_the_first_steps_only(dmx, cfd):
+    """Segments beyond the records are recomputed: the gradient that recomputing every
+    segment gives (the same right-hand sides along the same steps: 1e-12)."""
+    _run(r'''
+cfd = %r
+model, inp = dmx.Model(W.box_scene(**(W.CFD_OPTIONS if cfd else {}))), W.box_push_inputs(64, seed=5)
+bar = dev(np.random.default_rng(2).normal(size=(13, 64)))
+filler = torch.empty(free() - 4 * GiB, dtype=torch.uint8, device="cuda")
+got = {}
+for mode in ("reverse", "recompute"):
+    model.set_adjoint(mode)
+    t = tape(model, inp, 0.1, K=16, rtol=1e-9, atol=1e-11, h0=1e-3)
+    n, records = t.read()[1], used()
+    got[mode] = dmx.rollout_grad(t, bar, cfd=cfd)[0]
+    del t; gc.collect()
+    assert (records > 128 << 20) == (mode == "reverse"), records
+assert int(n.max()) > 288, int(n.max())         # half a GiB: at most 17 segments of 64 boxes' steps (31 KB each)
+a, b = got["reverse"], got["recompute"]
+assert torch.isfinite(b).all()
+assert float(((a - b).abs().amax(0) / b.abs().amax(0)).max()) < 1e-12
+''' % cfd)
